@@ -79,13 +79,18 @@ struct DevBuf {
     template <typename T> T *as() const { return (T *)p; }
 };
 
+// Words of StreamScratch::words: u's extremes [2], the kept lists' lengths
+// (int64 [2]), the hops' work queues ([2] a hop).
+constexpr int CW_EXT = 0, CW_KEPT = 2, CW_QUEUE = 6, CW_COUNT = CW_QUEUE + 2 * AKASHIC_MAX_HOPS;
+
 struct StreamScratch {
-    DevBuf qp, shift, u, sa, sb, zpart, partial, cand, counters;
+    DevBuf qp, shift, u, sa, sb, zpart, partial, cand;
+    DevBuf words;                // a call's counters (CallWords), zeroed by its first kernel
     DevBuf samp, ext_s, zsamp;   // retrieval without hops: the score's row sample
     DevBuf qns, ns_s, dead_s;    // scope: per query column, per sample row
     DevBuf rmax_u, rmin_u;       // u's row maxima / minima over the real queries
-    DevBuf ub, lb, ext, pfloor;  // the last hop's row bounds, extremes, floor
-    DevBuf skip_split, skip_slot, kept_rows, kept_count, kept_segs, kflag, kpos, ktmp;
+    DevBuf pfloor;               // the last hop's floor and what it keeps
+    DevBuf skip_split, kept_rows, kept_segs, keep_chain;
     DevBuf reach_keep, reach_part, reach_plan;   // flags + bad + done, partials, plan
     DevBuf nsf;                  // scoped last hop: tags, their floors, their count
     // every candidate's combined coefficients (bf16 hi, lo), and their key
@@ -1241,26 +1246,19 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
         if (eff_hops >= 1) AK_TRY(ensure_spare(sc->sa, (size_t)n * bp * 4));
         if (eff_hops >= 2) AK_TRY(ensure_spare(sc->sb, (size_t)n * bp * 4));
         if (eff_hops >= 1 && m->n_segs > 0) AK_TRY(ensure_spare(sc->partial, (size_t)m->n_segs * bp * 4));
-        if (eff_hops >= 1) AK_TRY(sc->counters.ensure(64));
+        if (eff_hops >= 1) AK_TRY(sc->words.ensure(CW_COUNT * 4));
         // row bounds for the last hop (fused filter only)
         const bool prune = eff_hops >= 1 && m->fuse_filter && m->hop_prune;
         if (prune) {
             AK_TRY(ensure_spare(sc->rmax_u, (size_t)n * 4));
             AK_TRY(ensure_spare(sc->rmin_u, (size_t)n * 4));
-            AK_TRY(ensure_spare(sc->ub, (size_t)n * 4));
-            AK_TRY(ensure_spare(sc->lb, (size_t)n * 4));
-            AK_TRY(sc->ext.ensure(16));
             AK_TRY(ensure_spare(sc->skip_split, (size_t)(m->n_split + 1) * 4));
             AK_TRY(ensure_spare(sc->kept_rows, (size_t)n * 4));
-            AK_TRY(sc->kept_count.ensure(16));
             AK_TRY(ensure_spare(sc->kept_segs, (size_t)(m->n_segs + 1) * 4));
-            const int64_t nk = n > m->n_segs ? n : m->n_segs;
-            AK_TRY(ensure_spare(sc->kflag, (size_t)(nk + 1) * 8));
-            AK_TRY(ensure_spare(sc->kpos, (size_t)(nk + 1) * 8));
-            AK_TRY(ensure_spare(sc->ktmp, scan_tmp_bytes(nk + 1) + 4096));
-            AK_TRY(ensure_spare(sc->skip_slot, (size_t)(m->n_segs + 1) * 4));
             AK_TRY(sc->pfloor.ensure(16));
         }
+        unsigned int *ext = eff_hops >= 1 ? sc->words.as<unsigned int>() + CW_EXT : nullptr;
+        int64_t *kept_count = (int64_t *)(sc->words.as<int32_t>() + CW_KEPT);
         const uint16_t *qb = q + (int64_t)off * m->dim;
         // namespace scope of this batch's queries (padding columns get -1)
         NsScope ns{};
@@ -1294,17 +1292,18 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                                 sc->zpart.as<float>(), m->status.as<int>(), st, launches, &zrows,
                                 ns.dead, prune ? sc->rmax_u.as<float>() : nullptr,
                                 prune ? sc->rmin_u.as<float>() : nullptr, b,
-                                prune ? sc->ext.as<unsigned int>() : nullptr);
+                                prune ? ext : nullptr);
         };
         {
             PhaseScope ph(m, AKASHIC_PHASE_SCORE, st);
             // with the row bounds (never with the dense fused filter) the
-            // score GEMM's epilogue reduces u's row extremes into sc->ext,
-            // zeroed here
+            // score GEMM's epilogue reduces u's row extremes into the call's
+            // words, which are zeroed here
             CUDA_TRY(launch_prep_queries(qb, b, bp, m->dim, m->tau, m->max_norm.as<float>(),
                                          sc->qp.as<uint16_t>(), sc->shift.as<float>(),
                                          m->status.as<int>(), st,
-                                         prune ? sc->ext.as<unsigned int>() : nullptr));
+                                         sc->words.as<unsigned int>(),
+                                         eff_hops >= 1 ? CW_COUNT : 0));
             ph.launches += 1;
             if (reach_try)
                 CUDA_TRY(launch_score_split(m->emb.as<uint16_t>(), n, m->dim,
@@ -1312,7 +1311,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                                             m->tau, u_hi, u_lo, sc->zpart.as<float>(),
                                             m->status.as<int>(), st, &ph.launches, &zrows, ns.dead,
                                             sc->rmax_u.as<float>(), sc->rmin_u.as<float>(), b,
-                                            sc->ext.as<unsigned int>()));
+                                            ext));
             else if (!dense_fused)
                 CUDA_TRY(score_fp32(&ph.launches));
         }
@@ -1383,28 +1382,14 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
             rc.in_src = hp.in_src;
             rc.in_w = hp.in_w;
             rc.alpha = alpha;
-            // scalar row bounds of the last hop's output, from u's row extremes
-            // (the two-hop reach path evaluates them only where it needs them
-            // and writes the arrays only when the hops run after all)
-            const float *row_ub = nullptr, *row_lb = nullptr;
-            auto row_bounds = [&]() -> akashic_status_t {
-                PhaseScope ph(m, AKASHIC_PHASE_BOUND, st);
-                CUDA_TRY(launch_final_bounds(sc->rmax_u.as<float>(), sc->rmin_u.as<float>(),
-                                             m->mass_up.as<float>(), m->mass_dn.as<float>(), n,
-                                             eff_hops, alpha, sc->ext.as<unsigned int>(),
-                                             sc->ub.as<float>(), sc->lb.as<float>(), st,
-                                             &ph.launches, true));
-                row_ub = sc->ub.as<float>();
-                row_lb = sc->lb.as<float>();
-                return AKASHIC_OK;
-            };
             if (prune) {
-                {
-                    std::lock_guard<std::mutex> lk(m->table_mu);
-                    AK_TRY(ensure_mass(m, hp, eff_hops, st));
-                }
-                if (!reach_try) AK_TRY(row_bounds());
+                std::lock_guard<std::mutex> lk(m->table_mu);
+                AK_TRY(ensure_mass(m, hp, eff_hops, st));
             }
+            // the row bounds of the last hop's output
+            const RowBounds rb{sc->rmax_u.as<float>(), sc->rmin_u.as<float>(),
+                               m->mass_up.as<float>(), m->mass_dn.as<float>(), ext, n, eff_hops,
+                               alpha};
             // Two hops without running them: when every row whose upper bound
             // reaches the floor (here the k-th largest lower bound) is a
             // candidate with reach coefficients, their final scores come from
@@ -1427,7 +1412,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                     rf.l0 = sc->rmin_u.as<float>();
                     rf.mup = m->mass_up.as<float>();
                     rf.mdn = m->mass_dn.as<float>();
-                    rf.ext = sc->ext.as<unsigned int>();
+                    rf.ext = ext;
                     rf.n = n;
                     rf.H = eff_hops;
                     rf.alpha = alpha;
@@ -1483,27 +1468,23 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                     reach_done = true;
                 } else {
                     // the hops run: they read u in fp32 (the same scores again)
-                    // and need every row's bounds
-                    {
-                        PhaseScope ph(m, AKASHIC_PHASE_SCORE, st);
-                        CUDA_TRY(score_fp32(&ph.launches));
-                    }
-                    AK_TRY(row_bounds());
+                    PhaseScope ph(m, AKASHIC_PHASE_SCORE, st);
+                    CUDA_TRY(score_fp32(&ph.launches));
                 }
             }
             for (int h = 0; h < eff_hops && !reach_done; ++h) {
                 float *out = bufs[h & 1];
                 const bool last = m->fuse_filter && h == eff_hops - 1;
                 if (last) {
-                    // Top-k filter fused into the last hop.  With w >= 0 and
-                    // alpha >= 0 every hop only adds to a score, and in fp32
-                    // too (same summation order, monotone rounding), so the
-                    // k-th largest key of s^(H-1) over the row sample is a
-                    // safe bound for s^(H).
+                    // Top-k filter fused into the last hop, its bound from the
+                    // hop's own values on the row sample.
                     {
                         PhaseScope ps(m, AKASHIC_PHASE_SELECT, st);
-                        CUDA_TRY(launch_sample_bound(sp, fin, b, m->ext_of.as<int32_t>(), ws, st,
-                                                     &ps.launches, 0u, ns));
+                        CUDA_TRY(launch_hop_sample(hp, sp, sc->u.as<float>(), fin, alpha, ns,
+                                                   (uint32_t *)(ws + sp.off_tr), st,
+                                                   &ps.launches));
+                        CUDA_TRY(launch_sample_bound(sp, nullptr, b, m->ext_of.as<int32_t>(), ws,
+                                                     st, &ps.launches, 0u, ns));
                     }
                     if (prune) {
                         PhaseScope ps(m, AKASHIC_PHASE_BOUND, st);
@@ -1511,10 +1492,13 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                         // scope to the k-th largest lower bound of the heaviest
                         // split rows (where the top scores lie)
                         const int64_t n_lb = m->n_split < 1024 ? m->n_split : 1024;
-                        CUDA_TRY(launch_prune_floor(ws + sp.off_bound, b, row_lb,
+                        const int64_t cw = keep_chain_words(hp);
+                        AK_TRY(ensure_spare(sc->keep_chain, (size_t)cw * 8));
+                        unsigned long long *chain = sc->keep_chain.as<unsigned long long>();
+                        CUDA_TRY(launch_prune_floor(ws + sp.off_bound, b, rb,
                                                     q_ns ? nullptr : hp.split_row,
                                                     hp.split_order, n_lb, k,
-                                                    sc->pfloor.as<float>(), st));
+                                                    sc->pfloor.as<float>(), chain, cw, st));
                         // with a scope, each namespace of the batch gets its own
                         // floor (its rows can only be selected by its queries)
                         NsFloors nf{};
@@ -1524,35 +1508,29 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                             float *tag_floor = (float *)(tags + PF_TAGS);
                             int *n_tags = (int *)(tag_floor + PF_TAGS);
                             CUDA_TRY(launch_ns_floors(ws + sp.off_bound, sc->qns.as<int32_t>(), b,
-                                                      row_lb, m->ns_row.as<int32_t>(),
-                                                      hp.split_row, hp.split_order, m->n_split, k,
-                                                      tags, n_tags, tag_floor, st));
+                                                      rb, m->ns_row.as<int32_t>(), hp.split_row,
+                                                      hp.split_order, m->n_split, k, tags, n_tags,
+                                                      tag_floor, st));
                             nf = NsFloors{m->ns_row.as<int32_t>(), tags, n_tags, tag_floor};
                             ps.launches += m->n_split > 0 ? 2 : 1;
                         }
-                        KeptScratch ks{sc->kflag.as<int64_t>(), sc->kpos.as<int64_t>(),
-                                       sc->ktmp.p, sc->ktmp.cap};
-                        CUDA_TRY(launch_split_flags(hp, row_ub, sc->pfloor.as<float>(),
-                                                    q_ns ? &nf : nullptr,
-                                                    sc->skip_split.as<int32_t>(),
-                                                    sc->skip_slot.as<int32_t>(),
-                                                    sc->kept_rows.as<int32_t>(),
-                                                    sc->kept_count.as<int64_t>(),
-                                                    sc->kept_segs.as<int32_t>(), ks, st,
-                                                    &ps.launches));
+                        CUDA_TRY(launch_keep(hp, rb, sc->pfloor.as<float>(), q_ns ? &nf : nullptr,
+                                             sc->skip_split.as<int32_t>(),
+                                             sc->kept_rows.as<int32_t>(),
+                                             sc->kept_segs.as<int32_t>(), kept_count, chain,
+                                             m->status.as<int>(), st, &ps.launches));
                         ps.launches += 1;
                     }
                 }
                 const HopFilter flt{m->ext_of.as<int32_t>(), ws + sp.off_bound,
                                     (unsigned int *)(ws + sp.off_cnt), ws + sp.off_buf, sp.cap,
                                     ns};
-                const HopBound hb{row_ub, sc->pfloor.as<float>(), sc->skip_split.as<int32_t>(),
-                                  sc->skip_slot.as<int32_t>(), sc->kept_rows.as<int32_t>(),
-                                  sc->kept_count.as<int64_t>(), sc->kept_segs.as<int32_t>()};
+                const HopBound hb{sc->skip_split.as<int32_t>(), sc->kept_rows.as<int32_t>(),
+                                  kept_count, sc->kept_segs.as<int32_t>()};
                 PhaseScope ph(m, last ? AKASHIC_PHASE_LAST_HOP : AKASHIC_PHASE_PROPAGATE, st);
                 CUDA_TRY(launch_hop(hp, sc->u.as<float>(), fin, out, bp, alpha,
-                                    sc->partial.as<float>(), sc->counters.as<int>(),
-                                    last ? &flt : nullptr, st, &ph.launches,
+                                    sc->partial.as<float>(),
+                                    sc->words.as<int>() + CW_QUEUE + 2 * h, last ? &flt : nullptr, st, &ph.launches,
                                     (last && prune) ? &hb : nullptr));
                 if (last) {
                     rc.kind = 1;

@@ -189,10 +189,11 @@ cudaError_t launch_dots_keys_t(const uint16_t *emb, int64_t n, int64_t row_strid
 
 // Query preparation: pad q (b rows) to bp rows of zeros and compute
 // shift[c] = tau * |q_c| * max_norm (0 for padding); flags ERANGE.
-// ext_zero (or NULL): two words set to 0 (the row extremes' initial value).
+// zero (or NULL): n_zero <= 128 words set to 0 (the call's counters).
 cudaError_t launch_prep_queries(const uint16_t *q, int b, int bp, int dim, float tau,
                                 const float *max_norm, uint16_t *qp, float *shift, int *status,
-                                cudaStream_t st, unsigned int *ext_zero = nullptr);
+                                cudaStream_t st, unsigned int *zero = nullptr,
+                                int n_zero = 0);
 
 // Running maximum of row norms of emb[0..n) into *max_norm (monotone).
 cudaError_t launch_row_norm_max(const uint16_t *emb, int64_t n, int dim, float *max_norm,
@@ -485,27 +486,15 @@ struct HopFilter {
     int64_t cap;
     NsScope ns;                       // candidates only within the query's namespace
 };
-// Row bounds for the last hop, whose output only feeds the fused top-k
-// filter: row_ub[j] bounds every real query column's fp32 value of the
-// hop's output s_j from above (launch_row_bounds), `floor` is at most every
-// real query's k-th largest final value (launch_prune_floor); a row with
-// row_ub < floor appends nothing in any column and is skipped, so the
-// filter's output is unchanged.
+// What the last hop may leave out, given a floor that every real query's k-th
+// largest final value reaches (launch_prune_floor): rows whose upper bound
+// (RowBounds) stays below it append nothing in any column, so the filter's
+// output is unchanged without them (launch_keep).
 struct HopBound {
-    const float *row_ub;       // [n]
-    const float *floor;        // device scalar
-    const int32_t *split_skip; // [n_split_rows] split rows to skip (launch_split_flags)
-    const int32_t *slot_skip;  // [n_segs] their partial slots
+    const int32_t *split_skip; // [n_split_rows] 1: split row to skip
     const int32_t *kept_rows;  // [n] rows kept whole that reach the floor ...
     const int64_t *kept_count; // ... [0] their number, [1] that of kept_segs (device)
     const int32_t *kept_segs;  // [n_segs] segments of the unpruned split rows
-};
-// Scratch of the kept lists' compaction: flag / pos [max(n, n_segs) + 1]
-// int64, tmp of scan_tmp_bytes(max(n, n_segs)) bytes.
-struct KeptScratch {
-    int64_t *flag, *pos;
-    void *tmp;
-    size_t tmp_bytes;
 };
 // Graph-only mass vectors for the row bounds, levels t0..t1 (level 0, all
 // ones, already in place): mup[t] >= g (1 + eps) sum_i w_ij mup[t-1]_i and
@@ -521,8 +510,9 @@ struct KeptScratch {
 cudaError_t launch_mass_levels(const HopPlan &p, int t0, int t1, float *mup, float *mdn,
                                const float *zeros, float *split_vu, float *split_vl,
                                cudaStream_t st);
-// The row bounds of the last hop's output (one row; k_final_bounds writes
-// them for every row, the reach path evaluates them where it needs them):
+// The row bounds of the last hop's output, evaluated where they are needed
+// (the at most ~3H roundings of the evaluation stay far below the 1e-5,
+// ~168 eps, for H <= 16):
 // ub_j = (U0_j + Umax sum_t alpha^t Mup[t]_j)(1 + 1e-5),
 // lb_j = (L0_j + Lmin sum_t alpha^t Mdn[t]_j)(1 - 1e-5), Horner over t.
 __device__ __forceinline__ float row_upper_bound(const float *u0, const float *mup, int64_t n,
@@ -542,15 +532,17 @@ __device__ __forceinline__ float ext_umax(const unsigned int *ext) { return __ui
 __device__ __forceinline__ float ext_lmin(const unsigned int *ext) {
     return __uint_as_float(0x7f800000u - ext[1]);
 }
-// Per call: ub / lb [n] from u's row extremes u0 / l0 and the mass levels
-// 1..H.  ext [2]: ext[0] the bits of Umax = max_j u0_j, ext[1] 0x7f800000
-// minus the bits of Lmin = min over u0_j > 0 of l0_j (both maxima, so zero
-// is the empty value); computed here unless ext_ready (the score GEMM's
-// epilogue already reduced them).
-cudaError_t launch_final_bounds(const float *u0, const float *l0, const float *mup,
-                                const float *mdn, int64_t n, int H, float alpha,
-                                unsigned int *ext, float *ub, float *lb, cudaStream_t st,
-                                int *launches, bool ext_ready = false);
+// What the bounds of a call's last hop come from: u's row maxima and minima,
+// the mass levels 0..H [H + 1][n], and ext [2] from the score GEMM's epilogue:
+// ext[0] the bits of Umax = max_j u0_j, ext[1] 0x7f800000 minus the bits of
+// Lmin = min over u0_j > 0 of l0_j (both maxima, so zero is the empty value).
+struct RowBounds {
+    const float *u0, *l0, *mup, *mdn;
+    const unsigned int *ext;
+    int64_t n;
+    int H;
+    float alpha;
+};
 // Floors of a namespace-scoped last hop: a row can only be selected by the
 // batch's queries of its own namespace, so its floor is that namespace's
 // (tag_floor[i] for tags[i] == its tag; the tags are the batch's distinct
@@ -563,41 +555,35 @@ struct NsFloors {
     const float *tag_floor;   // [<= PF_TAGS]
 };
 constexpr int PF_TAGS = 256;
-__device__ __forceinline__ float row_floor(const NsFloors &f, float floor_, int64_t row) {
-    if (!f.ns_row) return floor_;
-    const int32_t t = f.ns_row[row];
-    int lo = 0, hi = *f.n_tags;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (f.tags[mid] < t) lo = mid + 1;
-        else hi = mid;
-    }
-    if (lo < *f.n_tags && f.tags[lo] == t) return fmaxf(floor_, f.tag_floor[lo]);
-    return INFINITY;
-}
-// nf: the per-namespace floors, or NULL (one floor for all rows)
-cudaError_t launch_split_flags(const HopPlan &p, const float *row_ub, const float *floor_p,
-                               const NsFloors *nf, int32_t *split_skip, int32_t *slot_skip,
-                               int32_t *kept_rows, int64_t *kept_count, int32_t *kept_segs,
-                               KeptScratch &ks, cudaStream_t st, int *launches);
+// split_skip, kept_rows, kept_segs and kept_count (HopBound; kept_count zeroed
+// before) against the floor, or with nf the rows' namespaces' floors.
+// chain: keep_chain_words words of scratch, zeroed before.
+int64_t keep_chain_words(const HopPlan &p);
+cudaError_t launch_keep(const HopPlan &p, const RowBounds &rb, const float *floor_p,
+                        const NsFloors *nf, int32_t *split_skip, int32_t *kept_rows,
+                        int32_t *kept_segs, int64_t *kept_count, unsigned long long *chain,
+                        int *status, cudaStream_t st, int *launches);
 // The floors of a scoped batch: tags = the distinct q_ns of the n_real query
 // columns, and for each tag the largest of (a) the smallest score that the
-// filter bound of any of its queries admits and (b) the k-th largest lb over
-// the split rows of that namespace, taken heaviest first (split_order), at
+// filter bound of any of its queries admits and (b) the k-th largest lower
+// bound over the split rows of that namespace, taken heaviest first (split_order), at
 // most PF_ROWS of them (any subset of a namespace's rows gives a floor that
 // each of its queries' k-th largest final score reaches).
-cudaError_t launch_ns_floors(const unsigned long long *bound, const int32_t *q_ns, int n_real,
-                             const float *lb, const int32_t *ns_row, const int32_t *split_row,
+// The filter bounds are raised to the floors, which hold for them too.
+cudaError_t launch_ns_floors(unsigned long long *bound, const int32_t *q_ns, int n_real,
+                             const RowBounds &rb, const int32_t *ns_row, const int32_t *split_row,
                              const int32_t *split_order, int64_t n_split, int k, int32_t *tags,
                              int *n_tags, float *tag_floor, cudaStream_t st);
 // floor = max(the smallest score any real column's filter bound admits,
-// and, if lb_rows != NULL, the k-th largest lb over the rows
-// lb_rows[order[i]], i < n_lb_rows), written to floor_out.  The second term
-// is only valid when every row may be selected by every query (no namespace
-// scope).
-cudaError_t launch_prune_floor(const unsigned long long *bound, int n_real, const float *lb,
+// and, if lb_rows != NULL, the k-th largest lower bound over the rows
+// lb_rows[order[i]], i < n_lb_rows), written to floor_out; the filter bounds
+// are raised to it.  The second term is only valid when every row may be
+// selected by every query (no namespace scope).  zero[0 .. n_zero) are set to
+// 0 (launch_keep's chain).
+cudaError_t launch_prune_floor(unsigned long long *bound, int n_real, const RowBounds &rb,
                                const int32_t *lb_rows, const int32_t *order, int64_t n_lb_rows,
-                               int k, float *floor_out, cudaStream_t st);
+                               int k, float *floor_out, unsigned long long *zero, int64_t n_zero,
+                               cudaStream_t st);
 cudaError_t launch_fill_f32(float *v, int64_t n, float x, cudaStream_t st);
 
 // ------------------------------------------------------------------ reach (ak_reach.cu)
@@ -672,7 +658,7 @@ cudaError_t launch_reach_scores(const uint16_t *u_hi, const uint16_t *u_lo, int 
 // slot_split[s] = r for every partial slot s of split row r.
 cudaError_t launch_slot_owner(const int64_t *split_slot0, int64_t n_split, int32_t *slot_split,
                               cudaStream_t st);
-// `counters` = 2 device ints, zeroed by the launcher (work queues).
+// `counters` = 2 device ints (work queues), zeroed before.
 // `flt` may be NULL (no filter), `hb` NULL (no row bounds).
 cudaError_t launch_hop(const HopPlan &p, const float *u, const float *in, float *out, int bp,
                        float alpha, float *partial, int *counters, const HopFilter *flt,
@@ -693,6 +679,12 @@ struct SelectPlan {
 };
 // force_stride > 0 samples every force_stride-th row instead of the default.
 SelectPlan select_plan(int64_t n, int bp, int k, int sm_count, int64_t force_stride = 0);
+
+// keysT [sp.bp][sp.n_sample]: the last hop's selection keys of the sample
+// rows, none above its row's final key (see k_hop_sample).
+cudaError_t launch_hop_sample(const HopPlan &p, const SelectPlan &sp, const float *u,
+                              const float *in, float alpha, NsScope ns, uint32_t *keysT,
+                              cudaStream_t st, int *launches);
 
 // Retrieval: rows are store rows; keys and outputs carry chunk IDs
 // (ext_of), so ties resolve to the lower chunk ID; page_row is indexed by
@@ -716,8 +708,9 @@ cudaError_t launch_select_signed(const SelectPlan &sp, const float *s, int b,
 // Bound pass alone over signed values: bound[c] for the b real columns
 // (the k-th largest sampled key; padding columns get an all-ones bound).
 // Bound only, unsigned keys (retrieval): ws + sp.off_bound gets the bound,
-// the column counts are cleared.  For a filter fused into the last hop or
-// into the score.  `slack` lowers each bound by that many units of the
+// the column counts are cleared.  For a filter fused into the score, from
+// the sampled score slab `s`, or (s == NULL) into the last hop, from the keys
+// that launch_hop_sample left at ws + sp.off_tr.  `slack` lowers each bound by that many units of the
 // score's last place (margin for a sample computed by another launch).
 cudaError_t launch_sample_bound(const SelectPlan &sp, const float *s, int b,
                                 const int32_t *ext_of, unsigned long long *ws, cudaStream_t st,

@@ -17,10 +17,10 @@ template <bool VEC>
 __global__ void k_prep_queries(const uint16_t *__restrict__ q, int b, int dim, float tau,
                                const float *__restrict__ max_norm, uint16_t *__restrict__ qp,
                                float *__restrict__ shift, int *status,
-                               unsigned int *__restrict__ ext_zero) {
+                               unsigned int *__restrict__ zero, int n_zero) {
     griddep_wait();
     const int c = blockIdx.x;
-    if (ext_zero && c == 0 && threadIdx.x < 2) ext_zero[threadIdx.x] = 0u;
+    if (c == 0 && (int)threadIdx.x < n_zero) zero[threadIdx.x] = 0u;
     __shared__ float red[32];
     float ss = 0.f;
     if constexpr (VEC) {
@@ -59,11 +59,12 @@ __global__ void k_prep_queries(const uint16_t *__restrict__ q, int b, int dim, f
 
 cudaError_t launch_prep_queries(const uint16_t *q, int b, int bp, int dim, float tau,
                                 const float *max_norm, uint16_t *qp, float *shift, int *status,
-                                cudaStream_t st, unsigned int *ext_zero) {
+                                cudaStream_t st, unsigned int *zero, int n_zero) {
+    if (n_zero < 0 || n_zero > 128 || (n_zero > 0 && !zero)) return cudaErrorInvalidValue;
     const bool vec = ((uintptr_t)q & 15) == 0 && dim % 8 == 0;
     cudaError_t e = launch_pdl(vec ? k_prep_queries<true> : k_prep_queries<false>, dim3(bp),
                                dim3(128), 0, st, q, b, dim, tau, max_norm, qp, shift, status,
-                               ext_zero);
+                               zero, n_zero);
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 

@@ -137,6 +137,7 @@ __global__ __launch_bounds__(256) void k_sample_transpose(
     const int32_t *__restrict__ ext_of, int64_t id_limit, NsScope ns,
     uint32_t *__restrict__ keysT) {
     __shared__ uint32_t tile[32][33];
+    griddep_wait();
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int64_t v0 = (int64_t)blockIdx.x * 32;
     const int c0 = blockIdx.y * 32;
@@ -183,6 +184,7 @@ __global__ __launch_bounds__(SEL_THREADS) void k_sample_kth(
     __shared__ uint32_t cbuf[KTH_CBUF];
     __shared__ uint32_t s_prefix;
     __shared__ int s_rem, s_match, s_cn;
+    griddep_wait();
     const int c = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (c >= b) {   // padding column: nothing passes the filter
         if (tid == 0) {
@@ -720,25 +722,31 @@ cudaError_t launch_buf_merge_signed(const unsigned int *cnt, const unsigned long
 // subset of the rows gives a valid floor).  One CTA, one key per thread:
 // (b) sorts the unique keys (lb bits, position) descending with a bitonic
 // network (partners within a warp by shuffles, farther ones through a
-// ping-pong pair of shared arrays) and reads the k-th.
+// ping-pong pair of shared arrays) and reads the k-th.  The filter bounds are
+// then raised to the floor (fewer keys to merge).
 constexpr int PF_ROWS = 1024;
 
 __global__ __launch_bounds__(PF_ROWS) void k_prune_floor(
-    const unsigned long long *__restrict__ bound, int n_real, const float *__restrict__ lb,
+    unsigned long long *__restrict__ bound, int n_real, const RowBounds rb,
     const int32_t *__restrict__ lb_rows, const int32_t *__restrict__ order, int64_t n_rows,
-    int k, float *__restrict__ floor_out) {
+    int k, float *__restrict__ floor_out, unsigned long long *__restrict__ zero, int64_t n_zero) {
     __shared__ unsigned long long xk[2][PF_ROWS];
     __shared__ unsigned int s_min;
+    __shared__ float s_floor;
+    griddep_wait();
     const int t = threadIdx.x;
     if (t == 0) s_min = 0x7f800000u;
+    for (int64_t i = t; i < n_zero; i += PF_ROWS) zero[i] = 0ull;
     __syncthreads();
-    if (bound && t < n_real) atomicMin(&s_min, (unsigned int)(bound[t] >> 32));
+    if (t < n_real) atomicMin(&s_min, (unsigned int)(bound[t] >> 32));
     const bool want_lb = lb_rows && n_rows >= k;
     // absent keys are 0, below every real key but (lb = 0, position 0),
     // which they equal
     unsigned long long key =
         want_lb && t < n_rows
-            ? ((unsigned long long)__float_as_uint(lb[lb_rows[order[t]]]) << 32) |
+            ? ((unsigned long long)__float_as_uint(row_lower_bound(
+                   rb.l0, rb.mdn, rb.n, rb.H, rb.alpha, ext_lmin(rb.ext), lb_rows[order[t]]))
+               << 32) |
                   (unsigned long long)(uint32_t)t
             : 0ull;
     int cur = 0;
@@ -764,10 +772,15 @@ __global__ __launch_bounds__(PF_ROWS) void k_prune_floor(
     }
     __syncthreads();
     if (t == 0) {
-        // without filter bounds (no first term) the floor starts at 0
-        float fl = bound ? __uint_as_float(s_min) : 0.f;
+        float fl = __uint_as_float(s_min);
         if (want_lb) fl = fmaxf(fl, __uint_as_float((uint32_t)(xk[cur][0] >> 32)));
         *floor_out = fl;
+        s_floor = fl;
+    }
+    __syncthreads();
+    if (t < n_real) {
+        const unsigned long long fk = (unsigned long long)__float_as_uint(s_floor) << 32;
+        if (bound[t] < fk) bound[t] = fk;
     }
 }
 
@@ -783,6 +796,7 @@ __global__ __launch_bounds__(PF_TAGS) void k_ns_tags(const unsigned long long *_
     __shared__ unsigned long long key[PF_TAGS];
     __shared__ int pos[PF_TAGS];
     __shared__ unsigned int mn[PF_TAGS];
+    griddep_wait();
     const int t = threadIdx.x;
     // valid tags first, in signed order; padding (1 << 32) last
     key[t] = t < n_real ? (unsigned long long)((uint32_t)q_ns[t] ^ 0x80000000u) : (1ull << 32);
@@ -814,7 +828,7 @@ __global__ __launch_bounds__(PF_TAGS) void k_ns_tags(const unsigned long long *_
     if (first) tags[pos[t] - 1] = (int32_t)((uint32_t)key[t] ^ 0x80000000u);
     if (t == 0) *n_tags = nt;
     __syncthreads();
-    if (t < n_real && bound) {
+    if (t < n_real) {
         const int32_t mine = q_ns[t];
         int lo = 0, hi = nt;
         while (lo < hi) {
@@ -825,12 +839,15 @@ __global__ __launch_bounds__(PF_TAGS) void k_ns_tags(const unsigned long long *_
         atomicMin(&mn[lo], (unsigned int)(bound[t] >> 32));
     }
     __syncthreads();
-    if (t < nt) tag_floor[t] = bound ? __uint_as_float(mn[t]) : 0.f;
+    if (t < nt) tag_floor[t] = __uint_as_float(mn[t]);
 }
 
-// tag_floor[d] = max(tag_floor[d], k-th largest lb over the first PF_ROWS
-// split rows, heaviest first, of namespace tags[d]); one CTA per tag.
-__global__ __launch_bounds__(PF_ROWS) void k_ns_floor(const float *__restrict__ lb,
+// tag_floor[d] = max(tag_floor[d], k-th largest lower bound over the first
+// PF_ROWS split rows, heaviest first, of namespace tags[d]), and the filter
+// bounds of that namespace's queries raised to it; one CTA per tag.
+__global__ __launch_bounds__(PF_ROWS) void k_ns_floor(unsigned long long *__restrict__ bound,
+                                                      const int32_t *__restrict__ q_ns, int n_real,
+                                                      const RowBounds rb,
                                                       const int32_t *__restrict__ ns_row,
                                                       const int32_t *__restrict__ split_row,
                                                       const int32_t *__restrict__ order,
@@ -841,8 +858,10 @@ __global__ __launch_bounds__(PF_ROWS) void k_ns_floor(const float *__restrict__ 
     __shared__ unsigned int key[PF_ROWS];
     __shared__ int wcount[PF_ROWS / 32];
     __shared__ int got_s;
+    griddep_wait();
     const int d = blockIdx.x;
     if (d >= *n_tags) return;
+    const float lmin = ext_lmin(rb.ext);
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int32_t tag = tags[d];
     key[t] = 0u;
@@ -860,7 +879,9 @@ __global__ __launch_bounds__(PF_ROWS) void k_ns_floor(const float *__restrict__ 
         int before = got;
         for (int x = 0; x < w; ++x) before += wcount[x];
         before += __popc(bal & ((1u << lane) - 1u));
-        if (match && before < PF_ROWS) key[before] = __float_as_uint(lb[r]);   // lb >= 0
+        if (match && before < PF_ROWS)                // (lower bounds are >= 0)
+            key[before] = __float_as_uint(
+                row_lower_bound(rb.l0, rb.mdn, rb.n, rb.H, rb.alpha, lmin, r));
         __syncthreads();
         if (t == 0) {
             int tot = got;
@@ -885,28 +906,35 @@ __global__ __launch_bounds__(PF_ROWS) void k_ns_floor(const float *__restrict__ 
             }
             __syncthreads();
         }
-    if (t == 0) tag_floor[d] = fmaxf(tag_floor[d], __uint_as_float(key[k - 1]));
+    const float kth = __uint_as_float(key[k - 1]);
+    if (t == 0) tag_floor[d] = fmaxf(tag_floor[d], kth);
+    const unsigned long long fk = (unsigned long long)__float_as_uint(kth) << 32;
+    if (t < n_real && q_ns[t] == tag && bound[t] < fk) bound[t] = fk;
 }
 
-cudaError_t launch_ns_floors(const unsigned long long *bound, const int32_t *q_ns, int n_real,
-                             const float *lb, const int32_t *ns_row, const int32_t *split_row,
+cudaError_t launch_ns_floors(unsigned long long *bound, const int32_t *q_ns, int n_real,
+                             const RowBounds &rb, const int32_t *ns_row, const int32_t *split_row,
                              const int32_t *split_order, int64_t n_split, int k, int32_t *tags,
                              int *n_tags, float *tag_floor, cudaStream_t st) {
     if (n_real < 1 || n_real > PF_TAGS || k < 1) return cudaErrorInvalidValue;
-    k_ns_tags<<<1, PF_TAGS, 0, st>>>(bound, q_ns, n_real, tags, n_tags, tag_floor);
-    if (n_split > 0 && k <= PF_ROWS)
-        k_ns_floor<<<PF_TAGS, PF_ROWS, 0, st>>>(lb, ns_row, split_row, split_order, n_split, k,
-                                                tags, n_tags, tag_floor);
-    return cudaGetLastError();
+    cudaError_t e = launch_pdl(k_ns_tags, dim3(1), dim3(PF_TAGS), 0, st,
+                               (const unsigned long long *)bound, q_ns, n_real, tags, n_tags,
+                               tag_floor);
+    if (e == cudaSuccess && n_split > 0 && k <= PF_ROWS)
+        e = launch_pdl(k_ns_floor, dim3((unsigned)n_real), dim3(PF_ROWS), 0, st, bound, q_ns,
+                       n_real, rb, ns_row, split_row, split_order, n_split, k,
+                       (const int32_t *)tags, (const int *)n_tags, tag_floor);
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
-cudaError_t launch_prune_floor(const unsigned long long *bound, int n_real, const float *lb,
+cudaError_t launch_prune_floor(unsigned long long *bound, int n_real, const RowBounds &rb,
                                const int32_t *lb_rows, const int32_t *order, int64_t n_lb_rows,
-                               int k, float *floor_out, cudaStream_t st) {
+                               int k, float *floor_out, unsigned long long *zero, int64_t n_zero,
+                               cudaStream_t st) {
     if (n_lb_rows > PF_ROWS || n_real > PF_ROWS || k < 1) return cudaErrorInvalidValue;
-    k_prune_floor<<<1, PF_ROWS, 0, st>>>(bound, n_real, lb, lb_rows, order, n_lb_rows, k,
-                                         floor_out);
-    return cudaGetLastError();
+    cudaError_t e = launch_pdl(k_prune_floor, dim3(1), dim3(PF_ROWS), 0, st, bound, n_real, rb,
+                               lb_rows, order, n_lb_rows, k, floor_out, zero, n_zero);
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 // ------------------------------------------------------------------ launchers
@@ -926,15 +954,17 @@ static cudaError_t launch_kth(const SelectPlan &sp, const float *s, int b, const
         attr[dev] = true;
     }
     uint32_t *keysT = (uint32_t *)(ws + sp.off_tr);
-    const dim3 tgrid((unsigned)ceil_div<int64_t>(sp.n_sample, 32), (unsigned)(sp.bp / 32));
-    k_sample_transpose<SIGNED><<<tgrid, 256, 0, st>>>(s, sp.n_sample, sp.stride, sp.bp, ext_of,
-                                                      id_limit, ns, keysT);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    if (s) {
+        const dim3 tgrid((unsigned)ceil_div<int64_t>(sp.n_sample, 32), (unsigned)(sp.bp / 32));
+        e = launch_pdl(k_sample_transpose<SIGNED>, tgrid, dim3(256), 0, st, s, sp.n_sample,
+                       sp.stride, sp.bp, ext_of, id_limit, ns, keysT);
+        if (e != cudaSuccess) return e;
+    }
     const size_t smem = sp.n_sample <= KTH_STAGE ? (size_t)sp.n_sample * sizeof(uint32_t) : 0;
-    k_sample_kth<<<sp.bp, SEL_THREADS, smem, st>>>(keysT, sp.n_sample, b, sp.k, slack, bound,
-                                                   cnt);
-    return cudaGetLastError();
+    e = launch_pdl(k_sample_kth, dim3(sp.bp), dim3(SEL_THREADS), smem, st,
+                   (const uint32_t *)keysT, sp.n_sample, b, sp.k, slack, bound, cnt);
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 template <bool SIGNED>
@@ -971,7 +1001,7 @@ static cudaError_t sample_bound(const SelectPlan &sp, const float *s, int b,
                                 NsScope ns = NsScope{}) {
     cudaError_t e = launch_kth<SIGNED>(sp, s, b, ext_of, id_limit, ws, bound,
                                        (unsigned int *)(ws + sp.off_cnt), st, slack, ns);
-    if (launches) *launches += 2;
+    if (launches) *launches += s ? 2 : 1;
     return e;
 }
 
