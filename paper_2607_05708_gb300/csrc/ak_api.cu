@@ -103,6 +103,13 @@ struct StreamScratch {
     // their copy (the host waits for that point only)
     int32_t *plan_host = nullptr;
     cudaEvent_t plan_ev = nullptr;
+    // the fp32 pass: the combined coefficients and their key; the last
+    // attempt's outcome (plan_host[2], written by the device) and its key
+    DevBuf coef_f, coef_sum;
+    uint64_t cf_build = ~0ull, try_build = ~0ull;
+    float cf_alpha = -1.f, try_alpha = -1.f;
+    int cf_H = 0, try_H = 0, try_k = 0, try_skip = 0;
+    int64_t cf_n = -1, try_n = -1;
     ~StreamScratch() {
         if (plan_host) cudaFreeHost(plan_host);
         if (plan_ev) cudaEventDestroy(plan_ev);
@@ -168,10 +175,11 @@ struct akashic_mem {
     int mass_levels = -1;
     int64_t mass_n = -1;      // rows they were computed for
     // reach coefficients of the candidate rows (ak_reach.cu), same lifetime
-    DevBuf reach_rows, reach_t, reach_map, reach_c;
-    int reach_levels = -1;
-    int reach_T = 0;          // candidate rows (host copy)
+    DevBuf reach_rows, reach_t, reach_map, reach_c[REACH_MAX_H];
+    int reach_levels = -1;    // levels C_1.. in place (0 or less: no candidates either)
     int64_t reach_n = -1;     // rows they were computed for
+    double hop_work = 0;      // query columns x hops run through the hops since the
+    int64_t hop_work_n = -1;  // graph (or the number of rows) last changed
     uint64_t reach_build = 0; // incremented by every rebuild
     bool reach_on = true;     // AKASHIC_REACH=0: always run the hops
     // the mass levels and reach tables are built by whichever retrieve needs
@@ -410,6 +418,7 @@ static akashic_status_t build_split_plan(akashic_mem *m, cudaStream_t st) {
     const int64_t n = m->n;
     m->mass_levels = -1;   // the graph changed
     m->reach_levels = -1;
+    m->hop_work = 0;
     // temporaries from the store's scratch (slots SCR_SPLIT0..11)
     akashic_status_t sc_rc = AKASHIC_OK;
     auto get = [&](int i, size_t bytes) -> Tmp {
@@ -1174,20 +1183,17 @@ static akashic_status_t ensure_mass(akashic_mem *m, const HopPlan &hp, int H, cu
     return tables_built(m, st);
 }
 
-// Reach coefficients of the candidate rows for H hops (after the mass
-// levels).  table_mu held.
+// The candidate rows and their reach coefficients for H >= 2 hops (after the
+// mass levels).  A level is never rewritten while the graph stays the same, so
+// a call with another hop count only adds levels that no other call reads yet.
+// table_mu held.
 static akashic_status_t ensure_reach(akashic_mem *m, const HopPlan &hp, int H, cudaStream_t st) {
     const int64_t n = m->n;
     AK_TRY(wait_tables(m, st));
-    if (m->reach_levels == H && m->reach_n == n) return AKASHIC_OK;
-    AK_TRY(m->reach_rows.ensure(REACH_T * 4));
-    AK_TRY(m->reach_t.ensure(16));
-    AK_TRY(ensure_spare(m->reach_map, (size_t)n * 4));
-    AK_TRY(ensure_spare(m->reach_c, (size_t)H * n * REACH_T * 4));
+    if (m->reach_levels >= H && m->reach_n == n) return AKASHIC_OK;
     ReachBuild rb{};
     rb.n = n;
     rb.n_split = m->n_split;
-    rb.H = H;
     rb.split_row = hp.split_row;
     rb.split_order = hp.split_order;
     rb.mup = m->mass_up.as<float>();
@@ -1198,19 +1204,33 @@ static akashic_status_t ensure_reach(akashic_mem *m, const HopPlan &hp, int H, c
     rb.col = m->col.as<int32_t>();
     rb.row_of = m->row_of.as<int32_t>();
     rb.w = m->w.as<float>();
-    rb.rows = m->reach_rows.as<int32_t>();
-    rb.t_cnt = m->reach_t.as<int>();
-    rb.map = m->reach_map.as<int32_t>();
-    rb.C = m->reach_c.as<float>();
-    CUDA_TRY(launch_reach_build(rb, st));
-    int t = 0;
-    CUDA_TRY(cudaMemcpyAsync(&t, m->reach_t.p, 4, cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    m->reach_T = t;
-    m->reach_levels = H;
-    m->reach_n = n;
-    ++m->reach_build;
+    if (m->reach_levels < 1 || m->reach_n != n) {
+        m->reach_levels = -1;
+        AK_TRY(m->reach_rows.ensure(REACH_T * 4));
+        AK_TRY(m->reach_t.ensure(16));
+        AK_TRY(ensure_spare(m->reach_map, (size_t)n * 4));
+        AK_TRY(ensure_spare(m->reach_c[0], (size_t)n * REACH_T * 4));
+        rb.rows = m->reach_rows.as<int32_t>();
+        rb.t_cnt = m->reach_t.as<int>();
+        rb.map = m->reach_map.as<int32_t>();
+        CUDA_TRY(launch_reach_pick(rb, m->reach_c[0].as<float>(), st));
+        m->reach_levels = 1;
+        m->reach_n = n;
+        ++m->reach_build;
+    }
+    for (int t = m->reach_levels; t < H; ++t) {
+        AK_TRY(ensure_spare(m->reach_c[t], (size_t)n * REACH_T * 4));
+        CUDA_TRY(launch_reach_level(rb, m->reach_c[t - 1].as<float>(), m->reach_c[t].as<float>(),
+                                    st));
+        m->reach_levels = t + 1;
+    }
     return tables_built(m, st);
+}
+
+static ReachLevels reach_levels_of(const akashic_mem *m) {
+    ReachLevels c{};
+    for (int t = 0; t < REACH_MAX_H; ++t) c.level[t] = m->reach_c[t].as<float>();
+    return c;
 }
 
 static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t B, int32_t k,
@@ -1361,7 +1381,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
         }
         const float *fin = sc->u.as<float>();
         if (eff_hops >= 1) {
-            HopPlan hp;
+            HopPlan hp{};
             hp.split = m->split;
             hp.in_ptr = m->in_ptr.as<int64_t>();
             hp.in_src = m->in_src.as<int32_t>();
@@ -1386,6 +1406,73 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                 std::lock_guard<std::mutex> lk(m->table_mu);
                 AK_TRY(ensure_mass(m, hp, eff_hops, st));
             }
+            // Two to four hops in fp32 without running them, from the same
+            // candidates and floor (launch_reach_fma).  The hops are queued
+            // behind and return at once when the plan says the candidates
+            // suffice, so the host waits for nothing.  The coefficients cost
+            // about what the hops cost over 128 columns a level past the
+            // first, and are worth it only if the graph stays as it is: they
+            // are built once the hops have cost that much since it changed (so
+            // never more than twice the work of either way alone).  One GB300,
+            // hops against candidates: 1,048,576 chunks, 1 query, two hops 1533
+            // -> 444 us; 262,147 chunks, 24 queries 384 -> 143; 262,144 chunks,
+            // 200 queries, three hops 1589 -> 564.
+            bool reach_fma = false;
+            if (prune && !reach_try && !q_ns && m->reach_on && eff_hops >= 2 &&
+                eff_hops <= REACH_MAX_H && m->n_split >= k) {
+                std::lock_guard<std::mutex> lk(m->table_mu);
+                if (m->reach_levels < eff_hops || m->reach_n != n) {
+                    if (m->hop_work_n != n) m->hop_work = 0;
+                    m->hop_work_n = n;
+                    if (m->hop_work >= REACH_T * (eff_hops - 1) + 64) reach_fma = true;
+                    else m->hop_work += (double)eff_hops * bp;
+                } else {
+                    reach_fma = true;
+                }
+                if (reach_fma) {
+                    // no room for the tables: the hops run, as they would without
+                    akashic_status_t r = ensure_reach(m, hp, eff_hops, st);
+                    if (r == AKASHIC_OK)
+                        r = ensure_spare(sc->reach_part,
+                                         (size_t)reach_fma_parts(n, b) * REACH_T * bp * 4);
+                    if (r == AKASHIC_OK) r = ensure_spare(sc->coef_f, (size_t)n * REACH_T * 4);
+                    if (r == AKASHIC_OK) r = sc->coef_sum.ensure((size_t)reach_sum_words() * 8);
+                    if (r != AKASHIC_OK && r != AKASHIC_ENOMEM) return r;
+                    if (r == AKASHIC_ENOMEM) {
+                        g_last_error.clear();
+                        reach_fma = false;
+                        m->hop_work = -1e300;   // not again for this graph
+                        m->reach_levels = -1;
+                    }
+                }
+                // where the candidates did not suffice (the device has said so
+                // by now, or has not yet), the next 15 calls like it run the
+                // hops alone
+                if (reach_fma) {
+                    if (!sc->plan_host) {
+                        CUDA_TRY(cudaMallocHost((void **)&sc->plan_host, 16));
+                        memset(sc->plan_host, 0, 16);
+                    }
+                    volatile int32_t *outcome = sc->plan_host + 2;
+                    if (sc->try_build != m->reach_build || sc->try_alpha != alpha ||
+                        sc->try_H != eff_hops || sc->try_k != k || sc->try_n != n) {
+                        sc->try_build = m->reach_build;
+                        sc->try_alpha = alpha;
+                        sc->try_H = eff_hops;
+                        sc->try_k = k;
+                        sc->try_n = n;
+                        sc->try_skip = 0;
+                        *outcome = 0;
+                    } else if (sc->try_skip > 0) {
+                        --sc->try_skip;
+                        reach_fma = false;
+                    } else if (*outcome == 2) {
+                        sc->try_skip = 14;
+                        *outcome = 0;
+                        reach_fma = false;
+                    }
+                }
+            }
             // the row bounds of the last hop's output
             const RowBounds rb{sc->rmax_u.as<float>(), sc->rmin_u.as<float>(),
                                m->mass_up.as<float>(), m->mass_dn.as<float>(), ext, n, eff_hops,
@@ -1395,6 +1482,57 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
             // candidate with reach coefficients, their final scores come from
             // one pass over u and they alone are the selection's candidates.
             bool reach_done = false;
+            auto reach_flags = [&](int32_t *outcome, int *launches) -> akashic_status_t {
+                AK_TRY(sc->reach_keep.ensure((REACH_T + 2) * 4));
+                AK_TRY(sc->reach_plan.ensure(REACH_PLAN_INTS * 4));
+                ReachFlags rf{};
+                rf.u0 = rb.u0;
+                rf.l0 = rb.l0;
+                rf.mup = rb.mup;
+                rf.mdn = rb.mdn;
+                rf.ext = ext;
+                rf.n = n;
+                rf.H = eff_hops;
+                rf.alpha = alpha;
+                rf.split_row = hp.split_row;
+                rf.split_order = hp.split_order;
+                rf.n_lb = m->n_split < 1024 ? m->n_split : 1024;
+                rf.k = k;
+                rf.map = m->reach_map.as<int32_t>();
+                rf.t_cnt = m->reach_t.as<int>();
+                rf.floor_out = sc->pfloor.as<float>();
+                rf.ws = sc->reach_keep.as<int32_t>();
+                rf.plan = sc->reach_plan.as<int32_t>();
+                rf.outcome = outcome;
+                CUDA_TRY(launch_reach_flags(rf, st, launches));
+                return AKASHIC_OK;
+            };
+            if (reach_fma) {
+                {
+                    PhaseScope ph(m, AKASHIC_PHASE_BOUND, st);
+                    AK_TRY(reach_flags(sc->plan_host + 2, &ph.launches));
+                }
+                PhaseScope ph(m, AKASHIC_PHASE_LAST_HOP, st);
+                if (sc->cf_build != m->reach_build || sc->cf_alpha != alpha ||
+                    sc->cf_H != eff_hops || sc->cf_n != n) {
+                    CUDA_TRY(launch_reach_combine(reach_levels_of(m), n, eff_hops, alpha,
+                                                  sc->coef_f.as<float>(),
+                                                  sc->coef_sum.as<double>(), st));
+                    ph.launches += 2;
+                    sc->cf_build = m->reach_build;
+                    sc->cf_alpha = alpha;
+                    sc->cf_H = eff_hops;
+                    sc->cf_n = n;
+                }
+                CUDA_TRY(launch_reach_fma(sc->u.as<float>(), bp, b, n, sc->coef_f.as<float>(),
+                                          sc->coef_sum.as<double>(), ext,
+                                          sc->reach_plan.as<int32_t>(),
+                                          m->reach_rows.as<int32_t>(), m->ext_of.as<int32_t>(),
+                                          sc->reach_part.as<float>(),
+                                          (unsigned int *)(ws + sp.off_cnt), ws + sp.off_buf,
+                                          sp.cap, st, &ph.launches));
+                hp.done = sc->reach_plan.as<int32_t>();
+            }
             if (reach_try) {
                 {
                     PhaseScope ph(m, AKASHIC_PHASE_BOUND, st);
@@ -1402,30 +1540,13 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                         std::lock_guard<std::mutex> lk(m->table_mu);
                         AK_TRY(ensure_reach(m, hp, eff_hops, st));
                     }
-                    AK_TRY(sc->reach_keep.ensure((REACH_T + 2) * 4));
-                    AK_TRY(sc->reach_plan.ensure(REACH_PLAN_INTS * 4));
-                    if (!sc->plan_host) CUDA_TRY(cudaMallocHost((void **)&sc->plan_host, 16));
+                    if (!sc->plan_host) {
+                        CUDA_TRY(cudaMallocHost((void **)&sc->plan_host, 16));
+                        memset(sc->plan_host, 0, 16);
+                    }
                     if (!sc->plan_ev)
                         CUDA_TRY(cudaEventCreateWithFlags(&sc->plan_ev, cudaEventDisableTiming));
-                    ReachFlags rf{};
-                    rf.u0 = sc->rmax_u.as<float>();
-                    rf.l0 = sc->rmin_u.as<float>();
-                    rf.mup = m->mass_up.as<float>();
-                    rf.mdn = m->mass_dn.as<float>();
-                    rf.ext = ext;
-                    rf.n = n;
-                    rf.H = eff_hops;
-                    rf.alpha = alpha;
-                    rf.split_row = hp.split_row;
-                    rf.split_order = hp.split_order;
-                    rf.n_lb = m->n_split < 1024 ? m->n_split : 1024;
-                    rf.k = k;
-                    rf.map = m->reach_map.as<int32_t>();
-                    rf.t_cnt = m->reach_t.as<int>();
-                    rf.floor_out = sc->pfloor.as<float>();
-                    rf.ws = sc->reach_keep.as<int32_t>();
-                    rf.plan = sc->reach_plan.as<int32_t>();
-                    CUDA_TRY(launch_reach_flags(rf, st, &ph.launches));
+                    AK_TRY(reach_flags(nullptr, &ph.launches));
                     CUDA_TRY(cudaMemcpyAsync(sc->plan_host, sc->reach_plan.p, 8,
                                              cudaMemcpyDeviceToHost, st));
                     CUDA_TRY(cudaEventRecord(sc->plan_ev, st));
@@ -1435,7 +1556,8 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                     // plan (its kernels return at once when the plan says the
                     // hops run), so the GPU goes on while the host waits.
                     PhaseScope ph(m, AKASHIC_PHASE_LAST_HOP, st);
-                    AK_TRY(sc->reach_part.ensure((size_t)reach_parts() * REACH_T * bp * 4));
+                    AK_TRY(ensure_spare(sc->reach_part,
+                                        (size_t)reach_parts() * REACH_T * bp * 4));
                     // every candidate's packed coefficients, kept while the
                     // graph, alpha and the hop count stay the same
                     if (sc->coef_build != m->reach_build || sc->coef_alpha != alpha ||
@@ -1443,7 +1565,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                         const size_t cb = (size_t)REACH_T * reach_pad_rows(n) * 2;
                         AK_TRY(ensure_spare(sc->coef_hi, cb));
                         AK_TRY(ensure_spare(sc->coef_lo, cb));
-                        CUDA_TRY(launch_reach_pack(m->reach_c.as<float>(), n, eff_hops, alpha,
+                        CUDA_TRY(launch_reach_pack(reach_levels_of(m), n, eff_hops, alpha,
                                                    sc->coef_hi.as<uint16_t>(),
                                                    sc->coef_lo.as<uint16_t>(), st));
                         ph.launches += 1;
@@ -1484,7 +1606,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                                                    (uint32_t *)(ws + sp.off_tr), st,
                                                    &ps.launches));
                         CUDA_TRY(launch_sample_bound(sp, nullptr, b, m->ext_of.as<int32_t>(), ws,
-                                                     st, &ps.launches, 0u, ns));
+                                                     st, &ps.launches, 0u, ns, hp.done));
                     }
                     if (prune) {
                         PhaseScope ps(m, AKASHIC_PHASE_BOUND, st);
@@ -1498,7 +1620,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                         CUDA_TRY(launch_prune_floor(ws + sp.off_bound, b, rb,
                                                     q_ns ? nullptr : hp.split_row,
                                                     hp.split_order, n_lb, k,
-                                                    sc->pfloor.as<float>(), chain, cw, st));
+                                                    sc->pfloor.as<float>(), chain, cw, hp.done, st));
                         // with a scope, each namespace of the batch gets its own
                         // floor (its rows can only be selected by its queries)
                         NsFloors nf{};

@@ -459,6 +459,8 @@ cudaError_t launch_drop_dead_edges(const DropDead &d, cudaStream_t st);
 
 // Propagation hop (a2): out[j,:] = u[j,:] + alpha * sum_{i->j} w_ij * in[i,:].
 struct HopPlan {
+    const int32_t *done;        // a reach plan (or NULL): with done[0] = 1 the call's
+                                // kernels from the first hop on return at once
     SplitParams split;
     const int64_t *in_ptr;      // n+1
     const int32_t *in_src;      // nnz
@@ -583,18 +585,18 @@ cudaError_t launch_ns_floors(unsigned long long *bound, const int32_t *q_ns, int
 cudaError_t launch_prune_floor(unsigned long long *bound, int n_real, const RowBounds &rb,
                                const int32_t *lb_rows, const int32_t *order, int64_t n_lb_rows,
                                int k, float *floor_out, unsigned long long *zero, int64_t n_zero,
-                               cudaStream_t st);
+                               const int32_t *done, cudaStream_t st);
 cudaError_t launch_fill_f32(float *v, int64_t n, float x, cudaStream_t st);
 
 // ------------------------------------------------------------------ reach (ak_reach.cu)
 // Final scores of a few candidate rows straight from u: s^(H)_j = u_j +
 // sum_t alpha^t sum_k C_t[k][j] u_k with graph-only reach coefficients.
 constexpr int REACH_T = 128;         // candidate rows kept
+constexpr int REACH_MAX_H = 4;       // hop counts it serves: 2 .. REACH_MAX_H
 struct ReachBuild {
     int64_t n, n_split;
-    int H;
     const int32_t *split_row, *split_order;
-    const float *mup;                // mass levels [H + 1][n] (candidate choice)
+    const float *mup;                // mass levels 0..2 [3][n] (candidate choice)
     const int64_t *in_ptr;           // in-edge CSR (row space)
     const int32_t *in_src;
     const float *in_w;
@@ -604,9 +606,13 @@ struct ReachBuild {
     int32_t *rows;                   // [REACH_T] candidate rows
     int *t_cnt;                      // their number (device)
     int32_t *map;                    // [n] row -> candidate slot or -1
-    float *C;                        // [H][n][REACH_T]
 };
-cudaError_t launch_reach_build(const ReachBuild &rb, cudaStream_t st);
+struct ReachLevels {
+    const float *level[REACH_MAX_H]; // C_1, C_2, ...: [n][REACH_T] each
+};
+// The candidates, their map and C_1; then Cn = C_{t+1} from Cp = C_t.
+cudaError_t launch_reach_pick(const ReachBuild &rb, float *C1, cudaStream_t st);
+cudaError_t launch_reach_level(const ReachBuild &rb, const float *Cp, float *Cn, cudaStream_t st);
 // The reach path's floor, flags and plan, without the per-row bound arrays:
 // floor = the k-th largest lower bound over the (up to 1024) heaviest split
 // rows, computed for those rows only; then every row's upper bound against
@@ -628,6 +634,8 @@ struct ReachFlags {
     float *floor_out;
     int32_t *ws;
     int32_t *plan;                   // [REACH_PLAN_INTS]
+    int32_t *outcome;                // host-visible word (or NULL): 1 the candidates
+                                     // suffice, 2 the hops run
 };
 cudaError_t launch_reach_flags(const ReachFlags &f, cudaStream_t st, int *launches);
 int reach_parts();                   // CTAs of the candidates' pass (partial rows)
@@ -643,7 +651,7 @@ int64_t reach_pad_rows(int64_t n);
 // Every candidate's combined coefficients sum_t alpha^t C_t as bf16 hi + lo,
 // [REACH_T][reach_pad_rows(n)] each (graph-only; repacked when the graph,
 // alpha or H change).
-cudaError_t launch_reach_pack(const float *C, int64_t n, int H, float alpha, uint16_t *coef_hi,
+cudaError_t launch_reach_pack(const ReachLevels &C, int64_t n, int H, float alpha, uint16_t *coef_hi,
                               uint16_t *coef_lo, cudaStream_t st);
 // partial: [reach_parts()][REACH_T][bp] scratch; with plan[0] = 1 the
 // flagged candidates' keys are written to each real column's buffer
@@ -655,6 +663,19 @@ cudaError_t launch_reach_scores(const uint16_t *u_hi, const uint16_t *u_lo, int 
                                 const int32_t *ext_of, float *partial, unsigned int *cnt,
                                 unsigned long long *buf, int64_t cap, int *status, cudaStream_t st,
                                 int *launches);
+// The same in fp32 (any hop count and bp): coef [n][REACH_T] the combined
+// coefficients, sums [REACH_T] their column sums (of reach_sum_words() words,
+// the rest scratch), u [n][bp] the score slab, ext u's extremes, partial
+// [reach_fma_parts(n, B)][REACH_T][bp] scratch.
+int64_t reach_sum_words();
+cudaError_t launch_reach_combine(const ReachLevels &C, int64_t n, int H, float alpha, float *coef,
+                                 double *sums, cudaStream_t st);
+int reach_fma_parts(int64_t n, int B);
+cudaError_t launch_reach_fma(const float *u, int bp, int B, int64_t n, const float *coef,
+                             const double *sums, const unsigned int *ext, const int32_t *plan,
+                             const int32_t *rows, const int32_t *ext_of, float *partial,
+                             unsigned int *cnt, unsigned long long *buf, int64_t cap,
+                             cudaStream_t st, int *launches);
 // slot_split[s] = r for every partial slot s of split row r.
 cudaError_t launch_slot_owner(const int64_t *split_slot0, int64_t n_split, int32_t *slot_split,
                               cudaStream_t st);
@@ -714,7 +735,8 @@ cudaError_t launch_select_signed(const SelectPlan &sp, const float *s, int b,
 // score's last place (margin for a sample computed by another launch).
 cudaError_t launch_sample_bound(const SelectPlan &sp, const float *s, int b,
                                 const int32_t *ext_of, unsigned long long *ws, cudaStream_t st,
-                                int *launches, uint32_t slack = 0, NsScope ns = NsScope{});
+                                int *launches, uint32_t slack = 0, NsScope ns = NsScope{},
+                                const int32_t *done = nullptr);
 // A column of the last hop recomputed by the merge when the filter fused
 // into that hop (which writes no output slab) overflowed its buffer:
 // dst[j,c] = u[j,c] + alpha * sum_{e in in(j)} in_w[e] * prev[in_src[e],c].

@@ -1190,13 +1190,15 @@ __global__ __launch_bounds__(256) void k_keep(const RowBounds rb, const float *_
                                               int32_t *__restrict__ kept_rows,
                                               int32_t *__restrict__ kept_segs,
                                               unsigned long long *__restrict__ kept_count,
-                                              unsigned long long *chain, int *status) {
+                                              unsigned long long *chain, int *status,
+                                              const int32_t *__restrict__ done) {
     __shared__ int32_t tag_s[PF_TAGS];
     __shared__ float tag_floor_s[PF_TAGS];
     __shared__ int wcnt[32];
     __shared__ unsigned long long base_s;
     __shared__ int64_t tile_s;
     griddep_wait();
+    if (done && done[0] == 1) return;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const float floor_ = *floor_p, umax = ext_umax(rb.ext);
     int n_tags = 0;
@@ -1327,7 +1329,7 @@ cudaError_t launch_keep(const HopPlan &p, const RowBounds &rb, const float *floo
                                st, rb, floor_p, f, p.in_ptr, p.split.split_t, p.n_split_rows,
                                p.split_row, p.n_segs, p.seg_slot, p.slot_split, split_skip,
                                kept_rows, kept_segs, (unsigned long long *)kept_count, chain,
-                               status);
+                               status, p.done);
     if (launches) *launches += 1;
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
@@ -1462,9 +1464,11 @@ __global__ __launch_bounds__(256, WIDTH > 1 ? 2 : 3) void k_hop_rows(const int64
                                                   const int32_t *__restrict__ split_skip,
                                                   const int32_t *__restrict__ kept_rows,
                                                   const int64_t *__restrict__ kept_count,
-                                                  int *__restrict__ queue) {
+                                                  int *__restrict__ queue,
+                                                  const int32_t *__restrict__ done) {
     using S = HopShape<BP>;
     griddep_wait();
+    if (done && done[0] == 1) return;
     const int lane = threadIdx.x & 31;
     const int sub = lane % S::LW;
     // with the skip (last hop), the rows kept whole that reach the floor
@@ -1557,9 +1561,11 @@ __global__ __launch_bounds__(256, WIDTH > 1 ? 2 : 3) void k_hop_segs(const int64
                                                   float4 *__restrict__ part4,
                                                   const int32_t *__restrict__ kept_segs,
                                                   const int64_t *__restrict__ kept_count,
-                                                  int *__restrict__ queue) {
+                                                  int *__restrict__ queue,
+                                                  const int32_t *__restrict__ done) {
     using S = HopShape<BP>;
     griddep_wait();
+    if (done && done[0] == 1) return;
     const int lane = threadIdx.x & 31;
     const int sub = lane % S::LW;
     // last hop: only the listed segments (those of unpruned split rows)
@@ -1596,7 +1602,7 @@ static cudaError_t hop_bp(const HopPlan &p, const float *u, const float *in, flo
         e = launch_pdl(prune ? k_hop_segs<BP, 2> : k_hop_segs<BP>, dim3(g2), dim3(256), 0, st,
                        p.seg_e0, p.seg_e1, p.seg_slot, p.n_segs, p.in_src, p.in_w,
                        (const float4 *)in, (float4 *)partial, prune ? hbp->kept_segs : nullptr,
-                       prune ? hbp->kept_count + 1 : nullptr, counters + 1);
+                       prune ? hbp->kept_count + 1 : nullptr, counters + 1, p.done);
         if (e != cudaSuccess) return e;
         if (launches) *launches += 1;
     }
@@ -1612,7 +1618,8 @@ static cudaError_t hop_bp(const HopPlan &p, const float *u, const float *in, flo
                    (const float4 *)u, (const float4 *)in, (float4 *)out, alpha, p.split.split_t,
                    p.n_split_rows, p.split_order, p.split_row, p.split_slot0,
                    (const float4 *)partial, f, prune ? hbp->split_skip : nullptr,
-                   prune ? hbp->kept_rows : nullptr, prune ? hbp->kept_count : nullptr, counters);
+                   prune ? hbp->kept_rows : nullptr, prune ? hbp->kept_count : nullptr, counters,
+                   p.done);
     if (launches) *launches += 1;
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
@@ -1652,10 +1659,11 @@ __global__ __launch_bounds__(256, BP >= 256 ? 2 : BP >= 128 ? 3 : 4) void k_hop_
     const int64_t *__restrict__ in_ptr, const int32_t *__restrict__ in_src,
     const float *__restrict__ in_w, int64_t n_sample, int64_t stride, int64_t max_edges,
     const float4 *__restrict__ u4, const float4 *__restrict__ in4, float alpha, const NsScope ns,
-    uint32_t *__restrict__ keysT) {
+    uint32_t *__restrict__ keysT, const int32_t *__restrict__ done) {
     using S = HopShape<BP>;
     __shared__ uint32_t tile[SMP_ROWS][BP + 1];
     griddep_wait();
+    if (done && done[0] == 1) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane % S::LW;
     const int64_t v0 = (int64_t)blockIdx.x * SMP_ROWS;
     static_assert(SMP_ROWS == 8, "a row a warp");
@@ -1700,7 +1708,7 @@ cudaError_t launch_hop_sample(const HopPlan &p, const SelectPlan &sp, const floa
                           dim3(256), 0, st, p.in_ptr, p.in_src, p.in_w, sp.n_sample, sp.stride,
                           p.n_split_rows >= sp.k && SMP_EDGES < p.split.split_t
                               ? SMP_EDGES : p.split.split_t,
-                          (const float4 *)u, (const float4 *)in, alpha, ns, keysT);
+                          (const float4 *)u, (const float4 *)in, alpha, ns, keysT, p.done);
     };
     cudaError_t e = cudaErrorInvalidValue;
     switch (sp.bp) {

@@ -19,14 +19,15 @@
 namespace ak {
 
 // ------------------------------------------------------------------ graph-only
-// Candidates: the REACH_T rows of largest upper mass sum_{t<=H} mup[t]
-// among the (up to 1024) heaviest split rows; ties to the lower row.  One
+// Candidates: the REACH_T rows of largest upper mass mup[1] + mup[2] among
+// the (up to 1024) heaviest split rows, whatever the hop count (so that the
+// levels of one hop count serve the others); ties to the lower row.  One
 // CTA of 1024 threads, bitonic sort of the keys in shared memory.
 __global__ __launch_bounds__(1024) void k_reach_pick(const int32_t *__restrict__ split_row,
                                                       const int32_t *__restrict__ split_order,
                                                       int64_t n_split,
                                                       const float *__restrict__ mup, int64_t n,
-                                                      int H, int32_t *__restrict__ rows,
+                                                      int32_t *__restrict__ rows,
                                                       int *__restrict__ t_out) {
     __shared__ unsigned long long key[1024];
     const int tid = threadIdx.x;
@@ -34,8 +35,7 @@ __global__ __launch_bounds__(1024) void k_reach_pick(const int32_t *__restrict__
     unsigned long long k = 0ull;
     if (tid < nc) {
         const int32_t r = split_row[split_order[tid]];
-        float m = 0.f;
-        for (int t = 1; t <= H; ++t) m += mup[(int64_t)t * n + r];
+        const float m = mup[n + r] + mup[2 * n + r];
         k = ((unsigned long long)__float_as_uint(m) << 32) | (unsigned long long)(~(uint32_t)r);
     }
     key[tid] = k;
@@ -99,20 +99,20 @@ __global__ void k_reach_spmm(const int64_t *__restrict__ row_ptr, const int32_t 
     }
 }
 
-cudaError_t launch_reach_build(const ReachBuild &rb, cudaStream_t st) {
-    const int sms = device_sm_count();
+cudaError_t launch_reach_pick(const ReachBuild &rb, float *C1, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(rb.map, 0xff, (size_t)rb.n * 4, st);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(rb.C, 0, (size_t)rb.H * rb.n * REACH_T * 4, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(C1, 0, (size_t)rb.n * REACH_T * 4, st);
     if (e != cudaSuccess) return e;
-    k_reach_pick<<<1, 1024, 0, st>>>(rb.split_row, rb.split_order, rb.n_split, rb.mup, rb.n, rb.H,
+    k_reach_pick<<<1, 1024, 0, st>>>(rb.split_row, rb.split_order, rb.n_split, rb.mup, rb.n,
                                      rb.rows, rb.t_cnt);
     k_reach_map<<<1, REACH_T, 0, st>>>(rb.rows, rb.t_cnt, rb.map);
-    k_reach_c1<<<REACH_T, 256, 0, st>>>(rb.rows, rb.t_cnt, rb.in_ptr, rb.in_src, rb.in_w, rb.C);
-    for (int t = 2; t <= rb.H; ++t)
-        k_reach_spmm<<<sms * 8, 256, 0, st>>>(rb.row_ptr, rb.col, rb.w, rb.row_of, rb.n,
-                                              rb.C + (int64_t)(t - 2) * rb.n * REACH_T,
-                                              rb.C + (int64_t)(t - 1) * rb.n * REACH_T);
+    k_reach_c1<<<REACH_T, 256, 0, st>>>(rb.rows, rb.t_cnt, rb.in_ptr, rb.in_src, rb.in_w, C1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reach_level(const ReachBuild &rb, const float *Cp, float *Cn, cudaStream_t st) {
+    k_reach_spmm<<<device_sm_count() * 8, 256, 0, st>>>(rb.row_ptr, rb.col, rb.w, rb.row_of, rb.n,
+                                                        Cp, Cn);
     return cudaGetLastError();
 }
 
@@ -235,6 +235,8 @@ __global__ __launch_bounds__(256) void k_reach_flags(const ReachFlags f) {
     if (threadIdx.x < REACH_T) kf[threadIdx.x] = vk[threadIdx.x];
     __syncthreads();
     reach_build_plan(kf, *(volatile int *)bad, *f.t_cnt, f.k, f.plan);
+    if (f.outcome && threadIdx.x == REACH_T - 1)       // (the thread that wrote plan[0])
+        *(volatile int32_t *)f.outcome = f.plan[0] ? 1 : 2;
 }
 
 cudaError_t launch_reach_flags(const ReachFlags &f, cudaStream_t st, int *launches) {
@@ -498,7 +500,7 @@ __global__ __launch_bounds__(RM_THREADS, 1) void k_reach_mma(
 // hi + lo, zero for k >= n.  One CTA per 64 rows k: the rows' slots are
 // read contiguously (coalesced), transposed through shared memory and
 // written along k (coalesced).
-__global__ __launch_bounds__(256) void k_reach_pack(const float *__restrict__ C, int64_t n,
+__global__ __launch_bounds__(256) void k_reach_pack(const ReachLevels C, int64_t n,
                                                     int64_t n_pad, int H, float alpha,
                                                     uint16_t *__restrict__ hi,
                                                     uint16_t *__restrict__ lo) {
@@ -510,7 +512,7 @@ __global__ __launch_bounds__(256) void k_reach_pack(const float *__restrict__ C,
         float c = 0.f;
         if (k < n) {
             const int64_t at = k * REACH_T + i;
-            for (int t = H; t >= 1; --t) c = alpha * (c + C[(int64_t)(t - 1) * n * REACH_T + at]);
+            for (int t = H; t >= 1; --t) c = alpha * (c + C.level[t - 1][at]);
         }
         tile[kk][i] = c;
     }
@@ -528,14 +530,17 @@ __global__ __launch_bounds__(256) void k_reach_pack(const float *__restrict__ C,
 
 // Final score of each flagged candidate for each real query column: its u
 // plus the CTAs' partials, appended as a filter key (score bits, ~chunk ID)
-// to the column's buffer; the buffer then holds exactly them.  bp / 64
-// blocks per candidate slot of the plan, each on 64 query columns (blocks
+// to the column's buffer; the buffer then holds exactly them.  bp / Q
+// blocks per candidate slot of the plan, each on Q query columns (blocks
 // past nk, and every block when the plan says the hops run, return at
-// once): thread t takes column t % 64 of its block's and every 16th
-// partial from t / 64 on (coalesced rows of the partials), and the groups
+// once): thread t takes column t % Q of its block's and every G-th
+// partial from t / Q on (coalesced rows of the partials), and the groups
 // are added in group order (the same order on every run).
-constexpr int EMIT_Q = 64, EMIT_G = 1024 / EMIT_Q;
-__global__ __launch_bounds__(1024) void k_reach_emit(const uint16_t *__restrict__ u_hi,
+// F32: u is fp32 in `u` (32 query columns a block) and the partials are of
+// u - Lmin; else split bf16 in u_hi, u_lo (64 columns).
+template <bool F32>
+__global__ __launch_bounds__(1024) void k_reach_emit(const float *__restrict__ u,
+                                                     const uint16_t *__restrict__ u_hi,
                                                      const uint16_t *__restrict__ u_lo, int bp, int B,
                                                      const float *__restrict__ partial,
                                                      int n_parts, const int32_t *__restrict__ plan,
@@ -543,29 +548,37 @@ __global__ __launch_bounds__(1024) void k_reach_emit(const uint16_t *__restrict_
                                                      const int32_t *__restrict__ ext_of,
                                                      unsigned int *__restrict__ cnt,
                                                      unsigned long long *__restrict__ buf,
-                                                     int64_t cap) {
+                                                     int64_t cap, const double *__restrict__ sums,
+                                                     const unsigned int *__restrict__ ext) {
+    constexpr int Q = F32 ? 32 : 64, G = 1024 / Q;
     __shared__ float red[1024];
     griddep_wait();
     if (plan[0] == 0) return;
     const int nk = plan[1];
-    const int qb_n = bp / EMIT_Q;
+    const int qb_n = bp / Q;
     const int i = blockIdx.x / qb_n;
     if (i >= nk) return;
     const int slot = plan[2 + i];
-    const int b = (blockIdx.x % qb_n) * EMIT_Q + threadIdx.x % EMIT_Q;
-    const int g = threadIdx.x / EMIT_Q;
+    const int b = (blockIdx.x % qb_n) * Q + threadIdx.x % Q;
+    const int g = threadIdx.x / Q;
     float acc = 0.f;
+    if (!F32 || b < B) {   // (the fp32 pass writes the real columns only)
 #pragma unroll 4
-    for (int p = g; p < n_parts; p += EMIT_G) acc += partial[((int64_t)p * REACH_T + slot) * bp + b];
+        for (int p = g; p < n_parts; p += G) acc += partial[((int64_t)p * REACH_T + slot) * bp + b];
+    }
     red[threadIdx.x] = acc;
     __syncthreads();
     if (g == 0 && b < B) {
         float sum = red[threadIdx.x];
-        for (int h = 1; h < EMIT_G; ++h) sum += red[h * EMIT_Q + threadIdx.x];
+        for (int h = 1; h < G; ++h) sum += red[h * Q + threadIdx.x];
         const int64_t j = rows[slot];
-        const float uj = __bfloat162float(__ushort_as_bfloat16(u_hi[j * bp + b])) +
-                         __bfloat162float(__ushort_as_bfloat16(u_lo[j * bp + b]));
-        const float s = uj + sum;
+        const float uj = F32 ? u[j * bp + b]
+                             : __bfloat162float(__ushort_as_bfloat16(u_hi[j * bp + b])) +
+                                   __bfloat162float(__ushort_as_bfloat16(u_lo[j * bp + b]));
+        // (F32: the partials are of u - Lmin)
+        const float s = F32 ? (float)((double)uj + ((double)ext_lmin(ext) * sums[slot] +
+                                                    (double)sum))
+                            : uj + sum;
         buf[(int64_t)b * cap + i] = ((unsigned long long)__float_as_uint(s) << 32) |
                                     (unsigned long long)(~(uint32_t)ext_of[j]);
         if (i == 0) cnt[b] = (unsigned int)nk;
@@ -577,7 +590,7 @@ int reach_parts() { return device_sm_count(); }
 int64_t reach_pad_rows(int64_t n) { return (n + RM_BK - 1) / RM_BK * RM_BK; }
 
 
-cudaError_t launch_reach_pack(const float *C, int64_t n, int H, float alpha, uint16_t *coef_hi,
+cudaError_t launch_reach_pack(const ReachLevels &C, int64_t n, int H, float alpha, uint16_t *coef_hi,
                               uint16_t *coef_lo, cudaStream_t st) {
     const int64_t n_pad = reach_pad_rows(n);
     if (n_pad <= 0) return cudaSuccess;
@@ -639,9 +652,258 @@ cudaError_t launch_reach_scores(const uint16_t *u_hi, const uint16_t *u_lo, int 
                               : reach_mma_bp<128>(coef_hi, coef_lo, u_hi, u_lo, n, plan, partial,
                                                   parts, status, st);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(k_reach_emit, dim3(REACH_T * (bp / EMIT_Q)), dim3(1024), 0, st, u_hi, u_lo, bp, B,
-                   (const float *)partial, parts, plan, rows, ext_of, cnt, buf, cap);
+    e = launch_pdl(k_reach_emit<false>, dim3(REACH_T * (bp / 64)), dim3(1024), 0, st,
+                   (const float *)nullptr, u_hi, u_lo, bp, B, (const float *)partial, parts, plan,
+                   rows, ext_of, cnt, buf, cap, (const double *)nullptr,
+                   (const unsigned int *)nullptr);
     if (launches) *launches += 2;
+    return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
+// ------------------------------------------------------------------ fp32 terms
+// The same partial sums in fp32 on the CUDA cores, for the calls that had run
+// the hops in fp32: three hops and more, and batches of at most 64 queries.
+// (Split-bf16 products would take their error from ~1e-7 to ~6e-6.)
+//   sum_k coef[k][i] u[k][b] = m S_i + sum_k coef[k][i] (u[k][b] - m)
+// with m = Lmin, the smallest u of any live row and real query, and S_i the
+// coefficients' sum in 64 bits: u - m is exact where u <= 2 m, every term
+// stays >= 0, and the terms are as much smaller as u is flat, and the sums'
+// rounding with them.  (Plain sums of nearly equal terms all round the same
+// way: three hops on 262,144 chunks were 1.4e-6 off, 3e-8 so, 2.8e-7 the hops.)
+// Bound by the loads for few queries (64 coefficients and the query columns a
+// row) and by the FMAs for many: n * 64 * columns of them, 96 or 128 where
+// flagged slots lie there.  The hops gather nnz columns a hop instead, an
+// order of magnitude more, from L2.
+// A warp works alone: it takes groups of RF_ROWS rows, copies their
+// coefficients and query columns into its own ring of RF_STAGES stages
+// (cp.async), and keeps an ST-slot x CT-column tile of sums in registers, a
+// lane's part SPL slots x CPL columns: SPL * CPL FMAs a row for (SPL + CPL) / 4
+// 16-byte shared loads of four cycles each, which is why the wide batches take
+// 16 x 8 (8 x 8 ran at 47% of the FMA rate).  The eight warps' tiles, then the
+// CTAs' partials, are added in a fixed order.
+constexpr int RF_ROWS = 8, RF_STAGES = 4, RF_WARPS = 8;
+
+template <int ST, int CT>
+struct RfCfg {
+    static constexpr int SPL = CT == 64 ? ST / 4 : (ST * CT == 512 ? 4 : 8);
+    static constexpr int SG = ST / SPL, CG = 32 / SG;           // lanes over slots, columns
+    static constexpr int CPL = CT / CG;
+    static constexpr int STAGE = RF_ROWS * (ST + CT);           // floats a stage
+    static constexpr int SMEM = RF_WARPS * RF_STAGES * STAGE * 4;
+    static constexpr int CTAS = SPL * CPL > 64 ? 1 : 2;         // an SM
+    static_assert(SPL % 4 == 0 && CPL % 4 == 0 && SG * CG == 32, "16-byte shared loads");
+    static_assert(RF_WARPS * ST * CT * 4 <= SMEM, "the tiles' sum reuses the rings");
+};
+
+__device__ __forceinline__ void cp_async16(float *dst, const float *src, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src),
+                 "r"(valid ? 16 : 0)
+                 : "memory");
+}
+
+template <int ST, int CT>
+__global__ __launch_bounds__(RF_WARPS * 32, RfCfg<ST, CT>::CTAS) void k_reach_fma(
+    const float *__restrict__ u, int bp, int64_t n, const float *__restrict__ coef, int slot0,
+    const int32_t *__restrict__ plan, const unsigned int *__restrict__ ext,
+    float *__restrict__ partial) {
+    using C = RfCfg<ST, CT>;
+    extern __shared__ float4 rf_smem[];
+    float *smem = reinterpret_cast<float *>(rf_smem);
+    griddep_wait();
+    if (plan[0] == 0) return;
+    const int s0 = slot0 + (int)blockIdx.y * ST;       // slots s0 .. s0 + ST - 1
+    if (plan[1 + plan[1]] < s0) return;                // the last flagged slot is below
+    const float m = ext_lmin(ext);
+    const int c0 = blockIdx.z * CT;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int sg = lane % C::SG, cg = lane / C::SG;
+    float *ring = smem + warp * RF_STAGES * C::STAGE;
+    const int64_t groups = (n + RF_ROWS - 1) / RF_ROWS;
+    const int64_t per = (groups + gridDim.x - 1) / gridDim.x;
+    const int64_t g0 = (int64_t)blockIdx.x * per + warp;
+    const int64_t g1 = min((int64_t)(blockIdx.x + 1) * per, groups);
+    auto load = [&](int64_t g, int stage) {
+        float *cs = ring + stage * C::STAGE, *us = cs + RF_ROWS * ST;
+#pragma unroll
+        for (int i = 0; i < RF_ROWS * ST / 128; ++i) {
+            const int c = lane + 32 * i, r = c / (ST / 4);
+            const int64_t row = g * RF_ROWS + r;
+            const bool ok = row < n;
+            cp_async16(cs + c * 4, coef + (ok ? row : 0) * REACH_T + s0 + (c % (ST / 4)) * 4, ok);
+        }
+#pragma unroll
+        for (int i = 0; i < (RF_ROWS * CT / 4 + 31) / 32; ++i) {
+            const int c = lane + 32 * i, r = c / (CT / 4);
+            const int64_t row = g * RF_ROWS + r;
+            const bool ok = row < n;
+            if (RF_ROWS * CT / 4 >= 32 || c < RF_ROWS * CT / 4)
+                cp_async16(us + c * 4, u + (ok ? row : 0) * bp + c0 + (c % (CT / 4)) * 4, ok);
+        }
+    };
+    float acc[C::SPL][C::CPL];
+#pragma unroll
+    for (int i = 0; i < C::SPL; ++i)
+#pragma unroll
+        for (int j = 0; j < C::CPL; ++j) acc[i][j] = 0.f;
+    int64_t gl = g0;                                   // next group to load
+#pragma unroll
+    for (int s = 0; s < RF_STAGES - 1; ++s, gl += RF_WARPS) {
+        if (gl < g1) load(gl, s);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    int stage = 0, next = RF_STAGES - 1;
+    for (int64_t g = g0; g < g1; g += RF_WARPS, gl += RF_WARPS) {
+        if (gl < g1) load(gl, next);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group %0;" ::"n"(RF_STAGES - 1) : "memory");
+        __syncwarp();
+        const float *cs = ring + stage * C::STAGE, *us = cs + RF_ROWS * ST;
+#pragma unroll
+        for (int r = 0; r < RF_ROWS; ++r) {
+            float a[C::SPL], x[C::CPL];
+#pragma unroll
+            for (int i = 0; i < C::SPL / 4; ++i)
+                *reinterpret_cast<float4 *>(a + 4 * i) =
+                    *reinterpret_cast<const float4 *>(cs + r * ST + (i * C::SG + sg) * 4);
+#pragma unroll
+            for (int j = 0; j < C::CPL / 4; ++j)
+                *reinterpret_cast<float4 *>(x + 4 * j) =
+                    *reinterpret_cast<const float4 *>(us + r * CT + (j * C::CG + cg) * 4);
+#pragma unroll
+            for (int j = 0; j < C::CPL; ++j) x[j] -= m;   // (rows past n have coefficient 0)
+#pragma unroll
+            for (int i = 0; i < C::SPL; ++i)
+#pragma unroll
+                for (int j = 0; j < C::CPL; ++j) acc[i][j] = fmaf(a[i], x[j], acc[i][j]);
+        }
+        __syncwarp();   // the stage is free for the next round's copies
+        if (++stage == RF_STAGES) stage = 0;
+        if (++next == RF_STAGES) next = 0;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    // the warps' tiles through shared memory, added in warp order
+    float *mine = smem + warp * ST * CT;
+#pragma unroll
+    for (int i = 0; i < C::SPL; ++i)
+#pragma unroll
+        for (int j = 0; j < C::CPL; j += 4)
+            *reinterpret_cast<float4 *>(mine + ((i / 4 * C::SG + sg) * 4 + i % 4) * CT +
+                                        (j / 4 * C::CG + cg) * 4) =
+                make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]);
+    __syncthreads();
+    for (int x = threadIdx.x; x < ST * CT; x += RF_WARPS * 32) {
+        float s = smem[x];
+#pragma unroll
+        for (int w = 1; w < RF_WARPS; ++w) s += smem[w * ST * CT + x];
+        partial[((int64_t)blockIdx.x * REACH_T + s0 + x / CT) * bp + c0 + x % CT] = s;
+    }
+}
+
+// coef[k][i] = sum_t alpha^t C_t[k][i] (Horner over t), fp32, and its column
+// sums in 64 bits: each CTA's in part[cta][i], added in CTA order by
+// k_reach_colsum.  128 threads a row.
+__global__ __launch_bounds__(256) void k_reach_combine(const ReachLevels C, int64_t n, int H,
+                                                       float alpha, float *__restrict__ coef,
+                                                       double *__restrict__ part) {
+    __shared__ double half[REACH_T];
+    const int i = threadIdx.x % REACH_T, h = threadIdx.x / REACH_T;
+    double s = 0.0;
+    for (int64_t k = (int64_t)blockIdx.x * 2 + h; k < n; k += (int64_t)gridDim.x * 2) {
+        float c = 0.f;
+        for (int t = H; t >= 1; --t) c = alpha * (c + C.level[t - 1][k * REACH_T + i]);
+        coef[k * REACH_T + i] = c;
+        s += (double)c;
+    }
+    if (h == 1) half[i] = s;
+    __syncthreads();
+    if (h == 0) part[(int64_t)blockIdx.x * REACH_T + i] = s + half[i];
+}
+__global__ __launch_bounds__(REACH_T) void k_reach_colsum(const double *__restrict__ part,
+                                                          int n_parts, double *__restrict__ sum) {
+    double s = 0.0;
+    for (int p = 0; p < n_parts; ++p) s += part[(int64_t)p * REACH_T + threadIdx.x];
+    sum[threadIdx.x] = s;
+}
+
+static int combine_ctas() { return device_sm_count() * 8; }
+int64_t reach_sum_words() { return (int64_t)REACH_T * (1 + combine_ctas()); }
+
+cudaError_t launch_reach_combine(const ReachLevels &C, int64_t n, int H, float alpha, float *coef,
+                                 double *sums, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    k_reach_combine<<<combine_ctas(), 256, 0, st>>>(C, n, H, alpha, coef, sums + REACH_T);
+    k_reach_colsum<<<1, REACH_T, 0, st>>>(sums + REACH_T, combine_ctas(), sums);
+    return cudaGetLastError();
+}
+
+// Columns of a warp's tile, and CTAs along the rows: as many as the SMs hold at
+// a time over all column tiles, at least a group of rows a warp.
+static int fma_columns(int B) { return B <= 8 ? 8 : (B <= 16 ? 16 : (B <= 32 ? 32 : 64)); }
+int reach_fma_parts(int64_t n, int B) {
+    const int ct = fma_columns(B);
+    const int64_t most = ceil_div<int64_t>(n, RF_ROWS * RF_WARPS);
+    const int64_t want = ceil_div<int64_t>((ct == 64 ? 1 : 2) * device_sm_count(),
+                                           ceil_div<int64_t>(B, ct));
+    return (int)(want < most ? want : most);
+}
+
+template <int ST, int CT>
+static cudaError_t reach_fma_tile(const float *u, int bp, int B, int64_t n, const float *coef,
+                                  int slot0, const int32_t *plan, const unsigned int *ext,
+                                  float *partial, int parts, cudaStream_t st) {
+    static bool attr[64] = {false};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !attr[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(k_reach_fma<ST, CT>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             RfCfg<ST, CT>::SMEM);
+        if (e != cudaSuccess) return e;
+        attr[dev] = true;
+    }
+    const int slots = slot0 == 0 ? 64 : REACH_T - slot0;
+    return launch_pdl(k_reach_fma<ST, CT>, dim3(parts, slots / ST, (B + CT - 1) / CT),
+                      dim3(RF_WARPS * 32), RfCfg<ST, CT>::SMEM, st, u, bp, n, coef, slot0, plan,
+                      ext, partial);
+}
+
+// Slots 0..63, then the two groups of 32 above (CTAs of a group without a
+// flagged slot return at once).
+cudaError_t launch_reach_fma(const float *u, int bp, int B, int64_t n, const float *coef,
+                             const double *sums, const unsigned int *ext, const int32_t *plan,
+                             const int32_t *rows, const int32_t *ext_of, float *partial,
+                             unsigned int *cnt, unsigned long long *buf, int64_t cap,
+                             cudaStream_t st, int *launches) {
+    if (n <= 0 || B < 1 || B > bp || bp % 32 != 0 || (B > 32 && bp % 64 != 0))
+        return cudaErrorInvalidValue;
+    const int parts = reach_fma_parts(n, B);
+    cudaError_t e;
+#define RF_TILE(ST, CT, S0) reach_fma_tile<ST, CT>(u, bp, B, n, coef, S0, plan, ext, partial, parts, st)
+    switch (fma_columns(B)) {
+    case 8:
+        e = RF_TILE(64, 8, 0);
+        if (e == cudaSuccess) e = RF_TILE(32, 16, 64);   // (bp >= 32: columns 8..15 exist)
+        break;
+    case 16:
+        e = RF_TILE(64, 16, 0);
+        if (e == cudaSuccess) e = RF_TILE(32, 16, 64);
+        break;
+    case 32:
+        e = RF_TILE(64, 32, 0);
+        if (e == cudaSuccess) e = RF_TILE(32, 32, 64);
+        break;
+    default:
+        e = RF_TILE(64, 64, 0);
+        if (e == cudaSuccess) e = RF_TILE(32, 64, 64);
+        break;
+    }
+#undef RF_TILE
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(k_reach_emit<true>, dim3(REACH_T * (bp / 32)), dim3(1024), 0, st, u,
+                   (const uint16_t *)nullptr, (const uint16_t *)nullptr, bp, B,
+                   (const float *)partial, parts, plan, rows, ext_of, cnt, buf, cap, sums, ext);
+    if (launches) *launches += 3;
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 

@@ -176,7 +176,8 @@ constexpr int KTH_CBUF = 4096;                    // keys kept after the first d
 
 __global__ __launch_bounds__(SEL_THREADS) void k_sample_kth(
     const uint32_t *__restrict__ keysT, int64_t n_sample, int b, int k, uint32_t slack,
-    unsigned long long *__restrict__ bound, unsigned int *__restrict__ cnt) {
+    unsigned long long *__restrict__ bound, unsigned int *__restrict__ cnt,
+    const int32_t *__restrict__ done) {
     extern __shared__ uint32_t kst[];                 // [n_sample] when staged
     __shared__ int hist[KTH_REP * 256];
     __shared__ int wsum[SEL_THREADS / 32];
@@ -185,6 +186,7 @@ __global__ __launch_bounds__(SEL_THREADS) void k_sample_kth(
     __shared__ uint32_t s_prefix;
     __shared__ int s_rem, s_match, s_cn;
     griddep_wait();
+    if (done && done[0] == 1) return;
     const int c = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (c >= b) {   // padding column: nothing passes the filter
         if (tid == 0) {
@@ -729,11 +731,13 @@ constexpr int PF_ROWS = 1024;
 __global__ __launch_bounds__(PF_ROWS) void k_prune_floor(
     unsigned long long *__restrict__ bound, int n_real, const RowBounds rb,
     const int32_t *__restrict__ lb_rows, const int32_t *__restrict__ order, int64_t n_rows,
-    int k, float *__restrict__ floor_out, unsigned long long *__restrict__ zero, int64_t n_zero) {
+    int k, float *__restrict__ floor_out, unsigned long long *__restrict__ zero, int64_t n_zero,
+    const int32_t *__restrict__ done) {
     __shared__ unsigned long long xk[2][PF_ROWS];
     __shared__ unsigned int s_min;
     __shared__ float s_floor;
     griddep_wait();
+    if (done && done[0] == 1) return;
     const int t = threadIdx.x;
     if (t == 0) s_min = 0x7f800000u;
     for (int64_t i = t; i < n_zero; i += PF_ROWS) zero[i] = 0ull;
@@ -930,10 +934,10 @@ cudaError_t launch_ns_floors(unsigned long long *bound, const int32_t *q_ns, int
 cudaError_t launch_prune_floor(unsigned long long *bound, int n_real, const RowBounds &rb,
                                const int32_t *lb_rows, const int32_t *order, int64_t n_lb_rows,
                                int k, float *floor_out, unsigned long long *zero, int64_t n_zero,
-                               cudaStream_t st) {
+                               const int32_t *done, cudaStream_t st) {
     if (n_lb_rows > PF_ROWS || n_real > PF_ROWS || k < 1) return cudaErrorInvalidValue;
     cudaError_t e = launch_pdl(k_prune_floor, dim3(1), dim3(PF_ROWS), 0, st, bound, n_real, rb,
-                               lb_rows, order, n_lb_rows, k, floor_out, zero, n_zero);
+                               lb_rows, order, n_lb_rows, k, floor_out, zero, n_zero, done);
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
@@ -942,7 +946,7 @@ template <bool SIGNED>
 static cudaError_t launch_kth(const SelectPlan &sp, const float *s, int b, const int32_t *ext_of,
                               int64_t id_limit, unsigned long long *ws, unsigned long long *bound,
                               unsigned int *cnt, cudaStream_t st, uint32_t slack = 0,
-                              NsScope ns = NsScope{}) {
+                              NsScope ns = NsScope{}, const int32_t *done = nullptr) {
     static bool attr[64] = {false};
     int dev = 0;
     cudaGetDevice(&dev);
@@ -963,7 +967,7 @@ static cudaError_t launch_kth(const SelectPlan &sp, const float *s, int b, const
     }
     const size_t smem = sp.n_sample <= KTH_STAGE ? (size_t)sp.n_sample * sizeof(uint32_t) : 0;
     e = launch_pdl(k_sample_kth, dim3(sp.bp), dim3(SEL_THREADS), smem, st,
-                   (const uint32_t *)keysT, sp.n_sample, b, sp.k, slack, bound, cnt);
+                   (const uint32_t *)keysT, sp.n_sample, b, sp.k, slack, bound, cnt, done);
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
@@ -998,9 +1002,9 @@ static cudaError_t sample_bound(const SelectPlan &sp, const float *s, int b,
                                 const int32_t *ext_of, int64_t id_limit,
                                 unsigned long long *ws, unsigned long long *bound,
                                 cudaStream_t st, int *launches, uint32_t slack = 0,
-                                NsScope ns = NsScope{}) {
+                                NsScope ns = NsScope{}, const int32_t *done = nullptr) {
     cudaError_t e = launch_kth<SIGNED>(sp, s, b, ext_of, id_limit, ws, bound,
-                                       (unsigned int *)(ws + sp.off_cnt), st, slack, ns);
+                                       (unsigned int *)(ws + sp.off_cnt), st, slack, ns, done);
     if (launches) *launches += s ? 2 : 1;
     return e;
 }
@@ -1014,9 +1018,9 @@ cudaError_t launch_sample_bound_signed(const SelectPlan &sp, const float *s, int
 
 cudaError_t launch_sample_bound(const SelectPlan &sp, const float *s, int b,
                                 const int32_t *ext_of, unsigned long long *ws, cudaStream_t st,
-                                int *launches, uint32_t slack, NsScope ns) {
+                                int *launches, uint32_t slack, NsScope ns, const int32_t *done) {
     return sample_bound<false>(sp, s, b, ext_of, (int64_t)1 << 40, ws, ws + sp.off_bound, st,
-                               launches, slack, ns);
+                               launches, slack, ns, done);
 }
 
 cudaError_t launch_select(const SelectPlan &sp, const float *s, int b, unsigned long long *ws,

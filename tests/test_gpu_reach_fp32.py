@@ -1,0 +1,85 @@
+"""Two to four hops from reach coefficients in fp32 (batches of at most 64
+queries, or three hops and more): the path is taken once the hops have run
+often enough on one graph, selects what the hops select, and its scores agree
+with theirs to fp32 rounding; a graph whose candidates do not suffice goes
+through the hops."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import synth
+from _parity import assert_retrieval_parity, gpu_retrieve, gpu_store, oracle_retrieve
+
+pytestmark = pytest.mark.gpu
+
+# fp32 sums of non-negative terms in two orders: at most a few hundred
+# roundings on any path (a warp's rows, the warps, the CTAs; a hop's
+# segments), 2^-24 each, and three levels of coefficients
+REL = 1e-5
+
+
+def _launches(store, wl, q):
+    store.set_profiling(True)
+    store.phase_times()
+    _, out = gpu_retrieve(wl, "clustered", store=store, queries=q)
+    ph = store.phase_times()
+    store.set_profiling(False)
+    return out, ph["last_hop"][1]
+
+
+@pytest.mark.parametrize("n,B,hops,k", [
+    (16384, 1, 2, 32),          # one column tile of 8
+    (16383, 9, 2, 8),           # 16 columns, ragged rows
+    (16384, 33, 2, 32),         # two tiles of 32
+    (9001, 64, 3, 16),
+    (16384, 200, 3, 64),        # both halves of the candidates
+    (16001, 256, 4, 5),
+])
+def test_equals_the_hops(n, B, hops, k, monkeypatch):
+    base = synth.workload(2, scale=1 / 64)
+    rp = base.row_ptr[:n + 1]
+    keep = base.col[:rp[-1]] < n
+    new_rp = np.concatenate([[0], np.cumsum(np.add.reduceat(keep, rp[:-1].astype(np.int64)))])
+    wl = dataclasses.replace(base, emb=base.emb[:n], row_ptr=new_rp.astype(np.int64),
+                             col=base.col[:rp[-1]][keep], aff=base.aff[:rp[-1]][keep],
+                             page_of={"clustered": base.page_of["clustered"][:n]},
+                             component=base.component[:n], hops=hops, k=k)
+    q = wl.queries[:B]
+    monkeypatch.setenv("AKASHIC_REACH", "0")
+    _, ref = gpu_retrieve(wl, "clustered", queries=q)
+    monkeypatch.setenv("AKASHIC_REACH", "1")
+    store = gpu_store(wl, "clustered")
+    for _ in range(12):                      # the hops, until the coefficients pay
+        got, launches = _launches(store, wl, q)
+    assert launches == 5, launches           # the candidates' three kernels before the hop's
+    hit = got["ids"] == ref["ids"]
+    assert hit.mean() > 0.99
+    np.testing.assert_allclose(got["scores"][hit], ref["scores"][hit], rtol=REL, atol=0)
+    assert_retrieval_parity(wl, "clustered", got, oracle_retrieve(wl, "clustered", queries=q))
+    # a change of the graph starts over with the hops
+    import torch
+    victims = got["ids"][0][:1].astype(np.int64)
+    store.delete(torch.from_numpy(victims).cuda())
+    got, launches = _launches(store, wl, q)
+    assert launches == 2 and victims[0] not in got["ids"]
+
+
+def test_candidates_that_do_not_suffice():
+    """300 rows of equal in-weight above the split limit: more rows reach the
+    floor than there are candidates, so every call goes through the hops."""
+    base = synth.workload(2, scale=1 / 64)
+    n = base.n
+    rng = np.random.default_rng(3)
+    hubs = np.sort(rng.choice(n, 300, replace=False))
+    col = np.sort(np.stack([rng.permutation(hubs)[:8] for _ in range(n)]), axis=1)
+    ok = col != np.arange(n)[:, None]
+    rp = np.concatenate([[0], np.cumsum(ok.sum(1))]).astype(np.int64)
+    wl = dataclasses.replace(base, row_ptr=rp, col=col[ok].astype(np.int32),
+                             aff=np.zeros(int(ok.sum()), np.float32), k=16, hops=2)
+    q = wl.queries[:20]
+    store = gpu_store(wl, "clustered")
+    ref = oracle_retrieve(wl, "clustered", queries=q)
+    for _ in range(24):
+        _, got = gpu_retrieve(wl, "clustered", store=store, queries=q)
+        assert_retrieval_parity(wl, "clustered", got, ref)
