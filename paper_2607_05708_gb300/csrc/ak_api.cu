@@ -80,8 +80,9 @@ struct DevBuf {
 };
 
 // Words of StreamScratch::words: u's extremes [2], the kept lists' lengths
-// (int64 [2]), the hops' work queues ([2] a hop).
-constexpr int CW_EXT = 0, CW_KEPT = 2, CW_QUEUE = 6, CW_COUNT = CW_QUEUE + 2 * AKASHIC_MAX_HOPS;
+// (int64 [2]), the hops' work queues ([2] a hop), the candidates' flags.
+constexpr int CW_EXT = 0, CW_KEPT = 2, CW_QUEUE = 6, CW_REACH = CW_QUEUE + 2 * AKASHIC_MAX_HOPS,
+              CW_COUNT = CW_REACH + REACH_WS;
 
 struct StreamScratch {
     DevBuf qp, shift, u, sa, sb, zpart, partial, cand;
@@ -91,10 +92,10 @@ struct StreamScratch {
     DevBuf rmax_u, rmin_u;       // u's row maxima / minima over the real queries
     DevBuf pfloor;               // the last hop's floor and what it keeps
     DevBuf skip_split, kept_rows, kept_segs, keep_chain;
-    DevBuf reach_keep, reach_part, reach_plan;   // flags + bad + done, partials, plan
+    DevBuf reach_part, reach_plan;   // the candidates' partials, the plan
     DevBuf nsf;                  // scoped last hop: tags, their floors, their count
     // every candidate's combined coefficients (bf16 hi, lo), and their key
-    DevBuf coef_hi, coef_lo;
+    DevBuf coef_hi, coef_lo, coef_sum;
     uint64_t coef_build = ~0ull;
     float coef_alpha = -1.f;
     int coef_H = 0;
@@ -105,7 +106,8 @@ struct StreamScratch {
     cudaEvent_t plan_ev = nullptr;
     // the fp32 pass: the combined coefficients and their key; the last
     // attempt's outcome (plan_host[2], written by the device) and its key
-    DevBuf coef_f, coef_sum;
+    DevBuf coef_f, cf_sum;
+    int64_t no_room_n = -1;      // rows at which the tables did not fit
     uint64_t cf_build = ~0ull, try_build = ~0ull;
     float cf_alpha = -1.f, try_alpha = -1.f;
     int cf_H = 0, try_H = 0, try_k = 0, try_skip = 0;
@@ -175,7 +177,7 @@ struct akashic_mem {
     int mass_levels = -1;
     int64_t mass_n = -1;      // rows they were computed for
     // reach coefficients of the candidate rows (ak_reach.cu), same lifetime
-    DevBuf reach_rows, reach_t, reach_map, reach_c[REACH_MAX_H];
+    DevBuf reach_rows, reach_t, reach_map, reach_pick, reach_c[REACH_MAX_H];
     int reach_levels = -1;    // levels C_1.. in place (0 or less: no candidates either)
     int64_t reach_n = -1;     // rows they were computed for
     double hop_work = 0;      // query columns x hops run through the hops since the
@@ -1193,9 +1195,6 @@ static akashic_status_t ensure_reach(akashic_mem *m, const HopPlan &hp, int H, c
     if (m->reach_levels >= H && m->reach_n == n) return AKASHIC_OK;
     ReachBuild rb{};
     rb.n = n;
-    rb.n_split = m->n_split;
-    rb.split_row = hp.split_row;
-    rb.split_order = hp.split_order;
     rb.mup = m->mass_up.as<float>();
     rb.in_ptr = hp.in_ptr;
     rb.in_src = hp.in_src;
@@ -1208,11 +1207,13 @@ static akashic_status_t ensure_reach(akashic_mem *m, const HopPlan &hp, int H, c
         m->reach_levels = -1;
         AK_TRY(m->reach_rows.ensure(REACH_T * 4));
         AK_TRY(m->reach_t.ensure(16));
+        AK_TRY(m->reach_pick.ensure((size_t)reach_pick_words() * 8));
         AK_TRY(ensure_spare(m->reach_map, (size_t)n * 4));
         AK_TRY(ensure_spare(m->reach_c[0], (size_t)n * REACH_T * 4));
         rb.rows = m->reach_rows.as<int32_t>();
         rb.t_cnt = m->reach_t.as<int>();
         rb.map = m->reach_map.as<int32_t>();
+        rb.pick = m->reach_pick.as<unsigned long long>();
         CUDA_TRY(launch_reach_pick(rb, m->reach_c[0].as<float>(), st));
         m->reach_levels = 1;
         m->reach_n = n;
@@ -1231,6 +1232,14 @@ static ReachLevels reach_levels_of(const akashic_mem *m) {
     ReachLevels c{};
     for (int t = 0; t < REACH_MAX_H; ++t) c.level[t] = m->reach_c[t].as<float>();
     return c;
+}
+
+// The pinned words a stream's plans are read back through.
+static akashic_status_t plan_words(StreamScratch *sc) {
+    if (sc->plan_host) return AKASHIC_OK;
+    CUDA_TRY(cudaMallocHost((void **)&sc->plan_host, 16));
+    memset(sc->plan_host, 0, 16);
+    return AKASHIC_OK;
 }
 
 static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t B, int32_t k,
@@ -1298,21 +1307,116 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                                  sp2.words <= sp.words;
         unsigned long long *ws = sc->cand.as<unsigned long long>();
         ColumnRecompute rc{};
-        // the two-hop reach path is tried (its plan may still send the call
-        // through the hops): the score GEMM then writes u as split bf16, the
-        // operand form the candidates' tensor-core pass loads, in the bytes
-        // of the fp32 slab (hi [n][bp], then lo [n][bp])
-        const bool reach_try = prune && eff_hops == 2 && !q_ns && m->reach_on &&
-                               m->n_split > 0 && (bp == 256 || bp == 128);
-        uint16_t *u_hi = reach_try ? sc->u.as<uint16_t>() : nullptr;
-        uint16_t *u_lo = reach_try ? u_hi + (size_t)n * bp : nullptr;
-        auto score_fp32 = [&](int *launches) -> cudaError_t {
+        HopPlan hp{};
+        hp.split = m->split;
+        hp.in_ptr = m->in_ptr.as<int64_t>();
+        hp.in_src = m->in_src.as<int32_t>();
+        hp.in_w = m->in_w.as<float>();
+        hp.n = n;
+        hp.n_split_rows = m->n_split;
+        hp.split_row = m->split_row.as<int32_t>();
+        hp.split_slot0 = m->split_slot0.as<int64_t>();
+        hp.n_segs = m->n_segs;
+        hp.seg_e0 = m->seg_e0.as<int64_t>();
+        hp.seg_e1 = m->seg_e1.as<int64_t>();
+        hp.seg_slot = m->seg_slot.as<int32_t>();
+        hp.split_order = m->split_order.as<int32_t>();
+        hp.slot_split = m->slot_split.as<int32_t>();
+        // How a call with two to four hops gets its candidates' scores without
+        // running the hops (each form's plan, on the device, may still send the
+        // call through them):
+        //   RC_SYNC  two hops, 65 queries and more: on the tensor cores; the host
+        //            waits for the plan before it queues the hops (or not)
+        //   RC_MMA   other hop counts, or 33 to 64 queries: the same, with the
+        //            score in fp32 and the hops queued behind; their kernels
+        //            return at once when the plan says the candidates suffice
+        //   RC_FMA   at most 32 queries: in fp32 on the CUDA cores, then the hops
+        //            likewise
+        // The first builds the graph-only coefficients at once; they cost about
+        // what the hops cost over 128 columns a level past the first, far less
+        // than the hops of such a batch.  For the others they are built once the
+        // hops have cost that much since the graph changed, so that a graph that
+        // changes every few calls costs at most twice the hops alone.  One GB300,
+        // hops -> candidates: 1,048,576 chunks, 1 query, two hops 1533 -> 440 us;
+        // 262,147 chunks, 24 queries 384 -> 142; 262,144 chunks, 200 queries, three
+        // hops 1589 -> 237 (564 in fp32).
+        enum { RUN_HOPS, RC_SYNC, RC_MMA, RC_FMA } mode = RUN_HOPS;
+        if (prune) {
+            std::lock_guard<std::mutex> lk(m->table_mu);
+            AK_TRY(ensure_mass(m, hp, eff_hops, st));
+            const bool can = !q_ns && m->reach_on && eff_hops >= 2 && eff_hops <= REACH_MAX_H;
+            if (can && eff_hops == 2 && bp >= 128 && m->n_split > 0) {
+                AK_TRY(ensure_reach(m, hp, eff_hops, st));
+                mode = RC_SYNC;
+            } else if (can && m->n_split >= k && sc->no_room_n != n) {
+                bool go = m->reach_levels >= eff_hops && m->reach_n == n;
+                if (!go) {
+                    if (m->hop_work_n != n) m->hop_work = 0;
+                    m->hop_work_n = n;
+                    go = m->hop_work >= REACH_T * (eff_hops - 1) + 64;
+                    if (!go) m->hop_work += (double)eff_hops * bp;
+                }
+                if (go) {
+                    // no room for the tables: the hops run, as they would without
+                    const size_t cb = (size_t)REACH_T * reach_pad_rows(n) * 2;
+                    const int parts = bp == 32 ? reach_fma_parts(n) : reach_parts();
+                    akashic_status_t r = ensure_reach(m, hp, eff_hops, st);
+                    if (r == AKASHIC_OK)
+                        r = ensure_spare(sc->reach_part, (size_t)parts * REACH_T * bp * 4);
+                    if (r == AKASHIC_OK)
+                        r = bp == 32 ? ensure_spare(sc->coef_f, (size_t)n * REACH_T * 4)
+                                     : ensure_spare(sc->coef_hi, cb);
+                    if (r == AKASHIC_OK && bp != 32) r = ensure_spare(sc->coef_lo, cb);
+                    if (r == AKASHIC_OK)
+                        r = ensure_spare(bp == 32 ? sc->cf_sum : sc->coef_sum,
+                                         (size_t)reach_sum_words(n) * 8);
+                    if (r != AKASHIC_OK && r != AKASHIC_ENOMEM) return r;
+                    if (r == AKASHIC_ENOMEM) {
+                        g_last_error.clear();
+                        go = false;
+                        sc->no_room_n = n;   // not again on this stream at this size
+                    }
+                }
+                // where the candidates did not suffice (the device has said so
+                // by now, or has not yet), the next 15 calls like it run the
+                // hops alone
+                if (go) {
+                    AK_TRY(plan_words(sc));
+                    volatile int32_t *outcome = sc->plan_host + 2;
+                    if (sc->try_build != m->reach_build || sc->try_alpha != alpha ||
+                        sc->try_H != eff_hops || sc->try_k != k || sc->try_n != n) {
+                        sc->try_build = m->reach_build;
+                        sc->try_alpha = alpha;
+                        sc->try_H = eff_hops;
+                        sc->try_k = k;
+                        sc->try_n = n;
+                        sc->try_skip = 0;
+                        *outcome = 0;
+                    } else if (sc->try_skip > 0) {
+                        --sc->try_skip;
+                        go = false;
+                    } else if (*outcome == 2) {
+                        sc->try_skip = 14;
+                        *outcome = 0;
+                        go = false;
+                    }
+                }
+                if (go) mode = bp == 32 ? RC_FMA : RC_MMA;
+            }
+        }
+        // on the tensor cores the candidates' pass loads u - m as split bf16,
+        // which the score GEMM writes in the bytes of the fp32 slab (hi [n][bp],
+        // then lo [n][bp])
+        const bool split_u = mode == RC_SYNC || mode == RC_MMA;
+        uint16_t *u_hi = split_u ? sc->u.as<uint16_t>() : nullptr;
+        uint16_t *u_lo = split_u ? u_hi + (size_t)n * bp : nullptr;
+        auto score_fp32 = [&](int *launches, const int32_t *done) -> cudaError_t {
             return launch_score(m->emb.as<uint16_t>(), n, m->dim, sc->qp.as<uint16_t>(), bp,
                                 sc->shift.as<float>(), m->tau, sc->u.as<float>(),
                                 sc->zpart.as<float>(), m->status.as<int>(), st, launches, &zrows,
                                 ns.dead, prune ? sc->rmax_u.as<float>() : nullptr,
                                 prune ? sc->rmin_u.as<float>() : nullptr, b,
-                                prune ? ext : nullptr);
+                                prune ? ext : nullptr, done);
         };
         {
             PhaseScope ph(m, AKASHIC_PHASE_SCORE, st);
@@ -1325,7 +1429,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                                          sc->words.as<unsigned int>(),
                                          eff_hops >= 1 ? CW_COUNT : 0));
             ph.launches += 1;
-            if (reach_try)
+            if (split_u)
                 CUDA_TRY(launch_score_split(m->emb.as<uint16_t>(), n, m->dim,
                                             sc->qp.as<uint16_t>(), bp, sc->shift.as<float>(),
                                             m->tau, u_hi, u_lo, sc->zpart.as<float>(),
@@ -1333,7 +1437,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                                             sc->rmax_u.as<float>(), sc->rmin_u.as<float>(), b,
                                             ext));
             else if (!dense_fused)
-                CUDA_TRY(score_fp32(&ph.launches));
+                CUDA_TRY(score_fp32(&ph.launches, nullptr));
         }
         if (dense_fused) {
             {
@@ -1381,218 +1485,119 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
         }
         const float *fin = sc->u.as<float>();
         if (eff_hops >= 1) {
-            HopPlan hp{};
-            hp.split = m->split;
-            hp.in_ptr = m->in_ptr.as<int64_t>();
-            hp.in_src = m->in_src.as<int32_t>();
-            hp.in_w = m->in_w.as<float>();
-            hp.n = n;
-            hp.n_split_rows = m->n_split;
-            hp.split_row = m->split_row.as<int32_t>();
-            hp.split_slot0 = m->split_slot0.as<int64_t>();
-            hp.n_segs = m->n_segs;
-            hp.seg_e0 = m->seg_e0.as<int64_t>();
-            hp.seg_e1 = m->seg_e1.as<int64_t>();
-            hp.seg_slot = m->seg_slot.as<int32_t>();
-            hp.split_order = m->split_order.as<int32_t>();
-            hp.slot_split = m->slot_split.as<int32_t>();
             float *bufs[2] = {sc->sa.as<float>(), sc->sb.as<float>()};
             rc.u = sc->u.as<float>();
             rc.in_ptr = hp.in_ptr;
             rc.in_src = hp.in_src;
             rc.in_w = hp.in_w;
             rc.alpha = alpha;
-            if (prune) {
-                std::lock_guard<std::mutex> lk(m->table_mu);
-                AK_TRY(ensure_mass(m, hp, eff_hops, st));
-            }
-            // Two to four hops in fp32 without running them, from the same
-            // candidates and floor (launch_reach_fma).  The hops are queued
-            // behind and return at once when the plan says the candidates
-            // suffice, so the host waits for nothing.  The coefficients cost
-            // about what the hops cost over 128 columns a level past the
-            // first, and are worth it only if the graph stays as it is: they
-            // are built once the hops have cost that much since it changed (so
-            // never more than twice the work of either way alone).  One GB300,
-            // hops against candidates: 1,048,576 chunks, 1 query, two hops 1533
-            // -> 444 us; 262,147 chunks, 24 queries 384 -> 143; 262,144 chunks,
-            // 200 queries, three hops 1589 -> 564.
-            bool reach_fma = false;
-            if (prune && !reach_try && !q_ns && m->reach_on && eff_hops >= 2 &&
-                eff_hops <= REACH_MAX_H && m->n_split >= k) {
-                std::lock_guard<std::mutex> lk(m->table_mu);
-                if (m->reach_levels < eff_hops || m->reach_n != n) {
-                    if (m->hop_work_n != n) m->hop_work = 0;
-                    m->hop_work_n = n;
-                    if (m->hop_work >= REACH_T * (eff_hops - 1) + 64) reach_fma = true;
-                    else m->hop_work += (double)eff_hops * bp;
-                } else {
-                    reach_fma = true;
-                }
-                if (reach_fma) {
-                    // no room for the tables: the hops run, as they would without
-                    akashic_status_t r = ensure_reach(m, hp, eff_hops, st);
-                    if (r == AKASHIC_OK)
-                        r = ensure_spare(sc->reach_part,
-                                         (size_t)reach_fma_parts(n, b) * REACH_T * bp * 4);
-                    if (r == AKASHIC_OK) r = ensure_spare(sc->coef_f, (size_t)n * REACH_T * 4);
-                    if (r == AKASHIC_OK) r = sc->coef_sum.ensure((size_t)reach_sum_words() * 8);
-                    if (r != AKASHIC_OK && r != AKASHIC_ENOMEM) return r;
-                    if (r == AKASHIC_ENOMEM) {
-                        g_last_error.clear();
-                        reach_fma = false;
-                        m->hop_work = -1e300;   // not again for this graph
-                        m->reach_levels = -1;
-                    }
-                }
-                // where the candidates did not suffice (the device has said so
-                // by now, or has not yet), the next 15 calls like it run the
-                // hops alone
-                if (reach_fma) {
-                    if (!sc->plan_host) {
-                        CUDA_TRY(cudaMallocHost((void **)&sc->plan_host, 16));
-                        memset(sc->plan_host, 0, 16);
-                    }
-                    volatile int32_t *outcome = sc->plan_host + 2;
-                    if (sc->try_build != m->reach_build || sc->try_alpha != alpha ||
-                        sc->try_H != eff_hops || sc->try_k != k || sc->try_n != n) {
-                        sc->try_build = m->reach_build;
-                        sc->try_alpha = alpha;
-                        sc->try_H = eff_hops;
-                        sc->try_k = k;
-                        sc->try_n = n;
-                        sc->try_skip = 0;
-                        *outcome = 0;
-                    } else if (sc->try_skip > 0) {
-                        --sc->try_skip;
-                        reach_fma = false;
-                    } else if (*outcome == 2) {
-                        sc->try_skip = 14;
-                        *outcome = 0;
-                        reach_fma = false;
-                    }
-                }
-            }
             // the row bounds of the last hop's output
             const RowBounds rb{sc->rmax_u.as<float>(), sc->rmin_u.as<float>(),
                                m->mass_up.as<float>(), m->mass_dn.as<float>(), ext, n, eff_hops,
                                alpha};
-            // Two hops without running them: when every row whose upper bound
+            // The hops without running them: when every row whose upper bound
             // reaches the floor (here the k-th largest lower bound) is a
             // candidate with reach coefficients, their final scores come from
             // one pass over u and they alone are the selection's candidates.
             bool reach_done = false;
-            auto reach_flags = [&](int32_t *outcome, int *launches) -> akashic_status_t {
-                AK_TRY(sc->reach_keep.ensure((REACH_T + 2) * 4));
-                AK_TRY(sc->reach_plan.ensure(REACH_PLAN_INTS * 4));
-                ReachFlags rf{};
-                rf.u0 = rb.u0;
-                rf.l0 = rb.l0;
-                rf.mup = rb.mup;
-                rf.mdn = rb.mdn;
-                rf.ext = ext;
-                rf.n = n;
-                rf.H = eff_hops;
-                rf.alpha = alpha;
-                rf.split_row = hp.split_row;
-                rf.split_order = hp.split_order;
-                rf.n_lb = m->n_split < 1024 ? m->n_split : 1024;
-                rf.k = k;
-                rf.map = m->reach_map.as<int32_t>();
-                rf.t_cnt = m->reach_t.as<int>();
-                rf.floor_out = sc->pfloor.as<float>();
-                rf.ws = sc->reach_keep.as<int32_t>();
-                rf.plan = sc->reach_plan.as<int32_t>();
-                rf.outcome = outcome;
-                CUDA_TRY(launch_reach_flags(rf, st, launches));
-                return AKASHIC_OK;
-            };
-            if (reach_fma) {
+            if (mode != RUN_HOPS) {
                 {
                     PhaseScope ph(m, AKASHIC_PHASE_BOUND, st);
-                    AK_TRY(reach_flags(sc->plan_host + 2, &ph.launches));
+                    AK_TRY(plan_words(sc));
+                    AK_TRY(sc->reach_plan.ensure(REACH_PLAN_INTS * 4));
+                    ReachFlags rf{};
+                    rf.u0 = rb.u0;
+                    rf.l0 = rb.l0;
+                    rf.mup = rb.mup;
+                    rf.mdn = rb.mdn;
+                    rf.ext = ext;
+                    rf.n = n;
+                    rf.H = eff_hops;
+                    rf.alpha = alpha;
+                    rf.rows = m->reach_rows.as<int32_t>();
+                    rf.k = k;
+                    rf.map = m->reach_map.as<int32_t>();
+                    rf.t_cnt = m->reach_t.as<int>();
+                    rf.ws = sc->words.as<int32_t>() + CW_REACH;
+                    rf.plan = sc->reach_plan.as<int32_t>();
+                    rf.outcome = mode == RC_SYNC ? nullptr : sc->plan_host + 2;
+                    CUDA_TRY(launch_reach_flags(rf, st, &ph.launches));
+                    if (mode == RC_SYNC) {
+                        if (!sc->plan_ev)
+                            CUDA_TRY(cudaEventCreateWithFlags(&sc->plan_ev,
+                                                              cudaEventDisableTiming));
+                        CUDA_TRY(cudaMemcpyAsync(sc->plan_host, sc->reach_plan.p, 8,
+                                                 cudaMemcpyDeviceToHost, st));
+                        CUDA_TRY(cudaEventRecord(sc->plan_ev, st));
+                    }
                 }
+                // The candidates' pass is queued before the host learns the
+                // plan (its kernels return at once when the plan says the
+                // hops run), so the GPU goes on while the host waits.  Every
+                // candidate's packed coefficients are kept while the graph,
+                // alpha and the hop count stay the same.
                 PhaseScope ph(m, AKASHIC_PHASE_LAST_HOP, st);
-                if (sc->cf_build != m->reach_build || sc->cf_alpha != alpha ||
-                    sc->cf_H != eff_hops || sc->cf_n != n) {
-                    CUDA_TRY(launch_reach_combine(reach_levels_of(m), n, eff_hops, alpha,
-                                                  sc->coef_f.as<float>(),
-                                                  sc->coef_sum.as<double>(), st));
-                    ph.launches += 2;
-                    sc->cf_build = m->reach_build;
-                    sc->cf_alpha = alpha;
-                    sc->cf_H = eff_hops;
-                    sc->cf_n = n;
-                }
-                CUDA_TRY(launch_reach_fma(sc->u.as<float>(), bp, b, n, sc->coef_f.as<float>(),
-                                          sc->coef_sum.as<double>(), ext,
-                                          sc->reach_plan.as<int32_t>(),
-                                          m->reach_rows.as<int32_t>(), m->ext_of.as<int32_t>(),
-                                          sc->reach_part.as<float>(),
-                                          (unsigned int *)(ws + sp.off_cnt), ws + sp.off_buf,
-                                          sp.cap, st, &ph.launches));
-                hp.done = sc->reach_plan.as<int32_t>();
-            }
-            if (reach_try) {
-                {
-                    PhaseScope ph(m, AKASHIC_PHASE_BOUND, st);
-                    {
-                        std::lock_guard<std::mutex> lk(m->table_mu);
-                        AK_TRY(ensure_reach(m, hp, eff_hops, st));
+                const int32_t *plan = sc->reach_plan.as<int32_t>();
+                unsigned int *cnt = (unsigned int *)(ws + sp.off_cnt);
+                if (mode == RC_FMA) {
+                    if (sc->cf_build != m->reach_build || sc->cf_alpha != alpha ||
+                        sc->cf_H != eff_hops || sc->cf_n != n) {
+                        CUDA_TRY(launch_reach_combine(reach_levels_of(m), n, eff_hops, alpha,
+                                                      sc->coef_f.as<float>(),
+                                                      sc->cf_sum.as<double>(), st));
+                        ph.launches += 2;
+                        sc->cf_build = m->reach_build;
+                        sc->cf_alpha = alpha;
+                        sc->cf_H = eff_hops;
+                        sc->cf_n = n;
                     }
-                    if (!sc->plan_host) {
-                        CUDA_TRY(cudaMallocHost((void **)&sc->plan_host, 16));
-                        memset(sc->plan_host, 0, 16);
-                    }
-                    if (!sc->plan_ev)
-                        CUDA_TRY(cudaEventCreateWithFlags(&sc->plan_ev, cudaEventDisableTiming));
-                    AK_TRY(reach_flags(nullptr, &ph.launches));
-                    CUDA_TRY(cudaMemcpyAsync(sc->plan_host, sc->reach_plan.p, 8,
-                                             cudaMemcpyDeviceToHost, st));
-                    CUDA_TRY(cudaEventRecord(sc->plan_ev, st));
-                }
-                {
-                    // The candidates' pass is queued before the host learns the
-                    // plan (its kernels return at once when the plan says the
-                    // hops run), so the GPU goes on while the host waits.
-                    PhaseScope ph(m, AKASHIC_PHASE_LAST_HOP, st);
+                    CUDA_TRY(launch_reach_fma(sc->u.as<float>(), bp, b, n, sc->coef_f.as<float>(),
+                                              sc->cf_sum.as<double>(), ext, plan,
+                                              m->reach_rows.as<int32_t>(),
+                                              m->ext_of.as<int32_t>(),
+                                              sc->reach_part.as<float>(), cnt, ws + sp.off_buf,
+                                              sp.cap, st, &ph.launches));
+                } else {
                     AK_TRY(ensure_spare(sc->reach_part,
                                         (size_t)reach_parts() * REACH_T * bp * 4));
-                    // every candidate's packed coefficients, kept while the
-                    // graph, alpha and the hop count stay the same
                     if (sc->coef_build != m->reach_build || sc->coef_alpha != alpha ||
                         sc->coef_H != eff_hops || sc->coef_n != n) {
                         const size_t cb = (size_t)REACH_T * reach_pad_rows(n) * 2;
                         AK_TRY(ensure_spare(sc->coef_hi, cb));
                         AK_TRY(ensure_spare(sc->coef_lo, cb));
+                        AK_TRY(ensure_spare(sc->coef_sum, (size_t)reach_sum_words(n) * 8));
                         CUDA_TRY(launch_reach_pack(reach_levels_of(m), n, eff_hops, alpha,
                                                    sc->coef_hi.as<uint16_t>(),
-                                                   sc->coef_lo.as<uint16_t>(), st));
-                        ph.launches += 1;
+                                                   sc->coef_lo.as<uint16_t>(),
+                                                   sc->coef_sum.as<double>(), st));
+                        ph.launches += 2;
                         sc->coef_build = m->reach_build;
                         sc->coef_alpha = alpha;
                         sc->coef_H = eff_hops;
                         sc->coef_n = n;
                     }
-                    CUDA_TRY(launch_reach_scores(u_hi, u_lo, bp, b, n,
+                    CUDA_TRY(launch_reach_scores(u_hi, u_lo, sc->shift.as<float>(), bp, b, n,
                                                  sc->coef_hi.as<uint16_t>(),
                                                  sc->coef_lo.as<uint16_t>(),
-                                                 sc->reach_plan.as<int32_t>(),
+                                                 sc->coef_sum.as<double>(), plan,
                                                  m->reach_rows.as<int32_t>(),
                                                  m->ext_of.as<int32_t>(),
-                                                 sc->reach_part.as<float>(),
-                                                 (unsigned int *)(ws + sp.off_cnt), ws + sp.off_buf,
+                                                 sc->reach_part.as<float>(), cnt, ws + sp.off_buf,
                                                  sp.cap, m->status.as<int>(), st, &ph.launches));
                 }
-                CUDA_TRY(cudaEventSynchronize(sc->plan_ev));
-                if (sc->plan_host[0] == 1) {
-                    rc = ColumnRecompute{};   // the buffers hold every candidate
-                    reach_done = true;
+                if (mode == RC_SYNC) {
+                    ph.end();
+                    CUDA_TRY(cudaEventSynchronize(sc->plan_ev));
+                    reach_done = sc->plan_host[0] == 1;   // the buffers hold every candidate
+                    if (reach_done) rc = ColumnRecompute{};
                 } else {
-                    // the hops run: they read u in fp32 (the same scores again)
-                    PhaseScope ph(m, AKASHIC_PHASE_SCORE, st);
-                    CUDA_TRY(score_fp32(&ph.launches));
+                    hp.done = plan;
                 }
+            }
+            // the hops read u in fp32 (the same scores again)
+            if (split_u && !reach_done) {
+                PhaseScope ph(m, AKASHIC_PHASE_SCORE, st);
+                CUDA_TRY(score_fp32(&ph.launches, hp.done));
             }
             for (int h = 0; h < eff_hops && !reach_done; ++h) {
                 float *out = bufs[h & 1];

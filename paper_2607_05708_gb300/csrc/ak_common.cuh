@@ -132,10 +132,22 @@ cudaError_t launch_score(const uint16_t *emb, int64_t n, int dim, const uint16_t
                          const float *shift, float tau, float *u, float *zpart, int *status,
                          cudaStream_t st, int *launches, int *zrows,
                          const int32_t *dead_row = nullptr, float *row_max = nullptr,
-                         float *row_min = nullptr, int n_real = 0, unsigned int *ext = nullptr);
-// The same scores with u written as split bf16 instead of fp32: u_hi and u_lo
-// [n][bp] each, u = hi + lo to within 2^-17 relative (the operand form the
-// candidates' tensor-core pass reads); Z's column sums from the fp32 values.
+                         float *row_min = nullptr, int n_real = 0, unsigned int *ext = nullptr,
+                         const int32_t *done = nullptr);
+// At most any score of the batch: exp(-2 c) for the largest shift c of its
+// columns (z >= -c in every column).  The same bits wherever a whole warp calls
+// it.
+__device__ __forceinline__ float batch_u_min(const float *__restrict__ shift, int bp) {
+    float c = 0.f;
+    for (int i = threadIdx.x & 31; i < bp; i += 32) c = fmaxf(c, shift[i]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c = fmaxf(c, __shfl_xor_sync(0xffffffffu, c, o));
+    return exp2f(-2.f * c * LOG2E_F);
+}
+// The same scores with u - batch_u_min(shift) written as split bf16 instead of
+// u in fp32: u_hi and u_lo [n][bp] each, their sum within 2^-17 relative (the
+// operand form the candidates' tensor-core pass reads); Z's column sums from
+// the fp32 values of u.
 cudaError_t launch_score_split(const uint16_t *emb, int64_t n, int dim, const uint16_t *qp, int bp,
                                const float *shift, float tau, uint16_t *u_hi, uint16_t *u_lo,
                                float *zpart, int *status, cudaStream_t st, int *launches,
@@ -189,7 +201,7 @@ cudaError_t launch_dots_keys_t(const uint16_t *emb, int64_t n, int64_t row_strid
 
 // Query preparation: pad q (b rows) to bp rows of zeros and compute
 // shift[c] = tau * |q_c| * max_norm (0 for padding); flags ERANGE.
-// zero (or NULL): n_zero <= 128 words set to 0 (the call's counters).
+// zero (or NULL): n_zero words set to 0 (the call's counters).
 cudaError_t launch_prep_queries(const uint16_t *q, int b, int bp, int dim, float tau,
                                 const float *max_norm, uint16_t *qp, float *shift, int *status,
                                 cudaStream_t st, unsigned int *zero = nullptr,
@@ -594,8 +606,7 @@ cudaError_t launch_fill_f32(float *v, int64_t n, float x, cudaStream_t st);
 constexpr int REACH_T = 128;         // candidate rows kept
 constexpr int REACH_MAX_H = 4;       // hop counts it serves: 2 .. REACH_MAX_H
 struct ReachBuild {
-    int64_t n, n_split;
-    const int32_t *split_row, *split_order;
+    int64_t n;
     const float *mup;                // mass levels 0..2 [3][n] (candidate choice)
     const int64_t *in_ptr;           // in-edge CSR (row space)
     const int32_t *in_src;
@@ -606,19 +617,21 @@ struct ReachBuild {
     int32_t *rows;                   // [REACH_T] candidate rows
     int *t_cnt;                      // their number (device)
     int32_t *map;                    // [n] row -> candidate slot or -1
+    unsigned long long *pick;        // [reach_pick_words()] scratch
 };
+int64_t reach_pick_words();
 struct ReachLevels {
     const float *level[REACH_MAX_H]; // C_1, C_2, ...: [n][REACH_T] each
 };
 // The candidates, their map and C_1; then Cn = C_{t+1} from Cp = C_t.
 cudaError_t launch_reach_pick(const ReachBuild &rb, float *C1, cudaStream_t st);
 cudaError_t launch_reach_level(const ReachBuild &rb, const float *Cp, float *Cn, cudaStream_t st);
-// The reach path's floor, flags and plan, without the per-row bound arrays:
-// floor = the k-th largest lower bound over the (up to 1024) heaviest split
-// rows, computed for those rows only; then every row's upper bound against
-// it: keep[REACH_T] flags the candidates that reach it, *bad counts the
-// other rows that do, and the last CTA to finish writes the plan
-// (REACH_PLAN_INTS below).  ws: int32[REACH_T + 2] scratch (keep, bad, done).
+// The reach path's floor, flags and plan: floor = the k-th largest lower bound
+// over the candidates; then every row's upper bound against it: keep[REACH_T]
+// flags the candidates that reach it, *bad counts the other rows that do, and
+// the last CTA to finish writes the plan (REACH_PLAN_INTS below).  ws:
+// int32[REACH_WS] scratch (keep, bad, done), zeroed before.
+constexpr int REACH_WS = REACH_T + 2;
 struct ReachFlags {
     const float *u0, *l0;            // u's row maxima / minima [n]
     const float *mup, *mdn;          // mass levels [H + 1][n]
@@ -626,12 +639,10 @@ struct ReachFlags {
     int64_t n;
     int H;
     float alpha;
-    const int32_t *split_row, *split_order;
-    int64_t n_lb;                    // heaviest split rows taken for the floor (<= 1024)
+    const int32_t *rows;             // the candidates
     int k;
     const int32_t *map;              // row -> candidate slot or -1
     const int *t_cnt;                // candidates (device)
-    float *floor_out;
     int32_t *ws;
     int32_t *plan;                   // [REACH_PLAN_INTS]
     int32_t *outcome;                // host-visible word (or NULL): 1 the candidates
@@ -649,28 +660,28 @@ constexpr int REACH_PLAN_INTS = REACH_T + 3;
 // Rows of the packed coefficients: n rounded up to a whole 64-row stage.
 int64_t reach_pad_rows(int64_t n);
 // Every candidate's combined coefficients sum_t alpha^t C_t as bf16 hi + lo,
-// [REACH_T][reach_pad_rows(n)] each (graph-only; repacked when the graph,
-// alpha or H change).
-cudaError_t launch_reach_pack(const ReachLevels &C, int64_t n, int H, float alpha, uint16_t *coef_hi,
-                              uint16_t *coef_lo, cudaStream_t st);
+// [REACH_T][reach_pad_rows(n)] each, and their column sums in 64 bits
+// (sums[REACH_T]; reach_sum_words(n) words in all, the rest scratch)
+// (graph-only; repacked when the graph, alpha or H change).
+int64_t reach_sum_words(int64_t n);
+cudaError_t launch_reach_pack(const ReachLevels &C, int64_t n, int H, float alpha,
+                              uint16_t *coef_hi, uint16_t *coef_lo, double *sums, cudaStream_t st);
 // partial: [reach_parts()][REACH_T][bp] scratch; with plan[0] = 1 the
 // flagged candidates' keys are written to each real column's buffer
-// (cnt[b] = nk); with plan[0] = 0 both kernels return at once.  bp = 128
-// or 256.  u_hi, u_lo: the score GEMM's split-bf16 u, [n][bp] each.
-cudaError_t launch_reach_scores(const uint16_t *u_hi, const uint16_t *u_lo, int bp, int B,
-                                int64_t n, const uint16_t *coef_hi,
-                                const uint16_t *coef_lo, const int32_t *plan, const int32_t *rows,
-                                const int32_t *ext_of, float *partial, unsigned int *cnt,
-                                unsigned long long *buf, int64_t cap, int *status, cudaStream_t st,
-                                int *launches);
-// The same in fp32 (any hop count and bp): coef [n][REACH_T] the combined
-// coefficients, sums [REACH_T] their column sums (of reach_sum_words() words,
-// the rest scratch), u [n][bp] the score slab, ext u's extremes, partial
-// [reach_fma_parts(n, B)][REACH_T][bp] scratch.
-int64_t reach_sum_words();
+// (cnt[b] = nk); with plan[0] = 0 both kernels return at once.  bp = 64, 128
+// or 256.  u_hi, u_lo: the score GEMM's split-bf16 u - batch_u_min(shift).
+cudaError_t launch_reach_scores(const uint16_t *u_hi, const uint16_t *u_lo, const float *shift,
+                                int bp, int B, int64_t n, const uint16_t *coef_hi,
+                                const uint16_t *coef_lo, const double *sums, const int32_t *plan,
+                                const int32_t *rows, const int32_t *ext_of, float *partial,
+                                unsigned int *cnt, unsigned long long *buf, int64_t cap,
+                                int *status, cudaStream_t st, int *launches);
+// The same in fp32, for B <= 32: coef [n][REACH_T] the combined coefficients,
+// sums as above, u [n][bp] the score slab, ext u's extremes, partial
+// [reach_fma_parts(n)][REACH_T][bp] scratch.
 cudaError_t launch_reach_combine(const ReachLevels &C, int64_t n, int H, float alpha, float *coef,
                                  double *sums, cudaStream_t st);
-int reach_fma_parts(int64_t n, int B);
+int reach_fma_parts(int64_t n);
 cudaError_t launch_reach_fma(const float *u, int bp, int B, int64_t n, const float *coef,
                              const double *sums, const unsigned int *ext, const int32_t *plan,
                              const int32_t *rows, const int32_t *ext_of, float *partial,

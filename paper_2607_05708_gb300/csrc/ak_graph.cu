@@ -974,13 +974,16 @@ __device__ __forceinline__ void hop_accumulate(const int32_t *__restrict__ in_sr
 // and L[j] at most every real query column's value of s^(h)_j.  Level 0 is
 // u's row maximum / minimum (from the score step); level h follows the hop
 // s^(h)_j = fma(alpha, sum_{i->j} w_ij s^(h-1)_i, u_j) with the sums of
-// w * U and w * L over the row's in-edges (w, s >= 0), widened for rounding:
-// the hop's sum takes at most 2n + 10 roundings on any term's path
-// (segments and partial slots included) and the bound's own sum at most
-// n + 5, so exp(+-x), x = 3.25 (n + 8) 2^-24, covers both (with 1 + x + x^2
-// >= exp(x) and 1 - x <= exp(-x) for 0 <= x <= 1), and a factor 1 -+ 4e-6
-// (~67 ulp) covers the final rounding of the hop and of evaluating the
-// bound in fp32.
+// w * U and w * L over the row's in-edges (w, s >= 0), widened for rounding by
+// n, the terms one after another in either sum: the row's in-edges where it is
+// kept whole, else a segment's edges and the row's segments (what the hop adds
+// in sequence; the bound's own sums add a 32nd of a segment, then the
+// segments).  The hop's sum takes at most 2n + 10 roundings on any term's path
+// and the bound's own sum at most n + 5, so exp(+-x), x = 3.25 (n + 8) 2^-24,
+// covers both (with 1 + x + x^2 >= exp(x) and 1 - x <= exp(-x) for 0 <= x <=
+// 1), and a factor 1 -+ 4e-6 (~67 ulp) covers the final rounding of the hop
+// and of evaluating the bound in fp32.  (n = the in-degree widened a hub of
+// 2 * 10^5 in-edges by 4% a level, as much as u itself varies.)
 __device__ __forceinline__ float bound_x(int64_t n) {
     return 3.25f * (float)(n + 8) * 5.9604645e-8f;
 }
@@ -1064,8 +1067,8 @@ __global__ void k_bound_rows(const int64_t *__restrict__ in_ptr, const int32_t *
 
 // Split rows: one warp per segment, its sums added into the owning row's
 // totals (the order of the additions does not change the bound: every
-// term is >= 0 and a term's path stays within the row's edge count + 5
-// roundings) ...
+// term is >= 0 and a term's path stays within a segment's edges + the row's
+// segments + 5 roundings) ...
 __global__ void k_seg_bound(const int64_t *__restrict__ seg_e0, const int64_t *__restrict__ seg_e1,
                             const int32_t *__restrict__ seg_slot, int64_t n_segs,
                             const int32_t *__restrict__ slot_split,
@@ -1088,13 +1091,16 @@ __global__ void k_seg_bound(const int64_t *__restrict__ seg_e0, const int64_t *_
 // ... then each split row's bounds.
 __global__ void k_split_bound(const int64_t *__restrict__ in_ptr, int64_t n_split,
                               const int32_t *__restrict__ split_row,
+                              const int64_t *__restrict__ split_slot0, int64_t seg_len,
                               const float *__restrict__ u0, const float *__restrict__ l0,
                               const float *__restrict__ split_vu, const float *__restrict__ split_vl,
                               float alpha, float *__restrict__ Un, float *__restrict__ Ln) {
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n_split;
          r += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = split_row[r];
-        const int64_t n = in_ptr[j + 1] - in_ptr[j];
+        const int64_t edges = in_ptr[j + 1] - in_ptr[j];
+        const int64_t path = seg_len + (split_slot0[r + 1] - split_slot0[r]);
+        const int64_t n = edges < path ? edges : path;
         Un[j] = bound_up(u0[j], split_vu[r], n, alpha);
         Ln[j] = bound_dn(l0[j], split_vl[r], n, alpha);
     }
@@ -1153,7 +1159,8 @@ cudaError_t launch_mass_levels(const HopPlan &p, int t0, int t1, float *mup, flo
                                             split_vl);
             const int64_t wr = ceil_div<int64_t>(p.n_split_rows, 256);
             const int gr = (int)(wr < (int64_t)sms * 2 ? wr : (int64_t)sms * 2);
-            k_split_bound<<<gr, 256, 0, st>>>(p.in_ptr, p.n_split_rows, p.split_row, zeros, zeros,
+            k_split_bound<<<gr, 256, 0, st>>>(p.in_ptr, p.n_split_rows, p.split_row, p.split_slot0,
+                                              p.split.seg_len, zeros, zeros,
                                               split_vu, split_vl, 1.f, Un, Ln);
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;

@@ -19,43 +19,98 @@
 namespace ak {
 
 // ------------------------------------------------------------------ graph-only
-// Candidates: the REACH_T rows of largest upper mass mup[1] + mup[2] among
-// the (up to 1024) heaviest split rows, whatever the hop count (so that the
-// levels of one hop count serve the others); ties to the lower row.  One
-// CTA of 1024 threads, bitonic sort of the keys in shared memory.
-__global__ __launch_bounds__(1024) void k_reach_pick(const int32_t *__restrict__ split_row,
-                                                      const int32_t *__restrict__ split_order,
-                                                      int64_t n_split,
-                                                      const float *__restrict__ mup, int64_t n,
+// Candidates: the REACH_T rows of largest upper mass mup[1] + mup[2],
+// whatever the hop count (so that the levels of one hop count serve the others);
+// ties to the lower row.  Mass counts, not in-degree: a row with few in-edges
+// from chunks that link to little else outranks many hubs.  A histogram of the
+// masses' upper bits gives a threshold that at least REACH_T rows reach, those
+// rows are collected, and one CTA sorts them.  More than PICK_MAX of them (all
+// within 3% of the last): no candidates, as the plan would hardly ever take
+// them.
+constexpr int PICK_SHIFT = 18, PICK_BINS = 1 << (31 - PICK_SHIFT), PICK_MAX = 4096;
+__device__ __forceinline__ uint32_t mass_bits(const float *__restrict__ mup, int64_t n, int64_t r) {
+    return __float_as_uint(mup[n + r] + mup[2 * n + r]);   // >= 0: ordered like the values
+}
+
+__global__ __launch_bounds__(256) void k_mass_hist(const float *__restrict__ mup, int64_t n,
+                                                   int *__restrict__ hist) {
+    __shared__ int h[PICK_BINS];
+    for (int i = threadIdx.x; i < PICK_BINS; i += 256) h[i] = 0;
+    __syncthreads();
+    for (int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x; r < n; r += (int64_t)gridDim.x * 256)
+        atomicAdd(&h[mass_bits(mup, n, r) >> PICK_SHIFT], 1);
+    __syncthreads();
+    for (int i = threadIdx.x; i < PICK_BINS; i += 256)
+        if (h[i]) atomicAdd(&hist[i], h[i]);
+}
+
+// The lower edge of the highest bin with at least REACH_T rows in it and above
+// (0 if there are fewer rows): every CTA finds it, then collects its rows.
+__global__ __launch_bounds__(256) void k_mass_collect(const float *__restrict__ mup, int64_t n,
+                                                      const int *__restrict__ hist,
+                                                      unsigned long long *__restrict__ keys,
+                                                      int *__restrict__ count) {
+    __shared__ int sum[256];
+    __shared__ int bin_s;
+    constexpr int PER = PICK_BINS / 256;
+    const int t = threadIdx.x;
+    int mine = 0;                       // thread t: bins from the top, PER a thread
+    for (int i = 0; i < PER; ++i) mine += hist[PICK_BINS - 1 - (t * PER + i)];
+    sum[t] = mine;
+    if (t == 0) bin_s = 0;
+    __syncthreads();
+    int above = 0;
+    for (int i = 0; i < t; ++i) above += sum[i];
+    if (above < REACH_T && above + mine >= REACH_T) {
+        int b = PICK_BINS - 1 - t * PER;
+        for (int i = 0; i < PER; ++i, --b) {
+            above += hist[b];
+            if (above >= REACH_T) break;
+        }
+        bin_s = b;
+    }
+    __syncthreads();
+    // (rows without mass are nobody's candidates)
+    const uint32_t lo = bin_s > 0 ? (uint32_t)bin_s << PICK_SHIFT : 1u;
+    for (int64_t r = (int64_t)blockIdx.x * 256 + t; r < n; r += (int64_t)gridDim.x * 256) {
+        const uint32_t m = mass_bits(mup, n, r);
+        if (m < lo) continue;
+        const int p = atomicAdd(count, 1);
+        if (p < PICK_MAX)
+            keys[p] = ((unsigned long long)m << 32) | (unsigned long long)(~(uint32_t)r);
+    }
+}
+
+__global__ __launch_bounds__(1024) void k_reach_pick(const unsigned long long *__restrict__ keys,
+                                                      const int *__restrict__ count,
                                                       int32_t *__restrict__ rows,
                                                       int *__restrict__ t_out) {
-    __shared__ unsigned long long key[1024];
-    const int tid = threadIdx.x;
-    const int nc = (int)(n_split < 1024 ? n_split : 1024);
-    unsigned long long k = 0ull;
-    if (tid < nc) {
-        const int32_t r = split_row[split_order[tid]];
-        const float m = mup[n + r] + mup[2 * n + r];
-        k = ((unsigned long long)__float_as_uint(m) << 32) | (unsigned long long)(~(uint32_t)r);
+    __shared__ unsigned long long key[PICK_MAX];
+    const int tid = threadIdx.x, m = *count;
+    if (m > PICK_MAX) {
+        if (tid == 0) *t_out = 0;
+        return;
     }
-    key[tid] = k;
+    for (int i = tid; i < PICK_MAX; i += 1024) key[i] = i < m ? keys[i] : 0ull;
     __syncthreads();
     // descending bitonic sort
-    for (int size = 2; size <= 1024; size <<= 1) {
+    for (int size = 2; size <= PICK_MAX; size <<= 1) {
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            const int other = tid ^ stride;
-            if (other > tid) {
-                const unsigned long long a = key[tid], b = key[other];
-                const bool desc = (tid & size) == 0;
-                if (desc ? a < b : a > b) {
-                    key[tid] = b;
-                    key[other] = a;
+            for (int i = tid; i < PICK_MAX; i += 1024) {
+                const int other = i ^ stride;
+                if (other > i) {
+                    const unsigned long long a = key[i], b = key[other];
+                    const bool desc = (i & size) == 0;
+                    if (desc ? a < b : a > b) {
+                        key[i] = b;
+                        key[other] = a;
+                    }
                 }
             }
             __syncthreads();
         }
     }
-    const int T = nc < REACH_T ? nc : REACH_T;
+    const int T = m < REACH_T ? m : REACH_T;
     if (tid < T) rows[tid] = (int32_t)~(uint32_t)(key[tid] & 0xffffffffull);
     if (tid == 0) *t_out = T;
 }
@@ -99,12 +154,20 @@ __global__ void k_reach_spmm(const int64_t *__restrict__ row_ptr, const int32_t 
     }
 }
 
+int64_t reach_pick_words() { return PICK_MAX + (PICK_BINS + 2) / 2; }
+
 cudaError_t launch_reach_pick(const ReachBuild &rb, float *C1, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(rb.map, 0xff, (size_t)rb.n * 4, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(C1, 0, (size_t)rb.n * REACH_T * 4, st);
     if (e != cudaSuccess) return e;
-    k_reach_pick<<<1, 1024, 0, st>>>(rb.split_row, rb.split_order, rb.n_split, rb.mup, rb.n,
-                                     rb.rows, rb.t_cnt);
+    int *hist = (int *)(rb.pick + PICK_MAX);
+    e = cudaMemsetAsync(hist, 0, (PICK_BINS + 1) * 4, st);
+    if (e != cudaSuccess) return e;
+    const int64_t want = ceil_div<int64_t>(rb.n, 1024), sms = device_sm_count();
+    const unsigned g = (unsigned)(want < 2 * sms ? want : 2 * sms);
+    k_mass_hist<<<g, 256, 0, st>>>(rb.mup, rb.n, hist);
+    k_mass_collect<<<g, 256, 0, st>>>(rb.mup, rb.n, hist, rb.pick, hist + PICK_BINS);
+    k_reach_pick<<<1, 1024, 0, st>>>(rb.pick, hist + PICK_BINS, rb.rows, rb.t_cnt);
     k_reach_map<<<1, REACH_T, 0, st>>>(rb.rows, rb.t_cnt, rb.map);
     k_reach_c1<<<REACH_T, 256, 0, st>>>(rb.rows, rb.t_cnt, rb.in_ptr, rb.in_src, rb.in_w, C1);
     return cudaGetLastError();
@@ -146,49 +209,37 @@ __device__ void reach_build_plan(const int32_t *keep, int bad, int t_cnt, int k,
     }
 }
 
-// The floor: the k-th largest lower bound over the n_lb heaviest split
-// rows (each query's k-th largest final score reaches it: those k rows
-// score at least their lb for every query), computed for those rows only;
-// one CTA, one (lb bits, position) key per thread, a descending bitonic
-// network (partners within a warp by shuffles, farther ones through a
-// ping-pong pair of shared arrays).  Also clears the flags' scratch.
-__global__ __launch_bounds__(1024) void k_reach_floor(const ReachFlags f) {
-    __shared__ unsigned long long xk[2][1024];
-    griddep_wait();
-    const int t = threadIdx.x;
-    if (t < REACH_T + 2) f.ws[t] = 0;                  // keep[], bad, done
-    const float lmin = ext_lmin(f.ext);
-    unsigned long long key =
-        t < f.n_lb ? ((unsigned long long)__float_as_uint(row_lower_bound(
-                          f.l0, f.mdn, f.n, f.H, f.alpha, lmin, f.split_row[f.split_order[t]]))
-                      << 32) | (unsigned long long)(uint32_t)t
-                   : 0ull;
-    int cur = 0;
-    for (int size = 2; size <= 1024; size <<= 1)
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            unsigned long long other;
-            if (stride >= 32) {
-                xk[cur][t] = key;
-                __syncthreads();
-                other = xk[cur][t ^ stride];
-                cur ^= 1;          // the next write goes to the other array
-            } else {
-                other = __shfl_xor_sync(0xffffffffu, key, stride);
-            }
-            const bool keep_max = ((t & size) == 0) == ((t & stride) == 0);
-            key = keep_max ? (key > other ? key : other) : (key < other ? key : other);
-        }
-    if (t == f.k - 1)   // keys now descend with the thread index
-        *f.floor_out = f.n_lb >= f.k ? __uint_as_float((uint32_t)(key >> 32)) : 0.f;
-}
-
-// Rows whose upper bound reaches the floor: a candidate's slot is flagged,
-// any other row counted in bad; the last CTA to finish builds the plan.
+// The floor: the k-th largest lower bound over the candidates (each query's
+// k-th largest final score reaches it: those k rows score at least their lb
+// for every query); every CTA evaluates it, 128 bounds ranked against each
+// other (a CTA of its own that sorted 1024 hubs' bounds took 10 us more a
+// call).  Then the rows whose upper bound reaches it: a candidate's slot is
+// flagged, any other row counted in bad; the last CTA to finish builds the
+// plan.
 __global__ __launch_bounds__(256) void k_reach_flags(const ReachFlags f) {
     __shared__ int last;
+    __shared__ float floor_s;
+    __shared__ unsigned int lb_s[REACH_T];
     griddep_wait();
     int32_t *keep = f.ws, *bad = f.ws + REACH_T, *done = f.ws + REACH_T + 1;
-    const float floor_ = *f.floor_out, umax = ext_umax(f.ext);
+    const int t_cnt = *f.t_cnt;
+    {
+        const int t = threadIdx.x;
+        unsigned int lb = 0u;                            // (bounds are >= 0)
+        if (t < t_cnt)
+            lb = __float_as_uint(row_lower_bound(f.l0, f.mdn, f.n, f.H, f.alpha, ext_lmin(f.ext),
+                                                 f.rows[t]));
+        if (t < REACH_T) lb_s[t] = lb;
+        if (t == 0) floor_s = 0.f;
+        __syncthreads();
+        if (t < t_cnt) {
+            int rank = 0;
+            for (int i = 0; i < t_cnt; ++i) rank += lb_s[i] > lb || (lb_s[i] == lb && i < t) ? 1 : 0;
+            if (rank == f.k - 1) floor_s = __uint_as_float(lb);
+        }
+        __syncthreads();
+    }
+    const float floor_ = floor_s, umax = ext_umax(f.ext);
     int nb = 0;
     auto visit = [&](int64_t j, float ub) {
         if (ub >= floor_) {
@@ -234,22 +285,21 @@ __global__ __launch_bounds__(256) void k_reach_flags(const ReachFlags f) {
     __shared__ int32_t kf[REACH_T];
     if (threadIdx.x < REACH_T) kf[threadIdx.x] = vk[threadIdx.x];
     __syncthreads();
-    reach_build_plan(kf, *(volatile int *)bad, *f.t_cnt, f.k, f.plan);
+    reach_build_plan(kf, *(volatile int *)bad, t_cnt, f.k, f.plan);
     if (f.outcome && threadIdx.x == REACH_T - 1)       // (the thread that wrote plan[0])
         *(volatile int32_t *)f.outcome = f.plan[0] ? 1 : 2;
 }
 
 cudaError_t launch_reach_flags(const ReachFlags &f, cudaStream_t st, int *launches) {
-    if (f.n_lb > 1024 || f.k < 1) return cudaErrorInvalidValue;
-    cudaError_t e = launch_pdl(k_reach_floor, dim3(1), dim3(1024), 0, st, f);
-    if (e != cudaSuccess) return e;
+    if (f.k < 1) return cudaErrorInvalidValue;
     // four rows per thread (one where n is not a multiple of 4): a few
     // independent loads per row, so the rows in flight set the rate; a
     // quarter of the CTAs also takes three quarters of the done counter's
     // atomics off the tail
     const int64_t g = ceil_div<int64_t>(f.n, (f.n & 3) == 0 ? 1024 : 256);
-    e = launch_pdl(k_reach_flags, dim3((unsigned)(g > 0 ? g : 1)), dim3(256), 0, st, f);
-    if (launches) *launches += 2;
+    cudaError_t e =
+        launch_pdl(k_reach_flags, dim3((unsigned)(g > 0 ? g : 1)), dim3(256), 0, st, f);
+    if (launches) *launches += 1;
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
@@ -260,7 +310,11 @@ cudaError_t launch_reach_flags(const ReachFlags &f, cudaStream_t st, int *launch
 //   rest, so hi + lo holds 16 significant bits),
 //   coef u ~= A_hi B_hi + A_hi B_lo + A_lo B_hi,
 // three MMAs per 16-row slice into an fp32 accumulator in TMEM (the
-// dropped A_lo B_lo term is below 2^-16 of the product).
+// dropped A_lo B_lo term is below 2^-16 of the product).  u stands for
+// u - m here, m = batch_u_min: most of every u is the same constant, and
+//   sum_k coef[k][i] u[k][b] = m S_i + sum_k coef[k][i] (u[k][b] - m)
+// with S_i the coefficients' sum in 64 bits, so the products' and the
+// accumulation's errors shrink with the terms.
 //   A = the combined coefficients sum_t alpha^t C_t, packed by
 //       k_reach_pack as [REACH_T slots][n_pad rows] bf16 (hi, lo), loaded
 //       by TMA as K-major tiles [128 slots][64 rows] in the 128-byte swizzle;
@@ -271,14 +325,14 @@ cudaError_t launch_reach_flags(const ReachFlags &f, cudaStream_t st, int *launch
 //       queries, the BP / 64 boxes RM_BK * 128 bytes apart.
 // D[slot][query] (M = 128 slots = TMEM lanes, N = BP queries = columns).
 // The tensor core's accumulation of many positive terms drifts (each add
-// into the fp32 accumulator may round the same way), so an accumulator
-// takes only RM_CHUNK stages (1024 rows, 192 MMAs): two accumulators
-// alternate, and the flush warps add each finished one into the CTA's
-// partial with ordinary round-to-nearest fp32 adds while the MMAs fill the
-// other.  The operands' loads carry an L2 evict-first hint and the partial
-// rows' loads and stores an evict-last one, so that the partials stay in L2
-// while u streams past; slots 64 and above are flushed only when the plan
-// is wide.
+// into the fp32 accumulator rounds the same way, ~2^-25 an MMA), so an
+// accumulator takes only RM_CHUNK stages (RM_CHUNK * 12 MMAs): two
+// accumulators alternate, and the flush warps add each finished one to the
+// CTA's sums, which they hold in registers, with ordinary round-to-nearest
+// fp32 adds while the MMAs fill the other.  (Sums kept in memory cost so much
+// per flush that an accumulator took 16 stages: scores 5.6e-6 off on 1,048,576
+// chunks and 256 queries, 3.8e-8 with this and u - m.)  The operands' loads carry an L2 evict-first hint;
+// slots 64 and above are flushed only when the plan is wide.
 // Warps: 0 TMA producer (A and B), 1 MMA issuer, 2..9 flush (warp w reads
 // TMEM lanes 32 (w % 4) .., column half (w - 2) / 4).  Both operands
 // arrive by TMA, so the bytes in flight are the two stages' 192 KB of
@@ -289,7 +343,7 @@ constexpr int RM_M = REACH_T;            // candidate slots (M)
 constexpr int RM_STAGES = 2;
 constexpr int RM_FLUSH_W = 8;            // flush warps
 constexpr int RM_THREADS = 64 + 32 * RM_FLUSH_W;
-constexpr int RM_CHUNK = 16;             // stages per accumulator
+constexpr int RM_CHUNK = 2;              // stages per accumulator
 
 template <int BP>
 struct RmCfg {
@@ -301,7 +355,7 @@ struct RmCfg {
     static constexpr int SMEM = 1024 + RM_STAGES * STAGE_BYTES + 256;
     static constexpr int PARTS = RM_FLUSH_W / 4;     // column parts of a flush
     static constexpr int TMEM_COLS = 2 * BP; // two accumulators
-    static_assert(BP == 128 || BP == 256, "query widths 128 and 256");
+    static_assert(BP == 64 || BP == 128 || BP == 256, "query widths 64, 128 and 256");
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
@@ -439,21 +493,17 @@ __global__ __launch_bounds__(RM_THREADS, 1) void k_reach_mma(
         }
     } else {
         // ---------------- flush warps: each finished accumulator into the
-        // CTA's partial rows (the first chunk stores, the later ones add)
+        // warp's share of the CTA's sums (registers), written at the end
         const int fw = warp - 2;
         const int q = warp & 3;                       // TMEM lanes 32 q ..
         const int part = fw >> 2;                     // column part
         const int slot = q * 32 + lane;
         constexpr int PW = BP / C::PARTS;             // columns of a part
-        float *o = partial + ((int64_t)blockIdx.x * REACH_T + slot) * BP + part * PW;
         // slots 64..127 are read only when the plan is wide
         const bool live = wide || q < 2;
-        // the partial rows are re-read every chunk: keep them in L2
-        const uint64_t pol = l2_evict_last_policy();
-        if (ns == 0 && live) {
-            for (int b = 0; b < PW; b += 4)
-                *reinterpret_cast<float4 *>(o + b) = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+        float sum[PW];
+#pragma unroll
+        for (int i = 0; i < PW; ++i) sum[i] = 0.f;
         for (int64_t c = 0; c < n_chunks; ++c) {
             const int acc = (int)(c & 1);
             int f_ok = lane == 0 ? (mbar_wait(&dfull[acc], (uint32_t)((c >> 1) & 1), status) ? 1 : 0)
@@ -461,32 +511,28 @@ __global__ __launch_bounds__(RM_THREADS, 1) void k_reach_mma(
             f_ok = __shfl_sync(0xffffffffu, f_ok, 0);
             if (!f_ok) break;
             tc_fence_after();
-#pragma unroll 1
-            for (int ch = 0; ch < (live ? PW / 32 : 0); ++ch) {
-                uint32_t r[32];
-                tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) +
-                              (uint32_t)(acc * BP + part * PW + ch * 32),
-                          r);
-                tmem_ld_wait();
-                float4 *dst = reinterpret_cast<float4 *>(o + ch * 32);
+            if (live) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    float4 v = make_float4(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]),
-                                           __uint_as_float(r[4 * i + 2]),
-                                           __uint_as_float(r[4 * i + 3]));
-                    if (c > 0) {
-                        const float4 p = ld_f4_hint(dst + i, pol);
-                        v.x += p.x;
-                        v.y += p.y;
-                        v.z += p.z;
-                        v.w += p.w;
-                    }
-                    st_f4_hint(dst + i, v, pol);
+                for (int ch = 0; ch < PW / 32; ++ch) {
+                    uint32_t r[32];
+                    tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) +
+                                  (uint32_t)(acc * BP + part * PW + ch * 32),
+                              r);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) sum[ch * 32 + i] += __uint_as_float(r[i]);
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&dfree[acc]);
+        }
+        if (live) {
+            float *o = partial + ((int64_t)blockIdx.x * REACH_T + slot) * BP + part * PW;
+#pragma unroll
+            for (int i = 0; i < PW; i += 4)
+                *reinterpret_cast<float4 *>(o + i) =
+                    make_float4(sum[i], sum[i + 1], sum[i + 2], sum[i + 3]);
         }
     }
     tc_fence_before();
@@ -499,11 +545,12 @@ __global__ __launch_bounds__(RM_THREADS, 1) void k_reach_mma(
 // combined coefficient sum_t alpha^t C_t[k][i] (Horner over t) split into
 // hi + lo, zero for k >= n.  One CTA per 64 rows k: the rows' slots are
 // read contiguously (coalesced), transposed through shared memory and
-// written along k (coalesced).
+// written along k (coalesced).  part[cta][i]: the rows' sums in 64 bits.
 __global__ __launch_bounds__(256) void k_reach_pack(const ReachLevels C, int64_t n,
                                                     int64_t n_pad, int H, float alpha,
                                                     uint16_t *__restrict__ hi,
-                                                    uint16_t *__restrict__ lo) {
+                                                    uint16_t *__restrict__ lo,
+                                                    double *__restrict__ part) {
     __shared__ float tile[64][REACH_T + 1];
     const int64_t k0 = (int64_t)blockIdx.x * 64;
     for (int x = threadIdx.x; x < 64 * REACH_T; x += blockDim.x) {
@@ -517,6 +564,11 @@ __global__ __launch_bounds__(256) void k_reach_pack(const ReachLevels C, int64_t
         tile[kk][i] = c;
     }
     __syncthreads();
+    if (threadIdx.x < REACH_T) {
+        double s = 0.0;
+        for (int kk = 0; kk < 64; ++kk) s += (double)tile[kk][threadIdx.x];
+        part[(int64_t)blockIdx.x * REACH_T + threadIdx.x] = s;
+    }
     for (int x = threadIdx.x; x < 32 * REACH_T; x += blockDim.x) {
         const int i = x / 32, kk = 2 * (x % 32);
         const int64_t k = k0 + kk;
@@ -537,7 +589,7 @@ __global__ __launch_bounds__(256) void k_reach_pack(const ReachLevels C, int64_t
 // partial from t / Q on (coalesced rows of the partials), and the groups
 // are added in group order (the same order on every run).
 // F32: u is fp32 in `u` (32 query columns a block) and the partials are of
-// u - Lmin; else split bf16 in u_hi, u_lo (64 columns).
+// u - Lmin; else u - m is split bf16 in u_hi, u_lo (64 columns), m = batch_u_min.
 template <bool F32>
 __global__ __launch_bounds__(1024) void k_reach_emit(const float *__restrict__ u,
                                                      const uint16_t *__restrict__ u_hi,
@@ -549,7 +601,8 @@ __global__ __launch_bounds__(1024) void k_reach_emit(const float *__restrict__ u
                                                      unsigned int *__restrict__ cnt,
                                                      unsigned long long *__restrict__ buf,
                                                      int64_t cap, const double *__restrict__ sums,
-                                                     const unsigned int *__restrict__ ext) {
+                                                     const unsigned int *__restrict__ ext,
+                                                     const float *__restrict__ shift) {
     constexpr int Q = F32 ? 32 : 64, G = 1024 / Q;
     __shared__ float red[1024];
     griddep_wait();
@@ -567,18 +620,18 @@ __global__ __launch_bounds__(1024) void k_reach_emit(const float *__restrict__ u
         for (int p = g; p < n_parts; p += G) acc += partial[((int64_t)p * REACH_T + slot) * bp + b];
     }
     red[threadIdx.x] = acc;
+    const float m = F32 ? ext_lmin(ext) : batch_u_min(shift, bp);
     __syncthreads();
     if (g == 0 && b < B) {
         float sum = red[threadIdx.x];
         for (int h = 1; h < G; ++h) sum += red[h * Q + threadIdx.x];
         const int64_t j = rows[slot];
-        const float uj = F32 ? u[j * bp + b]
-                             : __bfloat162float(__ushort_as_bfloat16(u_hi[j * bp + b])) +
-                                   __bfloat162float(__ushort_as_bfloat16(u_lo[j * bp + b]));
-        // (F32: the partials are of u - Lmin)
-        const float s = F32 ? (float)((double)uj + ((double)ext_lmin(ext) * sums[slot] +
-                                                    (double)sum))
-                            : uj + sum;
+        // the partials are of u - m; in the split form so is u itself
+        const double uj = F32 ? (double)u[j * bp + b]
+                              : (double)__bfloat162float(__ushort_as_bfloat16(u_hi[j * bp + b])) +
+                                    (double)__bfloat162float(__ushort_as_bfloat16(u_lo[j * bp + b])) +
+                                    (double)m;
+        const float s = (float)(uj + ((double)m * sums[slot] + (double)sum));
         buf[(int64_t)b * cap + i] = ((unsigned long long)__float_as_uint(s) << 32) |
                                     (unsigned long long)(~(uint32_t)ext_of[j]);
         if (i == 0) cnt[b] = (unsigned int)nk;
@@ -590,11 +643,35 @@ int reach_parts() { return device_sm_count(); }
 int64_t reach_pad_rows(int64_t n) { return (n + RM_BK - 1) / RM_BK * RM_BK; }
 
 
-cudaError_t launch_reach_pack(const ReachLevels &C, int64_t n, int H, float alpha, uint16_t *coef_hi,
-                              uint16_t *coef_lo, cudaStream_t st) {
+// sum[i] = the column sums' parts part[p][i], p < n_parts, in a fixed order.
+__global__ __launch_bounds__(256) void k_reach_colsum(const double *__restrict__ part,
+                                                      int64_t n_parts, double *__restrict__ sum) {
+    __shared__ double red[256];
+    double s = 0.0;
+    for (int64_t p = threadIdx.x; p < n_parts; p += 256) s += part[p * REACH_T + blockIdx.x];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) sum[blockIdx.x] = red[0];
+}
+
+static int combine_ctas() { return device_sm_count() * 8; }
+int64_t reach_sum_words(int64_t n) {
+    const int64_t tiles = reach_pad_rows(n) / 64;
+    return (int64_t)REACH_T * (1 + (tiles > combine_ctas() ? tiles : combine_ctas()));
+}
+
+cudaError_t launch_reach_pack(const ReachLevels &C, int64_t n, int H, float alpha,
+                              uint16_t *coef_hi, uint16_t *coef_lo, double *sums,
+                              cudaStream_t st) {
     const int64_t n_pad = reach_pad_rows(n);
     if (n_pad <= 0) return cudaSuccess;
-    k_reach_pack<<<(unsigned)(n_pad / 64), 256, 0, st>>>(C, n, n_pad, H, alpha, coef_hi, coef_lo);
+    k_reach_pack<<<(unsigned)(n_pad / 64), 256, 0, st>>>(C, n, n_pad, H, alpha, coef_hi, coef_lo,
+                                                         sums + REACH_T);
+    k_reach_colsum<<<REACH_T, 256, 0, st>>>(sums + REACH_T, n_pad / 64, sums);
     return cudaGetLastError();
 }
 
@@ -634,63 +711,61 @@ static cudaError_t reach_mma_bp(const uint16_t *coef_hi, const uint16_t *coef_lo
         e = make_tmap_2d(&tbl, u_lo, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, BP, (uint64_t)n,
                          (uint64_t)BP * 2, 64, RM_BK);
     if (e != cudaSuccess) return e;
-    k_reach_mma<BP><<<parts, RM_THREADS, C::SMEM, st>>>(thi, tlo, thi64, tlo64, tbh, tbl, n, plan,
-                                                         partial, status);
-    return cudaGetLastError();
+    return launch_pdl(k_reach_mma<BP>, dim3(parts), dim3(RM_THREADS), C::SMEM, st, thi, tlo, thi64,
+                      tlo64, tbh, tbl, n, plan, partial, status);
 }
 
-cudaError_t launch_reach_scores(const uint16_t *u_hi, const uint16_t *u_lo, int bp, int B,
-                                int64_t n, const uint16_t *coef_hi,
-                                const uint16_t *coef_lo, const int32_t *plan, const int32_t *rows,
-                                const int32_t *ext_of, float *partial, unsigned int *cnt,
-                                unsigned long long *buf, int64_t cap, int *status, cudaStream_t st,
-                                int *launches) {
-    if (n <= 0 || (bp != 128 && bp != 256)) return cudaErrorInvalidValue;
+cudaError_t launch_reach_scores(const uint16_t *u_hi, const uint16_t *u_lo, const float *shift,
+                                int bp, int B, int64_t n, const uint16_t *coef_hi,
+                                const uint16_t *coef_lo, const double *sums, const int32_t *plan,
+                                const int32_t *rows, const int32_t *ext_of, float *partial,
+                                unsigned int *cnt, unsigned long long *buf, int64_t cap,
+                                int *status, cudaStream_t st, int *launches) {
     const int parts = reach_parts();
-    cudaError_t e = bp == 256 ? reach_mma_bp<256>(coef_hi, coef_lo, u_hi, u_lo, n, plan, partial,
-                                                  parts, status, st)
-                              : reach_mma_bp<128>(coef_hi, coef_lo, u_hi, u_lo, n, plan, partial,
-                                                  parts, status, st);
+    cudaError_t e = cudaErrorInvalidValue;
+    if (n <= 0) return e;
+    switch (bp) {
+    case 64: e = reach_mma_bp<64>(coef_hi, coef_lo, u_hi, u_lo, n, plan, partial, parts, status, st); break;
+    case 128: e = reach_mma_bp<128>(coef_hi, coef_lo, u_hi, u_lo, n, plan, partial, parts, status, st); break;
+    case 256: e = reach_mma_bp<256>(coef_hi, coef_lo, u_hi, u_lo, n, plan, partial, parts, status, st); break;
+    }
     if (e != cudaSuccess) return e;
     e = launch_pdl(k_reach_emit<false>, dim3(REACH_T * (bp / 64)), dim3(1024), 0, st,
                    (const float *)nullptr, u_hi, u_lo, bp, B, (const float *)partial, parts, plan,
-                   rows, ext_of, cnt, buf, cap, (const double *)nullptr,
-                   (const unsigned int *)nullptr);
+                   rows, ext_of, cnt, buf, cap, sums, (const unsigned int *)nullptr, shift);
     if (launches) *launches += 2;
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 // ------------------------------------------------------------------ fp32 terms
-// The same partial sums in fp32 on the CUDA cores, for the calls that had run
-// the hops in fp32: three hops and more, and batches of at most 64 queries.
-// (Split-bf16 products would take their error from ~1e-7 to ~6e-6.)
+// The same partial sums in fp32 on the CUDA cores, for at most 32 queries (the
+// tensor cores' tiles have 64 columns, and a slab of 64 would cost more than
+// the FMAs):
 //   sum_k coef[k][i] u[k][b] = m S_i + sum_k coef[k][i] (u[k][b] - m)
-// with m = Lmin, the smallest u of any live row and real query, and S_i the
-// coefficients' sum in 64 bits: u - m is exact where u <= 2 m, every term
-// stays >= 0, and the terms are as much smaller as u is flat, and the sums'
-// rounding with them.  (Plain sums of nearly equal terms all round the same
-// way: three hops on 262,144 chunks were 1.4e-6 off, 3e-8 so, 2.8e-7 the hops.)
+// with m = Lmin, the smallest u of any live row and real query: u - m is exact
+// where u <= 2 m, every term stays >= 0, and the terms are as much smaller as u
+// is flat, and the sums' rounding with them.  (Plain sums of nearly equal
+// terms all round the same way: three hops on 262,144 chunks were 1.4e-6 off,
+// 3e-8 so, 2.8e-7 the hops.)
 // Bound by the loads for few queries (64 coefficients and the query columns a
-// row) and by the FMAs for many: n * 64 * columns of them, 96 or 128 where
-// flagged slots lie there.  The hops gather nnz columns a hop instead, an
-// order of magnitude more, from L2.
+// row: 268 MB at 1,048,576 chunks) and by the FMAs and shared loads towards 32:
+// n * 64 * columns of them, 96 or 128 where flagged slots lie there.  The hops
+// gather nnz columns a hop instead, an order of magnitude more, from L2.
 // A warp works alone: it takes groups of RF_ROWS rows, copies their
 // coefficients and query columns into its own ring of RF_STAGES stages
 // (cp.async), and keeps an ST-slot x CT-column tile of sums in registers, a
 // lane's part SPL slots x CPL columns: SPL * CPL FMAs a row for (SPL + CPL) / 4
-// 16-byte shared loads of four cycles each, which is why the wide batches take
-// 16 x 8 (8 x 8 ran at 47% of the FMA rate).  The eight warps' tiles, then the
-// CTAs' partials, are added in a fixed order.
+// 16-byte shared loads.  The eight warps' tiles, then the CTAs' partials, are
+// added in a fixed order.
 constexpr int RF_ROWS = 8, RF_STAGES = 4, RF_WARPS = 8;
 
 template <int ST, int CT>
 struct RfCfg {
-    static constexpr int SPL = CT == 64 ? ST / 4 : (ST * CT == 512 ? 4 : 8);
+    static constexpr int SPL = ST * CT == 512 ? 4 : 8;
     static constexpr int SG = ST / SPL, CG = 32 / SG;           // lanes over slots, columns
     static constexpr int CPL = CT / CG;
     static constexpr int STAGE = RF_ROWS * (ST + CT);           // floats a stage
     static constexpr int SMEM = RF_WARPS * RF_STAGES * STAGE * 4;
-    static constexpr int CTAS = SPL * CPL > 64 ? 1 : 2;         // an SM
     static_assert(SPL % 4 == 0 && CPL % 4 == 0 && SG * CG == 32, "16-byte shared loads");
     static_assert(RF_WARPS * ST * CT * 4 <= SMEM, "the tiles' sum reuses the rings");
 };
@@ -702,7 +777,7 @@ __device__ __forceinline__ void cp_async16(float *dst, const float *src, bool va
 }
 
 template <int ST, int CT>
-__global__ __launch_bounds__(RF_WARPS * 32, RfCfg<ST, CT>::CTAS) void k_reach_fma(
+__global__ __launch_bounds__(RF_WARPS * 32, 2) void k_reach_fma(
     const float *__restrict__ u, int bp, int64_t n, const float *__restrict__ coef, int slot0,
     const int32_t *__restrict__ plan, const unsigned int *__restrict__ ext,
     float *__restrict__ partial) {
@@ -801,8 +876,8 @@ __global__ __launch_bounds__(RF_WARPS * 32, RfCfg<ST, CT>::CTAS) void k_reach_fm
 }
 
 // coef[k][i] = sum_t alpha^t C_t[k][i] (Horner over t), fp32, and its column
-// sums in 64 bits: each CTA's in part[cta][i], added in CTA order by
-// k_reach_colsum.  128 threads a row.
+// sums in 64 bits: each CTA's in part[cta][i], added by k_reach_colsum.  128
+// threads a row.
 __global__ __launch_bounds__(256) void k_reach_combine(const ReachLevels C, int64_t n, int H,
                                                        float alpha, float *__restrict__ coef,
                                                        double *__restrict__ part) {
@@ -819,32 +894,17 @@ __global__ __launch_bounds__(256) void k_reach_combine(const ReachLevels C, int6
     __syncthreads();
     if (h == 0) part[(int64_t)blockIdx.x * REACH_T + i] = s + half[i];
 }
-__global__ __launch_bounds__(REACH_T) void k_reach_colsum(const double *__restrict__ part,
-                                                          int n_parts, double *__restrict__ sum) {
-    double s = 0.0;
-    for (int p = 0; p < n_parts; ++p) s += part[(int64_t)p * REACH_T + threadIdx.x];
-    sum[threadIdx.x] = s;
-}
-
-static int combine_ctas() { return device_sm_count() * 8; }
-int64_t reach_sum_words() { return (int64_t)REACH_T * (1 + combine_ctas()); }
-
 cudaError_t launch_reach_combine(const ReachLevels &C, int64_t n, int H, float alpha, float *coef,
                                  double *sums, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     k_reach_combine<<<combine_ctas(), 256, 0, st>>>(C, n, H, alpha, coef, sums + REACH_T);
-    k_reach_colsum<<<1, REACH_T, 0, st>>>(sums + REACH_T, combine_ctas(), sums);
+    k_reach_colsum<<<REACH_T, 256, 0, st>>>(sums + REACH_T, combine_ctas(), sums);
     return cudaGetLastError();
 }
 
-// Columns of a warp's tile, and CTAs along the rows: as many as the SMs hold at
-// a time over all column tiles, at least a group of rows a warp.
-static int fma_columns(int B) { return B <= 8 ? 8 : (B <= 16 ? 16 : (B <= 32 ? 32 : 64)); }
-int reach_fma_parts(int64_t n, int B) {
-    const int ct = fma_columns(B);
-    const int64_t most = ceil_div<int64_t>(n, RF_ROWS * RF_WARPS);
-    const int64_t want = ceil_div<int64_t>((ct == 64 ? 1 : 2) * device_sm_count(),
-                                           ceil_div<int64_t>(B, ct));
+// CTAs along the rows: two an SM, at least a group of rows a warp.
+int reach_fma_parts(int64_t n) {
+    const int64_t most = ceil_div<int64_t>(n, RF_ROWS * RF_WARPS), want = 2 * device_sm_count();
     return (int)(want < most ? want : most);
 }
 
@@ -875,34 +935,20 @@ cudaError_t launch_reach_fma(const float *u, int bp, int B, int64_t n, const flo
                              const int32_t *rows, const int32_t *ext_of, float *partial,
                              unsigned int *cnt, unsigned long long *buf, int64_t cap,
                              cudaStream_t st, int *launches) {
-    if (n <= 0 || B < 1 || B > bp || bp % 32 != 0 || (B > 32 && bp % 64 != 0))
-        return cudaErrorInvalidValue;
-    const int parts = reach_fma_parts(n, B);
+    if (n <= 0 || B < 1 || B > 32 || bp != 32) return cudaErrorInvalidValue;
+    const int parts = reach_fma_parts(n);
     cudaError_t e;
 #define RF_TILE(ST, CT, S0) reach_fma_tile<ST, CT>(u, bp, B, n, coef, S0, plan, ext, partial, parts, st)
-    switch (fma_columns(B)) {
-    case 8:
-        e = RF_TILE(64, 8, 0);
-        if (e == cudaSuccess) e = RF_TILE(32, 16, 64);   // (bp >= 32: columns 8..15 exist)
-        break;
-    case 16:
-        e = RF_TILE(64, 16, 0);
-        if (e == cudaSuccess) e = RF_TILE(32, 16, 64);
-        break;
-    case 32:
-        e = RF_TILE(64, 32, 0);
-        if (e == cudaSuccess) e = RF_TILE(32, 32, 64);
-        break;
-    default:
-        e = RF_TILE(64, 64, 0);
-        if (e == cudaSuccess) e = RF_TILE(32, 64, 64);
-        break;
-    }
+    if (B <= 8) e = RF_TILE(64, 8, 0);
+    else if (B <= 16) e = RF_TILE(64, 16, 0);
+    else e = RF_TILE(64, 32, 0);
+    if (e == cudaSuccess) e = B <= 16 ? RF_TILE(32, 16, 64) : RF_TILE(32, 32, 64);
 #undef RF_TILE
     if (e != cudaSuccess) return e;
     e = launch_pdl(k_reach_emit<true>, dim3(REACH_T * (bp / 32)), dim3(1024), 0, st, u,
                    (const uint16_t *)nullptr, (const uint16_t *)nullptr, bp, B,
-                   (const float *)partial, parts, plan, rows, ext_of, cnt, buf, cap, sums, ext);
+                   (const float *)partial, parts, plan, rows, ext_of, cnt, buf, cap, sums, ext,
+                   (const float *)nullptr);
     if (launches) *launches += 3;
     return e == cudaSuccess ? cudaGetLastError() : e;
 }

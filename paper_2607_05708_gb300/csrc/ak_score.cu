@@ -20,7 +20,8 @@ __global__ void k_prep_queries(const uint16_t *__restrict__ q, int b, int dim, f
                                unsigned int *__restrict__ zero, int n_zero) {
     griddep_wait();
     const int c = blockIdx.x;
-    if (c == 0 && (int)threadIdx.x < n_zero) zero[threadIdx.x] = 0u;
+    if (c == 0)
+        for (int i = threadIdx.x; i < n_zero; i += blockDim.x) zero[i] = 0u;
     __shared__ float red[32];
     float ss = 0.f;
     if constexpr (VEC) {
@@ -60,7 +61,7 @@ __global__ void k_prep_queries(const uint16_t *__restrict__ q, int b, int dim, f
 cudaError_t launch_prep_queries(const uint16_t *q, int b, int bp, int dim, float tau,
                                 const float *max_norm, uint16_t *qp, float *shift, int *status,
                                 cudaStream_t st, unsigned int *zero, int n_zero) {
-    if (n_zero < 0 || n_zero > 128 || (n_zero > 0 && !zero)) return cudaErrorInvalidValue;
+    if (n_zero < 0 || (n_zero > 0 && !zero)) return cudaErrorInvalidValue;
     const bool vec = ((uintptr_t)q & 15) == 0 && dim % 8 == 0;
     cudaError_t e = launch_pdl(vec ? k_prep_queries<true> : k_prep_queries<false>, dim3(bp),
                                dim3(128), 0, st, q, b, dim, tau, max_norm, qp, shift, status,
@@ -175,8 +176,10 @@ struct GemmEpi {
     const int32_t *dead_row;            // EXP, EXP_FILTER, FILTER: deleted rows (or NULL):
                                         // no score (u = 0) / never a filter candidate
     uint32_t *keys_t;                   // KEYS_T: [n_ctiles * BP][n_rows]
-    uint16_t *u_hi, *u_lo;              // EXP (or NULL): u as split bf16, [n_rows][n_ctiles * BP]
-                                        // each (u = hi + lo to 2^-17), instead of fp32
+    uint16_t *u_hi, *u_lo;              // EXP (or NULL): u - batch_u_min(shift) as split
+                                        // bf16, [n_rows][n_ctiles * BP] each (the sum of
+                                        // the two to 2^-17), instead of u in fp32
+    const int32_t *done;                // or NULL: with done[0] = 1 the kernel returns at once
     float *row_max, *row_min;           // EXP (or NULL): [n_rows] largest / smallest u of
     int n_real;                         // the row over the first n_real columns
     unsigned int *ext;                  // with row_max (or NULL), atomically maxed, zeroed
@@ -223,7 +226,7 @@ struct GemmCfg {
                                           ? (BP * 12 < 1024 ? 1024 : BP * 12)
                                       : MODE == GEMM_EXP_FILTER ? 2 * OUT_BYTES + BP * 12
                                                                 : 2 * HALVES * OUT_BYTES;
-    static constexpr int MISC = 4096;   // shift, Z sums, flags, barriers
+    static constexpr int MISC = 4096;   // shift, row extremes, flags, barriers
     static constexpr int BUDGET = 227 * 1024 - 1024;
     static constexpr int S_FIT = (BUDGET - OUT_REGION - MISC) / STAGE_BYTES;
     static constexpr int STAGES = S_FIT > 8 ? 8 : S_FIT;
@@ -245,6 +248,7 @@ __global__ __launch_bounds__(GemmCfg<BP, MODE, P2>::THREADS, 1) void k_gemm_umma
                                                       const GemmEpi ep) {
     using C = GemmCfg<BP, MODE, P2>;
     griddep_wait();
+    if (MODE == GEMM_EXP && ep.done && ep.done[0] == 1) return;
     constexpr bool EXPF = MODE == GEMM_EXP_FILTER;
     constexpr bool EXP = MODE == GEMM_EXP || EXPF;
     constexpr bool FILTER = MODE == GEMM_FILTER;
@@ -437,6 +441,7 @@ __global__ __launch_bounds__(GemmCfg<BP, MODE, P2>::THREADS, 1) void k_gemm_umma
 #pragma unroll
         for (int i = 0; i < BP / 32; ++i) zl[i] = 0.f;
         float emx = 0.f, emn = INFINITY;                 // this thread's rows' extremes
+        const float u_min = MODE == GEMM_EXP && ep.u_hi ? batch_u_min(ep.shift, BP) : 0.f;
         int it = 0, cc = 0;
         for (int64_t u = u_first; u < n_units; u += u_step, ++it) {
             const int64_t ct = u % n_ctiles;
@@ -537,14 +542,17 @@ __global__ __launch_bounds__(GemmCfg<BP, MODE, P2>::THREADS, 1) void k_gemm_umma
                         }
                 }
                 if (MODE == GEMM_EXP && ep.u_hi) {
-                    // u as split bf16: hi and lo tiles [128 rows][32 cols] of
-                    // 64-byte rows in the 64-byte swizzle (the 16-byte chunk c
-                    // of row r at c ^ ((r >> 1) & 3)), one TMA store each
+                    // u - u_min as split bf16 (nearly all of u is the same
+                    // constant, which the candidates' pass adds back exactly):
+                    // hi and lo tiles [128 rows][32 cols] of 64-byte rows in
+                    // the 64-byte swizzle (the 16-byte chunk c of row r at
+                    // c ^ ((r >> 1) & 3)), one TMA store each
                     named_bar(2 + hsel, 128);                 // staging[buf] free again
                     uint8_t *sb = (uint8_t *)(sOut + (hsel * 2 + buf) * (C::OUT_BYTES / 4));
                     uint32_t hw[16], lw[16];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) hw[i] = split_bf16_pair(v[2 * i], v[2 * i + 1], lw[i]);
+                    for (int i = 0; i < 16; ++i)
+                        hw[i] = split_bf16_pair(v[2 * i] - u_min, v[2 * i + 1] - u_min, lw[i]);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const int pos = row * 64 + ((j ^ ((row >> 1) & 3)) << 4);
@@ -899,8 +907,10 @@ static cudaError_t gemm_dispatch(const uint16_t *emb, int64_t n_rows, int64_t ro
 cudaError_t launch_score(const uint16_t *emb, int64_t n, int dim, const uint16_t *qp, int bp,
                          const float *shift, float tau, float *u, float *zpart, int *status,
                          cudaStream_t st, int *launches, int *zrows, const int32_t *dead_row,
-                         float *row_max, float *row_min, int n_real, unsigned int *ext) {
+                         float *row_max, float *row_min, int n_real, unsigned int *ext,
+                         const int32_t *done) {
     GemmEpi ep{};
+    ep.done = done;
     ep.dead_row = dead_row;
     ep.row_max = row_max;
     ep.row_min = row_min;

@@ -1,8 +1,8 @@
-"""Two to four hops from reach coefficients in fp32 (batches of at most 64
-queries, or three hops and more): the path is taken once the hops have run
-often enough on one graph, selects what the hops select, and its scores agree
-with theirs to fp32 rounding; a graph whose candidates do not suffice goes
-through the hops."""
+"""Two to four hops from reach coefficients, in fp32 (batches of at most 32
+queries) or on the tensor cores (33 to 64 queries, or three hops and more): the
+path is taken once the hops have run often enough on one graph, selects what
+the hops select, and its scores agree with theirs within the bound below; a
+graph whose candidates do not suffice goes through the hops."""
 import dataclasses
 
 import numpy as np
@@ -13,9 +13,11 @@ from _parity import assert_retrieval_parity, gpu_retrieve, gpu_store, oracle_ret
 
 pytestmark = pytest.mark.gpu
 
-# fp32 sums of non-negative terms in two orders: at most a few hundred
-# roundings on any path (a warp's rows, the warps, the CTAs; a hop's
-# segments), 2^-24 each, and three levels of coefficients
+# fp32: sums of non-negative terms in two orders, at most a few hundred
+# roundings on any path (a warp's rows, the warps, the CTAs; a hop's segments),
+# 2^-24 each.  Tensor cores: split-bf16 products of u - u_min, each within
+# 3 * 2^-16 = 4.6e-5, and u - u_min is at most 1 - exp(-2 tau |q| |e|) = 6% of u
+# here (dim 1024): 2.9e-6 of the sum.
 REL = 1e-5
 
 
@@ -52,7 +54,7 @@ def test_equals_the_hops(n, B, hops, k, monkeypatch):
     store = gpu_store(wl, "clustered")
     for _ in range(12):                      # the hops, until the coefficients pay
         got, launches = _launches(store, wl, q)
-    assert launches == 5, launches           # the candidates' three kernels before the hop's
+    assert launches == (5 if B <= 32 else 4), launches   # the candidates' and the last hop's
     hit = got["ids"] == ref["ids"]
     assert hit.mean() > 0.99
     np.testing.assert_allclose(got["scores"][hit], ref["scores"][hit], rtol=REL, atol=0)
