@@ -146,8 +146,8 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
  * per batch for the device's decision between the two-hop path from reach
  * coefficients and the hops (an event recorded after a 12-byte copy, not the
  * whole stream; the candidates' pass is already queued behind it, so the
- * GPU does not idle); the first such call after the graph changed also waits
- * while it builds their graph-only tables.
+ * GPU does not idle).  The other calls with two to four hops decide on the
+ * device.
  * Graph-only tables built by a call on one stream are waited for (an event,
  * not a host wait) by calls on every other stream. */
 akashic_status_t akashic_mem_retrieve(akashic_mem_t *m, const uint16_t *q, int32_t B, int32_t k,
