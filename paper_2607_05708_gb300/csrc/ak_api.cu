@@ -163,7 +163,7 @@ struct akashic_mem {
     DevBuf rstat;                // per chunk ID: (max, 1/sum) of its out-row softmax
     // spares the relation update writes the next CSR / transpose into (then
     // swapped with the live arrays), and grow-only scratch for its temporaries
-    DevBuf rp2, col2, aff2, in_ptr2, in_src2, in_aff2, in_w2;
+    DevBuf rp2, col2, aff2, w2, in_ptr2, in_src2, in_aff2, in_w2;
     DevBuf scr[SCR_COUNT];
     bool inc_transpose = true;   // relation updates patch the transpose instead of re-sorting
     SplitParams split;
@@ -428,65 +428,61 @@ static akashic_status_t build_split_plan(akashic_mem *m, cudaStream_t st) {
         if (!q) sc_rc = AKASHIC_ENOMEM;
         return Tmp{q, bytes};
     };
-    const Tmp tmp = get(0, scan_tmp_bytes(n + 1) + 4096);
-    const Tmp nseg = get(1, (size_t)(n + 1) * 8), flag = get(2, (size_t)(n + 1) * 8);
-    const Tmp slot_off = get(3, (size_t)(n + 1) * 8), split_idx = get(4, (size_t)(n + 1) * 8);
+    // sizes first (read back once), then the plan
+    const int64_t max_hubs = m->nnz / (m->split.split_t + 1);
+    const Tmp chain = get(0, (size_t)hub_plan_words(n, max_hubs) * 8);
+    const Tmp rows = get(1, (size_t)(max_hubs + 1) * 4), slot0 = get(2, (size_t)(max_hubs + 1) * 8);
+    const Tmp counts = get(3, 16);
     if (sc_rc != AKASHIC_OK) return fail(sc_rc, "relation graph rebuild: out of device memory");
-    CUDA_TRY(launch_split_count(m->split, m->in_ptr.as<int64_t>(), m->in_src.as<int32_t>(), n,
-                                nseg.as<int64_t>(), flag.as<int64_t>(), st));
-    CUDA_TRY(scan_exclusive(nseg.as<int64_t>(), slot_off.as<int64_t>(), n, tmp.p, tmp.cap, st));
-    CUDA_TRY(scan_exclusive(flag.as<int64_t>(), split_idx.as<int64_t>(), n, tmp.p, tmp.cap, st));
-    int64_t n_segs = 0, n_split = 0;
-    CUDA_TRY(cudaMemcpyAsync(&n_segs, slot_off.as<int64_t>() + n, 8, cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaMemcpyAsync(&n_split, split_idx.as<int64_t>() + n, 8, cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(launch_hub_count(m->split, m->in_ptr.as<int64_t>(), m->in_src.as<int32_t>(), n,
+                              max_hubs, rows.as<int32_t>(), slot0.as<int64_t>(),
+                              counts.as<int64_t>(), chain.as<unsigned long long>(),
+                              m->status.as<int>(), st));
+    int64_t got[2] = {0, 0};
+    CUDA_TRY(cudaMemcpyAsync(got, counts.p, 16, cudaMemcpyDeviceToHost, st));
     AK_TRY(check_status(m, st, "relation graph rebuild"));
+    const int64_t n_split = got[0], n_segs = got[1];
     if (n_segs > 0x7fffffffLL) return fail(AKASHIC_ECAPACITY, "too many hub segments");
     m->n_segs = n_segs;
     m->n_split = n_split;
-    if (n_split > 0) {
-        // grown with headroom: every relation update adds a few segments, and
-        // a reallocation would synchronise the device
-        AK_TRY(ensure_spare(m->split_row, (size_t)n_split * 4));
-        AK_TRY(ensure_spare(m->split_slot0, (size_t)(n_split + 1) * 8));
-        AK_TRY(ensure_spare(m->seg_e0, (size_t)n_segs * 8));
-        AK_TRY(ensure_spare(m->seg_e1, (size_t)n_segs * 8));
-        AK_TRY(ensure_spare(m->seg_slot, (size_t)n_segs * 4));
-        const Tmp e0 = get(5, (size_t)n_segs * 8), e1 = get(6, (size_t)n_segs * 8);
-        const Tmp win = get(7, (size_t)n_segs * 4), order = get(8, (size_t)n_segs * 4);
-        const Tmp win2 = get(9, (size_t)n_segs * 4), order2 = get(10, (size_t)n_segs * 4);
-        const Tmp rtmp = get(11, radix_tmp_bytes(n_segs) + 4096);
-        if (sc_rc != AKASHIC_OK) return fail(sc_rc, "relation graph rebuild: out of device memory");
-        CUDA_TRY(launch_split_fill(m->split, m->in_ptr.as<int64_t>(), m->in_src.as<int32_t>(), n,
-                                   nseg.as<int64_t>(), slot_off.as<int64_t>(),
-                                   split_idx.as<int64_t>(), m->split_row.as<int32_t>(),
-                                   m->split_slot0.as<int64_t>(), e0.as<int64_t>(),
-                                   e1.as<int64_t>(), win.as<uint32_t>(), st));
-        CUDA_TRY(cudaMemcpyAsync(m->split_slot0.as<int64_t>() + n_split, &n_segs, 8,
-                                 cudaMemcpyHostToDevice, st));
-        CUDA_TRY(launch_iota(order.as<uint32_t>(), n_segs, st));
-        bool alt = false;
-        CUDA_TRY(radix_sort_pairs(win.as<uint32_t>(), order.as<uint32_t>(), win2.as<uint32_t>(),
-                                  order2.as<uint32_t>(), n_segs, bits_for((n - 1) / m->split.win_rows),
-                                  rtmp.p, rtmp.cap, st, &alt));
-        CUDA_TRY(launch_seg_permute(alt ? order2.as<uint32_t>() : order.as<uint32_t>(),
-                                    e0.as<int64_t>(), e1.as<int64_t>(), n_segs,
-                                    m->seg_e0.as<int64_t>(), m->seg_e1.as<int64_t>(),
-                                    m->seg_slot.as<int32_t>(), st));
-        // split rows heaviest first (the hop's fixup order)
-        AK_TRY(ensure_spare(m->split_order, (size_t)n_split * 4));
-        CUDA_TRY(launch_split_keys(m->split_slot0.as<int64_t>(), n_split, win.as<uint32_t>(),
-                                   order.as<uint32_t>(), st));
-        bool alt2 = false;
-        CUDA_TRY(radix_sort_pairs(win.as<uint32_t>(), order.as<uint32_t>(), win2.as<uint32_t>(),
-                                  order2.as<uint32_t>(), n_split, 32, rtmp.p, rtmp.cap, st, &alt2));
-        CUDA_TRY(cudaMemcpyAsync(m->split_order.p, alt2 ? order2.p : order.p, (size_t)n_split * 4,
-                                 cudaMemcpyDeviceToDevice, st));
-        AK_TRY(ensure_spare(m->slot_split, (size_t)n_segs * 4));
-        CUDA_TRY(launch_slot_owner(m->split_slot0.as<int64_t>(), n_split,
-                                   m->slot_split.as<int32_t>(), st));
-        AK_TRY(check_status(m, st, "relation graph rebuild"));
-    }
-    return check_status(m, st, "relation graph rebuild");
+    if (n_split <= 0) return AKASHIC_OK;
+    // grown with headroom: every relation update adds a few segments, and
+    // a reallocation would synchronise the device
+    AK_TRY(ensure_spare(m->split_row, (size_t)n_split * 4));
+    AK_TRY(ensure_spare(m->split_slot0, (size_t)(n_split + 1) * 8));
+    AK_TRY(ensure_spare(m->seg_e0, (size_t)n_segs * 8));
+    AK_TRY(ensure_spare(m->seg_e1, (size_t)n_segs * 8));
+    AK_TRY(ensure_spare(m->seg_slot, (size_t)n_segs * 4));
+    AK_TRY(ensure_spare(m->split_order, (size_t)n_split * 4));
+    AK_TRY(ensure_spare(m->slot_split, (size_t)n_segs * 4));
+    const Tmp e0 = get(4, (size_t)n_segs * 8), e1 = get(5, (size_t)n_segs * 8);
+    const Tmp win = get(6, (size_t)n_segs * 4), order = get(7, (size_t)n_segs * 4);
+    const Tmp win2 = get(8, (size_t)n_segs * 4), order2 = get(9, (size_t)n_segs * 4);
+    const Tmp rkey = get(10, (size_t)n_split * 8), rtmp = get(11, radix_tmp_bytes(n_segs) + 4096);
+    if (sc_rc != AKASHIC_OK) return fail(sc_rc, "relation graph rebuild: out of device memory");
+    uint32_t *row_key = rkey.as<uint32_t>(), *row_id = row_key + n_split;
+    CUDA_TRY(launch_hub_fill(m->split, m->in_ptr.as<int64_t>(), m->in_src.as<int32_t>(),
+                             rows.as<int32_t>(), slot0.as<int64_t>(), n_split, n_segs,
+                             m->split_row.as<int32_t>(), m->split_slot0.as<int64_t>(),
+                             e0.as<int64_t>(), e1.as<int64_t>(), win.as<uint32_t>(),
+                             order.as<uint32_t>(), m->slot_split.as<int32_t>(), row_key, row_id,
+                             st));
+    bool alt = false;
+    CUDA_TRY(radix_sort_pairs(win.as<uint32_t>(), order.as<uint32_t>(), win2.as<uint32_t>(),
+                              order2.as<uint32_t>(), n_segs, bits_for((n - 1) / m->split.win_rows),
+                              rtmp.p, rtmp.cap, st, &alt));
+    CUDA_TRY(launch_seg_permute(alt ? order2.as<uint32_t>() : order.as<uint32_t>(),
+                                e0.as<int64_t>(), e1.as<int64_t>(), n_segs,
+                                m->seg_e0.as<int64_t>(), m->seg_e1.as<int64_t>(),
+                                m->seg_slot.as<int32_t>(), st));
+    // split rows heaviest first (the hop's fixup order); the segments' sort
+    // buffers are free again
+    bool alt2 = false;
+    CUDA_TRY(radix_sort_pairs(row_key, row_id, win.as<uint32_t>(), win2.as<uint32_t>(), n_split,
+                              bits_for(n_segs), rtmp.p, rtmp.cap, st, &alt2));
+    CUDA_TRY(cudaMemcpyAsync(m->split_order.p, alt2 ? win2.p : row_id, (size_t)n_split * 4,
+                             cudaMemcpyDeviceToDevice, st));
+    return AKASHIC_OK;
 }
 
 // ================================================================== ABI
@@ -734,6 +730,7 @@ akashic_status_t akashic_mem_append_chunks(akashic_mem_t *m, const uint16_t *emb
         return check_status(m, st, "append");
     }
     AK_TRY(rebuild_in_edges(m, st));
+    CUDA_TRY(cudaStreamSynchronize(st));
     return AKASHIC_OK;
 }
 
@@ -874,6 +871,7 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
             AK_TRY(build_split_plan(m, st));
         }
     }
+    CUDA_TRY(cudaStreamSynchronize(st));
     return AKASHIC_OK;
 }
 
@@ -942,54 +940,93 @@ akashic_status_t akashic_mem_delete(akashic_mem_t *m, const int64_t *ids, int64_
     m->has_dead = true;
     const int64_t rows = m->n, nnz = m->nnz;
     if (nnz == 0) return AKASHIC_OK;
-    const size_t tb = scan_tmp_bytes(nnz + 1) + 4096;
-    int64_t *keep = (int64_t *)store_scratch(m, SCR_DEL_KEEP, (size_t)(nnz + 1) * 8);
-    int64_t *pos = (int64_t *)store_scratch(m, SCR_DEL_POS, (size_t)(nnz + 1) * 8);
-    void *tmp = store_scratch(m, SCR_DEL_TMP, tb);
-    if (!keep || !pos || !tmp) return fail(AKASHIC_ENOMEM, "delete: out of device memory");
-    // out-edge CSR (rows are chunk IDs, targets chunk IDs)
+    // bitmaps of the deleted chunks and of the rows whose weights change, and
+    // the compaction's scratch; what has to start at zero comes first
+    const size_t rb = (size_t)ceil_div<int64_t>(rows, 32) * 4;
+    const size_t eb = (size_t)ceil_div<int64_t>(nnz, 32) * 4;
+    const size_t cb = (size_t)(drop_tiles(nnz) + 1) * 8;
+    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t zero = 2 * up(cb) + 2 * up(rb) + 2 * up(eb);
+    uint8_t *scr = (uint8_t *)store_scratch(m, SCR_DEL, zero + up(rb) + 2 * up(eb));
+    if (!scr) return fail(AKASHIC_ENOMEM, "delete: out of device memory");
+    unsigned long long *chain = (unsigned long long *)scr;
+    unsigned long long *chain_in = (unsigned long long *)(scr + up(cb));
+    uint32_t *dead_id = (uint32_t *)(scr + 2 * up(cb));
+    uint32_t *touched = (uint32_t *)(scr + 2 * up(cb) + up(rb));
+    uint32_t *drop = (uint32_t *)(scr + 2 * up(cb) + 2 * up(rb));
+    uint32_t *drop_in = (uint32_t *)(scr + 2 * up(cb) + 2 * up(rb) + up(eb));
+    uint32_t *dead_bits = (uint32_t *)(scr + zero);
+    uint32_t *keep = (uint32_t *)(scr + zero + up(rb));
+    int32_t *word_pos = (int32_t *)(scr + zero + up(rb) + up(eb));
     AK_TRY(ensure_spare(m->rp2, (size_t)(m->cap + 1) * 8));
     AK_TRY(ensure_spare(m->col2, (size_t)nnz * 4));
     AK_TRY(ensure_spare(m->aff2, (size_t)nnz * 4));
-    DropDead d{rows, nnz, m->row_ptr.as<int64_t>(), m->col.as<int32_t>(), m->aff.as<float>(),
-               m->row_of.as<int32_t>(), m->dead_row.as<int32_t>(), ids, n, rows, nullptr,
-               keep, pos, tmp, tb, m->rp2.as<int64_t>(), m->col2.as<int32_t>(),
-               m->aff2.as<float>()};
-    CUDA_TRY(launch_drop_dead_edges(d, st));
-    int64_t nnz_new = 0;
-    CUDA_TRY(cudaMemcpyAsync(&nnz_new, pos + nnz, 8, cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    std::swap(m->row_ptr.p, m->rp2.p);
-    std::swap(m->row_ptr.cap, m->rp2.cap);
-    std::swap(m->col.p, m->col2.p);
-    std::swap(m->col.cap, m->col2.cap);
-    std::swap(m->aff.p, m->aff2.p);
-    std::swap(m->aff.cap, m->aff2.cap);
-    m->nnz = nnz_new;
-    AK_TRY(m->w.ensure(m->col.cap > 4 ? m->col.cap : 4, false));
-    CUDA_TRY(launch_row_softmax(m->row_ptr.as<int64_t>(), m->aff.as<float>(), m->w.as<float>(),
-                                rows, m->rstat.as<float2>(), st));
-    // in-edge transpose (rows are store rows, sources rows); the same edges go
+    AK_TRY(ensure_spare(m->w2, (size_t)nnz * 4));
     AK_TRY(ensure_spare(m->in_ptr2, (size_t)(m->cap + 1) * 8));
     AK_TRY(ensure_spare(m->in_src2, (size_t)nnz * 4));
     AK_TRY(ensure_spare(m->in_aff2, (size_t)nnz * 4));
     AK_TRY(ensure_spare(m->in_w2, (size_t)nnz * 4));
-    DropDead di{rows, nnz, m->in_ptr.as<int64_t>(), m->in_src.as<int32_t>(), m->in_aff.as<float>(),
-                nullptr, m->dead_row.as<int32_t>(), ids, n, rows, m->row_of.as<int32_t>(),
-                keep, pos, tmp, tb, m->in_ptr2.as<int64_t>(), m->in_src2.as<int32_t>(),
-                m->in_aff2.as<float>()};
+    CUDA_TRY(cudaMemsetAsync(scr, 0, zero, st));
+    CUDA_TRY(launch_dead_bits(m->dead_row.as<int32_t>(), m->ext_of.as<int32_t>(), rows, dead_bits,
+                              dead_id, st));
+    // out-edge CSR (rows are chunk IDs, targets chunk IDs)
+    DropDead d{};
+    d.n_rows = rows;
+    d.nnz = nnz;
+    d.ptr = m->row_ptr.as<int64_t>();
+    d.tgt = m->col.as<int32_t>();
+    d.val = m->aff.as<float>();
+    d.w = m->w.as<float>();
+    d.dead_bits = dead_id;
+    d.ids = ids;
+    d.n_ids = n;
+    d.n_total = rows;
+    d.drop_bits = drop;
+    d.keep_bits = keep;
+    d.word_pos = word_pos;
+    d.chain = chain;
+    d.status = m->status.as<int>();
+    d.tgt_out = m->col2.as<int32_t>();
+    d.val_out = m->aff2.as<float>();
+    d.w_out = m->w2.as<float>();
+    CUDA_TRY(launch_drop_dead_edges(d, st));
+    CUDA_TRY(launch_drop_row_ptr(d, m->rp2.as<int64_t>(), m->w2.as<float>(),
+                                 m->rstat.as<float2>(), m->row_of.as<int32_t>(), touched, st));
+    int64_t nnz_new = 0;
+    CUDA_TRY(cudaMemcpyAsync(&nnz_new, m->rp2.as<int64_t>() + rows, 8, cudaMemcpyDeviceToHost, st));
+    // in-edge transpose (rows are store rows, sources rows); the same edges go
+    DropDead di = d;
+    di.ptr = m->in_ptr.as<int64_t>();
+    di.tgt = m->in_src.as<int32_t>();
+    di.val = m->in_aff.as<float>();
+    di.w = m->in_w.as<float>();
+    di.dead_bits = dead_bits;
+    di.own_row_of = m->row_of.as<int32_t>();
+    di.touched = touched;
+    di.ext_of = m->ext_of.as<int32_t>();
+    di.rstat = m->rstat.as<float2>();
+    di.drop_bits = drop_in;
+    di.chain = chain_in;
+    di.tgt_out = m->in_src2.as<int32_t>();
+    di.val_out = m->in_aff2.as<float>();
+    di.w_out = m->in_w2.as<float>();
     CUDA_TRY(launch_drop_dead_edges(di, st));
-    CUDA_TRY(launch_in_weights(m->in_src2.as<int32_t>(), m->in_aff2.as<float>(), nnz_new,
-                               m->ext_of.as<int32_t>(), m->rstat.as<float2>(),
-                               m->in_w2.as<float>(), st));
-    std::swap(m->in_ptr.p, m->in_ptr2.p);
-    std::swap(m->in_ptr.cap, m->in_ptr2.cap);
-    std::swap(m->in_src.p, m->in_src2.p);
-    std::swap(m->in_src.cap, m->in_src2.cap);
-    std::swap(m->in_aff.p, m->in_aff2.p);
-    std::swap(m->in_aff.cap, m->in_aff2.cap);
-    std::swap(m->in_w.p, m->in_w2.p);
-    std::swap(m->in_w.cap, m->in_w2.cap);
+    CUDA_TRY(launch_drop_row_ptr(di, m->in_ptr2.as<int64_t>(), nullptr, nullptr, nullptr, nullptr,
+                                 st));
+    CUDA_TRY(cudaStreamSynchronize(st));
+    m->nnz = nnz_new;
+    auto swap = [](DevBuf &x, DevBuf &y) {
+        std::swap(x.p, y.p);
+        std::swap(x.cap, y.cap);
+    };
+    swap(m->row_ptr, m->rp2);
+    swap(m->col, m->col2);
+    swap(m->aff, m->aff2);
+    swap(m->w, m->w2);
+    swap(m->in_ptr, m->in_ptr2);
+    swap(m->in_src, m->in_src2);
+    swap(m->in_aff, m->in_aff2);
+    swap(m->in_w, m->in_w2);
     AK_TRY(build_split_plan(m, st));
     return check_status(m, st, "delete");
 }

@@ -42,6 +42,51 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// ------------------------------------------------------------------ ordered tiles
+// One-pass ordered compaction: CTAs take tiles by ticket, and a tile learns
+// where its survivors go from the tiles before it.  chain[] holds one word a
+// tile, zero at first: CHAIN_SUM | the tile's own count, then CHAIN_TOTAL | the
+// count of all tiles up to it.  Called by one whole warp once the tile's count
+// `own` is known; returns the count of the tiles first .. tile - 1.  A tile
+// only waits for tiles whose ticket was taken before its own, so the wait
+// ends; it is bounded all the same (ETIMEOUT, and a value too small).
+constexpr unsigned long long CHAIN_SUM = 1ull << 62, CHAIN_TOTAL = 2ull << 62;
+constexpr unsigned long long CHAIN_VALUE = CHAIN_SUM - 1;
+constexpr uint32_t CHAIN_POLLS = 1u << 24;
+__device__ __forceinline__ unsigned long long chain_before(volatile unsigned long long *chain,
+                                                           int64_t first, int64_t tile,
+                                                           unsigned long long own, int *status) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long before = 0ull;
+    if (tile > first) {
+        if (lane == 0) chain[tile] = CHAIN_SUM | own;
+        bool more = true;
+        for (int64_t hi = tile - 1; more; hi -= 32) {
+            const int64_t at = hi - lane;
+            unsigned long long v = CHAIN_TOTAL;      // before the first: 0 in all
+            uint32_t polls = 0;
+            if (at >= first)
+                while (((v = chain[at]) >> 62) == 0ull) {
+                    if (++polls > CHAIN_POLLS) {
+                        set_status(status, AKASHIC_ETIMEOUT);
+                        v = CHAIN_TOTAL;
+                        break;
+                    }
+                }
+            __syncwarp();
+            const unsigned tot = __ballot_sync(0xffffffffu, (v >> 62) == 2ull);
+            const int stop = tot ? __ffs(tot) - 1 : 31;   // the nearest total
+            unsigned long long x = lane <= stop ? v & CHAIN_VALUE : 0ull;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            before += x;
+            more = tot == 0u;
+        }
+    }
+    if (lane == 0) chain[tile] = CHAIN_TOTAL | (before + own);
+    return before;
+}
+
 // ------------------------------------------------------------------ small helpers
 __device__ __forceinline__ float bf16_to_f32(uint16_t h) {
     return __uint_as_float(((uint32_t)h) << 16);
@@ -354,32 +399,32 @@ struct InEdgeScratch {
 };
 cudaError_t launch_in_edges_update(const InEdgeUpdate &u, const InEdgeScratch &s, cudaStream_t st,
                                    int *launches);
-// in_w[e] = row_softmax_weight(in_aff[e], rstat[ext_of[in_src[e]]])
-cudaError_t launch_in_weights(const int32_t *in_src, const float *in_aff, int64_t nnz,
-                              const int32_t *ext_of, const float2 *rstat, float *in_w,
-                              cudaStream_t st);
 cudaError_t launch_batch_layout(const uint32_t *order, int64_t first, int64_t n, int dim,
                                 const uint16_t *emb_in, uint16_t *emb, const int32_t *page_in,
                                 int64_t first_page, int per_page, int32_t *page_row,
                                 int32_t *ext_of, int32_t *row_of, cudaStream_t st);
-// Split plan (see SPLIT_T): per row the number of segments (0 for rows kept
-// whole) and a split flag; then the segments themselves with their window.
-cudaError_t launch_split_count(const SplitParams &sp, const int64_t *in_ptr, const int32_t *in_src,
-                               int64_t n, int64_t *nseg, int64_t *flag, cudaStream_t st);
-cudaError_t launch_split_fill(const SplitParams &sp, const int64_t *in_ptr, const int32_t *in_src,
-                              int64_t n,
-                              const int64_t *nseg, const int64_t *slot_off,
-                              const int64_t *split_idx, int32_t *split_row, int64_t *split_slot0,
-                              int64_t *seg_e0, int64_t *seg_e1, uint32_t *seg_win,
-                              cudaStream_t st);
+// Hub plan (see SplitParams), first its sizes: rows = the hub rows in row order
+// (at most max_hubs), slot0 = their first partial slots, counts[0] / [1] = the
+// number of hub rows / segments.  chain: hub_plan_words(n, max_hubs) words.
+int64_t hub_plan_words(int64_t n, int64_t max_hubs);
+cudaError_t launch_hub_count(const SplitParams &sp, const int64_t *in_ptr, const int32_t *in_src,
+                             int64_t n, int64_t max_hubs, int32_t *rows, int64_t *slot0,
+                             int64_t *counts, unsigned long long *chain, int *status,
+                             cudaStream_t st);
+// Then the plan: the split rows and their slots, the segments (by row, then
+// window) with their window as sort key and their index as value, the split row
+// that owns each slot, and sort keys / values that order the split rows by
+// segment count, largest first, ties in row order.
+cudaError_t launch_hub_fill(const SplitParams &sp, const int64_t *in_ptr, const int32_t *in_src,
+                            const int32_t *rows, const int64_t *slot0, int64_t n_rows,
+                            int64_t n_segs, int32_t *split_row, int64_t *split_slot0,
+                            int64_t *seg_e0, int64_t *seg_e1, uint32_t *seg_win, uint32_t *seg_id,
+                            int32_t *slot_split, uint32_t *row_key, uint32_t *row_id,
+                            cudaStream_t st);
 // Permute segments into window-major order: dst[i] = src[order[i]], slot[i] = order[i].
 cudaError_t launch_seg_permute(const uint32_t *order, const int64_t *e0, const int64_t *e1,
                                int64_t n_segs, int64_t *e0s, int64_t *e1s, int32_t *slot,
                                cudaStream_t st);
-
-// keys[r] = ~(slot count of split row r), vals[r] = r (sorted: heaviest first).
-cudaError_t launch_split_keys(const int64_t *slot0, int64_t n_split, uint32_t *keys,
-                              uint32_t *vals, cudaStream_t st);
 
 // Memory Manager tables (ak_mm.cu): the page directory's slot counters,
 // the co-retrieval statistics and the running counters.
@@ -446,28 +491,43 @@ cudaError_t launch_mark_dead(const int64_t *ids, int64_t n, int64_t n_total, con
 cudaError_t launch_check_dead_targets(const int32_t *col, int64_t nnz, int64_t first,
                                       const int32_t *row_of, const int32_t *dead_row, int *status,
                                       cudaStream_t st);
-// One CSR without the edges that touch a dead row: an edge survives if its
-// target (tgt[e], mapped through tgt_row_of unless NULL) is not dead and it
-// is not in the row of a listed ID (rows found through own_row_of unless
-// NULL).  Survivors keep their order; ptr_out[r] = new start of row r.
+// Bitmaps of the deleted chunks, by row and by chunk ID ((n + 31) / 32 words
+// each, by_id zeroed before), from dead_row.
+cudaError_t launch_dead_bits(const int32_t *dead_row, const int32_t *ext_of, int64_t n,
+                             uint32_t *by_row, uint32_t *by_id, cudaStream_t st);
+// One edge list without the edges that touch a deleted chunk: an edge survives
+// if its target is not deleted (bit tgt of dead_bits) and it is not in the row
+// of a listed ID (rows found through own_row_of unless NULL).  Survivors keep
+// their order and their logit and weight; where touched is given, an edge whose
+// target's bit is set there gets its weight anew, row_softmax_weight(val,
+// rstat[ext_of[target]]).
 struct DropDead {
     int64_t n_rows, nnz;
-    const int64_t *ptr;                 // [n_rows+1]
+    const int64_t *ptr;                 // [n_rows + 1]
     const int32_t *tgt;                 // [nnz]
-    const float *val;                   // [nnz] carried along (logits)
-    const int32_t *tgt_row_of;          // chunk ID -> row for targets, or NULL (targets are rows)
-    const int32_t *dead_row;            // [rows]
+    const float *val, *w;               // [nnz] logits, weights
+    const uint32_t *dead_bits;          // by what tgt holds
     const int64_t *ids;                 // [n_ids] deleted chunk IDs
     int64_t n_ids, n_total;
-    const int32_t *own_row_of;          // chunk ID -> row of the CSR, or NULL (CSR rows are IDs)
-    int64_t *keep, *pos;                // scratch [nnz+1] each
-    void *tmp;                          // scan scratch
-    size_t tmp_bytes;
-    int64_t *ptr_out;                   // [n_rows+1]
+    const int32_t *own_row_of;          // chunk ID -> row of the list, or NULL (rows are IDs)
+    const uint32_t *touched;            // or NULL
+    const int32_t *ext_of;
+    const float2 *rstat;
+    uint32_t *drop_bits;                // scratch [(nnz + 31) / 32], zeroed before
+    uint32_t *keep_bits;                // scratch [(nnz + 31) / 32]: the survivors
+    int32_t *word_pos;                  // scratch [(nnz + 31) / 32]: survivors before a word
+    unsigned long long *chain;          // scratch [drop_tiles(nnz) + 1], zeroed before
+    int *status;
     int32_t *tgt_out;                   // [nnz]
-    float *val_out;                     // [nnz]
+    float *val_out, *w_out;             // [nnz]
 };
+int64_t drop_tiles(int64_t nnz);
 cudaError_t launch_drop_dead_edges(const DropDead &d, cudaStream_t st);
+// The row starts after launch_drop_dead_edges.  w (or NULL): rows that lost an
+// edge get their softmax anew (w, rstat) and their row's bit in touched
+// (row_of maps the list's rows, chunk IDs; zeroed before).
+cudaError_t launch_drop_row_ptr(const DropDead &d, int64_t *ptr_out, float *w, float2 *rstat,
+                                const int32_t *row_of, uint32_t *touched, cudaStream_t st);
 
 // Propagation hop (a2): out[j,:] = u[j,:] + alpha * sum_{i->j} w_ij * in[i,:].
 struct HopPlan {
@@ -687,9 +747,6 @@ cudaError_t launch_reach_fma(const float *u, int bp, int B, int64_t n, const flo
                              const int32_t *rows, const int32_t *ext_of, float *partial,
                              unsigned int *cnt, unsigned long long *buf, int64_t cap,
                              cudaStream_t st, int *launches);
-// slot_split[s] = r for every partial slot s of split row r.
-cudaError_t launch_slot_owner(const int64_t *split_slot0, int64_t n_split, int32_t *slot_split,
-                              cudaStream_t st);
 // `counters` = 2 device ints (work queues), zeroed before.
 // `flt` may be NULL (no filter), `hb` NULL (no row bounds).
 cudaError_t launch_hop(const HopPlan &p, const float *u, const float *in, float *out, int bp,

@@ -2,9 +2,10 @@
 // copies are logically tombstoned, §4.2): a deleted chunk keeps its row but
 // is marked dead, gets no score, is never a candidate, and every relation
 // edge into or out of it is dropped from both the out-edge CSR and the
-// in-edge transpose.  Compaction is edge-parallel: per-edge keep flags, one
-// exclusive scan for the new positions, a scatter, and the new row pointers
-// read from the scan at the old row starts.
+// in-edge transpose.  Each list is compacted in one edge-parallel pass over
+// its targets, logits and weights, in ordered tiles; what it keeps of every 32
+// edges (a mask and the count before them) gives the new row starts.  Rows
+// that lost nothing keep their weights.
 #include "ak_common.cuh"
 
 namespace ak {
@@ -28,52 +29,196 @@ __global__ void k_mark_dead(const int64_t *__restrict__ ids, int64_t n, int64_t 
     }
 }
 
-// keep[e] = 1 unless the edge's target (a chunk ID for the out-CSR, mapped
-// to its row; a row for the transpose) or its listed source row is dead.
-// The other end is handled per row by k_drop_rows.
-__global__ void k_keep_by_target(const int32_t *__restrict__ tgt, int64_t nnz,
-                                 const int32_t *__restrict__ row_of,
-                                 const int32_t *__restrict__ dead_row, int64_t *__restrict__ keep) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nnz;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t t = tgt[e];
-        keep[e] = dead_row[row_of ? row_of[t] : t] ? 0 : 1;
+__global__ void k_dead_bits(const int32_t *__restrict__ dead_row,
+                            const int32_t *__restrict__ ext_of, int64_t n,
+                            uint32_t *__restrict__ by_row, uint32_t *__restrict__ by_id) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    // warp-uniform trip count: whole words
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < ((n + 31) & ~(int64_t)31);
+         r += stride) {
+        const bool dead = r < n && dead_row[r] != 0;
+        const unsigned bits = __ballot_sync(0xffffffffu, dead);
+        if ((threadIdx.x & 31) == 0) by_row[r >> 5] = bits;
+        if (dead) {
+            const uint32_t id = (uint32_t)ext_of[r];
+            atomicOr(&by_id[id >> 5], 1u << (id & 31));
+        }
     }
+}
+
+cudaError_t launch_dead_bits(const int32_t *dead_row, const int32_t *ext_of, int64_t n,
+                             uint32_t *by_row, uint32_t *by_id, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    k_dead_bits<<<device_sm_count() * 4, 256, 0, st>>>(dead_row, ext_of, n, by_row, by_id);
+    return cudaGetLastError();
 }
 
 // Every edge of the listed IDs' own rows is dropped (their out-edges in the
-// out-CSR, their in-edges in the transpose): one warp per deleted chunk.
+// out-CSR, their in-edges in the transpose): one CTA per deleted chunk, a word
+// of 32 edges a thread (a hub's row has 10^5 and more).
 __global__ void k_drop_rows(const int64_t *__restrict__ ids, int64_t n, int64_t n_total,
                             const int32_t *__restrict__ row_of, const int64_t *__restrict__ ptr,
-                            int64_t *__restrict__ keep) {
-    const int lane = threadIdx.x & 31;
-    int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (; i < n; i += stride) {
+                            uint32_t *__restrict__ drop_bits) {
+    for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
         const int64_t id = ids[i];
         if (id < 0 || id >= n_total) continue;
         const int64_t r = row_of ? row_of[id] : id;
-        for (int64_t e = ptr[r] + lane; e < ptr[r + 1]; e += 32) keep[e] = 0;
+        const int64_t a = ptr[r], b = ptr[r + 1];
+        if (a >= b) continue;
+        for (int64_t w = (a >> 5) + threadIdx.x; w <= (b - 1) >> 5; w += blockDim.x) {
+            const int lo = a > 32 * w ? (int)(a - 32 * w) : 0;
+            const int hi = b < 32 * (w + 1) ? (int)(b - 32 * w) : 32;
+            const uint32_t m = (hi == 32 ? ~0u : (1u << hi) - 1u) & ~((1u << lo) - 1u);
+            atomicOr(&drop_bits[w], m);
+        }
     }
 }
 
-__global__ void k_compact_edges(const int64_t *__restrict__ keep, const int64_t *__restrict__ pos,
-                                int64_t nnz, const int32_t *__restrict__ a_in,
-                                const float *__restrict__ b_in, int32_t *__restrict__ a_out,
-                                float *__restrict__ b_out) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nnz;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        if (!keep[e]) continue;
-        a_out[pos[e]] = a_in[e];
-        b_out[pos[e]] = b_in[e];
+// The compaction: DROP_TILE consecutive edges a tile, 16 words of 32 edges a
+// warp.  Bound by memory: 12 bytes an edge read and written once, the bitmaps
+// cached.  (It took flags, a scan and positions of 8 bytes an edge in memory
+// before, ~60 bytes an edge more, and a softmax of every row: 1.20 ms for 200
+// chunks of 524,288 with 16.8M edges, read-back included, 0.64 now; a list's
+// 403 MB take 114 us.  Eight words a warp: 135.)
+constexpr int DROP_WORDS = 16;                          // a warp
+constexpr int DROP_TILE = 8 * 32 * DROP_WORDS;
+int64_t drop_tiles(int64_t nnz) { return ceil_div<int64_t>(nnz, DROP_TILE); }
+
+__global__ __launch_bounds__(256, 4) void k_drop_edges(const DropDead d) {
+    __shared__ int warp_n[8];
+    __shared__ unsigned long long base_s;
+    __shared__ int64_t tile_s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const int64_t tiles = (d.nnz + DROP_TILE - 1) / DROP_TILE;
+    while (true) {
+        __syncthreads();   // the tile before is done with the shared words
+        if (threadIdx.x == 0) tile_s = (int64_t)atomicAdd(d.chain, 1ull);
+        __syncthreads();
+        const int64_t tile = tile_s;
+        if (tile >= tiles) break;
+        const int64_t e0 = tile * DROP_TILE + warp * 32 * DROP_WORDS;
+        int32_t t[DROP_WORDS];
+        float v[DROP_WORDS], w[DROP_WORDS];
+#pragma unroll
+        for (int j = 0; j < DROP_WORDS; ++j) {
+            const int64_t e = e0 + 32 * j + lane;
+            t[j] = e < d.nnz ? __ldcs(d.tgt + e) : -1;
+        }
+#pragma unroll
+        for (int j = 0; j < DROP_WORDS; ++j) {
+            const int64_t e = e0 + 32 * j + lane;
+            v[j] = e < d.nnz ? __ldcs(d.val + e) : 0.f;
+            w[j] = e < d.nnz ? __ldcs(d.w + e) : 0.f;
+        }
+        // lane j holds word j's bits from here on
+        const int64_t word0 = e0 >> 5;
+        const bool has_word = lane < DROP_WORDS && e0 + 32 * lane < d.nnz;
+        const uint32_t drop = has_word ? d.drop_bits[word0 + lane] : ~0u;
+        uint32_t mine = 0u;
+#pragma unroll
+        for (int j = 0; j < DROP_WORDS; ++j) {
+            const bool live = t[j] >= 0 && !((__ldg(d.dead_bits + (t[j] >> 5)) >> (t[j] & 31)) & 1u);
+            const uint32_t keep = __ballot_sync(0xffffffffu, live);
+            if (lane == j) mine = keep & ~drop;
+        }
+        // survivors before each word of the warp, then before each warp
+        int incl = __popc(mine);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += x;
+        }
+        const int pre = incl - __popc(mine);
+        if (lane == 31) warp_n[warp] = incl;
+        __syncthreads();
+        int own = 0, wpre = 0;
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+            if (x < warp) wpre += warp_n[x];
+            own += warp_n[x];
+        }
+        if (warp == 0) {
+            const unsigned long long before =
+                chain_before(d.chain + 1, 0, tile, (unsigned long long)own, d.status);
+            if (lane == 0) base_s = before;
+        }
+        __syncthreads();
+        const int64_t base = (int64_t)base_s + wpre;
+        if (has_word) {
+            d.keep_bits[word0 + lane] = mine;
+            d.word_pos[word0 + lane] = (int32_t)(base + pre);
+        }
+#pragma unroll
+        for (int j = 0; j < DROP_WORDS; ++j) {
+            const uint32_t keep = __shfl_sync(0xffffffffu, mine, j);
+            const int at = __shfl_sync(0xffffffffu, pre, j);
+            if (!((keep >> lane) & 1u)) continue;
+            const int64_t p = base + at + __popc(keep & lt);
+            float wj = w[j];
+            if (d.touched && ((__ldg(d.touched + (t[j] >> 5)) >> (t[j] & 31)) & 1u))
+                wj = row_softmax_weight(v[j], d.rstat[d.ext_of[t[j]]]);
+            __stcs(d.tgt_out + p, t[j]);
+            __stcs(d.val_out + p, v[j]);
+            __stcs(d.w_out + p, wj);
+        }
     }
 }
 
-__global__ void k_new_ptr(const int64_t *__restrict__ ptr, const int64_t *__restrict__ pos,
-                          int64_t n, int64_t *__restrict__ new_ptr) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r <= n;
-         r += (int64_t)gridDim.x * blockDim.x)
-        new_ptr[r] = pos[ptr[r]];
+// new start of a row = the survivors before its old first edge
+__device__ __forceinline__ int64_t kept_before(const DropDead &d, int64_t e, int64_t total) {
+    if (e >= d.nnz) return total;
+    return d.word_pos[e >> 5] + __popc(d.keep_bits[e >> 5] & ((1u << (e & 31)) - 1u));
+}
+
+// Eight lanes a row: the new starts, and (out-CSR) the softmax of the rows that
+// lost an edge, as k_row_softmax does it.
+__global__ __launch_bounds__(256) void k_drop_row_ptr(const DropDead d,
+                                                      int64_t *__restrict__ ptr_out,
+                                                      float *__restrict__ w,
+                                                      float2 *__restrict__ rstat,
+                                                      const int32_t *__restrict__ row_of,
+                                                      uint32_t *__restrict__ touched) {
+    constexpr int L = 8;
+    const int lane = threadIdx.x & 31, sub = lane % L;
+    const int64_t step = ((int64_t)gridDim.x * blockDim.x) / L;
+    const int64_t warp0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (32 / L);
+    const int64_t total =
+        (int64_t)d.chain[(d.nnz + DROP_TILE - 1) / DROP_TILE] & CHAIN_VALUE;
+    for (int64_t r0 = warp0; r0 <= d.n_rows; r0 += step) {   // (warp-uniform)
+        const int64_t r = r0 + lane / L;
+        int64_t old = 0, a = 0, b = 0;
+        if (r < d.n_rows) {
+            const int64_t p0 = d.ptr[r], p1 = d.ptr[r + 1];
+            old = p1 - p0;
+            a = kept_before(d, p0, total);
+            b = kept_before(d, p1, total);
+            if (sub == 0) ptr_out[r] = a;
+        } else if (r == d.n_rows && sub == 0) {
+            ptr_out[r] = total;
+        }
+        const bool lost = w && r < d.n_rows && b - a != old;
+        if (!__any_sync(0xffffffffu, lost)) continue;
+        float m = -INFINITY;
+        if (lost)
+            for (int64_t e = a + sub; e < b; e += L) m = fmaxf(m, d.val_out[e]);
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        float s = 0.f;
+        if (lost)
+            for (int64_t e = a + sub; e < b; e += L) s += expf(d.val_out[e] - m);
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lost && b > a) {
+            const float2 stat = make_float2(m, 1.f / s);
+            if (sub == 0) {
+                rstat[r] = stat;
+                const uint32_t row = (uint32_t)row_of[r];
+                atomicOr(&touched[row >> 5], 1u << (row & 31));
+            }
+            for (int64_t e = a + sub; e < b; e += L) w[e] = row_softmax_weight(d.val_out[e], stat);
+        }
+    }
 }
 
 // Edges handed to an append may not point at a deleted chunk (targets below
@@ -108,28 +253,24 @@ cudaError_t launch_mark_dead(const int64_t *ids, int64_t n, int64_t n_total, con
 
 cudaError_t launch_drop_dead_edges(const DropDead &d, cudaStream_t st) {
     const int sms = device_sm_count();
-    if (d.nnz > 0) {
-        k_keep_by_target<<<sms * 8, 256, 0, st>>>(d.tgt, d.nnz, d.tgt_row_of, d.dead_row, d.keep);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        if (d.n_ids > 0) {
-            k_drop_rows<<<sms * 2, 256, 0, st>>>(d.ids, d.n_ids, d.n_total, d.own_row_of, d.ptr,
-                                                 d.keep);
-            e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-        }
+    if (d.nnz <= 0) return cudaErrorInvalidValue;
+    if (d.n_ids > 0) {
+        const int64_t g = d.n_ids < (int64_t)sms * 16 ? d.n_ids : (int64_t)sms * 16;
+        k_drop_rows<<<(unsigned)g, 128, 0, st>>>(d.ids, d.n_ids, d.n_total, d.own_row_of, d.ptr,
+                                                 d.drop_bits);
     }
-    // keep[nnz] = 0 so that pos[nnz] is the surviving count
-    cudaError_t e = cudaMemsetAsync(d.keep + d.nnz, 0, 8, st);
-    if (e == cudaSuccess) e = scan_exclusive(d.keep, d.pos, d.nnz + 1, d.tmp, d.tmp_bytes, st);
-    if (e != cudaSuccess) return e;
-    if (d.nnz > 0) {
-        k_compact_edges<<<sms * 8, 256, 0, st>>>(d.keep, d.pos, d.nnz, d.tgt, d.val, d.tgt_out,
-                                                 d.val_out);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    k_new_ptr<<<sms * 4, 256, 0, st>>>(d.ptr, d.pos, d.n_rows, d.ptr_out);
+    const int64_t tiles = drop_tiles(d.nnz);
+    const int64_t cap = (int64_t)sms * 8;
+    k_drop_edges<<<(unsigned)(tiles < cap ? tiles : cap), 256, 0, st>>>(d);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_drop_row_ptr(const DropDead &d, int64_t *ptr_out, float *w, float2 *rstat,
+                                const int32_t *row_of, uint32_t *touched, cudaStream_t st) {
+    const int64_t want = ceil_div<int64_t>((d.n_rows + 1) * 8, 256);
+    const int64_t cap = (int64_t)device_sm_count() * 16;
+    k_drop_row_ptr<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(d, ptr_out, w, rstat,
+                                                                       row_of, touched);
     return cudaGetLastError();
 }
 

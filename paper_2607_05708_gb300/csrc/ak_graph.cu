@@ -688,102 +688,167 @@ __device__ __forceinline__ int64_t lower_bound_src(const int32_t *__restrict__ s
 }
 
 // A hub row (more than split_t in-edges, sorted by source row) cut by one
-// warp: lane l takes source windows w0 + l, w0 + l + 32, ...; the edge range
-// of each window comes from two binary searches, and its segments (at most
-// seg_len edges each) are numbered by a scan across the lanes in window
-// order.  Returns the row's segment count (on every lane).
-template <bool FILL>
+// warp: lane l takes source windows w0 + l, w0 + l + 32, ...; a window starts
+// where a binary search finds its first source and ends where the next lane's
+// starts, and its segments (at most seg_len edges each) are numbered by a scan
+// across the lanes in window order; emit(segment, first edge, end, window) for
+// each.  Returns the row's segment count (on every lane).
+template <typename Emit>
 __device__ int64_t warp_segments(const SplitParams &sp, const int32_t *__restrict__ in_src,
-                                 int64_t a, int64_t b, int64_t slot, int64_t *seg_e0,
-                                 int64_t *seg_e1, uint32_t *seg_win) {
+                                 int64_t a, int64_t b, Emit emit) {
     const int lane = threadIdx.x & 31;
     const int64_t w0 = (int64_t)in_src[a] / sp.win_rows, w1 = (int64_t)in_src[b - 1] / sp.win_rows;
     int64_t base = 0;
     for (int64_t wb = w0; wb <= w1; wb += 32) {
         const int64_t w = wb + lane;
-        int64_t lo = 0, cnt = 0, hi = 0;
-        if (w <= w1) {
-            lo = w == w0 ? a : lower_bound_src(in_src, a, b, w * sp.win_rows);
-            hi = w == w1 ? b : lower_bound_src(in_src, lo, b, (w + 1) * sp.win_rows);
-            cnt = (hi - lo + sp.seg_len - 1) / sp.seg_len;
-        }
+        const int64_t lo = w == w0 ? a : (w <= w1 ? lower_bound_src(in_src, a, b, w * sp.win_rows) : b);
+        int64_t hi = __shfl_down_sync(0xffffffffu, lo, 1);
+        if (lane == 31) hi = w < w1 ? lower_bound_src(in_src, lo, b, (w + 1) * sp.win_rows) : b;
+        const int64_t cnt = w <= w1 ? (hi - lo + sp.seg_len - 1) / sp.seg_len : 0;
         int64_t incl = cnt;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int64_t t = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += t;
         }
-        if (FILL) {
-            const int64_t at = slot + base + incl - cnt;
-            for (int64_t t = 0; t < cnt; ++t) {
-                const int64_t e = lo + t * sp.seg_len;
-                seg_e0[at + t] = e;
-                seg_e1[at + t] = e + sp.seg_len < hi ? e + sp.seg_len : hi;
-                seg_win[at + t] = (uint32_t)w;
-            }
+        for (int64_t t = 0; t < cnt; ++t) {
+            const int64_t e = lo + t * sp.seg_len;
+            emit(base + incl - cnt + t, e, e + sp.seg_len < hi ? e + sp.seg_len : hi, w);
         }
         base += __shfl_sync(0xffffffffu, incl, 31);
     }
     return base;
 }
 
-// Segment count of every row (0 below split_t).  A warp takes 32 rows; its
-// hub rows are then cut one after another by the whole warp.
-__global__ void k_split_count(SplitParams sp, const int64_t *__restrict__ in_ptr,
-                              const int32_t *__restrict__ in_src, int64_t n,
-                              int64_t *__restrict__ nseg, int64_t *__restrict__ flag) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t r0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; r0 < n;
-         r0 += nw * 32) {
-        const int64_t j = r0 + lane;
-        bool heavy = false;
-        if (j < n) {
-            heavy = in_ptr[j + 1] - in_ptr[j] > sp.split_t;
-            if (!heavy) {
-                nseg[j] = 0;
-                flag[j] = 0;
+// The hub rows (more than split_t in-edges) in row order, and their number: one
+// pass over the row starts in ordered tiles.
+constexpr int HEAVY_TILE = 1024;
+__global__ __launch_bounds__(256) void k_heavy_rows(const int64_t *__restrict__ in_ptr, int64_t n,
+                                                    int64_t split_t, int32_t *__restrict__ rows,
+                                                    int64_t *__restrict__ n_rows,
+                                                    unsigned long long *chain, int *status) {
+    __shared__ int wcnt[32];
+    __shared__ int64_t tile_s, base_s;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int64_t tiles = (n + HEAVY_TILE - 1) / HEAVY_TILE;
+    while (true) {
+        __syncthreads();
+        if (t == 0) tile_s = (int64_t)atomicAdd(chain, 1ull);
+        __syncthreads();
+        const int64_t tile = tile_s;
+        if (tile >= tiles) break;
+        unsigned bal[HEAVY_TILE / 256];
+#pragma unroll
+        for (int q = 0; q < HEAVY_TILE / 256; ++q) {
+            const int64_t i = tile * HEAVY_TILE + q * 256 + t;
+            bal[q] = __ballot_sync(0xffffffffu, i < n && in_ptr[i + 1] - in_ptr[i] > split_t);
+            if (lane == 0) wcnt[q * 8 + warp] = __popc(bal[q]);
+        }
+        __syncthreads();
+        if (warp == 0) {
+            const int c = wcnt[lane];
+            int incl = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += x;
+            }
+            wcnt[lane] = incl - c;
+            const unsigned long long own = (unsigned long long)__shfl_sync(0xffffffffu, incl, 31);
+            const unsigned long long before = chain_before(chain + 1, 0, tile, own, status);
+            if (lane == 0) {
+                base_s = (int64_t)before;
+                if (tile == tiles - 1) *n_rows = (int64_t)(before + own);
             }
         }
-        unsigned hv = __ballot_sync(0xffffffffu, heavy);
-        while (hv) {
-            const int l = __ffs(hv) - 1;
-            hv &= hv - 1;
-            const int64_t h = r0 + l;
-            const int64_t s = warp_segments<false>(sp, in_src, in_ptr[h], in_ptr[h + 1], 0, nullptr,
-                                                   nullptr, nullptr);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < HEAVY_TILE / 256; ++q)
+            if ((bal[q] >> lane) & 1u)
+                rows[base_s + wcnt[q * 8 + warp] + __popc(bal[q] & ((1u << lane) - 1u))] =
+                    (int32_t)(tile * HEAVY_TILE + q * 256 + t);
+    }
+}
+
+// First partial slot of every hub row and the number of segments: a warp a
+// row, a CTA eight consecutive ones, in ordered tiles.  (A warp that walked 32
+// rows of the store and cut the hubs among them one after another took 56 us
+// at 524,288 chunks, as a cut is a chain of ~20 dependent loads.)
+__global__ __launch_bounds__(256) void k_hub_slots(SplitParams sp,
+                                                   const int64_t *__restrict__ in_ptr,
+                                                   const int32_t *__restrict__ in_src,
+                                                   const int32_t *__restrict__ rows,
+                                                   const int64_t *__restrict__ n_rows,
+                                                   int64_t *__restrict__ slot0,
+                                                   int64_t *__restrict__ n_segs,
+                                                   unsigned long long *chain, int *status) {
+    __shared__ int64_t cnt[8];
+    __shared__ int64_t tile_s, base_s;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int64_t n = *n_rows, tiles = (n + 7) / 8;
+    while (true) {
+        __syncthreads();
+        if (t == 0) tile_s = (int64_t)atomicAdd(chain, 1ull);
+        __syncthreads();
+        const int64_t tile = tile_s;
+        if (tile >= tiles) break;
+        const int64_t i = tile * 8 + warp;
+        int64_t mine = 0;
+        if (i < n) {
+            const int64_t r = rows[i];
+            mine = warp_segments(sp, in_src, in_ptr[r], in_ptr[r + 1],
+                                 [](int64_t, int64_t, int64_t, int64_t) {});
+        }
+        if (lane == 0) cnt[warp] = mine;
+        __syncthreads();
+        if (warp == 0) {
+            int64_t own = 0;
+            for (int w = 0; w < 8; ++w) own += cnt[w];
+            const unsigned long long before =
+                chain_before(chain + 1, 0, tile, (unsigned long long)own, status);
             if (lane == 0) {
-                nseg[h] = s;
-                flag[h] = s > 0;
+                base_s = (int64_t)before;
+                if (tile == tiles - 1) *n_segs = (int64_t)before + own;
             }
+        }
+        __syncthreads();
+        if (lane == 0 && i < n) {
+            int64_t at = base_s;
+            for (int w = 0; w < warp; ++w) at += cnt[w];
+            slot0[i] = at;
         }
     }
 }
 
-__global__ void k_split_fill(SplitParams sp, const int64_t *__restrict__ in_ptr,
-                             const int32_t *__restrict__ in_src, int64_t n,
-                             const int64_t *__restrict__ nseg,
-                             const int64_t *__restrict__ slot_off,
-                             const int64_t *__restrict__ split_idx, int32_t *__restrict__ split_row,
-                             int64_t *__restrict__ split_slot0, int64_t *__restrict__ seg_e0,
-                             int64_t *__restrict__ seg_e1, uint32_t *__restrict__ seg_win) {
+// The plan of every hub row, a warp each: its segments with their window and
+// their owner, and the row's place by segment count (key n_segs - count, so
+// that ascending keys are heaviest first).
+__global__ void k_hub_fill(SplitParams sp, const int64_t *__restrict__ in_ptr,
+                           const int32_t *__restrict__ in_src, const int32_t *__restrict__ rows,
+                           const int64_t *__restrict__ slot0, int64_t n_rows, int64_t n_segs,
+                           int32_t *__restrict__ split_row, int64_t *__restrict__ split_slot0,
+                           int64_t *__restrict__ seg_e0, int64_t *__restrict__ seg_e1,
+                           uint32_t *__restrict__ seg_win, uint32_t *__restrict__ seg_id,
+                           int32_t *__restrict__ slot_split, uint32_t *__restrict__ row_key,
+                           uint32_t *__restrict__ row_id) {
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t r0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; r0 < n;
-         r0 += nw * 32) {
-        const int64_t j = r0 + lane;
-        unsigned hv = __ballot_sync(0xffffffffu, j < n && nseg[j] > 0);
-        while (hv) {
-            const int l = __ffs(hv) - 1;
-            hv &= hv - 1;
-            const int64_t h = r0 + l;
-            if (lane == 0) {
-                const int64_t idx = split_idx[h];
-                split_row[idx] = (int32_t)h;
-                split_slot0[idx] = slot_off[h];
-            }
-            warp_segments<true>(sp, in_src, in_ptr[h], in_ptr[h + 1], slot_off[h], seg_e0, seg_e1,
-                                seg_win);
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n_rows; i += nw) {
+        const int64_t r = rows[i], slot = slot0[i];
+        const int64_t cnt = warp_segments(
+            sp, in_src, in_ptr[r], in_ptr[r + 1], [&](int64_t s, int64_t e0, int64_t e1, int64_t w) {
+                seg_e0[slot + s] = e0;
+                seg_e1[slot + s] = e1;
+                seg_win[slot + s] = (uint32_t)w;
+                seg_id[slot + s] = (uint32_t)(slot + s);
+                slot_split[slot + s] = (int32_t)i;
+            });
+        if (lane == 0) {
+            split_row[i] = (int32_t)r;
+            split_slot0[i] = slot;
+            if (i == n_rows - 1) split_slot0[n_rows] = n_segs;
+            row_key[i] = (uint32_t)(n_segs - cnt);
+            row_id[i] = (uint32_t)i;
         }
     }
 }
@@ -801,22 +866,39 @@ __global__ void k_seg_permute(const uint32_t *__restrict__ order, const int64_t 
     }
 }
 
-cudaError_t launch_split_count(const SplitParams &sp, const int64_t *in_ptr, const int32_t *in_src,
-                               int64_t n, int64_t *nseg, int64_t *flag, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    k_split_count<<<device_sm_count() * 4, 256, 0, st>>>(sp, in_ptr, in_src, n, nseg, flag);
+int64_t hub_plan_words(int64_t n, int64_t max_hubs) {
+    return 2 + ceil_div<int64_t>(n, HEAVY_TILE) + ceil_div<int64_t>(max_hubs, 8);
+}
+
+cudaError_t launch_hub_count(const SplitParams &sp, const int64_t *in_ptr, const int32_t *in_src,
+                             int64_t n, int64_t max_hubs, int32_t *rows, int64_t *slot0,
+                             int64_t *counts, unsigned long long *chain, int *status,
+                             cudaStream_t st) {
+    const int64_t words = hub_plan_words(n, max_hubs), tiles = ceil_div<int64_t>(n, HEAVY_TILE);
+    cudaError_t e = cudaMemsetAsync(chain, 0, (size_t)words * 8, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, 16, st);
+    if (e != cudaSuccess || n <= 0) return e;
+    const int64_t cap = (int64_t)device_sm_count() * 8;
+    k_heavy_rows<<<(unsigned)(tiles < cap ? tiles : cap), 256, 0, st>>>(in_ptr, n, sp.split_t, rows,
+                                                                        counts, chain, status);
+    const int64_t ht = ceil_div<int64_t>(max_hubs > 0 ? max_hubs : 1, 8);
+    k_hub_slots<<<(unsigned)(ht < cap ? ht : cap), 256, 0, st>>>(sp, in_ptr, in_src, rows, counts,
+                                                                 slot0, counts + 1,
+                                                                 chain + 1 + tiles, status);
     return cudaGetLastError();
 }
 
-cudaError_t launch_split_fill(const SplitParams &sp, const int64_t *in_ptr, const int32_t *in_src,
-                              int64_t n, const int64_t *nseg, const int64_t *slot_off,
-                              const int64_t *split_idx, int32_t *split_row, int64_t *split_slot0,
-                              int64_t *seg_e0, int64_t *seg_e1, uint32_t *seg_win,
-                              cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    k_split_fill<<<device_sm_count() * 4, 256, 0, st>>>(sp, in_ptr, in_src, n, nseg, slot_off,
-                                                        split_idx, split_row, split_slot0, seg_e0,
-                                                        seg_e1, seg_win);
+cudaError_t launch_hub_fill(const SplitParams &sp, const int64_t *in_ptr, const int32_t *in_src,
+                            const int32_t *rows, const int64_t *slot0, int64_t n_rows,
+                            int64_t n_segs, int32_t *split_row, int64_t *split_slot0,
+                            int64_t *seg_e0, int64_t *seg_e1, uint32_t *seg_win, uint32_t *seg_id,
+                            int32_t *slot_split, uint32_t *row_key, uint32_t *row_id,
+                            cudaStream_t st) {
+    if (n_rows <= 0) return cudaSuccess;
+    const int64_t want = ceil_div<int64_t>(n_rows, 4), cap = (int64_t)device_sm_count() * 16;
+    k_hub_fill<<<(unsigned)(want < cap ? want : cap), 128, 0, st>>>(
+        sp, in_ptr, in_src, rows, slot0, n_rows, n_segs, split_row, split_slot0, seg_e0, seg_e1,
+        seg_win, seg_id, slot_split, row_key, row_id);
     return cudaGetLastError();
 }
 
@@ -825,26 +907,6 @@ cudaError_t launch_seg_permute(const uint32_t *order, const int64_t *e0, const i
                                cudaStream_t st) {
     if (n_segs <= 0) return cudaSuccess;
     k_seg_permute<<<device_sm_count() * 2, 256, 0, st>>>(order, e0, e1, n_segs, e0s, e1s, slot);
-    return cudaGetLastError();
-}
-
-// Split rows ordered by their number of partial slots, largest first (the
-// hop sums each split row's slots in one warp and hands the heaviest out
-// first, so that they finish early).  keys = ~count, so an ascending stable
-// sort gives descending counts with ties in row order.
-__global__ void k_split_keys(const int64_t *__restrict__ slot0, int64_t n_split,
-                             uint32_t *__restrict__ keys, uint32_t *__restrict__ vals) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n_split;
-         r += (int64_t)gridDim.x * blockDim.x) {
-        keys[r] = ~(uint32_t)(slot0[r + 1] - slot0[r]);
-        vals[r] = (uint32_t)r;
-    }
-}
-
-cudaError_t launch_split_keys(const int64_t *slot0, int64_t n_split, uint32_t *keys,
-                              uint32_t *vals, cudaStream_t st) {
-    if (n_split <= 0) return cudaSuccess;
-    k_split_keys<<<device_sm_count(), 256, 0, st>>>(slot0, n_split, keys, vals);
     return cudaGetLastError();
 }
 
@@ -1106,15 +1168,6 @@ __global__ void k_split_bound(const int64_t *__restrict__ in_ptr, int64_t n_spli
     }
 }
 
-__global__ void k_slot_owner(const int64_t *__restrict__ split_slot0, int64_t n_split,
-                             int32_t *__restrict__ slot_split) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n_split; r += nw)
-        for (int64_t s = split_slot0[r] + lane; s < split_slot0[r + 1]; s += 32)
-            slot_split[s] = (int32_t)r;
-}
-
 __global__ void k_fill_f32(float *__restrict__ v, int64_t n, float x) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
@@ -1124,13 +1177,6 @@ __global__ void k_fill_f32(float *__restrict__ v, int64_t n, float x) {
 cudaError_t launch_fill_f32(float *v, int64_t n, float x, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     k_fill_f32<<<device_sm_count() * 2, 256, 0, st>>>(v, n, x);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_slot_owner(const int64_t *split_slot0, int64_t n_split, int32_t *slot_split,
-                              cudaStream_t st) {
-    if (n_split <= 0) return cudaSuccess;
-    k_slot_owner<<<device_sm_count() * 4, 256, 0, st>>>(split_slot0, n_split, slot_split);
     return cudaGetLastError();
 }
 
@@ -1172,20 +1218,14 @@ cudaError_t launch_mass_levels(const HopPlan &p, int t0, int t1, float *mup, flo
 // Last hop, after the floor: the rows kept whole whose upper bound reaches
 // their floor (kept_rows), the split rows that do not (split_skip), and the
 // segments of the split rows that do (kept_segs), in one pass over rows,
-// split rows and segments.  A CTA takes a tile of KEEP_TILE consecutive items
-// by ticket and learns where its survivors go from the tiles before it (each
-// publishes its own count, then the total up to itself, in `chain`), so both
-// lists are in row order and in window-major order: the order that keeps
-// gathered source rows in L2 (in the order of the tiles' finish the last hop
-// took 363 instead of 317 us on 500,009 chunks, 100 scoped queries).  A tile
-// only waits for tiles that took their ticket earlier, so the wait ends; it is
-// bounded all the same.  The bounds are evaluated here: no per-row arrays are
+// split rows and segments, in ordered tiles (chain_before): both lists are in
+// row order and in window-major order, the order that keeps gathered source
+// rows in L2 (in the order of the tiles' finish the last hop took 363 instead
+// of 317 us on 500,009 chunks, 100 scoped queries).  The bounds are evaluated
+// here: no per-row arrays are
 // written (eleven launches did this; with the floor 102 -> 60 us there, 34 ->
 // 11 us on 4096 chunks).
 constexpr int KEEP_TILE = 1024;
-constexpr unsigned long long KEEP_SUM = 1ull << 62, KEEP_TOTAL = 2ull << 62;
-constexpr unsigned long long KEEP_VALUE = KEEP_SUM - 1;
-constexpr uint32_t KEEP_POLLS = 1u << 24;
 __global__ __launch_bounds__(256) void k_keep(const RowBounds rb, const float *__restrict__ floor_p,
                                               const NsFloors nf,
                                               const int64_t *__restrict__ in_ptr, int64_t split_t,
@@ -1271,40 +1311,11 @@ __global__ __launch_bounds__(256) void k_keep(const RowBounds rb, const float *_
             wcnt[lane] = incl - c;
             const unsigned long long own =
                 (unsigned long long)__shfl_sync(0xffffffffu, incl, 31);
-            // this tile's place in its list: the counts of the list's tiles
-            // before it, 32 at a time back to one that holds a total
-            volatile unsigned long long *ch = chain + 1;
+            // this tile's place in its list
             const int64_t first = rows ? 0 : row_tiles + split_tiles;
             const int64_t last = rows ? row_tiles : row_tiles + split_tiles + seg_tiles;
-            unsigned long long before = 0ull;
-            if (tile > first) {
-                if (lane == 0) ch[tile] = KEEP_SUM | own;
-                bool more = true;
-                for (int64_t hi = tile - 1; more; hi -= 32) {
-                    const int64_t at = hi - lane;
-                    unsigned long long v = KEEP_TOTAL;      // before the list: 0 in all
-                    uint32_t polls = 0;
-                    if (at >= first)
-                        while (((v = ch[at]) >> 62) == 0ull) {
-                            if (++polls > KEEP_POLLS) {
-                                set_status(status, AKASHIC_ETIMEOUT);
-                                v = KEEP_TOTAL;
-                                break;
-                            }
-                        }
-                    __syncwarp();
-                    const unsigned tot = __ballot_sync(0xffffffffu, (v >> 62) == 2ull);
-                    // lanes up to the nearest total count
-                    const int stop = tot ? __ffs(tot) - 1 : 31;
-                    unsigned long long x = lane <= stop ? v & KEEP_VALUE : 0ull;
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-                    before += x;
-                    more = tot == 0u;
-                }
-            }
+            const unsigned long long before = chain_before(chain + 1, first, tile, own, status);
             if (lane == 0) {
-                ch[tile] = KEEP_TOTAL | (before + own);
                 base_s = before;
                 if (tile == last - 1) kept_count[rows ? 0 : 1] = before + own;
             }

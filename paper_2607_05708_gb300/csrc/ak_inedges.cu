@@ -169,24 +169,6 @@ __global__ void k_place_recip(const int32_t *__restrict__ nbr_ids, const float *
     }
 }
 
-__global__ void k_in_weights(const int32_t *__restrict__ in_src, const float *__restrict__ in_aff,
-                             int64_t nnz, const int32_t *__restrict__ ext_of,
-                             const float2 *__restrict__ rstat, float *__restrict__ in_w) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nnz;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const float2 s = rstat[ext_of[in_src[e]]];
-        in_w[e] = row_softmax_weight(in_aff[e], s);
-    }
-}
-
-cudaError_t launch_in_weights(const int32_t *in_src, const float *in_aff, int64_t nnz,
-                              const int32_t *ext_of, const float2 *rstat, float *in_w,
-                              cudaStream_t st) {
-    if (nnz <= 0) return cudaSuccess;
-    k_in_weights<<<device_sm_count() * 8, 256, 0, st>>>(in_src, in_aff, nnz, ext_of, rstat, in_w);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_in_edges_update(const InEdgeUpdate &u, const InEdgeScratch &s, cudaStream_t st,
                                    int *launches) {
     const int sms = device_sm_count();

@@ -13,7 +13,7 @@ enum UpdateScratchSlot {
     SCR_NBR_IDS, SCR_NBR_COS,                                                // update results
     SCR_IN_INC, SCR_IN_DEG, SCR_IN_OFF, SCR_IN_RSTAT,                        // transpose patch
     SCR_DEAD_S,                                                              // relate sample
-    SCR_DEL_KEEP, SCR_DEL_POS, SCR_DEL_TMP,                                  // deletion
+    SCR_DEL,                                                                 // deletion
     SCR_MM_G, SCR_MM_GN, SCR_MM_CAND, SCR_MM_MOVING, SCR_MM_POS, SCR_MM_PARENT,  // memory
     SCR_MM_NS, SCR_MM_IDS, SCR_MM_ROOT, SCR_MM_NSK, SCR_MM_K2, SCR_MM_V2,          // manager
     SCR_MM_TMP,
