@@ -91,7 +91,7 @@ struct StreamScratch {
     DevBuf qns, ns_s, dead_s;    // scope: per query column, per sample row
     DevBuf rmax_u, rmin_u;       // u's row maxima / minima over the real queries
     DevBuf pfloor;               // the last hop's floor and what it keeps
-    DevBuf skip_split, kept_rows, kept_segs, keep_chain;
+    DevBuf skip_split, kept_rows, kept_segs, keep_scr;
     DevBuf reach_part, reach_plan;   // the candidates' partials, the plan
     DevBuf nsf;                  // scoped last hop: tags, their floors, their count
     // every candidate's combined coefficients (bf16 hi, lo), and their key
@@ -153,7 +153,7 @@ struct akashic_mem {
     bool has_dead = false;       // any chunk deleted (enables the masks)
     // memory manager: per-page slot counters, co-retrieval statistics
     DevBuf page_total, page_live, sel, co_key, co_val, mm_ctr;
-    int64_t page_cap = 0, co_cap = 0, co_upper = 0;
+    int64_t page_cap = 0, co_cap = 0, co_pairs = 0;
     int64_t appended = 0, moves = 0;
     // canonical out-edge CSR
     int64_t nnz = 0;
@@ -307,9 +307,8 @@ static MmTables mm_tables(akashic_mem *m) {
     t.co_key = m->co_key.as<unsigned long long>();
     t.co_val = m->co_val.as<uint32_t>();
     t.co_cap = m->co_cap;
-    t.next_page = m->mm_ctr.as<int64_t>();
-    t.writes = m->mm_ctr.as<int64_t>() + 1;
-    t.released = m->mm_ctr.as<unsigned long long>() + 2;
+    t.pairs = m->mm_ctr.as<unsigned long long>();
+    t.released = m->mm_ctr.as<unsigned long long>() + 1;
     return t;
 }
 
@@ -331,9 +330,9 @@ static akashic_status_t mm_ensure_pages(akashic_mem *m, int64_t need, cudaStream
 // Co-retrieval table able to take `more` new pairs at load <= 1/2.
 static akashic_status_t mm_ensure_pairs(akashic_mem *m, int64_t more, cudaStream_t st,
                                         int *launches = nullptr) {
-    if (m->co_cap > 0 && m->co_upper + more <= m->co_cap / 2) return AKASHIC_OK;
+    if (m->co_cap > 0 && m->co_pairs + more <= m->co_cap / 2) return AKASHIC_OK;
     int64_t cap = m->co_cap > 0 ? m->co_cap : ((int64_t)1 << 20);
-    while (m->co_upper + more > cap / 2) cap *= 2;
+    while (m->co_pairs + more > cap / 2) cap *= 2;
     DevBuf nk, nv;
     AK_TRY(nk.ensure((size_t)cap * 8));
     AK_TRY(nv.ensure((size_t)cap * 4));
@@ -430,16 +429,17 @@ static akashic_status_t build_split_plan(akashic_mem *m, cudaStream_t st) {
     };
     // sizes first (read back once), then the plan
     const int64_t max_hubs = m->nnz / (m->split.split_t + 1);
-    const Tmp chain = get(0, (size_t)hub_plan_words(n, max_hubs) * 8);
+    const Tmp words = get(0, (size_t)hub_plan_words(n, max_hubs) * 8);
     const Tmp rows = get(1, (size_t)(max_hubs + 1) * 4), slot0 = get(2, (size_t)(max_hubs + 1) * 8);
     const Tmp counts = get(3, 16);
     if (sc_rc != AKASHIC_OK) return fail(sc_rc, "relation graph rebuild: out of device memory");
     CUDA_TRY(launch_hub_count(m->split, m->in_ptr.as<int64_t>(), m->in_src.as<int32_t>(), n,
                               max_hubs, rows.as<int32_t>(), slot0.as<int64_t>(),
-                              counts.as<int64_t>(), chain.as<unsigned long long>(),
-                              m->status.as<int>(), st));
+                              counts.as<int64_t>(), words.as<int64_t>(), st));
     int64_t got[2] = {0, 0};
-    CUDA_TRY(cudaMemcpyAsync(got, counts.p, 16, cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaMemcpyAsync(got, counts.p, 8, cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaMemcpyAsync(got + 1, slot0.as<int64_t>() + max_hubs, 8, cudaMemcpyDeviceToHost,
+                             st));
     AK_TRY(check_status(m, st, "relation graph rebuild"));
     const int64_t n_split = got[0], n_segs = got[1];
     if (n_segs > 0x7fffffffLL) return fail(AKASHIC_ECAPACITY, "too many hub segments");
@@ -545,7 +545,7 @@ akashic_status_t akashic_mem_create(const akashic_mem_config_t *cfg, akashic_mem
         cudaMemset(m->dead_row.p, 0, (size_t)m->cap * 4) != cudaSuccess ||
         m->sel.ensure((size_t)m->cap * 4) != AKASHIC_OK ||
         cudaMemset(m->sel.p, 0, (size_t)m->cap * 4) != cudaSuccess ||
-        m->mm_ctr.ensure(32) != AKASHIC_OK || cudaMemset(m->mm_ctr.p, 0, 32) != cudaSuccess ||
+        m->mm_ctr.ensure(64) != AKASHIC_OK || cudaMemset(m->mm_ctr.p, 0, 64) != cudaSuccess ||
         mm_ensure_pages(m, 1024, 0) != AKASHIC_OK || mm_ensure_pairs(m, 0, 0) != AKASHIC_OK ||
         cudaDeviceSynchronize() != cudaSuccess) {
         delete m;
@@ -944,20 +944,19 @@ akashic_status_t akashic_mem_delete(akashic_mem_t *m, const int64_t *ids, int64_
     // the compaction's scratch; what has to start at zero comes first
     const size_t rb = (size_t)ceil_div<int64_t>(rows, 32) * 4;
     const size_t eb = (size_t)ceil_div<int64_t>(nnz, 32) * 4;
-    const size_t cb = (size_t)(drop_tiles(nnz) + 1) * 8;
+    const size_t cb = (size_t)drop_tiles(nnz) * 4;
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t zero = 2 * up(cb) + 2 * up(rb) + 2 * up(eb);
-    uint8_t *scr = (uint8_t *)store_scratch(m, SCR_DEL, zero + up(rb) + 2 * up(eb));
+    const size_t zero = 2 * up(rb) + 2 * up(eb);
+    uint8_t *scr = (uint8_t *)store_scratch(m, SCR_DEL, zero + up(rb) + 2 * up(eb) + up(cb));
     if (!scr) return fail(AKASHIC_ENOMEM, "delete: out of device memory");
-    unsigned long long *chain = (unsigned long long *)scr;
-    unsigned long long *chain_in = (unsigned long long *)(scr + up(cb));
-    uint32_t *dead_id = (uint32_t *)(scr + 2 * up(cb));
-    uint32_t *touched = (uint32_t *)(scr + 2 * up(cb) + up(rb));
-    uint32_t *drop = (uint32_t *)(scr + 2 * up(cb) + 2 * up(rb));
-    uint32_t *drop_in = (uint32_t *)(scr + 2 * up(cb) + 2 * up(rb) + up(eb));
+    uint32_t *dead_id = (uint32_t *)scr;
+    uint32_t *touched = (uint32_t *)(scr + up(rb));
+    uint32_t *drop = (uint32_t *)(scr + 2 * up(rb));
+    uint32_t *drop_in = (uint32_t *)(scr + 2 * up(rb) + up(eb));
     uint32_t *dead_bits = (uint32_t *)(scr + zero);
     uint32_t *keep = (uint32_t *)(scr + zero + up(rb));
     int32_t *word_pos = (int32_t *)(scr + zero + up(rb) + up(eb));
+    int32_t *counts = (int32_t *)(scr + zero + up(rb) + 2 * up(eb));
     AK_TRY(ensure_spare(m->rp2, (size_t)(m->cap + 1) * 8));
     AK_TRY(ensure_spare(m->col2, (size_t)nnz * 4));
     AK_TRY(ensure_spare(m->aff2, (size_t)nnz * 4));
@@ -984,8 +983,7 @@ akashic_status_t akashic_mem_delete(akashic_mem_t *m, const int64_t *ids, int64_
     d.drop_bits = drop;
     d.keep_bits = keep;
     d.word_pos = word_pos;
-    d.chain = chain;
-    d.status = m->status.as<int>();
+    d.counts = counts;
     d.tgt_out = m->col2.as<int32_t>();
     d.val_out = m->aff2.as<float>();
     d.w_out = m->w2.as<float>();
@@ -1006,7 +1004,6 @@ akashic_status_t akashic_mem_delete(akashic_mem_t *m, const int64_t *ids, int64_
     di.ext_of = m->ext_of.as<int32_t>();
     di.rstat = m->rstat.as<float2>();
     di.drop_bits = drop_in;
-    di.chain = chain_in;
     di.tgt_out = m->in_src2.as<int32_t>();
     di.val_out = m->in_aff2.as<float>();
     di.w_out = m->in_w2.as<float>();
@@ -1050,20 +1047,23 @@ akashic_status_t akashic_mem_relocate(akashic_mem_t *m, const int64_t *S, int32_
     int32_t *gb = (int32_t *)store_scratch(m, SCR_MM_G, (size_t)n_req * 64 * 4);
     int32_t *gn = (int32_t *)store_scratch(m, SCR_MM_GN, (size_t)n_req * 4);
     if (!gb || !gn) return fail(AKASHIC_ENOMEM, "relocate: out of device memory");
-    int64_t ctr[2] = {m->next_page, 0};
-    CUDA_TRY(cudaMemcpyAsync(m->mm_ctr.p, ctr, 16, cudaMemcpyHostToDevice, st));
     const int32_t *dead = m->has_dead ? m->dead_row.as<int32_t>() : nullptr;
     const MmTables t = mm_tables(m);
+    int64_t *result = m->mm_ctr.as<int64_t>() + 4;
     CUDA_TRY(launch_mm_count(S, n_req, s_len, m->n, m->row_of.as<int32_t>(), dead, t,
                              m->status.as<int>(), st));
     CUDA_TRY(launch_mm_relocate(S, n_req, s_len, m->n, m->row_of.as<int32_t>(), dead,
-                                m->page_of.as<int32_t>(), t, tau_assoc, m->per_page, gb, gn, st));
+                                m->page_of.as<int32_t>(), t, tau_assoc, m->next_page, m->per_page,
+                                gb, gn, m->status.as<int>(), result, st));
     ph.launches += 3;
-    CUDA_TRY(cudaMemcpyAsync(ctr, m->mm_ctr.p, 16, cudaMemcpyDeviceToHost, st));
-    AK_TRY(check_status(m, st, "relocate"));
-    m->next_page = ctr[0];
-    m->moves += ctr[1];
-    m->co_upper += pairs;
+    // everything the host needs in one read-back, the status word with it
+    int64_t got[4] = {0, 0, 0, 0};
+    CUDA_TRY(cudaMemcpyAsync(got, result, 32, cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaStreamSynchronize(st));
+    if (got[3] != 0) AK_TRY(check_status(m, st, "relocate"));
+    m->next_page = got[0];
+    m->moves += got[1];
+    m->co_pairs = got[2];
     return AKASHIC_OK;
 }
 
@@ -1080,59 +1080,75 @@ akashic_status_t akashic_mem_compact_pages(akashic_mem_t *m, float theta, float 
     const int64_t n = m->n, pages = m->next_page;
     if (released) *released = 0;
     if (n == 0) return AKASHIC_OK;
-    const size_t tb = (scan_tmp_bytes(n + 1) > radix_tmp_bytes(n) ? scan_tmp_bytes(n + 1)
-                                                                   : radix_tmp_bytes(n)) + 4096;
+    // the directory first: pages to compact and the live chunks on them, with
+    // the union of their groups, read back together
     int32_t *cand = (int32_t *)store_scratch(m, SCR_MM_CAND, (size_t)(pages + 1) * 4);
-    int64_t *moving = (int64_t *)store_scratch(m, SCR_MM_MOVING, (size_t)(n + 1) * 8);
-    int64_t *pos = (int64_t *)store_scratch(m, SCR_MM_POS, (size_t)(n + 1) * 8);
+    uint32_t *moving = (uint32_t *)store_scratch(m, SCR_MM_MOVING, (size_t)ceil_div<int64_t>(n, 32) * 4);
     int32_t *parent = (int32_t *)store_scratch(m, SCR_MM_PARENT, (size_t)n * 4);
-    int32_t *ns_id = (int32_t *)store_scratch(m, SCR_MM_NS, (size_t)n * 4);
+    int32_t *counts = (int32_t *)store_scratch(m, SCR_MM_COUNTS, (size_t)mm_tiles(n) * 4);
     uint32_t *ids = (uint32_t *)store_scratch(m, SCR_MM_IDS, (size_t)n * 4 + 16);
-    uint32_t *root = (uint32_t *)store_scratch(m, SCR_MM_ROOT, (size_t)n * 4 + 16);
     uint32_t *nsk = (uint32_t *)store_scratch(m, SCR_MM_NSK, (size_t)n * 4 + 16);
-    uint32_t *k2 = (uint32_t *)store_scratch(m, SCR_MM_K2, (size_t)n * 4 + 16);
-    uint32_t *v2 = (uint32_t *)store_scratch(m, SCR_MM_V2, (size_t)n * 4 + 16);
-    void *tmp = store_scratch(m, SCR_MM_TMP, tb);
-    if (!cand || !moving || !pos || !parent || !ns_id || !ids || !root || !nsk || !k2 || !v2 || !tmp)
+    if (!cand || !moving || !parent || !counts || !ids || !nsk)
         return fail(AKASHIC_ENOMEM, "compact: out of device memory");
     PhaseScope ph(m, AKASHIC_PHASE_COMPACT, st);
     const MmTables t = mm_tables(m);
     const int32_t *dead = m->has_dead ? m->dead_row.as<int32_t>() : nullptr;
-    const int32_t *row_of = m->row_of.as<int32_t>();
-    CUDA_TRY(cudaMemsetAsync(t.released, 0, 8, st));
-    CUDA_TRY(launch_mm_compact_prepare(t, pages, theta, n, row_of, dead, m->page_of.as<int32_t>(),
-                                       cand, moving, parent, st));
-    CUDA_TRY(cudaMemsetAsync(moving + n, 0, 8, st));
-    CUDA_TRY(launch_by_id(m->ns_row.as<int32_t>(), row_of, n, ns_id, st));
-    CUDA_TRY(launch_mm_union(t, moving, ns_id, tau_assoc, parent, m->status.as<int>(), st));
+    const int32_t *row_of = m->row_of.as<int32_t>(), *ns_row = m->ns_row.as<int32_t>();
+    CUDA_TRY(launch_mm_candidates(t, pages, theta, cand, st));
+    CUDA_TRY(launch_mm_collect(t, n, row_of, dead, m->page_of.as<int32_t>(), ns_row, cand, moving,
+                               parent, ids, nsk, counts, st));
+    CUDA_TRY(launch_mm_union(t, moving, row_of, ns_row, tau_assoc, parent, m->status.as<int>(), st));
     ph.launches += (pages > 0) + 3;
-    CUDA_TRY(scan_exclusive(moving, pos, n + 1, tmp, tb, st, &ph.launches));
-    // released pages and moving chunks, read back together
-    CUDA_TRY(cudaMemcpyAsync(t.released + 1, pos + n, 8, cudaMemcpyDeviceToDevice, st));
     int64_t rc[2] = {0, 0};
     CUDA_TRY(cudaMemcpyAsync(rc, t.released, 16, cudaMemcpyDeviceToHost, st));
     AK_TRY(check_status(m, st, "compact"));
     const int64_t n_rel = rc[0], count = rc[1];
+    if (n_rel == 0) return AKASHIC_OK;
+    int64_t new_pages = 0;
+    if (count > 0 && count <= mm_small_repack()) {
+        // (a fresh page a chunk at most)
+        AK_TRY(mm_ensure_pages(m, m->next_page + count + 1, st));
+        int64_t *np = m->mm_ctr.as<int64_t>() + 3;
+        CUDA_TRY(launch_mm_repack_small(mm_tables(m), pages, cand, ids, nsk, count, parent, row_of,
+                                        m->page_of.as<int32_t>(), m->next_page, m->per_page, np,
+                                        st));
+        ph.launches += 2;
+        CUDA_TRY(cudaMemcpyAsync(&new_pages, np, 8, cudaMemcpyDeviceToHost, st));
+        CUDA_TRY(cudaStreamSynchronize(st));
+        m->next_page += new_pages;
+        m->moves += count;
+        if (released) *released = n_rel;
+        return AKASHIC_OK;
+    }
     if (count > 0) {
-        CUDA_TRY(launch_mm_keys(moving, pos, n, parent, ns_id, ids, root, nsk, st));
+        const size_t tb = (scan_tmp_bytes(count + 1) > radix_tmp_bytes(count)
+                               ? scan_tmp_bytes(count + 1) : radix_tmp_bytes(count)) + 4096;
+        uint32_t *root = (uint32_t *)store_scratch(m, SCR_MM_ROOT, (size_t)count * 4 + 16);
+        uint32_t *k2 = (uint32_t *)store_scratch(m, SCR_MM_K2, (size_t)count * 4 + 16);
+        uint32_t *v2 = (uint32_t *)store_scratch(m, SCR_MM_V2, (size_t)count * 4 + 16);
+        // pages of each namespace's run, scanned into its base page
+        int64_t *part = (int64_t *)store_scratch(m, SCR_MM_POS, (size_t)(count + 1) * 16);
+        void *tmp = store_scratch(m, SCR_MM_TMP, tb);
+        if (!root || !k2 || !v2 || !part || !tmp)
+            return fail(AKASHIC_ENOMEM, "compact: out of device memory");
+        int64_t *pos = part + count + 1;
+        CUDA_TRY(launch_mm_roots(ids, count, parent, root, st));
         // order (namespace, group root, chunk ID): the list is in ID order;
         // stable sorts by root, then by namespace
         bool alt = false;
         CUDA_TRY(radix_sort_pairs(root, ids, k2, v2, count, 32, tmp, tb, st, &alt, &ph.launches));
         uint32_t *sid = alt ? v2 : ids, *spare_v = alt ? ids : v2;
         uint32_t *nk = alt ? root : k2;
-        CUDA_TRY(launch_mm_ns_keys(sid, count, ns_id, nsk, st));
+        CUDA_TRY(launch_mm_ns_keys(sid, count, row_of, ns_row, nsk, st));
         bool alt2 = false;
         CUDA_TRY(radix_sort_pairs(nsk, sid, nk, spare_v, count, 32, tmp, tb, st, &alt2,
                                   &ph.launches));
         const uint32_t *order = alt2 ? spare_v : sid;
         const uint32_t *ns_sorted = alt2 ? nk : nsk;
         // every namespace starts on a fresh page (compaction never mixes
-        // tenants or sessions): pages per namespace run, scanned into each
-        // run's base page; `moving` and `pos` are free again
-        CUDA_TRY(launch_mm_part_pages(ns_sorted, count, m->per_page, moving, st));
-        CUDA_TRY(scan_exclusive(moving, pos, count, tmp, tb, st, &ph.launches));
-        int64_t new_pages = 0;
+        // tenants or sessions)
+        CUDA_TRY(launch_mm_part_pages(ns_sorted, count, m->per_page, part, st));
+        CUDA_TRY(scan_exclusive(part, pos, count, tmp, tb, st, &ph.launches));
         CUDA_TRY(cudaMemcpyAsync(&new_pages, pos + count, 8, cudaMemcpyDeviceToHost, st));
         AK_TRY(check_status(m, st, "compact"));
         AK_TRY(mm_ensure_pages(m, m->next_page + new_pages + 1, st));
@@ -1142,7 +1158,7 @@ akashic_status_t akashic_mem_compact_pages(akashic_mem_t *m, float theta, float 
         ph.launches += 3 + (pages > 0) + 1;
         m->next_page += new_pages;
         m->moves += count;
-    } else if (n_rel > 0) {
+    } else {
         CUDA_TRY(launch_mm_release_repack(t, pages, cand, nullptr, nullptr, nullptr, 0, row_of,
                                           m->page_of.as<int32_t>(), m->next_page, m->per_page,
                                           st));
@@ -1656,13 +1672,11 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                         // scope to the k-th largest lower bound of the heaviest
                         // split rows (where the top scores lie)
                         const int64_t n_lb = m->n_split < 1024 ? m->n_split : 1024;
-                        const int64_t cw = keep_chain_words(hp);
-                        AK_TRY(ensure_spare(sc->keep_chain, (size_t)cw * 8));
-                        unsigned long long *chain = sc->keep_chain.as<unsigned long long>();
+                        AK_TRY(ensure_spare(sc->keep_scr, (size_t)keep_words(hp) * 4));
                         CUDA_TRY(launch_prune_floor(ws + sp.off_bound, b, rb,
                                                     q_ns ? nullptr : hp.split_row,
                                                     hp.split_order, n_lb, k,
-                                                    sc->pfloor.as<float>(), chain, cw, hp.done, st));
+                                                    sc->pfloor.as<float>(), hp.done, st));
                         // with a scope, each namespace of the batch gets its own
                         // floor (its rows can only be selected by its queries)
                         NsFloors nf{};
@@ -1681,8 +1695,8 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                         CUDA_TRY(launch_keep(hp, rb, sc->pfloor.as<float>(), q_ns ? &nf : nullptr,
                                              sc->skip_split.as<int32_t>(),
                                              sc->kept_rows.as<int32_t>(),
-                                             sc->kept_segs.as<int32_t>(), kept_count, chain,
-                                             m->status.as<int>(), st, &ps.launches));
+                                             sc->kept_segs.as<int32_t>(), kept_count,
+                                             sc->keep_scr.as<int32_t>(), st, &ps.launches));
                         ps.launches += 1;
                     }
                 }

@@ -2,10 +2,11 @@
 // copies are logically tombstoned, §4.2): a deleted chunk keeps its row but
 // is marked dead, gets no score, is never a candidate, and every relation
 // edge into or out of it is dropped from both the out-edge CSR and the
-// in-edge transpose.  Each list is compacted in one edge-parallel pass over
-// its targets, logits and weights, in ordered tiles; what it keeps of every 32
-// edges (a mask and the count before them) gives the new row starts.  Rows
-// that lost nothing keep their weights.
+// in-edge transpose.  Each list is compacted edge-parallel: a pass over its
+// targets marks what it keeps (a mask every 32 edges) and counts it by tile, a
+// pass over targets, logits and weights moves them; the masks and the counts
+// before them give the new row starts.  Rows that lost nothing keep their
+// weights.
 #include "ak_common.cuh"
 
 namespace ak {
@@ -74,100 +75,102 @@ __global__ void k_drop_rows(const int64_t *__restrict__ ids, int64_t n, int64_t 
     }
 }
 
-// The compaction: DROP_TILE consecutive edges a tile, 16 words of 32 edges a
-// warp.  Bound by memory: 12 bytes an edge read and written once, the bitmaps
-// cached.  (It took flags, a scan and positions of 8 bytes an edge in memory
-// before, ~60 bytes an edge more, and a softmax of every row: 1.20 ms for 200
-// chunks of 524,288 with 16.8M edges, read-back included, 0.64 now; a list's
-// 403 MB take 114 us.  Eight words a warp: 135.)
+// The compaction, DROP_TILE consecutive edges a CTA, DROP_WORDS words of 32
+// edges a warp: first the masks and the tiles' counts, then the move.  Bound by
+// memory: 4 bytes an edge read to mark it, 12 read and written to move it, the
+// bitmaps cached.  (It took flags, a scan and positions of 8 bytes an edge in
+// memory before, ~60 bytes an edge more, and a softmax of every row: 1.20 ms
+// for 200 chunks of 524,288 with 16.8M edges, read-back included, 0.59 now; a
+// list's 470 MB take 88 us.)
 constexpr int DROP_WORDS = 16;                          // a warp
 constexpr int DROP_TILE = 8 * 32 * DROP_WORDS;
 int64_t drop_tiles(int64_t nnz) { return ceil_div<int64_t>(nnz, DROP_TILE); }
 
+__global__ __launch_bounds__(256) void k_drop_mark(const DropDead d) {
+    __shared__ int warp_n[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t e0 = (int64_t)blockIdx.x * DROP_TILE + warp * 32 * DROP_WORDS;
+    int32_t t[DROP_WORDS];
+#pragma unroll
+    for (int j = 0; j < DROP_WORDS; ++j) {
+        const int64_t e = e0 + 32 * j + lane;
+        t[j] = e < d.nnz ? d.tgt[e] : -1;
+    }
+    // lane j holds word j's bits from here on
+    const bool has_word = lane < DROP_WORDS && e0 + 32 * lane < d.nnz;
+    const uint32_t drop = has_word ? d.drop_bits[(e0 >> 5) + lane] : ~0u;
+    uint32_t mine = 0u;
+#pragma unroll
+    for (int j = 0; j < DROP_WORDS; ++j) {
+        const bool live = t[j] >= 0 && !((__ldg(d.dead_bits + (t[j] >> 5)) >> (t[j] & 31)) & 1u);
+        const uint32_t keep = __ballot_sync(0xffffffffu, live);
+        if (lane == j) mine = keep & ~drop;
+    }
+    if (has_word) d.keep_bits[(e0 >> 5) + lane] = mine;
+    int n = __popc(mine);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+    if (lane == 0) warp_n[warp] = n;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int own = 0;
+        for (int w = 0; w < 8; ++w) own += warp_n[w];
+        d.counts[blockIdx.x] = own;
+    }
+}
+
 __global__ __launch_bounds__(256, 4) void k_drop_edges(const DropDead d) {
     __shared__ int warp_n[8];
-    __shared__ unsigned long long base_s;
-    __shared__ int64_t tile_s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    const int64_t tiles = (d.nnz + DROP_TILE - 1) / DROP_TILE;
-    while (true) {
-        __syncthreads();   // the tile before is done with the shared words
-        if (threadIdx.x == 0) tile_s = (int64_t)atomicAdd(d.chain, 1ull);
-        __syncthreads();
-        const int64_t tile = tile_s;
-        if (tile >= tiles) break;
-        const int64_t e0 = tile * DROP_TILE + warp * 32 * DROP_WORDS;
-        int32_t t[DROP_WORDS];
-        float v[DROP_WORDS], w[DROP_WORDS];
+    const int64_t e0 = (int64_t)blockIdx.x * DROP_TILE + warp * 32 * DROP_WORDS;
+    const int64_t word0 = e0 >> 5;
+    const bool has_word = lane < DROP_WORDS && e0 + 32 * lane < d.nnz;
+    const uint32_t mine = has_word ? d.keep_bits[word0 + lane] : 0u;   // lane j: word j
+    int32_t t[DROP_WORDS];
+    float v[DROP_WORDS], w[DROP_WORDS];
 #pragma unroll
-        for (int j = 0; j < DROP_WORDS; ++j) {
-            const int64_t e = e0 + 32 * j + lane;
-            t[j] = e < d.nnz ? __ldcs(d.tgt + e) : -1;
-        }
+    for (int j = 0; j < DROP_WORDS; ++j) {
+        const int64_t e = e0 + 32 * j + lane;
+        const bool ok = e < d.nnz;
+        t[j] = ok ? __ldcs(d.tgt + e) : 0;
+        v[j] = ok ? __ldcs(d.val + e) : 0.f;
+        w[j] = ok ? __ldcs(d.w + e) : 0.f;
+    }
+    // survivors before each word of the warp, before the warp, before the tile
+    int incl = __popc(mine);
 #pragma unroll
-        for (int j = 0; j < DROP_WORDS; ++j) {
-            const int64_t e = e0 + 32 * j + lane;
-            v[j] = e < d.nnz ? __ldcs(d.val + e) : 0.f;
-            w[j] = e < d.nnz ? __ldcs(d.w + e) : 0.f;
-        }
-        // lane j holds word j's bits from here on
-        const int64_t word0 = e0 >> 5;
-        const bool has_word = lane < DROP_WORDS && e0 + 32 * lane < d.nnz;
-        const uint32_t drop = has_word ? d.drop_bits[word0 + lane] : ~0u;
-        uint32_t mine = 0u;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+    }
+    const int pre = incl - __popc(mine);
+    if (lane == 31) warp_n[warp] = incl;
+    int64_t base = tile_base(d.counts, 0, blockIdx.x);   // (syncs the CTA)
+    for (int x = 0; x < warp; ++x) base += warp_n[x];
+    if (has_word) d.word_pos[word0 + lane] = (int32_t)(base + pre);
 #pragma unroll
-        for (int j = 0; j < DROP_WORDS; ++j) {
-            const bool live = t[j] >= 0 && !((__ldg(d.dead_bits + (t[j] >> 5)) >> (t[j] & 31)) & 1u);
-            const uint32_t keep = __ballot_sync(0xffffffffu, live);
-            if (lane == j) mine = keep & ~drop;
-        }
-        // survivors before each word of the warp, then before each warp
-        int incl = __popc(mine);
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int x = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += x;
-        }
-        const int pre = incl - __popc(mine);
-        if (lane == 31) warp_n[warp] = incl;
-        __syncthreads();
-        int own = 0, wpre = 0;
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            if (x < warp) wpre += warp_n[x];
-            own += warp_n[x];
-        }
-        if (warp == 0) {
-            const unsigned long long before =
-                chain_before(d.chain + 1, 0, tile, (unsigned long long)own, d.status);
-            if (lane == 0) base_s = before;
-        }
-        __syncthreads();
-        const int64_t base = (int64_t)base_s + wpre;
-        if (has_word) {
-            d.keep_bits[word0 + lane] = mine;
-            d.word_pos[word0 + lane] = (int32_t)(base + pre);
-        }
-#pragma unroll
-        for (int j = 0; j < DROP_WORDS; ++j) {
-            const uint32_t keep = __shfl_sync(0xffffffffu, mine, j);
-            const int at = __shfl_sync(0xffffffffu, pre, j);
-            if (!((keep >> lane) & 1u)) continue;
-            const int64_t p = base + at + __popc(keep & lt);
-            float wj = w[j];
-            if (d.touched && ((__ldg(d.touched + (t[j] >> 5)) >> (t[j] & 31)) & 1u))
-                wj = row_softmax_weight(v[j], d.rstat[d.ext_of[t[j]]]);
-            __stcs(d.tgt_out + p, t[j]);
-            __stcs(d.val_out + p, v[j]);
-            __stcs(d.w_out + p, wj);
-        }
+    for (int j = 0; j < DROP_WORDS; ++j) {
+        const uint32_t keep = __shfl_sync(0xffffffffu, mine, j);
+        const int at = __shfl_sync(0xffffffffu, pre, j);
+        if (!((keep >> lane) & 1u)) continue;
+        const int64_t p = base + at + __popc(keep & lt);
+        float wj = w[j];
+        if (d.touched && ((__ldg(d.touched + (t[j] >> 5)) >> (t[j] & 31)) & 1u))
+            wj = row_softmax_weight(v[j], d.rstat[d.ext_of[t[j]]]);
+        __stcs(d.tgt_out + p, t[j]);
+        __stcs(d.val_out + p, v[j]);
+        __stcs(d.w_out + p, wj);
     }
 }
 
 // new start of a row = the survivors before its old first edge
-__device__ __forceinline__ int64_t kept_before(const DropDead &d, int64_t e, int64_t total) {
-    if (e >= d.nnz) return total;
+// (e = nnz: all of them, by the last word)
+__device__ __forceinline__ int64_t kept_before(const DropDead &d, int64_t e) {
+    if (e >= d.nnz) {
+        const int64_t w = (d.nnz - 1) >> 5;
+        return d.word_pos[w] + __popc(d.keep_bits[w]);
+    }
     return d.word_pos[e >> 5] + __popc(d.keep_bits[e >> 5] & ((1u << (e & 31)) - 1u));
 }
 
@@ -183,19 +186,17 @@ __global__ __launch_bounds__(256) void k_drop_row_ptr(const DropDead d,
     const int lane = threadIdx.x & 31, sub = lane % L;
     const int64_t step = ((int64_t)gridDim.x * blockDim.x) / L;
     const int64_t warp0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (32 / L);
-    const int64_t total =
-        (int64_t)d.chain[(d.nnz + DROP_TILE - 1) / DROP_TILE] & CHAIN_VALUE;
     for (int64_t r0 = warp0; r0 <= d.n_rows; r0 += step) {   // (warp-uniform)
         const int64_t r = r0 + lane / L;
         int64_t old = 0, a = 0, b = 0;
         if (r < d.n_rows) {
             const int64_t p0 = d.ptr[r], p1 = d.ptr[r + 1];
             old = p1 - p0;
-            a = kept_before(d, p0, total);
-            b = kept_before(d, p1, total);
+            a = kept_before(d, p0);
+            b = kept_before(d, p1);
             if (sub == 0) ptr_out[r] = a;
         } else if (r == d.n_rows && sub == 0) {
-            ptr_out[r] = total;
+            ptr_out[r] = kept_before(d, d.nnz);
         }
         const bool lost = w && r < d.n_rows && b - a != old;
         if (!__any_sync(0xffffffffu, lost)) continue;
@@ -259,9 +260,9 @@ cudaError_t launch_drop_dead_edges(const DropDead &d, cudaStream_t st) {
         k_drop_rows<<<(unsigned)g, 128, 0, st>>>(d.ids, d.n_ids, d.n_total, d.own_row_of, d.ptr,
                                                  d.drop_bits);
     }
-    const int64_t tiles = drop_tiles(d.nnz);
-    const int64_t cap = (int64_t)sms * 8;
-    k_drop_edges<<<(unsigned)(tiles < cap ? tiles : cap), 256, 0, st>>>(d);
+    const unsigned tiles = (unsigned)drop_tiles(d.nnz);
+    k_drop_mark<<<tiles, 256, 0, st>>>(d);
+    k_drop_edges<<<tiles, 256, 0, st>>>(d);
     return cudaGetLastError();
 }
 

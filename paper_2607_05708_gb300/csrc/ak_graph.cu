@@ -720,104 +720,57 @@ __device__ int64_t warp_segments(const SplitParams &sp, const int32_t *__restric
     return base;
 }
 
-// The hub rows (more than split_t in-edges) in row order, and their number: one
-// pass over the row starts in ordered tiles.
+// The hub rows (more than split_t in-edges) in row order, and their number, in
+// ordered tiles (tile_base).
 constexpr int HEAVY_TILE = 1024;
+template <bool WRITE>
 __global__ __launch_bounds__(256) void k_heavy_rows(const int64_t *__restrict__ in_ptr, int64_t n,
                                                     int64_t split_t, int32_t *__restrict__ rows,
                                                     int64_t *__restrict__ n_rows,
-                                                    unsigned long long *chain, int *status) {
-    __shared__ int wcnt[32];
-    __shared__ int64_t tile_s, base_s;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int64_t tiles = (n + HEAVY_TILE - 1) / HEAVY_TILE;
-    while (true) {
-        __syncthreads();
-        if (t == 0) tile_s = (int64_t)atomicAdd(chain, 1ull);
-        __syncthreads();
-        const int64_t tile = tile_s;
-        if (tile >= tiles) break;
-        unsigned bal[HEAVY_TILE / 256];
+                                                    int32_t *__restrict__ counts) {
+    const int t = threadIdx.x;
+    const int64_t tile = blockIdx.x;
+    if (WRITE && counts[tile] == 0 && tile != gridDim.x - 1) return;
+    unsigned bal[4];
 #pragma unroll
-        for (int q = 0; q < HEAVY_TILE / 256; ++q) {
-            const int64_t i = tile * HEAVY_TILE + q * 256 + t;
-            bal[q] = __ballot_sync(0xffffffffu, i < n && in_ptr[i + 1] - in_ptr[i] > split_t);
-            if (lane == 0) wcnt[q * 8 + warp] = __popc(bal[q]);
-        }
-        __syncthreads();
-        if (warp == 0) {
-            const int c = wcnt[lane];
-            int incl = c;
+    for (int q = 0; q < 4; ++q) {
+        const int64_t i = tile * HEAVY_TILE + q * 256 + t;
+        bal[q] = __ballot_sync(0xffffffffu, i < n && in_ptr[i + 1] - in_ptr[i] > split_t);
+    }
+    int places[4];
+    const int own = tile_places(bal, places);
+    if constexpr (!WRITE) {
+        if (t == 0) counts[tile] = own;
+    } else {
+        const int64_t base = tile_base(counts, 0, tile);
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int x = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += x;
-            }
-            wcnt[lane] = incl - c;
-            const unsigned long long own = (unsigned long long)__shfl_sync(0xffffffffu, incl, 31);
-            const unsigned long long before = chain_before(chain + 1, 0, tile, own, status);
-            if (lane == 0) {
-                base_s = (int64_t)before;
-                if (tile == tiles - 1) *n_rows = (int64_t)(before + own);
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < HEAVY_TILE / 256; ++q)
-            if ((bal[q] >> lane) & 1u)
-                rows[base_s + wcnt[q * 8 + warp] + __popc(bal[q] & ((1u << lane) - 1u))] =
-                    (int32_t)(tile * HEAVY_TILE + q * 256 + t);
+        for (int q = 0; q < 4; ++q)
+            if ((bal[q] >> (t & 31)) & 1u)
+                rows[base + places[q]] = (int32_t)(tile * HEAVY_TILE + q * 256 + t);
+        if (t == 0 && tile == gridDim.x - 1) *n_rows = base + own;
     }
 }
 
-// First partial slot of every hub row and the number of segments: a warp a
-// row, a CTA eight consecutive ones, in ordered tiles.  (A warp that walked 32
-// rows of the store and cut the hubs among them one after another took 56 us
-// at 524,288 chunks, as a cut is a chain of ~20 dependent loads.)
-__global__ __launch_bounds__(256) void k_hub_slots(SplitParams sp,
-                                                   const int64_t *__restrict__ in_ptr,
-                                                   const int32_t *__restrict__ in_src,
-                                                   const int32_t *__restrict__ rows,
-                                                   const int64_t *__restrict__ n_rows,
-                                                   int64_t *__restrict__ slot0,
-                                                   int64_t *__restrict__ n_segs,
-                                                   unsigned long long *chain, int *status) {
-    __shared__ int64_t cnt[8];
-    __shared__ int64_t tile_s, base_s;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int64_t n = *n_rows, tiles = (n + 7) / 8;
-    while (true) {
-        __syncthreads();
-        if (t == 0) tile_s = (int64_t)atomicAdd(chain, 1ull);
-        __syncthreads();
-        const int64_t tile = tile_s;
-        if (tile >= tiles) break;
-        const int64_t i = tile * 8 + warp;
-        int64_t mine = 0;
-        if (i < n) {
-            const int64_t r = rows[i];
-            mine = warp_segments(sp, in_src, in_ptr[r], in_ptr[r + 1],
-                                 [](int64_t, int64_t, int64_t, int64_t) {});
-        }
-        if (lane == 0) cnt[warp] = mine;
-        __syncthreads();
-        if (warp == 0) {
-            int64_t own = 0;
-            for (int w = 0; w < 8; ++w) own += cnt[w];
-            const unsigned long long before =
-                chain_before(chain + 1, 0, tile, (unsigned long long)own, status);
-            if (lane == 0) {
-                base_s = (int64_t)before;
-                if (tile == tiles - 1) *n_segs = (int64_t)before + own;
-            }
-        }
-        __syncthreads();
-        if (lane == 0 && i < n) {
-            int64_t at = base_s;
-            for (int w = 0; w < warp; ++w) at += cnt[w];
-            slot0[i] = at;
-        }
+// Segment count of every hub row, a warp a row (0 past them, for the scan).  (A
+// warp that walked 32 rows of the store and cut the hubs among them one after
+// another took 56 us at 524,288 chunks, as a cut is a chain of ~20 dependent
+// loads.)
+__global__ __launch_bounds__(256) void k_hub_segs(SplitParams sp,
+                                                  const int64_t *__restrict__ in_ptr,
+                                                  const int32_t *__restrict__ in_src,
+                                                  const int32_t *__restrict__ rows,
+                                                  const int64_t *__restrict__ n_rows,
+                                                  int64_t max_hubs, int64_t *__restrict__ nseg) {
+    const int lane = threadIdx.x & 31;
+    const int64_t n = *n_rows, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (int64_t i = gt >> 5; i < n; i += nw) {
+        const int64_t r = rows[i];
+        const int64_t c = warp_segments(sp, in_src, in_ptr[r], in_ptr[r + 1],
+                                        [](int64_t, int64_t, int64_t, int64_t) {});
+        if (lane == 0) nseg[i] = c;
     }
+    for (int64_t i = n + gt; i < max_hubs; i += nw * 32) nseg[i] = 0;
 }
 
 // The plan of every hub row, a warp each: its segments with their window and
@@ -867,25 +820,28 @@ __global__ void k_seg_permute(const uint32_t *__restrict__ order, const int64_t 
 }
 
 int64_t hub_plan_words(int64_t n, int64_t max_hubs) {
-    return 2 + ceil_div<int64_t>(n, HEAVY_TILE) + ceil_div<int64_t>(max_hubs, 8);
+    return ceil_div<int64_t>(ceil_div<int64_t>(n, HEAVY_TILE), 2) + max_hubs +
+           (int64_t)(scan_tmp_bytes(max_hubs) / 8) + 1;
 }
 
 cudaError_t launch_hub_count(const SplitParams &sp, const int64_t *in_ptr, const int32_t *in_src,
                              int64_t n, int64_t max_hubs, int32_t *rows, int64_t *slot0,
-                             int64_t *counts, unsigned long long *chain, int *status,
-                             cudaStream_t st) {
-    const int64_t words = hub_plan_words(n, max_hubs), tiles = ceil_div<int64_t>(n, HEAVY_TILE);
-    cudaError_t e = cudaMemsetAsync(chain, 0, (size_t)words * 8, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, 16, st);
-    if (e != cudaSuccess || n <= 0) return e;
-    const int64_t cap = (int64_t)device_sm_count() * 8;
-    k_heavy_rows<<<(unsigned)(tiles < cap ? tiles : cap), 256, 0, st>>>(in_ptr, n, sp.split_t, rows,
-                                                                        counts, chain, status);
-    const int64_t ht = ceil_div<int64_t>(max_hubs > 0 ? max_hubs : 1, 8);
-    k_hub_slots<<<(unsigned)(ht < cap ? ht : cap), 256, 0, st>>>(sp, in_ptr, in_src, rows, counts,
-                                                                 slot0, counts + 1,
-                                                                 chain + 1 + tiles, status);
-    return cudaGetLastError();
+                             int64_t *counts, int64_t *scratch, cudaStream_t st) {
+    const int64_t tiles = ceil_div<int64_t>(n, HEAVY_TILE);
+    if (n <= 0 || max_hubs <= 0) {
+        cudaError_t e = cudaMemsetAsync(counts, 0, 8, st);
+        return e == cudaSuccess ? cudaMemsetAsync(slot0 + (max_hubs > 0 ? max_hubs : 0), 0, 8, st) : e;
+    }
+    int32_t *tc = (int32_t *)scratch;
+    int64_t *nseg = scratch + ceil_div<int64_t>(tiles, 2);
+    k_heavy_rows<false><<<(unsigned)tiles, 256, 0, st>>>(in_ptr, n, sp.split_t, rows, counts, tc);
+    k_heavy_rows<true><<<(unsigned)tiles, 256, 0, st>>>(in_ptr, n, sp.split_t, rows, counts, tc);
+    const int64_t want = ceil_div<int64_t>(max_hubs, 8), cap = (int64_t)device_sm_count() * 8;
+    k_hub_segs<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(sp, in_ptr, in_src, rows, counts,
+                                                                    max_hubs, nseg);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return scan_exclusive(nseg, slot0, max_hubs, nseg + max_hubs, scan_tmp_bytes(max_hubs), st);
 }
 
 cudaError_t launch_hub_fill(const SplitParams &sp, const int64_t *in_ptr, const int32_t *in_src,
@@ -1217,36 +1173,36 @@ cudaError_t launch_mass_levels(const HopPlan &p, int t0, int t1, float *mup, flo
 
 // Last hop, after the floor: the rows kept whole whose upper bound reaches
 // their floor (kept_rows), the split rows that do not (split_skip), and the
-// segments of the split rows that do (kept_segs), in one pass over rows,
-// split rows and segments, in ordered tiles (chain_before): both lists are in
-// row order and in window-major order, the order that keeps gathered source
-// rows in L2 (in the order of the tiles' finish the last hop took 363 instead
-// of 317 us on 500,009 chunks, 100 scoped queries).  The bounds are evaluated
+// segments of the split rows that do (kept_segs), over rows, split rows and
+// segments, in ordered tiles (tile_base): both lists are in row order and in
+// window-major order, the order that keeps gathered source rows in L2 (in the
+// order of the tiles' finish the last hop took 363 instead of 317 us on 500,009
+// chunks, 100 scoped queries).  The bounds are evaluated
 // here: no per-row arrays are
 // written (eleven launches did this; with the floor 102 -> 60 us there, 34 ->
 // 11 us on 4096 chunks).
 constexpr int KEEP_TILE = 1024;
-__global__ __launch_bounds__(256) void k_keep(const RowBounds rb, const float *__restrict__ floor_p,
-                                              const NsFloors nf,
-                                              const int64_t *__restrict__ in_ptr, int64_t split_t,
-                                              int64_t n_split,
-                                              const int32_t *__restrict__ split_row,
-                                              int64_t n_segs, const int32_t *__restrict__ seg_slot,
-                                              const int32_t *__restrict__ slot_split,
-                                              int32_t *__restrict__ split_skip,
-                                              int32_t *__restrict__ kept_rows,
-                                              int32_t *__restrict__ kept_segs,
-                                              unsigned long long *__restrict__ kept_count,
-                                              unsigned long long *chain, int *status,
-                                              const int32_t *__restrict__ done) {
+// k_keep_mark tests (a bit an item in bits, a count a tile), k_keep_list writes
+// the lists.
+__global__ __launch_bounds__(256) void k_keep_mark(const RowBounds rb,
+                                                   const float *__restrict__ floor_p,
+                                                   const NsFloors nf,
+                                                   const int64_t *__restrict__ in_ptr,
+                                                   int64_t split_t, int64_t n_split,
+                                                   const int32_t *__restrict__ split_row,
+                                                   int64_t n_segs,
+                                                   const int32_t *__restrict__ seg_slot,
+                                                   const int32_t *__restrict__ slot_split,
+                                                   int32_t *__restrict__ split_skip,
+                                                   int32_t *__restrict__ counts,
+                                                   uint32_t *__restrict__ bits,
+                                                   const int32_t *__restrict__ done) {
+    __shared__ int own;
     __shared__ int32_t tag_s[PF_TAGS];
     __shared__ float tag_floor_s[PF_TAGS];
-    __shared__ int wcnt[32];
-    __shared__ unsigned long long base_s;
-    __shared__ int64_t tile_s;
     griddep_wait();
     if (done && done[0] == 1) return;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int t = threadIdx.x;
     const float floor_ = *floor_p, umax = ext_umax(rb.ext);
     int n_tags = 0;
     if (nf.ns_row) {
@@ -1270,85 +1226,89 @@ __global__ __launch_bounds__(256) void k_keep(const RowBounds rb, const float *_
         }
         return lo < n_tags && tag_s[lo] == tag && ub >= tag_floor_s[lo];
     };
+    // tiles of rows, of segments, of split rows
     const int64_t row_tiles = (rb.n + KEEP_TILE - 1) / KEEP_TILE;
-    const int64_t split_tiles = (n_split + KEEP_TILE - 1) / KEEP_TILE;
     const int64_t seg_tiles = (n_segs + KEEP_TILE - 1) / KEEP_TILE;
-    while (true) {
-        __syncthreads();   // the tile before is done with wcnt, base_s, tile_s
-        if (t == 0) tile_s = (int64_t)atomicAdd(chain, 1ull);
-        __syncthreads();
-        const int64_t tile = tile_s;
-        if (tile >= row_tiles + split_tiles + seg_tiles) break;
-        if (tile >= row_tiles && tile < row_tiles + split_tiles) {
-            for (int q = 0; q < KEEP_TILE / 256; ++q) {
-                const int64_t r = (tile - row_tiles) * KEEP_TILE + q * 256 + t;
-                if (r < n_split) split_skip[r] = reaches(split_row[r]) ? 0 : 1;
-            }
-            continue;
-        }
-        const bool rows = tile < row_tiles;
-        const int64_t i0 = (rows ? tile : tile - row_tiles - split_tiles) * KEEP_TILE;
-        unsigned bal[KEEP_TILE / 256];
-#pragma unroll
+    const int64_t tile = blockIdx.x;
+    if (tile >= row_tiles + seg_tiles) {
         for (int q = 0; q < KEEP_TILE / 256; ++q) {
-            const int64_t i = i0 + q * 256 + t;
-            bool k = false;
-            if (rows) k = i < rb.n && reaches(i) && in_ptr[i + 1] - in_ptr[i] <= split_t;
-            else k = i < n_segs && reaches(split_row[slot_split[seg_slot[i]]]);
-            bal[q] = __ballot_sync(0xffffffffu, k);
-            if (lane == 0) wcnt[q * 8 + warp] = __popc(bal[q]);
+            const int64_t r = (tile - row_tiles - seg_tiles) * KEEP_TILE + q * 256 + t;
+            if (r < n_split) split_skip[r] = reaches(split_row[r]) ? 0 : 1;
         }
-        __syncthreads();
-        if (warp == 0) {
-            // exclusive offsets of the (step, warp) groups, in item order
-            const int c = wcnt[lane];
-            int incl = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int x = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += x;
-            }
-            wcnt[lane] = incl - c;
-            const unsigned long long own =
-                (unsigned long long)__shfl_sync(0xffffffffu, incl, 31);
-            // this tile's place in its list
-            const int64_t first = rows ? 0 : row_tiles + split_tiles;
-            const int64_t last = rows ? row_tiles : row_tiles + split_tiles + seg_tiles;
-            const unsigned long long before = chain_before(chain + 1, first, tile, own, status);
-            if (lane == 0) {
-                base_s = before;
-                if (tile == last - 1) kept_count[rows ? 0 : 1] = before + own;
-            }
-        }
-        __syncthreads();
-        int32_t *out = rows ? kept_rows : kept_segs;
-#pragma unroll
-        for (int q = 0; q < KEEP_TILE / 256; ++q)
-            if ((bal[q] >> lane) & 1u)
-                out[base_s + wcnt[q * 8 + warp] + __popc(bal[q] & ((1u << lane) - 1u))] =
-                    (int32_t)(i0 + q * 256 + t);
+        return;
     }
+    if (t == 0) own = 0;
+    __syncthreads();
+    const bool rows = tile < row_tiles;
+    const int64_t i0 = (rows ? tile : tile - row_tiles) * KEEP_TILE;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int64_t i = i0 + q * 256 + t;
+        bool k = false;
+        if (rows) k = i < rb.n && reaches(i) && in_ptr[i + 1] - in_ptr[i] <= split_t;
+        else k = i < n_segs && reaches(split_row[slot_split[seg_slot[i]]]);
+        const unsigned bal = __ballot_sync(0xffffffffu, k);
+        if ((t & 31) == 0) {
+            bits[tile * 32 + q * 8 + (t >> 5)] = bal;
+            if (bal) atomicAdd(&own, __popc(bal));
+        }
+    }
+    __syncthreads();
+    if (t == 0) counts[tile] = own;
 }
 
-int64_t keep_chain_words(const HopPlan &p) {
-    return 1 + ceil_div<int64_t>(p.n, KEEP_TILE) + ceil_div<int64_t>(p.n_split_rows, KEEP_TILE) +
-           ceil_div<int64_t>(p.n_segs, KEEP_TILE);
+__global__ __launch_bounds__(256) void k_keep_list(int64_t row_tiles, int64_t seg_tiles,
+                                                   const int32_t *__restrict__ counts,
+                                                   const uint32_t *__restrict__ bits,
+                                                   int32_t *__restrict__ kept_rows,
+                                                   int32_t *__restrict__ kept_segs,
+                                                   int64_t *__restrict__ kept_count,
+                                                   const int32_t *__restrict__ done) {
+    griddep_wait();
+    if (done && done[0] == 1) return;
+    const int t = threadIdx.x;
+    const int64_t tile = blockIdx.x;
+    const bool rows = tile < row_tiles;
+    const bool last = tile == (rows ? row_tiles : row_tiles + seg_tiles) - 1;
+    const int own = counts[tile];
+    if (own == 0 && !last) return;   // nothing to write, no total to tell
+    const int64_t base = tile_base(counts, rows ? 0 : row_tiles, tile);
+    if (last && t == 0) kept_count[rows ? 0 : 1] = base + own;
+    if (own == 0) return;
+    unsigned bal[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) bal[q] = bits[tile * 32 + q * 8 + (t >> 5)];
+    int places[4];
+    tile_places(bal, places);
+    int32_t *out = rows ? kept_rows : kept_segs;
+    const int64_t i0 = (rows ? tile : tile - row_tiles) * KEEP_TILE;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if ((bal[q] >> (t & 31)) & 1u) out[base + places[q]] = (int32_t)(i0 + q * 256 + t);
 }
+
+static int64_t keep_tiles(const HopPlan &p) {
+    return ceil_div<int64_t>(p.n, KEEP_TILE) + ceil_div<int64_t>(p.n_segs, KEEP_TILE);
+}
+int64_t keep_words(const HopPlan &p) { return keep_tiles(p) * (1 + KEEP_TILE / 32); }
 
 cudaError_t launch_keep(const HopPlan &p, const RowBounds &rb, const float *floor_p,
                         const NsFloors *nf, int32_t *split_skip, int32_t *kept_rows,
-                        int32_t *kept_segs, int64_t *kept_count, unsigned long long *chain,
-                        int *status, cudaStream_t st, int *launches) {
-    static_assert(KEEP_TILE / 256 * 8 == 32, "one lane per (step, warp) group");
-    const int64_t tiles = keep_chain_words(p) - 1;
-    const int64_t cap = (int64_t)device_sm_count() * 8;
+                        int32_t *kept_segs, int64_t *kept_count, int32_t *words, cudaStream_t st,
+                        int *launches) {
+    static_assert(KEEP_TILE == 1024, "tile_places");
+    const int64_t tiles = keep_tiles(p), row_tiles = ceil_div<int64_t>(p.n, KEEP_TILE);
     const NsFloors f = nf ? *nf : NsFloors{};
-    cudaError_t e = launch_pdl(k_keep, dim3((unsigned)(tiles < cap ? tiles : cap)), dim3(256), 0,
-                               st, rb, floor_p, f, p.in_ptr, p.split.split_t, p.n_split_rows,
-                               p.split_row, p.n_segs, p.seg_slot, p.slot_split, split_skip,
-                               kept_rows, kept_segs, (unsigned long long *)kept_count, chain,
-                               status, p.done);
-    if (launches) *launches += 1;
+    uint32_t *bits = (uint32_t *)(words + tiles);
+    cudaError_t e = launch_pdl(
+        k_keep_mark, dim3((unsigned)(tiles + ceil_div<int64_t>(p.n_split_rows, KEEP_TILE))),
+        dim3(256), 0, st, rb, floor_p, f, p.in_ptr, p.split.split_t, p.n_split_rows, p.split_row,
+        p.n_segs, p.seg_slot, p.slot_split, split_skip, words, bits, p.done);
+    if (e == cudaSuccess)
+        e = launch_pdl(k_keep_list, dim3((unsigned)tiles), dim3(256), 0, st, row_tiles,
+                       tiles - row_tiles, (const int32_t *)words, (const uint32_t *)bits, kept_rows,
+                       kept_segs, kept_count, p.done);
+    if (launches) *launches += 2;
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 

@@ -9,8 +9,7 @@
 //   LLMCoLocate(S) = the chunks of S with a partner in S at or above tau;
 //   LLMGroup(P) = connected components of those pairs within a namespace.
 // A batch of requests adds its statistics first; its relocations then run
-// in request order (one CTA walks the requests; lanes work on a request's
-// chunk set).
+// in request order (one CTA walks the requests, 32 at a time).
 #include "ak_common.cuh"
 
 namespace ak {
@@ -40,6 +39,7 @@ __device__ void mm_co_add(const MmTables &t, unsigned long long key, int *status
         const unsigned long long prev = atomicCAS(&t.co_key[h], MM_EMPTY, key);
         if (prev == MM_EMPTY || prev == key) {
             atomicAdd(&t.co_val[h], 1u);
+            if (prev == MM_EMPTY) atomicAdd(t.pairs, 1ull);
             return;
         }
         h = (h + 1) & (t.co_cap - 1);
@@ -117,7 +117,7 @@ __global__ void k_mm_count(const int64_t *__restrict__ S, int n_req, int s_len, 
 
 // LLMCoLocate stand-in for every request of the batch (the statistics of
 // the whole batch are in place): G = the chunks of the set associated with
-// some other chunk of it, in chunk ID order.  One warp per request.
+// some other chunk of it, their rows in chunk ID order.  One warp per request.
 __global__ void k_mm_colocate(const int64_t *__restrict__ S, int n_req, int s_len, int64_t n,
                               const int32_t *__restrict__ row_of,
                               const int32_t *__restrict__ dead_row, MmTables t, float tau,
@@ -147,45 +147,96 @@ __global__ void k_mm_colocate(const int64_t *__restrict__ S, int n_req, int s_le
             const int32_t a = sets[w][i];
             int rk = 0;
             for (int j = 0; j < cnt; ++j) rk += flags[w][j] && sets[w][j] < a;
-            g_out[(int64_t)r * MM_MAX_S + rk] = a;
+            g_out[(int64_t)r * MM_MAX_S + rk] = row_of[a];
         }
         if (lane == 0) g_n[r] = ng;
         __syncwarp();
     }
 }
 
-// Relocation in request order (one warp): a G of two or more chunks not all
-// on one page is written into fresh pages, old slots become invalid.
-__global__ void k_mm_relocate(const int32_t *__restrict__ g_in, const int32_t *__restrict__ g_n,
-                              int n_req, const int32_t *__restrict__ row_of,
-                              int32_t *__restrict__ page_row, MmTables t, int per_page) {
-    const int lane = threadIdx.x & 31;
-    int64_t next = *t.next_page;
-    int64_t writes = 0;
-    for (int r = 0; r < n_req; ++r) {
-        const int ng = g_n[r];
-        if (ng < 2) continue;
-        const int32_t *g = g_in + (int64_t)r * MM_MAX_S;
-        const int32_t p0 = page_row[row_of[g[0]]];
-        bool same = true;
-        for (int i = lane; i < ng; i += 32) same &= page_row[row_of[g[i]]] == p0;
-        if (__all_sync(0xffffffffu, same)) continue;
-        __syncwarp();
-        for (int i = lane; i < ng; i += 32) {
-            const int64_t row = row_of[g[i]];
-            atomicSub(&t.page_live[page_row[row]], 1);
-            const int32_t p = (int32_t)(next + i / per_page);
-            page_row[row] = p;
-            atomicAdd(&t.page_total[p], 1);
-            atomicAdd(&t.page_live[p], 1);
-        }
-        __syncwarp();
-        next += (ng + per_page - 1) / per_page;
-        writes += ng;
+// Relocation in request order: a G of two or more chunks not all on one page
+// is written into fresh pages, old slots become invalid.  One CTA, 32 requests
+// at a time, a warp each: every warp looks whether its G lies on one page; the
+// requests before the first that does not are done, that one moves, and the
+// ones after it look again (their chunks may just have moved).  A request that
+// stays costs a 32nd of a look (one warp that took the requests in turn, a
+// chain of four dependent loads each, needed ~0.9 us for every one of them:
+// relocation 238 us a batch of 256, 92 so).
+// result: the next fresh page, the chunks written, the pairs in the table, the
+// status word.
+__global__ __launch_bounds__(1024) void k_mm_relocate(const int32_t *__restrict__ g_in,
+                                                      const int32_t *__restrict__ g_n, int n_req,
+                                                      int32_t *page_row, MmTables t,
+                                                      int64_t next_page, int per_page,
+                                                      const int *status, int64_t *result) {
+    __shared__ int need[32];
+    __shared__ int64_t next_s, writes_s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        next_s = next_page;
+        writes_s = 0;
     }
-    if (lane == 0) {
-        *t.next_page = next;
-        *t.writes += writes;
+    // the next 32 requests' rows are loaded while these are looked at (slots
+    // past a request's count hold what an earlier batch left there)
+    int ng_n = warp < n_req ? g_n[warp] : 0;
+    int32_t row_n[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        row_n[h] = warp < n_req ? g_in[(int64_t)warp * MM_MAX_S + lane + 32 * h] : -1;
+    for (int r0 = 0; r0 < n_req; r0 += 32) {
+        const int ng = ng_n, r = r0 + 32 + warp;
+        int64_t row[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) row[h] = lane + 32 * h < ng ? (int64_t)row_n[h] : -1;
+        ng_n = r < n_req ? g_n[r] : 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            row_n[h] = r < n_req ? g_in[(int64_t)r * MM_MAX_S + lane + 32 * h] : -1;
+        bool done = ng < 2;
+        while (true) {
+            bool moves = false;
+            if (!done) {
+                // (pages are written by other warps: not through the L1)
+                int32_t p[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) p[h] = row[h] >= 0 ? __ldcg(page_row + row[h]) : 0;
+                const int32_t p0 = __shfl_sync(0xffffffffu, p[0], 0);
+                moves = __any_sync(0xffffffffu, (row[0] >= 0 && p[0] != p0) ||
+                                                    (row[1] >= 0 && p[1] != p0));
+            }
+            if (lane == 0) need[warp] = moves ? 1 : 0;
+            __syncthreads();
+            const unsigned nd = __ballot_sync(0xffffffffu, need[lane] != 0);
+            if (nd == 0u) break;
+            const int first = __ffs(nd) - 1;
+            if (warp < first) done = true;
+            if (warp == first) {
+                done = true;
+                const int64_t next = next_s;
+                __syncwarp();
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (row[h] < 0) continue;
+                    atomicSub(&t.page_live[__ldcg(page_row + row[h])], 1);
+                    const int32_t q = (int32_t)(next + (lane + 32 * h) / per_page);
+                    __stcg(page_row + row[h], q);
+                    atomicAdd(&t.page_total[q], 1);
+                    atomicAdd(&t.page_live[q], 1);
+                }
+                if (lane == 0) {
+                    next_s = next + (ng + per_page - 1) / per_page;
+                    writes_s += ng;
+                }
+            }
+            __syncthreads();
+        }
+        __syncthreads();   // need[] is rewritten by the next 32
+    }
+    if (threadIdx.x == 0) {
+        result[0] = next_s;
+        result[1] = writes_s;
+        result[2] = (int64_t)*t.pairs;
+        result[3] = *status;
     }
 }
 
@@ -207,18 +258,80 @@ __global__ void k_mm_candidates(MmTables t, int64_t n_pages, float theta, int32_
     }
 }
 
-// moving[c] = 1 for live chunks on candidate pages; parent[c] = c
-__global__ void k_mm_moving(int64_t n, const int32_t *__restrict__ row_of,
-                            const int32_t *__restrict__ dead_row,
-                            const int32_t *__restrict__ page_row, const int32_t *__restrict__ cand,
-                            int64_t *__restrict__ moving, int32_t *__restrict__ parent) {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t row = row_of[c];
-        const bool mv = !(dead_row && dead_row[row]) && cand[page_row[row]];
-        moving[c] = mv ? 1 : 0;
-        parent[c] = (int32_t)c;
+// The live chunks on candidate pages, in ID order: ids[] and their namespaces'
+// sort keys, a bitmap of them, parent[c] = c; count = how many.  The first pass
+// over the directory makes the bitmap and the tiles' counts (tile_base), the
+// second reads these alone.
+constexpr int MM_TILE = 1024;
+__global__ __launch_bounds__(256) void k_mm_moving(int64_t n, const int32_t *__restrict__ row_of,
+                                                   const int32_t *__restrict__ dead_row,
+                                                   const int32_t *__restrict__ page_row,
+                                                   const int32_t *__restrict__ cand,
+                                                   uint32_t *__restrict__ moving,
+                                                   int32_t *__restrict__ counts) {
+    const int t = threadIdx.x;
+    int64_t row[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int64_t c = (int64_t)blockIdx.x * MM_TILE + q * 256 + t;
+        row[q] = c < n ? row_of[c] : -1;
     }
+    int mine = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int64_t c = (int64_t)blockIdx.x * MM_TILE + q * 256 + t;
+        const bool mv =
+            row[q] >= 0 && cand[page_row[row[q]]] && !(dead_row && dead_row[row[q]]);
+        const unsigned bal = __ballot_sync(0xffffffffu, mv);
+        if ((t & 31) == 0 && c < n) moving[c >> 5] = bal;
+        mine += mv ? 1 : 0;
+    }
+    const int own = __syncthreads_count(mine > 0) ? 1 : 0;
+    // (mostly none moves: only then is there nothing to add up)
+    if (own == 0) {
+        if (t == 0) counts[blockIdx.x] = 0;
+        return;
+    }
+    __shared__ int sum;
+    if (t == 0) sum = 0;
+    __syncthreads();
+    if (mine) atomicAdd(&sum, mine);
+    __syncthreads();
+    if (t == 0) counts[blockIdx.x] = sum;
+}
+
+__global__ __launch_bounds__(256) void k_mm_list(int64_t n, const int32_t *__restrict__ row_of,
+                                                 const int32_t *__restrict__ ns_row,
+                                                 const uint32_t *__restrict__ moving,
+                                                 int32_t *__restrict__ parent,
+                                                 uint32_t *__restrict__ ids,
+                                                 uint32_t *__restrict__ ns_key,
+                                                 unsigned long long *__restrict__ count,
+                                                 const int32_t *__restrict__ counts) {
+    const int t = threadIdx.x;
+    const int64_t tile = blockIdx.x;
+    const int own = counts[tile];
+    if (own == 0 && tile != gridDim.x - 1) return;
+    const int64_t base = tile_base(counts, 0, tile);
+    if (t == 0 && tile == gridDim.x - 1) *count = (unsigned long long)(base + own);
+    if (own == 0) return;
+    unsigned bal[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int64_t c = tile * MM_TILE + q * 256 + t;
+        bal[q] = c < n ? moving[c >> 5] : 0u;
+        bal[q] = __shfl_sync(0xffffffffu, bal[q], 0);   // (a warp's 32 chunks share a word)
+    }
+    int places[4];
+    tile_places(bal, places);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if ((bal[q] >> (t & 31)) & 1u) {
+            const int64_t c = tile * MM_TILE + q * 256 + t, i = base + places[q];
+            ids[i] = (uint32_t)c;
+            ns_key[i] = (uint32_t)ns_row[row_of[c]] ^ 0x80000000u;   // signed order
+            parent[c] = (int32_t)c;
+        }
 }
 
 __device__ int32_t mm_find(volatile int32_t *parent, int32_t x) {
@@ -232,15 +345,18 @@ __device__ int32_t mm_find(volatile int32_t *parent, int32_t x) {
 
 // union of every associated pair of moving chunks in one namespace; roots
 // hook under the smaller root, so a group's root is its earliest chunk
-__global__ void k_mm_union(MmTables t, const int64_t *__restrict__ moving,
-                           const int32_t *__restrict__ ns_by_id, float tau,
-                           int32_t *__restrict__ parent, int *status) {
+__global__ void k_mm_union(MmTables t, const uint32_t *__restrict__ moving,
+                           const unsigned long long *__restrict__ count,
+                           const int32_t *__restrict__ row_of, const int32_t *__restrict__ ns_row,
+                           float tau, int32_t *__restrict__ parent, int *status) {
     for (int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; h < t.co_cap;
          h += (int64_t)gridDim.x * blockDim.x) {
         const unsigned long long key = t.co_key[h];
         if (key == MM_EMPTY) continue;
         const int32_t a = (int32_t)(key >> 32), b = (int32_t)(key & 0xffffffffu);
-        if (!moving[a] || !moving[b] || ns_by_id[a] != ns_by_id[b]) continue;
+        if (!((moving[a >> 5] >> (a & 31)) & 1u) || !((moving[b >> 5] >> (b & 31)) & 1u) ||
+            ns_row[row_of[a]] != ns_row[row_of[b]])
+            continue;
         if (!mm_assoc(t.co_val[h], t.sel[a], t.sel[b], tau)) continue;
         volatile int32_t *vp = parent;
         int it = 0;
@@ -254,33 +370,125 @@ __global__ void k_mm_union(MmTables t, const int64_t *__restrict__ moving,
     }
 }
 
-// keys for the ordered repack: (namespace, group root, chunk ID); the
-// moving chunks arrive in ID order (compacted by scan)
-__global__ void k_mm_keys(const int64_t *__restrict__ moving, const int64_t *__restrict__ pos,
-                          int64_t n, const int32_t *__restrict__ parent,
-                          const int32_t *__restrict__ ns_by_id, uint32_t *__restrict__ ids,
-                          uint32_t *__restrict__ root_key, uint32_t *__restrict__ ns_key) {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        if (!moving[c]) continue;
-        const int64_t i = pos[c];
-        ids[i] = (uint32_t)c;
-        root_key[i] = (uint32_t)mm_find((volatile int32_t *)parent, (int32_t)c);
-        ns_key[i] = (uint32_t)ns_by_id[c] ^ 0x80000000u;   // signed order
-    }
+// keys for the ordered repack: (namespace, group root, chunk ID); the moving
+// chunks arrive in ID order
+__global__ void k_mm_roots(const uint32_t *__restrict__ ids, int64_t count,
+                           const int32_t *__restrict__ parent, uint32_t *__restrict__ root_key) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
+         i += (int64_t)gridDim.x * blockDim.x)
+        root_key[i] = (uint32_t)mm_find((volatile int32_t *)parent, (int32_t)ids[i]);
 }
 
 __global__ void k_mm_ns_keys(const uint32_t *__restrict__ ids, int64_t count,
-                             const int32_t *__restrict__ ns_by_id, uint32_t *__restrict__ out) {
+                             const int32_t *__restrict__ row_of,
+                             const int32_t *__restrict__ ns_row, uint32_t *__restrict__ out) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = (uint32_t)ns_by_id[ids[i]] ^ 0x80000000u;
+        out[i] = (uint32_t)ns_row[row_of[ids[i]]] ^ 0x80000000u;
 }
 
-cudaError_t launch_mm_ns_keys(const uint32_t *ids, int64_t count, const int32_t *ns_by_id,
-                              uint32_t *out, cudaStream_t st) {
+// The whole repack of at most MM_SMALL chunks by one CTA: their order
+// (namespace, group root, chunk ID), the pages of each namespace's run (every
+// namespace starts on a fresh page), the chunks written there.  new_pages: the
+// pages used.  (Sorts, page counts, a scan and the writes took 15 launches and
+// a read-back for the few dozen chunks that a compaction mostly moves.)
+constexpr int MM_SMALL = 2048;
+__global__ __launch_bounds__(1024) void k_mm_repack_small(const uint32_t *__restrict__ ids,
+                                                          const uint32_t *__restrict__ ns_key,
+                                                          int count,
+                                                          const int32_t *__restrict__ parent,
+                                                          const int32_t *__restrict__ row_of,
+                                                          int32_t *__restrict__ page_row,
+                                                          MmTables t, int64_t first_page,
+                                                          int per_page, int64_t *new_pages) {
+    __shared__ unsigned long long key[MM_SMALL];   // (namespace, root)
+    __shared__ uint16_t at[MM_SMALL];              // place in ids
+    __shared__ int32_t run_page[MM_SMALL];         // at a run's head: its first page
+    __shared__ int wsum[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int size = 32;
+    while (size < count) size <<= 1;
+    for (int i = tid; i < size; i += 1024) {
+        key[i] = i < count ? ((unsigned long long)ns_key[i] << 32) |
+                                 (uint32_t)mm_find((volatile int32_t *)parent, (int32_t)ids[i])
+                           : ~0ull;
+        at[i] = (uint16_t)i;
+    }
+    __syncthreads();
+    // ascending by (key, place): places are in chunk ID order; absent ones last
+    for (int sz = 2; sz <= size; sz <<= 1)
+        for (int stride = sz >> 1; stride > 0; stride >>= 1) {
+            for (int i = tid; i < size; i += 1024) {
+                const int o = i ^ stride;
+                if (o > i) {
+                    const unsigned long long a = key[i], b = key[o];
+                    const uint16_t pa = at[i], pb = at[o];
+                    const bool gt = a > b || (a == b && pa > pb);
+                    if (gt == ((i & sz) == 0)) {
+                        key[i] = b;
+                        key[o] = a;
+                        at[i] = pb;
+                        at[o] = pa;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    // runs of equal namespaces: two places a thread, 0 .. 2047
+    int head[2], len[2] = {0, 0}, pages = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int i = 2 * tid + h;
+        head[h] = i < count && (i == 0 || (key[i] >> 32) != (key[i - 1] >> 32));
+        if (head[h]) {
+            // the run's end: first place with a larger namespace
+            int lo = i + 1, hi = count;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if ((key[mid] >> 32) > (key[i] >> 32)) hi = mid;
+                else lo = mid + 1;
+            }
+            len[h] = lo - i;
+        }
+        pages += (len[h] + per_page - 1) / per_page;
+    }
+    // base pages: exclusive scan of the runs' pages over the threads
+    int incl = pages;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    int base = incl - pages;
+    for (int w = 0; w < warp; ++w) base += wsum[w];
+    if (tid == 1023) *new_pages = base + pages;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if (head[h]) run_page[2 * tid + h] = base;
+        base += (len[h] + per_page - 1) / per_page;
+    }
+    __syncthreads();
+    // place i: its run's head is the first place with its namespace
+    for (int i = tid; i < count; i += 1024) {
+        int lo = 0, hi = i;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if ((key[mid] >> 32) < (key[i] >> 32)) lo = mid + 1;
+            else hi = mid;
+        }
+        const int32_t p = (int32_t)(first_page + run_page[lo] + (i - lo) / per_page);
+        page_row[row_of[ids[at[i]]]] = p;
+        atomicAdd(&t.page_total[p], 1);
+        atomicAdd(&t.page_live[p], 1);
+    }
+}
+
+cudaError_t launch_mm_ns_keys(const uint32_t *ids, int64_t count, const int32_t *row_of,
+                              const int32_t *ns_row, uint32_t *out, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
-    k_mm_ns_keys<<<device_sm_count() * 2, 256, 0, st>>>(ids, count, ns_by_id, out);
+    k_mm_ns_keys<<<device_sm_count() * 2, 256, 0, st>>>(ids, count, row_of, ns_row, out);
     return cudaGetLastError();
 }
 
@@ -420,42 +628,69 @@ cudaError_t launch_mm_count(const int64_t *S, int n_req, int s_len, int64_t n,
 
 cudaError_t launch_mm_relocate(const int64_t *S, int n_req, int s_len, int64_t n,
                                const int32_t *row_of, const int32_t *dead_row, int32_t *page_row,
-                               const MmTables &t, float tau, int per_page, int32_t *g_buf,
-                               int32_t *g_n, cudaStream_t st) {
+                               const MmTables &t, float tau, int64_t next_page, int per_page,
+                               int32_t *g_buf, int32_t *g_n, const int *status, int64_t *result,
+                               cudaStream_t st) {
     if (n_req <= 0) return cudaSuccess;
     const int grid = (int)ceil_div<int64_t>(n_req, 8);
     k_mm_colocate<<<grid < device_sm_count() * 8 ? grid : device_sm_count() * 8, 256, 0, st>>>(
         S, n_req, s_len, n, row_of, dead_row, t, tau, g_buf, g_n);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_mm_relocate<<<1, 32, 0, st>>>(g_buf, g_n, n_req, row_of, page_row, t, per_page);
+    k_mm_relocate<<<1, 1024, 0, st>>>(g_buf, g_n, n_req, page_row, t, next_page, per_page, status,
+                                      result);
     return cudaGetLastError();
 }
 
-cudaError_t launch_mm_compact_prepare(const MmTables &t, int64_t n_pages, float theta, int64_t n,
-                                      const int32_t *row_of, const int32_t *dead_row,
-                                      const int32_t *page_row, int32_t *cand, int64_t *moving,
-                                      int32_t *parent, cudaStream_t st) {
-    const int sms = device_sm_count();
-    if (n_pages > 0) k_mm_candidates<<<sms * 2, 256, 0, st>>>(t, n_pages, theta, cand);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || n <= 0) return e;
-    k_mm_moving<<<sms * 4, 256, 0, st>>>(n, row_of, dead_row, page_row, cand, moving, parent);
+cudaError_t launch_mm_candidates(const MmTables &t, int64_t n_pages, float theta, int32_t *cand,
+                                 cudaStream_t st) {
+    cudaError_t e = cudaMemsetAsync(t.released, 0, 8, st);
+    if (e != cudaSuccess || n_pages <= 0) return e;
+    const int64_t want = ceil_div<int64_t>(n_pages, 256), cap = (int64_t)device_sm_count() * 2;
+    k_mm_candidates<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(t, n_pages, theta, cand);
     return cudaGetLastError();
 }
 
-cudaError_t launch_mm_union(const MmTables &t, const int64_t *moving, const int32_t *ns_by_id,
-                            float tau, int32_t *parent, int *status, cudaStream_t st) {
-    k_mm_union<<<device_sm_count() * 8, 256, 0, st>>>(t, moving, ns_by_id, tau, parent, status);
+int64_t mm_tiles(int64_t n) { return ceil_div<int64_t>(n, MM_TILE); }
+
+cudaError_t launch_mm_collect(const MmTables &t, int64_t n, const int32_t *row_of,
+                              const int32_t *dead_row, const int32_t *page_row,
+                              const int32_t *ns_row, const int32_t *cand, uint32_t *moving,
+                              int32_t *parent, uint32_t *ids, uint32_t *ns_key, int32_t *counts,
+                              cudaStream_t st) {
+    if (n <= 0) return cudaErrorInvalidValue;
+    const unsigned tiles = (unsigned)mm_tiles(n);
+    k_mm_moving<<<tiles, 256, 0, st>>>(n, row_of, dead_row, page_row, cand, moving, counts);
+    k_mm_list<<<tiles, 256, 0, st>>>(n, row_of, ns_row, moving, parent, ids, ns_key,
+                                     t.released + 1, counts);
     return cudaGetLastError();
 }
 
-cudaError_t launch_mm_keys(const int64_t *moving, const int64_t *pos, int64_t n,
-                           const int32_t *parent, const int32_t *ns_by_id, uint32_t *ids,
-                           uint32_t *root_key, uint32_t *ns_key, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    k_mm_keys<<<device_sm_count() * 4, 256, 0, st>>>(moving, pos, n, parent, ns_by_id, ids,
-                                                     root_key, ns_key);
+cudaError_t launch_mm_union(const MmTables &t, const uint32_t *moving, const int32_t *row_of,
+                            const int32_t *ns_row, float tau, int32_t *parent, int *status,
+                            cudaStream_t st) {
+    k_mm_union<<<device_sm_count() * 8, 256, 0, st>>>(t, moving, t.released + 1, row_of, ns_row,
+                                                      tau, parent, status);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mm_roots(const uint32_t *ids, int64_t count, const int32_t *parent,
+                            uint32_t *root_key, cudaStream_t st) {
+    if (count <= 0) return cudaSuccess;
+    k_mm_roots<<<device_sm_count() * 2, 256, 0, st>>>(ids, count, parent, root_key);
+    return cudaGetLastError();
+}
+
+int mm_small_repack() { return MM_SMALL; }
+cudaError_t launch_mm_repack_small(const MmTables &t, int64_t n_pages, const int32_t *cand,
+                                   const uint32_t *ids, const uint32_t *ns_key, int64_t count,
+                                   const int32_t *parent, const int32_t *row_of,
+                                   int32_t *page_row, int64_t first_page, int per_page,
+                                   int64_t *new_pages, cudaStream_t st) {
+    if (count < 1 || count > MM_SMALL) return cudaErrorInvalidValue;
+    if (n_pages > 0) k_mm_release<<<device_sm_count() * 2, 256, 0, st>>>(t, n_pages, cand);
+    k_mm_repack_small<<<1, 1024, 0, st>>>(ids, ns_key, (int)count, parent, row_of, page_row, t,
+                                          first_page, per_page, new_pages);
     return cudaGetLastError();
 }
 

@@ -731,8 +731,7 @@ constexpr int PF_ROWS = 1024;
 __global__ __launch_bounds__(PF_ROWS) void k_prune_floor(
     unsigned long long *__restrict__ bound, int n_real, const RowBounds rb,
     const int32_t *__restrict__ lb_rows, const int32_t *__restrict__ order, int64_t n_rows,
-    int k, float *__restrict__ floor_out, unsigned long long *__restrict__ zero, int64_t n_zero,
-    const int32_t *__restrict__ done) {
+    int k, float *__restrict__ floor_out, const int32_t *__restrict__ done) {
     __shared__ unsigned long long xk[2][PF_ROWS];
     __shared__ unsigned int s_min;
     __shared__ float s_floor;
@@ -740,7 +739,6 @@ __global__ __launch_bounds__(PF_ROWS) void k_prune_floor(
     if (done && done[0] == 1) return;
     const int t = threadIdx.x;
     if (t == 0) s_min = 0x7f800000u;
-    for (int64_t i = t; i < n_zero; i += PF_ROWS) zero[i] = 0ull;
     __syncthreads();
     if (t < n_real) atomicMin(&s_min, (unsigned int)(bound[t] >> 32));
     const bool want_lb = lb_rows && n_rows >= k;
@@ -933,11 +931,10 @@ cudaError_t launch_ns_floors(unsigned long long *bound, const int32_t *q_ns, int
 
 cudaError_t launch_prune_floor(unsigned long long *bound, int n_real, const RowBounds &rb,
                                const int32_t *lb_rows, const int32_t *order, int64_t n_lb_rows,
-                               int k, float *floor_out, unsigned long long *zero, int64_t n_zero,
-                               const int32_t *done, cudaStream_t st) {
+                               int k, float *floor_out, const int32_t *done, cudaStream_t st) {
     if (n_lb_rows > PF_ROWS || n_real > PF_ROWS || k < 1) return cudaErrorInvalidValue;
     cudaError_t e = launch_pdl(k_prune_floor, dim3(1), dim3(PF_ROWS), 0, st, bound, n_real, rb,
-                               lb_rows, order, n_lb_rows, k, floor_out, zero, n_zero, done);
+                               lb_rows, order, n_lb_rows, k, floor_out, done);
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 

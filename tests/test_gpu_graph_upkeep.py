@@ -1,4 +1,4 @@
-"""Deletion's one-pass compaction at the edges of its words and tiles, and the
+"""Deletion's two-pass compaction at the edges of its words and tiles, and the
 hub plan with more source windows than a warp has lanes.  Against the oracle."""
 import dataclasses
 
