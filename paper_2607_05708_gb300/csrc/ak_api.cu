@@ -1329,9 +1329,17 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
         if (eff_hops >= 2) AK_TRY(ensure_spare(sc->sb, (size_t)n * bp * 4));
         if (eff_hops >= 1 && m->n_segs > 0) AK_TRY(ensure_spare(sc->partial, (size_t)m->n_segs * bp * 4));
         if (eff_hops >= 1) AK_TRY(sc->words.ensure(CW_COUNT * 4));
-        // row bounds for the last hop (fused filter only)
-        const bool prune = eff_hops >= 1 && m->fuse_filter && m->hop_prune;
-        if (prune) {
+        // a small store: the hops in full, the selection from the slab (8192
+        // chunks, 16 queries, two hops 163 -> 70 us), unless the candidates may
+        // do with a host wait (RC_SYNC: 256 queries 74 us, 190 with the hops)
+        const bool direct = m->fuse_filter && topk_direct(n);
+        const bool reach_small =
+            eff_hops == 2 && bp >= 128 && !q_ns && m->reach_on && m->n_split > 0;
+        // row bounds, for the candidates and for the last hop (fused filter only)
+        const bool bounds =
+            eff_hops >= 1 && m->fuse_filter && m->hop_prune && (!direct || reach_small);
+        const bool prune = bounds && !direct;
+        if (bounds) {
             AK_TRY(ensure_spare(sc->rmax_u, (size_t)n * 4));
             AK_TRY(ensure_spare(sc->rmin_u, (size_t)n * 4));
             AK_TRY(ensure_spare(sc->skip_split, (size_t)(m->n_split + 1) * 4));
@@ -1356,7 +1364,8 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
         // then writes no slab: the bound comes from the score of every
         // stride-th row, computed first by the same kernel (same values).
         const SelectPlan sp2 = select_plan(sp.n_sample, bp, k, sms, 1);
-        const bool dense_fused = eff_hops == 0 && m->fuse_filter && sp2.off_tr == sp.off_tr &&
+        const bool dense_fused = eff_hops == 0 && m->fuse_filter && !direct &&
+                                 sp2.off_tr == sp.off_tr &&
                                  sp2.words <= sp.words;
         unsigned long long *ws = sc->cand.as<unsigned long long>();
         ColumnRecompute rc{};
@@ -1394,14 +1403,14 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
         // 262,147 chunks, 24 queries 384 -> 142; 262,144 chunks, 200 queries, three
         // hops 1589 -> 237 (564 in fp32).
         enum { RUN_HOPS, RC_SYNC, RC_MMA, RC_FMA } mode = RUN_HOPS;
-        if (prune) {
+        if (bounds) {
             std::lock_guard<std::mutex> lk(m->table_mu);
             AK_TRY(ensure_mass(m, hp, eff_hops, st));
             const bool can = !q_ns && m->reach_on && eff_hops >= 2 && eff_hops <= REACH_MAX_H;
             if (can && eff_hops == 2 && bp >= 128 && m->n_split > 0) {
                 AK_TRY(ensure_reach(m, hp, eff_hops, st));
                 mode = RC_SYNC;
-            } else if (can && m->n_split >= k && sc->no_room_n != n) {
+            } else if (can && !direct && m->n_split >= k && sc->no_room_n != n) {
                 bool go = m->reach_levels >= eff_hops && m->reach_n == n;
                 if (!go) {
                     if (m->hop_work_n != n) m->hop_work = 0;
@@ -1467,9 +1476,9 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
             return launch_score(m->emb.as<uint16_t>(), n, m->dim, sc->qp.as<uint16_t>(), bp,
                                 sc->shift.as<float>(), m->tau, sc->u.as<float>(),
                                 sc->zpart.as<float>(), m->status.as<int>(), st, launches, &zrows,
-                                ns.dead, prune ? sc->rmax_u.as<float>() : nullptr,
-                                prune ? sc->rmin_u.as<float>() : nullptr, b,
-                                prune ? ext : nullptr, done);
+                                ns.dead, bounds ? sc->rmax_u.as<float>() : nullptr,
+                                bounds ? sc->rmin_u.as<float>() : nullptr, b,
+                                bounds ? ext : nullptr, done);
         };
         {
             PhaseScope ph(m, AKASHIC_PHASE_SCORE, st);
@@ -1537,6 +1546,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
             rc.dst = sc->u.as<float>();
         }
         const float *fin = sc->u.as<float>();
+        bool reached = false;   // the buffers hold every candidate
         if (eff_hops >= 1) {
             float *bufs[2] = {sc->sa.as<float>(), sc->sb.as<float>()};
             rc.u = sc->u.as<float>();
@@ -1641,7 +1651,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                 if (mode == RC_SYNC) {
                     ph.end();
                     CUDA_TRY(cudaEventSynchronize(sc->plan_ev));
-                    reach_done = sc->plan_host[0] == 1;   // the buffers hold every candidate
+                    reached = reach_done = sc->plan_host[0] == 1;
                     if (reach_done) rc = ColumnRecompute{};
                 } else {
                     hp.done = plan;
@@ -1654,7 +1664,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
             }
             for (int h = 0; h < eff_hops && !reach_done; ++h) {
                 float *out = bufs[h & 1];
-                const bool last = m->fuse_filter && h == eff_hops - 1;
+                const bool last = m->fuse_filter && !direct && h == eff_hops - 1;
                 if (last) {
                     // Top-k filter fused into the last hop, its bound from the
                     // hop's own values on the row sample.
@@ -1722,7 +1732,14 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
             PhaseScope ph(m, AKASHIC_PHASE_SELECT, st);
             int32_t *pids = page_ids ? page_ids + (int64_t)off * k : nullptr;
             int32_t *npg = n_pages ? n_pages + off : nullptr;
-            if ((eff_hops >= 1 && m->fuse_filter) || dense_fused)
+            if (direct && !reached)
+                CUDA_TRY(launch_topk_direct(fin, n, bp, b, k, sc->zpart.as<float>(), zrows,
+                                            m->ext_of.as<int32_t>(), m->row_of.as<int32_t>(),
+                                            m->page_of.as<int32_t>(), ids + (int64_t)off * k,
+                                            scores + (int64_t)off * k, pids, npg,
+                                            m->status.as<int>(), ns, sort_by_time, st,
+                                            &ph.launches));
+            else if ((eff_hops >= 1 && m->fuse_filter) || dense_fused)
                 CUDA_TRY(launch_topk_merge(sp, fin, b, sc->cand.as<unsigned long long>(),
                                            sc->zpart.as<float>(), zrows, m->ext_of.as<int32_t>(),
                                            m->row_of.as<int32_t>(), m->page_of.as<int32_t>(),

@@ -855,6 +855,14 @@ cudaError_t launch_topk_merge(const SelectPlan &sp, const float *s, int b,
                               int32_t *page_ids, int32_t *n_pages, int *status,
                               const ColumnRecompute *rc, NsScope ns, int sort_by_time,
                               cudaStream_t st, int *launches);
+// Small stores (topk_direct(n)): the same selection straight from the slab of
+// final scores, in one launch.
+bool topk_direct(int64_t n);
+cudaError_t launch_topk_direct(const float *s, int64_t n, int bp, int b, int k,
+                               const float *zpart, int64_t n_ztiles, const int32_t *ext_of,
+                               const int32_t *row_of, const int32_t *page_row, int64_t *ids,
+                               float *scores, int32_t *page_ids, int32_t *n_pages, int *status,
+                               NsScope ns, int sort_by_time, cudaStream_t st, int *launches);
 cudaError_t launch_sample_bound_signed(const SelectPlan &sp, const float *s, int b,
                                        const int32_t *ext_of, int64_t id_limit,
                                        unsigned long long *ws, unsigned long long *bound,

@@ -557,6 +557,58 @@ __device__ void column_top(const float *__restrict__ s, int64_t n, int bp, int k
     }
 }
 
+// The winners of query c (win[0..win_n), unordered, at least 64 slots) ordered
+// by key (score desc, id asc) or, with sort_by_time, by chunk ID; normalised by
+// the sum of zred[0..8); resolved to pages, and their distinct pages counted.
+// At least 64 threads; pg: 64 shared words.
+__device__ __forceinline__ void write_winners(const unsigned long long *win, int win_n, int k,
+                                              int c, const double *zred,
+                                              const int32_t *__restrict__ row_of,
+                                              const int32_t *__restrict__ page_row,
+                                              int64_t *__restrict__ ids, float *__restrict__ scores,
+                                              int32_t *__restrict__ page_ids,
+                                              int32_t *__restrict__ n_pages, int *status,
+                                              const NsScope &ns, int sort_by_time, int *pg) {
+    const int tid = threadIdx.x;
+    // without a scope every query has k winners; with one, a namespace
+    // holding fewer than k chunks pads its list
+    if (tid == 0 && (win_n > k || (!scope_active(ns) && win_n != k)))
+        set_status(status, AKASHIC_EDEVICE);
+    const int got = win_n < k ? win_n : k;
+    if (tid < got) {
+        const unsigned long long key = win[tid];
+        const uint32_t id = key_id(key);
+        // rank by score (key desc) or, with SortByTime, by chunk ID
+        int rank = 0;
+        for (int t = 0; t < got; ++t)
+            rank += sort_by_time ? (key_id(win[t]) < id) : (win[t] > key);
+        double zsum = 0.0;
+        for (int w = 0; w < SEL_THREADS / 32; ++w) zsum += zred[w];
+        const int64_t o = (int64_t)c * k + rank;
+        ids[o] = (int64_t)id;
+        scores[o] = (float)((double)sel_value<false>(key) / zsum);
+        const int32_t p = page_row ? page_row[row_of[id]] : 0;
+        pg[rank] = p;
+        if (page_ids) page_ids[o] = p;
+    } else if (tid < k) {
+        const int64_t o = (int64_t)c * k + tid;
+        ids[o] = -1;
+        scores[o] = 0.f;
+        if (page_ids) page_ids[o] = -1;
+    }
+    __syncthreads();
+    if (n_pages && tid < 32) {
+        int distinct = 0;
+        for (int a = tid; a < got; a += 32) {
+            bool first = true;
+            for (int b2 = 0; b2 < a; ++b2) first &= pg[b2] != pg[a];
+            distinct += first;
+        }
+        for (int o = 16; o > 0; o >>= 1) distinct += __shfl_xor_sync(0xffffffffu, distinct, o);
+        if (tid == 0) n_pages[c] = distinct;
+    }
+}
+
 // Retrieval merge, one CTA per real query column: the k winners ordered by
 // key (score desc, id asc), normalised by Z = sum of the score pass's
 // partials, resolved to pages, and their distinct pages counted.
@@ -607,43 +659,106 @@ __global__ __launch_bounds__(SEL_THREADS) void k_topk_merge(
     if ((tid & 31) == 0) zred[tid >> 5] = z;
     column_top<false>(s, n, bp, k, c, ext_of, (int64_t)1 << 40, cnt, buf, cap, stage, win, &win_n,
                       hist, &s_prefix, &s_remaining, ns);
-    // without a scope every query has k winners; with one, a namespace
-    // holding fewer than k chunks pads its list
-    if (tid == 0 && (win_n > k || (!scope_active(ns) && win_n != k)))
-        set_status(status, AKASHIC_EDEVICE);
-    const int got = win_n < k ? win_n : k;
-    if (tid < got) {
-        const unsigned long long key = win[tid];
-        const uint32_t id = key_id(key);
-        // rank by score (key desc) or, with SortByTime, by chunk ID
-        int rank = 0;
-        for (int t = 0; t < got; ++t)
-            rank += sort_by_time ? (key_id(win[t]) < id) : (win[t] > key);
-        double zsum = 0.0;
-        for (int w = 0; w < SEL_THREADS / 32; ++w) zsum += zred[w];
-        const int64_t o = (int64_t)c * k + rank;
-        ids[o] = (int64_t)id;
-        scores[o] = (float)((double)sel_value<false>(key) / zsum);
-        const int32_t p = page_row ? page_row[row_of[id]] : 0;
-        pg[rank] = p;
-        if (page_ids) page_ids[o] = p;
-    } else if (tid < k) {
-        const int64_t o = (int64_t)c * k + tid;
-        ids[o] = -1;
-        scores[o] = 0.f;
-        if (page_ids) page_ids[o] = -1;
+    write_winners(win, win_n, k, c, zred, row_of, page_row, ids, scores, page_ids, n_pages, status,
+                  ns, sort_by_time, pg);
+}
+
+// Small stores: the top k of column c straight from the slab, without a bound
+// and a filter.  One CTA a query, PER keys a thread in registers; the k-th
+// largest score by its bits from the top (each kept when at least k keys are
+// at or above the prefix with it set), then, only where scores tie across it,
+// the IDs likewise.  A count is a compare a key, a warp sum and one barrier.
+// (The sample, its k-th, the floor, the kept lists and the merge take as many
+// launches as all the rest: 4096 chunks, 4 queries, one hop 43 us, 30 so.)
+constexpr int DIRECT_T = 1024;
+constexpr int64_t DIRECT_N = 8192;
+template <int PER>
+__global__ __launch_bounds__(DIRECT_T) void k_topk_direct(
+    const float *__restrict__ s, int64_t n, int bp, int k, const int32_t *__restrict__ ext_of,
+    const float *__restrict__ zpart, int64_t n_ztiles, const int32_t *__restrict__ row_of,
+    const int32_t *__restrict__ page_row, int64_t *__restrict__ ids, float *__restrict__ scores,
+    int32_t *__restrict__ page_ids, int32_t *__restrict__ n_pages, int *status, const NsScope ns,
+    const int sort_by_time) {
+    __shared__ unsigned long long win[64];
+    __shared__ int win_n;
+    __shared__ int cnt[2][32];
+    __shared__ double zred[SEL_THREADS / 32];
+    __shared__ int pg[64];
+    griddep_wait();
+    const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned long long key[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int64_t j = (int64_t)i * DIRECT_T + tid;
+        key[i] = 0ull;
+        if (j < n && in_scope(ns, j, c))
+            key[i] = sel_key<false>(s[j * bp + c], (uint32_t)ext_of[j]);
     }
-    __syncthreads();
-    if (n_pages && tid < 32) {
-        int distinct = 0;
-        for (int a = tid; a < got; a += 32) {
-            bool first = true;
-            for (int b2 = 0; b2 < a; ++b2) first &= pg[b2] != pg[a];
-            distinct += first;
+    if (tid == 0) win_n = 0;
+    if (warp < SEL_THREADS / 32) {     // Z, as the merge adds it
+        double z = 0.0;
+        for (int64_t t = tid; t < n_ztiles; t += SEL_THREADS) z += (double)zpart[t * bp + c];
+        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+        if (lane == 0) zred[warp] = z;
+    }
+    int turn = 0;
+    auto count_ge = [&](unsigned long long t) {
+        unsigned m = 0u;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) m += key[i] >= t ? 1u : 0u;
+        m = __reduce_add_sync(0xffffffffu, m);
+        if (lane == 0) cnt[turn][warp] = (int)m;
+        __syncthreads();
+        const int all = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt[turn][lane]);
+        turn ^= 1;
+        return all;
+    };
+    // the smallest key that at least k keys reach (1 where fewer are in scope)
+    unsigned long long kth = 1ull;
+    if (count_ge(1ull) > k) {
+        unsigned long long prefix = 0ull;
+        int reach = k + 1;
+        for (int b = 62; b >= 0 && reach != k; --b) {   // (a score's sign bit is 0)
+            const unsigned long long cand = prefix | (1ull << b);
+            const int m = count_ge(cand);
+            if (m >= k) {
+                prefix = cand;
+                reach = m;
+            }
         }
-        for (int o = 16; o > 0; o >>= 1) distinct += __shfl_xor_sync(0xffffffffu, distinct, o);
-        if (tid == 0) n_pages[c] = distinct;
+        kth = prefix;
     }
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+        if (key[i] >= kth) {
+            const int p = atomicAdd(&win_n, 1);
+            if (p < 64) win[p] = key[i];
+        }
+    __syncthreads();
+    write_winners(win, win_n, k, c, zred, row_of, page_row, ids, scores, page_ids, n_pages, status,
+                  ns, sort_by_time, pg);
+}
+
+bool topk_direct(int64_t n) { return n <= DIRECT_N; }
+
+cudaError_t launch_topk_direct(const float *s, int64_t n, int bp, int b, int k,
+                               const float *zpart, int64_t n_ztiles, const int32_t *ext_of,
+                               const int32_t *row_of, const int32_t *page_row, int64_t *ids,
+                               float *scores, int32_t *page_ids, int32_t *n_pages, int *status,
+                               NsScope ns, int sort_by_time, cudaStream_t st, int *launches) {
+    if (n < 1 || n > DIRECT_N || k > 64) return cudaErrorInvalidValue;
+    auto go = [&](auto kernel) {
+        return launch_pdl(kernel, dim3(b), dim3(DIRECT_T), 0, st, s, n, bp, k, ext_of, zpart,
+                          n_ztiles, row_of, page_row, ids, scores, page_ids, n_pages, status, ns,
+                          sort_by_time);
+    };
+    cudaError_t e;
+    if (n <= DIRECT_T) e = go(k_topk_direct<1>);
+    else if (n <= 2 * DIRECT_T) e = go(k_topk_direct<2>);
+    else if (n <= 4 * DIRECT_T) e = go(k_topk_direct<4>);
+    else e = go(k_topk_direct<8>);
+    if (launches) *launches += 1;
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 // Relation-update merge: the M best prior chunks of new chunk c (ordered by
