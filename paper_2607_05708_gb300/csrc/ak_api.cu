@@ -279,9 +279,9 @@ static int bits_for(int64_t max_value) {
 }
 
 static akashic_status_t check_status(akashic_mem *m, cudaStream_t st, const char *what) {
-    CUDA_TRY(cudaStreamSynchronize(st));
     int code = 0;
-    CUDA_TRY(cudaMemcpy(&code, m->status.p, sizeof(int), cudaMemcpyDeviceToHost));
+    CUDA_TRY(cudaMemcpyAsync(&code, m->status.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaStreamSynchronize(st));
     if (code != 0) {
         CUDA_TRY(cudaMemset(m->status.p, 0, sizeof(int)));
         return fail((akashic_status_t)code, "%s: device reported status %d", what, code);
@@ -746,12 +746,6 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
     if (n == 0) return AKASHIC_OK;
     DeviceGuard g(m->device);
     cudaStream_t st = (cudaStream_t)stream;
-    // rows [first, first+n) must have no out-edges
-    int64_t a = 0, b = 0;
-    CUDA_TRY(cudaMemcpyAsync(&a, m->row_ptr.as<int64_t>() + first, 8, cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaMemcpyAsync(&b, m->row_ptr.as<int64_t>() + first + n, 8, cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    if (a != b) return fail(AKASHIC_EINVAL, "update: rows [first, first+n) already have out-edges");
     UpdateArgs ua;
     ua.emb = m->emb.as<uint16_t>();
     ua.dim = m->dim;
@@ -777,23 +771,32 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
     AK_TRY(ensure_spare(ncol, (size_t)nnz_new * 4));
     AK_TRY(ensure_spare(naff, (size_t)nnz_new * 4));
     AK_TRY(ensure_spare(nrp, (size_t)(m->cap + 1) * 8));
+    AK_TRY(ensure_spare(m->w2, (size_t)nnz_new * 4));
+    uint32_t *touched =
+        (uint32_t *)store_scratch(m, SCR_TOUCHED, (size_t)ceil_div<int64_t>(m->n, 32) * 4);
+    if (!touched) return fail(AKASHIC_ENOMEM, "update: out of device memory");
     {
+        // rows [first, first+n) must have no out-edges and no in-edges: checked on
+        // the device, read back with the top-M's outcome, before anything changes
         PhaseScope ph(m, AKASHIC_PHASE_RELATE, st);
-        akashic_status_t r = relate_top_m(ua, st, &ph.launches);
+        CUDA_TRY(launch_check_new_rows(m->row_ptr.as<int64_t>(), m->in_ptr.as<int64_t>(),
+                                       m->row_of.as<int32_t>(), first, n, m->status.as<int>(), st));
+        int code = 0;
+        akashic_status_t r = relate_top_m(ua, st, &ph.launches, &code);
         if (r != AKASHIC_OK) return fail(r, "update: relation GEMM / top-M failed");
-        AK_TRY(check_status(m, st, "update: top-M"));
+        if (code != 0) return check_status(m, st, "update");
     }
     {
         PhaseScope ph(m, AKASHIC_PHASE_GRAPH, st);
         {
             PhaseScope pc(m, AKASHIC_PHASE_CSR_INSERT, st);
             akashic_status_t r = csr_insert(ua, m->row_ptr.as<int64_t>(), m->col.as<int32_t>(),
-                                            m->aff.as<float>(), m->nnz, nrp.as<int64_t>(),
-                                            ncol.as<int32_t>(), naff.as<float>(), st,
-                                            &pc.launches);
+                                            m->aff.as<float>(), m->w.as<float>(), m->nnz,
+                                            nrp.as<int64_t>(), ncol.as<int32_t>(),
+                                            naff.as<float>(), m->w2.as<float>(),
+                                            m->rstat.as<float2>(), touched, st, &pc.launches);
             ph.launches += pc.launches;
             if (r != AKASHIC_OK) return fail(r, "update: CSR insert failed");
-            AK_TRY(check_status(m, st, "update"));
         }
         PhaseScope pt(m, AKASHIC_PHASE_TRANSPOSE, st);
         std::swap(m->row_ptr.p, nrp.p);
@@ -802,12 +805,10 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
         std::swap(m->col.cap, ncol.cap);
         std::swap(m->aff.p, naff.p);
         std::swap(m->aff.cap, naff.cap);
+        std::swap(m->w.p, m->w2.p);
+        std::swap(m->w.cap, m->w2.cap);
         const int64_t nnz_old = m->nnz;
         m->nnz = nnz_new;
-        AK_TRY(m->w.ensure(m->col.cap, false));
-        CUDA_TRY(launch_row_softmax(m->row_ptr.as<int64_t>(), m->aff.as<float>(), m->w.as<float>(),
-                                    m->n, m->rstat.as<float2>(), st));
-        pt.launches += 1;
         if (!m->inc_transpose || nnz_old == 0) {
             AK_TRY(rebuild_in_edges(m, st));
         } else {
@@ -819,18 +820,15 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
             AK_TRY(ensure_spare(src2, (size_t)nnz_new * 4));
             AK_TRY(ensure_spare(aff2, (size_t)nnz_new * 4));
             AK_TRY(ensure_spare(w2, (size_t)nnz_new * 4));
-            const size_t tb = (radix_tmp_bytes(pairs) > scan_tmp_bytes(rows + 1)
-                                   ? radix_tmp_bytes(pairs) : scan_tmp_bytes(rows + 1)) + 4096;
-            void *p_inc = store_scratch(m, SCR_IN_INC, (size_t)(rows + 1) * 8);
-            void *p_deg = store_scratch(m, SCR_IN_DEG, (size_t)(rows + 1) * 8);
-            void *p_off = store_scratch(m, SCR_IN_OFF, (size_t)(rows + 1) * 8);
-            void *p_rs = store_scratch(m, SCR_IN_RSTAT, (size_t)(rows > 0 ? rows : 1) * 8);
+            const size_t tb = radix_tmp_bytes(pairs) + 4096;
+            void *p_rows = store_scratch(m, SCR_IN_ROWS, (size_t)n * 16);
             void *p_k = store_scratch(m, SCR_KEYS, (size_t)pairs * 4 + 16);
             void *p_v = store_scratch(m, SCR_VALS, (size_t)pairs * 4 + 16);
             void *p_k2 = store_scratch(m, SCR_KEYS2, (size_t)pairs * 4 + 16);
             void *p_v2 = store_scratch(m, SCR_VALS2, (size_t)pairs * 4 + 16);
             void *p_tmp = store_scratch(m, SCR_TMP, tb);
-            if (!p_inc || !p_deg || !p_off || !p_rs || !p_k || !p_v || !p_k2 || !p_v2 || !p_tmp)
+            void *p_move = store_scratch(m, SCR_MOVE, (size_t)(1 + move_words(nnz_old, pairs, n)) * 4);
+            if (!p_rows || !p_move || !p_k || !p_v || !p_k2 || !p_v2 || !p_tmp)
                 return fail(AKASHIC_ENOMEM, "update: out of device memory");
             InEdgeUpdate u;
             u.n = rows;
@@ -838,6 +836,8 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
             u.in_ptr_old = m->in_ptr.as<int64_t>();
             u.in_src_old = m->in_src.as<int32_t>();
             u.in_aff_old = m->in_aff.as<float>();
+            u.in_w_old = m->in_w.as<float>();
+            u.touched = touched;
             u.in_ptr_new = ptr2.as<int64_t>();
             u.in_src_new = src2.as<int32_t>();
             u.in_aff_new = aff2.as<float>();
@@ -853,9 +853,8 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
             u.row_of = m->row_of.as<int32_t>();
             u.ext_of = m->ext_of.as<int32_t>();
             u.rstat = m->rstat.as<float2>();
-            InEdgeScratch sc{(int64_t *)p_inc, (int64_t *)p_deg, (int64_t *)p_off,
-                             (uint32_t *)p_k, (uint32_t *)p_v, (uint32_t *)p_k2, (uint32_t *)p_v2,
-                             p_tmp, tb, (float2 *)p_rs};
+            InEdgeScratch sc{(uint32_t *)p_k, (uint32_t *)p_v, (uint32_t *)p_k2, (uint32_t *)p_v2,
+                             (uint32_t *)p_rows, (uint32_t *)p_move, p_tmp, tb};
             CUDA_TRY(launch_in_edges_update(u, sc, st, &pt.launches));
             std::swap(m->in_ptr.p, ptr2.p);
             std::swap(m->in_ptr.cap, ptr2.cap);

@@ -302,61 +302,20 @@ __device__ __forceinline__ float row_softmax_weight(float aff, float2 stat) {
 }
 cudaError_t launch_row_softmax(const int64_t *row_ptr, const float *aff, float *w, int64_t n_rows,
                                float2 *rstat, cudaStream_t st);
-// Edge-parallel moves of CSR rows: a warp takes CHUNK_E consecutive edges
-// [base, base + CHUNK_E), lane l the edges base + 32 j + l (j < CHUNK_E / 32),
-// and finds their rows without a search per edge.  Given r_lo, the row of
-// edge `base` (ptr[r_lo] <= base < ptr[r_lo + 1]), the warp marks in its own
-// shared array rid[] the first edge of every later row that starts inside
-// the chunk, as row - r_lo (where several rows start at one edge, the empty
-// rows before it, the largest wins); a running maximum over the positions,
-// taken 32 at a time across the lanes, gives every edge its row:
-// rows[j] = row of edge base + 32 j + lane - r_lo.  ptr has n + 1 entries,
-// ptr[n] = nnz.
-// All 32 lanes call it.  Chunks are small (four edges a lane) so that the
-// moving kernels stay at high occupancy: their loads are latency-bound.
-constexpr int CHUNK_E = 128;
-__device__ __forceinline__ void chunk_rows(const int64_t *__restrict__ ptr, int64_t n,
-                                           int64_t nnz, int64_t base, int64_t r_lo, int *rid,
-                                           int (&rows)[CHUNK_E / 32]) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int j = 0; j < CHUNK_E / 32; ++j) rid[32 * j + lane] = 0;
-    __syncwarp();
-    // rows starting at or past nnz own no edge (the empty rows at the end)
-    const int64_t lim = base + CHUNK_E < nnz ? base + CHUNK_E : nnz;
-    for (int64_t r0 = r_lo + 1; r0 < n; r0 += 32) {
-        const int64_t r = r0 + lane;
-        const int64_t s = r < n ? ptr[r] : INT64_MAX;   // > base for every r > r_lo
-        if (s < lim) atomicMax(&rid[s - base], (int)(r - r_lo));
-        if (__shfl_sync(0xffffffffu, s, 31) >= lim) break;
-    }
-    __syncwarp();
-    int carry = 0;
-#pragma unroll
-    for (int j = 0; j < CHUNK_E / 32; ++j) {
-        int x = max(rid[32 * j + lane], carry);
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x = max(x, t);
-        }
-        rows[j] = x;
-        carry = __shfl_sync(0xffffffffu, x, 31);
-    }
-    __syncwarp();
-}
-// The row of edge e (e < ptr[n]) by binary search: the largest r with
-// ptr[r] <= e.
-__device__ __forceinline__ int64_t edge_row(const int64_t *__restrict__ ptr, int64_t n,
-                                            int64_t e) {
-    int64_t lo = 0, hi = n;
-    while (hi - lo > 1) {
+// How many of the sorted keys[0 .. count) are below v.
+__device__ __forceinline__ int64_t lower_bound_u32(const uint32_t *__restrict__ keys, int64_t count,
+                                                   uint64_t v) {
+    int64_t lo = 0, hi = count;
+    while (lo < hi) {
         const int64_t mid = (lo + hi) >> 1;
-        if (ptr[mid] <= e) lo = mid;
+        if ((uint64_t)keys[mid] < v) lo = mid + 1;
         else hi = mid;
     }
     return lo;
 }
+// keys[p] = map ? map[ids[p]] : ids[p], vals[p] = p, p < pairs.
+cudaError_t launch_pair_keys(const int32_t *ids, const int32_t *map, int64_t pairs, uint32_t *keys,
+                             uint32_t *vals, cudaStream_t st);
 // The store keeps chunks in HBM in page order: row r holds chunk ext_of[r],
 // chunk c lives in row row_of[c].  The out-edge CSR stays in chunk IDs; the
 // in-edge transpose used by propagation is in rows.
@@ -378,7 +337,7 @@ struct InEdgeUpdate {
     int64_t nnz_new;                    // edges after the update
     const int64_t *in_ptr_old;          // [n+1]
     const int32_t *in_src_old;
-    const float *in_aff_old;
+    const float *in_aff_old, *in_w_old;
     int64_t *in_ptr_new;                // [n+1]
     int32_t *in_src_new;                // [nnz_new]
     float *in_aff_new, *in_w_new;       // [nnz_new]
@@ -391,16 +350,35 @@ struct InEdgeUpdate {
     int row_bits;                       // key bits of a row index
     const int32_t *row_of, *ext_of;
     const float2 *rstat;                // per chunk ID: (max, inv) of its out-row
+    const uint32_t *touched;            // bits of the rows whose out-edges changed
 };
-// The update writes in_w_new for every edge as it places it (old edges
-// moved, new edges placed): row_softmax_weight(aff, rstat[ext_of[src]]).
+// The update writes in_w_new for every edge as it places it: the old weight, or
+// row_softmax_weight(aff, rstat[ext_of[src]]) for new edges and touched sources.
 struct InEdgeScratch {
-    int64_t *inc, *deg, *fwd_off;       // [n+1] each
     uint32_t *keys, *vals, *keys2, *vals2;   // [n_new * M] each
+    uint32_t *rows;                     // [4 * n_new]
+    uint32_t *move;                     // [move_words(old edges, n_new * M, n_new)]
     void *tmp;
-    size_t tmp_bytes;                   // >= radix and scan needs
-    float2 *rstat_row;                  // [n]: rstat[ext_of[r]], the statistics by row
+    size_t tmp_bytes;                   // >= radix needs
 };
+// An edge list moved to make room (ak_inedges.cu): `pairs` edges are inserted, one
+// at the end of each row sorted[p] (ascending), and blocks of mult2 edges in the
+// empty rows rows2[] (ascending); ptr: the old row starts.
+struct MoveEdges {
+    int64_t nnz;                        // old edges
+    const int32_t *tgt;
+    const float *val, *w;               // logits, weights
+    int32_t *tgt_out;
+    float *val_out, *w_out;
+    int64_t mult2;
+    const uint32_t *touched;            // or NULL: bit of an edge's tgt set: its weight is
+    const int32_t *ext_of;              // row_softmax_weight(val, rstat[ext_of[tgt]])
+    const float2 *rstat;
+};
+int64_t move_words(int64_t nnz, int64_t pairs, int64_t n_rows2);
+cudaError_t launch_move_edges(const MoveEdges &m, const int64_t *ptr, const uint32_t *sorted,
+                              int64_t pairs, const uint32_t *rows2, int64_t n_rows2,
+                              uint32_t *words, cudaStream_t st, int *launches);
 cudaError_t launch_in_edges_update(const InEdgeUpdate &u, const InEdgeScratch &s, cudaStream_t st,
                                    int *launches);
 cudaError_t launch_batch_layout(const uint32_t *order, int64_t first, int64_t n, int dim,

@@ -382,6 +382,35 @@ __global__ __launch_bounds__(RS_THREADS) void k_rs_scatter_small(
     }
 }
 
+// At most RS_ONE pairs: every thread counts the keys before its own (smaller
+// ones, and equal ones at an earlier place) and writes its pair there, in one
+// launch spread over n / 128 CTAs.  A radix sort's launches cost ~4 us each
+// whatever their size: 1280 pairs of 18 bits 19 -> 11 us (19 with a bitonic
+// network in one CTA).
+constexpr int64_t RS_ONE = 2048;
+__global__ __launch_bounds__(128) void k_sort_one(const uint32_t *__restrict__ keys,
+                                                  const uint32_t *__restrict__ vals, int n,
+                                                  uint32_t mask, uint32_t *__restrict__ okeys,
+                                                  uint32_t *__restrict__ ovals) {
+    __shared__ uint4 x4[RS_ONE / 4];
+    uint32_t *x = reinterpret_cast<uint32_t *>(x4);
+    for (int i = threadIdx.x; i < ((n + 3) & ~3); i += 128) x[i] = i < n ? keys[i] & mask : ~0u;
+    __syncthreads();
+    const int i = blockIdx.x * 128 + threadIdx.x;
+    if (i >= n) return;
+    const uint32_t mine = x[i];
+    int rank = 0;
+    for (int j = 0; j < n; j += 4) {
+        const uint4 k = x4[j >> 2];
+        rank += k.x < mine || (k.x == mine && j < i) ? 1 : 0;
+        rank += k.y < mine || (k.y == mine && j + 1 < i) ? 1 : 0;
+        rank += k.z < mine || (k.z == mine && j + 2 < i) ? 1 : 0;
+        rank += k.w < mine || (k.w == mine && j + 3 < i) ? 1 : 0;
+    }
+    okeys[rank] = keys[i];
+    ovals[rank] = vals[i];
+}
+
 size_t radix_tmp_bytes(int64_t n) {
     int64_t n_tiles = ceil_div<int64_t>(n, RS_TILE);
     int64_t m = 256 * n_tiles;
@@ -398,6 +427,13 @@ cudaError_t radix_sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt,
     *result_in_alt = false;
     if (n <= 1 || bits <= 0) return cudaSuccess;
     if (tmp_bytes < radix_tmp_bytes(n)) return cudaErrorInvalidValue;
+    if (n <= RS_ONE) {
+        k_sort_one<<<(unsigned)ceil_div<int64_t>(n, 128), 128, 0, st>>>(
+            keys, vals, (int)n, bits >= 32 ? 0xffffffffu : (1u << bits) - 1u, keys_alt, vals_alt);
+        if (launches) *launches += 1;
+        *result_in_alt = true;
+        return cudaGetLastError();
+    }
     const int64_t n_tiles = ceil_div<int64_t>(n, RS_TILE);
     const int64_t m = 256 * n_tiles;
     int64_t *hist = (int64_t *)tmp;

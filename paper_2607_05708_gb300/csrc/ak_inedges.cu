@@ -1,8 +1,8 @@
 // Incremental update of the in-edge transpose after a relation update
 // (a7, §4.1 cross-chunk relations): instead of re-sorting every edge of the
 // store, the old in-edge lists are moved to their new offsets and only the
-// new edges are placed, then every in-edge weight is recomputed from its
-// logit and its source row's softmax statistics.
+// new edges are placed; the in-edges of sources whose rows gained edges get
+// their weights anew from their logits and those rows' softmax statistics.
 //
 // Layout facts this relies on (all enforced by the update's preconditions):
 //   * the new chunks' rows come after every old row (appends grow the store
@@ -12,132 +12,166 @@
 //     each other, so a new chunk's in-edges are exactly its M reciprocal
 //     edges;
 //   * the out-edge weights are w = exp(aff - max_row) * inv_row with the
-//     per-row (max, inv) kept in `rstat`, so recomputing them here gives the
-//     same bits as the row softmax.
+//     per-row (max, inv) kept in `rstat`, so a weight recomputed here for a
+//     source whose row gained edges has the same bits as the out-edge's, and
+//     the other edges keep theirs.
 #include "ak_common.cuh"
 
 namespace ak {
 
-// inc[row of t] += 1 for every forward pair (new chunk -> old chunk t).
-__global__ void k_inc_fwd(const int32_t *__restrict__ nbr_ids, int64_t pairs,
-                          const int32_t *__restrict__ row_of, unsigned long long *__restrict__ inc) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < pairs;
-         p += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&inc[row_of[nbr_ids[p]]], 1ull);
-}
-
-// deg[r] = old in-degree + forward additions; new rows get M (reciprocal).
-__global__ void k_in_deg_new(const int64_t *__restrict__ in_ptr_old, int64_t n,
-                             const int64_t *__restrict__ inc, int64_t *__restrict__ deg) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n;
+// New list starts: the old ones moved by the forward pairs into the rows
+// before (counted in the sorted target rows) and by the new rows before (M
+// reciprocal edges each, counted in the sorted new rows).
+__global__ void k_new_in_ptr(const int64_t *__restrict__ in_ptr_old, int64_t n,
+                             const uint32_t *__restrict__ fwd, int64_t pairs,
+                             const uint32_t *__restrict__ new_rows, int64_t n_new, int M,
+                             int64_t *__restrict__ in_ptr_new) {
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r <= n;
          r += (int64_t)gridDim.x * blockDim.x)
-        deg[r] = (in_ptr_old[r + 1] - in_ptr_old[r]) + inc[r];
+        in_ptr_new[r] = in_ptr_old[r] + lower_bound_u32(fwd, pairs, (uint64_t)r) +
+                        (int64_t)M * lower_bound_u32(new_rows, n_new, (uint64_t)r);
 }
 
-__global__ void k_in_deg_recip(const int32_t *__restrict__ row_of, int64_t first, int64_t n_new,
-                               int M, int64_t *__restrict__ deg) {
+__global__ void k_row_keys(const int32_t *__restrict__ row_of, int64_t first, int64_t n_new,
+                           uint32_t *__restrict__ keys, uint32_t *__restrict__ vals) {
     for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < n_new;
-         a += (int64_t)gridDim.x * blockDim.x)
-        deg[row_of[first + a]] += M;
-}
-
-// Old lists to their new offsets, in order, each edge's weight recomputed
-// from its logit and its source's row statistics on the way (a moved edge
-// whose source row did not change gets its old weight back bit for bit).
-// Edge-parallel (a row-parallel copy would leave one warp copying a hub's
-// ~10^5..10^6 edges): chunks of CHUNK_E edges are dealt
-// round-robin to the warps; a warp finds the rows of a chunk at once
-// (chunk_rows), then issues all of a lane's loads for the chunk before any
-// store.
-__global__ __launch_bounds__(256) void k_copy_in_edges(
-    const int64_t *__restrict__ in_ptr_old, const int32_t *__restrict__ src_old,
-    const float *__restrict__ aff_old, int64_t n, int64_t nnz_old,
-    const int64_t *__restrict__ in_ptr_new, int32_t *__restrict__ src_new,
-    float *__restrict__ aff_new, const float2 *__restrict__ rstat_row,
-    float *__restrict__ w_new) {
-    __shared__ int rid_s[8][CHUNK_E];
-    constexpr int PER = CHUNK_E / 32;
-    const int lane = threadIdx.x & 31;
-    int *rid = rid_s[threadIdx.x >> 5];
-    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t n_chunks = (nnz_old + CHUNK_E - 1) / CHUNK_E;
-    // chunks dealt round-robin to the warps; the lanes find the first rows
-    // of a warp's next 32 chunks at once, one binary search each
-    int64_t first = 0;
-    int i = 0;
-    for (int64_t c = w0; c < n_chunks; c += nw, ++i) {
-        if ((i & 31) == 0) {
-            const int64_t cl = c + (int64_t)lane * nw;
-            first = cl < n_chunks ? edge_row(in_ptr_old, n, cl * CHUNK_E) : 0;
-        }
-        const int64_t base = c * CHUNK_E;
-        const int64_t r_lo = __shfl_sync(0xffffffffu, first, i & 31);
-        {
-            int rows[PER];
-            chunk_rows(in_ptr_old, n, nnz_old, base, r_lo, rid, rows);
-            int32_t src[PER];
-            float a[PER];
-            int64_t pos[PER];
-#pragma unroll
-            for (int j = 0; j < PER; ++j) {
-                const int64_t e = base + 32 * j + lane;
-                const int64_t row = r_lo + rows[j];
-                const bool ok = e < nnz_old;
-                src[j] = ok ? src_old[e] : 0;
-                a[j] = ok ? aff_old[e] : 0.f;
-                pos[j] = ok ? e + (in_ptr_new[row] - in_ptr_old[row]) : -1;
-            }
-            float2 st[PER];
-#pragma unroll
-            for (int j = 0; j < PER; ++j) st[j] = pos[j] >= 0 ? rstat_row[src[j]] : make_float2(0.f, 0.f);
-#pragma unroll
-            for (int j = 0; j < PER; ++j) {
-                if (pos[j] < 0) continue;
-                src_new[pos[j]] = src[j];
-                aff_new[pos[j]] = a[j];
-                w_new[pos[j]] = row_softmax_weight(a[j], st[j]);
-            }
-            __syncwarp();
-        }
+         a += (int64_t)gridDim.x * blockDim.x) {
+        keys[a] = (uint32_t)row_of[first + a];
+        vals[a] = (uint32_t)a;
     }
 }
 
-// The row statistics by row: rstat_row[r] = rstat[ext_of[r]] (one gather
-// per moved in-edge instead of two).
-__global__ void k_rstat_rows(const int32_t *__restrict__ ext_of, const float2 *__restrict__ rstat,
-                             int64_t n, float2 *__restrict__ rstat_row) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n;
-         r += (int64_t)gridDim.x * blockDim.x)
-        rstat_row[r] = rstat[ext_of[r]];
-}
+// ------------------------------------------------------------------ moved edges
+// Old edges to their new places, each with its logit and weight.  An edge moves
+// by the edges inserted before its row, so its shift only changes where a row
+// that gained edges ends: cut[] holds those ends (one entry an inserted edge,
+// ascending), cut2[] the starts of rows whose insertions come in equal blocks of
+// mult2 edges (the new rows, which had none).  A CTA takes MOVE_TILE consecutive
+// edges; 32 with no cut among them, as most, move together, else an edge
+// searches the few cuts there.  Bound by memory, 24 bytes an edge
+// (finding every edge's row instead: 60 us for 8.4M edges, 29 so; 16 edges a
+// thread 38, as the registers then cost a CTA an SM).
+// Weights are kept, or recomputed where touched has the bit of the edge's tgt.
+constexpr int MOVE_PER = 8, MOVE_TILE = 256 * MOVE_PER;
 
-// keys[p] = row of the new chunk of pair p (pairs are [new chunk][slot]).
-__global__ void k_pair_src_rows(const int32_t *__restrict__ row_of, int64_t first, int M,
-                                int64_t pairs, uint32_t *__restrict__ keys) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < pairs;
+// cut[p] = ptr[sorted[p] + end], p < count
+__global__ void k_move_cuts(const int64_t *__restrict__ ptr, const uint32_t *__restrict__ sorted,
+                            int64_t count, int end, uint32_t *__restrict__ cut) {
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < count;
          p += (int64_t)gridDim.x * blockDim.x)
-        keys[p] = (uint32_t)row_of[first + p / M];
+        cut[p] = (uint32_t)ptr[sorted[p] + end];
 }
 
-// Forward edges c -> t, pairs sorted by (row of t, row of c): the i-th
-// sorted pair is the (i - fwd_off[row t])-th new source of row t, after the
-// row's old list.
-__global__ void k_place_fwd(const uint32_t *__restrict__ order, int64_t pairs,
-                            const int32_t *__restrict__ nbr_ids, const float *__restrict__ nbr_cos,
-                            float scale, int64_t first, int M, const int32_t *__restrict__ row_of,
+// tile_cut[t] / tile_cut2[t]: the cuts before edge t * MOVE_TILE.
+__global__ void k_move_tiles(const uint32_t *__restrict__ cut, int64_t n_cut,
+                             const uint32_t *__restrict__ cut2, int64_t n_cut2, int64_t tiles,
+                             int32_t *__restrict__ tile_cut, int32_t *__restrict__ tile_cut2) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t > tiles) return;
+    tile_cut[t] = (int32_t)lower_bound_u32(cut, n_cut, (uint64_t)t * MOVE_TILE);
+    tile_cut2[t] = (int32_t)lower_bound_u32(cut2, n_cut2, (uint64_t)t * MOVE_TILE);
+}
+
+__global__ __launch_bounds__(256, 4) void k_move_edges(const MoveEdges m,
+                                                       const uint32_t *__restrict__ cut,
+                                                       const uint32_t *__restrict__ cut2,
+                                                       const int32_t *__restrict__ tile_cut,
+                                                       const int32_t *__restrict__ tile_cut2) {
+    const int64_t tile = blockIdx.x, e0 = tile * MOVE_TILE + threadIdx.x;
+    int32_t t[MOVE_PER];
+    float v[MOVE_PER], w[MOVE_PER];
+#pragma unroll
+    for (int j = 0; j < MOVE_PER; ++j) {
+        const int64_t e = e0 + 256 * j;
+        const bool ok = e < m.nnz;
+        t[j] = ok ? __ldcs(m.tgt + e) : 0;
+        v[j] = ok ? __ldcs(m.val + e) : 0.f;
+        w[j] = ok ? __ldcs(m.w + e) : 0.f;
+    }
+    const int32_t c0 = tile_cut[tile], c1 = tile_cut[tile + 1];
+    const int32_t d0 = tile_cut2[tile], d1 = tile_cut2[tile + 1];
+    // lane j: the cuts at or before the first and the last edge of the warp's j-th
+    // 32 edges
+    const int lane = threadIdx.x & 31;
+    const int64_t w0 = e0 - lane + 256 * (lane & (MOVE_PER - 1));
+    auto upto = [&](const uint32_t *c, int32_t lo, int32_t hi, int64_t e) {
+        return hi > lo ? lo + (int32_t)lower_bound_u32(c + lo, hi - lo, (uint64_t)e + 1) : lo;
+    };
+    const int32_t fa = upto(cut, c0, c1, w0), fb = upto(cut, c0, c1, w0 + 31);
+    const int32_t ga = upto(cut2, d0, d1, w0), gb = upto(cut2, d0, d1, w0 + 31);
+    // touched sources' statistics, all gathers in flight together
+    if (m.touched) {
+        uint32_t hit = 0u;
+#pragma unroll
+        for (int j = 0; j < MOVE_PER; ++j)
+            hit |= ((__ldg(m.touched + (t[j] >> 5)) >> (t[j] & 31)) & 1u) << j;
+        if (__any_sync(0xffffffffu, hit != 0u)) {
+            int32_t id[MOVE_PER];
+#pragma unroll
+            for (int j = 0; j < MOVE_PER; ++j) id[j] = (hit >> j) & 1u ? m.ext_of[t[j]] : -1;
+#pragma unroll
+            for (int j = 0; j < MOVE_PER; ++j)
+                if (id[j] >= 0) w[j] = row_softmax_weight(v[j], m.rstat[id[j]]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < MOVE_PER; ++j) {
+        const int64_t e = e0 + 256 * j;
+        const int32_t ca = __shfl_sync(0xffffffffu, fa, j), cb = __shfl_sync(0xffffffffu, fb, j);
+        const int32_t da = __shfl_sync(0xffffffffu, ga, j), db = __shfl_sync(0xffffffffu, gb, j);
+        if (e >= m.nnz) continue;
+        const int64_t by = cb > ca ? upto(cut, ca, cb, e) : ca;
+        const int64_t by2 = db > da ? upto(cut2, da, db, e) : da;
+        const int64_t p = e + by + by2 * m.mult2;
+        __stcs(m.tgt_out + p, t[j]);
+        __stcs(m.val_out + p, v[j]);
+        __stcs(m.w_out + p, w[j]);
+    }
+}
+
+int64_t move_words(int64_t nnz, int64_t pairs, int64_t rows2) {
+    return pairs + rows2 + 2 * (ceil_div<int64_t>(nnz, MOVE_TILE) + 1);
+}
+
+cudaError_t launch_move_edges(const MoveEdges &m, const int64_t *ptr, const uint32_t *sorted,
+                              int64_t pairs, const uint32_t *rows2, int64_t n_rows2,
+                              uint32_t *words, cudaStream_t st, int *launches) {
+    if (m.nnz <= 0) return cudaSuccess;
+    const int64_t tiles = ceil_div<int64_t>(m.nnz, MOVE_TILE), cap = (int64_t)device_sm_count() * 4;
+    uint32_t *cut = words, *cut2 = cut + pairs;
+    int32_t *tc = (int32_t *)(cut2 + n_rows2), *tc2 = tc + tiles + 1;
+    auto grid = [&](int64_t n) {
+        const int64_t want = ceil_div<int64_t>(n, 256);
+        return (unsigned)(want < cap ? want : cap);
+    };
+    if (pairs > 0) k_move_cuts<<<grid(pairs), 256, 0, st>>>(ptr, sorted, pairs, 1, cut);
+    if (n_rows2 > 0) k_move_cuts<<<grid(n_rows2), 256, 0, st>>>(ptr, rows2, n_rows2, 0, cut2);
+    k_move_tiles<<<(unsigned)ceil_div<int64_t>(tiles + 1, 256), 256, 0, st>>>(cut, pairs, cut2,
+                                                                             n_rows2, tiles, tc, tc2);
+    k_move_edges<<<(unsigned)tiles, 256, 0, st>>>(m, cut, cut2, tc, tc2);
+    if (launches) *launches += 2 + (pairs > 0) + (n_rows2 > 0);
+    return cudaGetLastError();
+}
+
+// Forward edges c -> t, pairs sorted by the row of t (fwd): after the row's old
+// list, by source row (rank by counting among the row's new sources).
+__global__ void k_place_fwd(const uint32_t *__restrict__ fwd, const uint32_t *__restrict__ order,
+                            int64_t pairs, const float *__restrict__ nbr_cos, float scale,
+                            int64_t first, int M, const int32_t *__restrict__ row_of,
                             const int64_t *__restrict__ in_ptr_old,
-                            const int64_t *__restrict__ in_ptr_new,
-                            const int64_t *__restrict__ fwd_off, int32_t *__restrict__ src_new,
+                            const int64_t *__restrict__ in_ptr_new, int32_t *__restrict__ src_new,
                             float *__restrict__ aff_new, const float2 *__restrict__ rstat,
                             float *__restrict__ w_new) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pairs;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t p = order[i];
-        const int64_t rt = row_of[nbr_ids[p]];
-        const int64_t pos = in_ptr_new[rt] + (in_ptr_old[rt + 1] - in_ptr_old[rt]) + (i - fwd_off[rt]);
+        const uint32_t p = order[i], rt = fwd[i];
+        const int32_t rs = row_of[first + p / M];
+        int64_t rank = 0;
+        for (int64_t q = lower_bound_u32(fwd, i, rt); q < pairs && fwd[q] == rt; ++q)
+            rank += row_of[first + order[q] / M] < rs ? 1 : 0;
+        const int64_t pos = in_ptr_new[rt] + (in_ptr_old[rt + 1] - in_ptr_old[rt]) + rank;
         const float a = scale * nbr_cos[p];
-        src_new[pos] = row_of[first + p / M];
+        src_new[pos] = rs;
         aff_new[pos] = a;
         w_new[pos] = row_softmax_weight(a, rstat[first + p / M]);   // source: chunk first + p / M
     }
@@ -173,65 +207,42 @@ cudaError_t launch_in_edges_update(const InEdgeUpdate &u, const InEdgeScratch &s
                                    int *launches) {
     const int sms = device_sm_count();
     const int64_t pairs = u.n_new * u.M;
-    int L = 0;
-    cudaError_t e = cudaMemsetAsync(s.inc, 0, (size_t)(u.n + 1) * 8, st);
-    if (e != cudaSuccess) return e;
-    if (pairs > 0) {
-        k_inc_fwd<<<sms * 4, 256, 0, st>>>(u.nbr_ids, pairs, u.row_of, (unsigned long long *)s.inc);
+    if (pairs <= 0) return cudaErrorInvalidValue;
+    int L = 3;
+    // forward pairs by target row; the new rows, which get M edges each
+    bool alt = false, alt_r = false;
+    cudaError_t e = launch_pair_keys(u.nbr_ids, u.row_of, pairs, s.keys, s.vals, st);
+    if (e == cudaSuccess)
+        e = radix_sort_pairs(s.keys, s.vals, s.keys2, s.vals2, pairs, u.row_bits, s.tmp,
+                             s.tmp_bytes, st, &alt, &L);
+    const int64_t recip_rows = u.reciprocal ? u.n_new : 0;
+    uint32_t *rk = s.rows, *rv = rk + u.n_new, *rk2 = rv + u.n_new, *rv2 = rk2 + u.n_new;
+    if (e == cudaSuccess && recip_rows > 0) {
+        const int64_t want = ceil_div<int64_t>(u.n_new, 256);
+        k_row_keys<<<(unsigned)(want < sms ? want : sms), 256, 0, st>>>(u.row_of, u.first, u.n_new,
+                                                                        rk, rv);
+        e = radix_sort_pairs(rk, rv, rk2, rv2, u.n_new, u.row_bits, s.tmp, s.tmp_bytes, st, &alt_r,
+                             &L);
         ++L;
     }
-    k_in_deg_new<<<sms * 4, 256, 0, st>>>(u.in_ptr_old, u.n, s.inc, s.deg);
-    ++L;
-    if (u.reciprocal && u.n_new > 0) {
-        k_in_deg_recip<<<sms, 256, 0, st>>>(u.row_of, u.first, u.n_new, u.M, s.deg);
-        ++L;
-    }
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = scan_exclusive(s.deg, u.in_ptr_new, u.n, s.tmp, s.tmp_bytes, st);
-    if (e == cudaSuccess) e = scan_exclusive(s.inc, s.fwd_off, u.n, s.tmp, s.tmp_bytes, st);
     if (e != cudaSuccess) return e;
+    const uint32_t *fwd = alt ? s.keys2 : s.keys, *order = alt ? s.vals2 : s.vals;
+    k_new_in_ptr<<<sms * 8, 256, 0, st>>>(u.in_ptr_old, u.n, fwd, pairs, alt_r ? rk2 : rk,
+                                          recip_rows, u.M, u.in_ptr_new);
     const int64_t nnz_old = u.nnz_new - pairs * (u.reciprocal ? 2 : 1);
-    if (nnz_old > 0) {
-        k_rstat_rows<<<sms * 4, 256, 0, st>>>(u.ext_of, u.rstat, u.n, s.rstat_row);
-        const int64_t warps = ceil_div<int64_t>(nnz_old, CHUNK_E);
-        const int64_t grid = ceil_div<int64_t>(warps, 8);
-        k_copy_in_edges<<<(unsigned)(grid < (int64_t)sms * 6 ? grid : (int64_t)sms * 6), 256, 0,
-                          st>>>(u.in_ptr_old, u.in_src_old, u.in_aff_old, u.n, nnz_old,
-                                u.in_ptr_new, u.in_src_new, u.in_aff_new, s.rstat_row,
-                                u.in_w_new);
-        L += 2;
-    }
-    if (pairs > 0) {
-        // forward pairs by (target row, source row): sort by source row,
-        // then stably by target row
-        k_pair_src_rows<<<sms * 2, 256, 0, st>>>(u.row_of, u.first, u.M, pairs, s.keys);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = launch_iota(s.vals, pairs, st);
-        bool alt = false;
-        if (e == cudaSuccess)
-            e = radix_sort_pairs(s.keys, s.vals, s.keys2, s.vals2, pairs, u.row_bits, s.tmp,
-                                 s.tmp_bytes, st, &alt);
-        if (e != cudaSuccess) return e;
-        uint32_t *k1 = alt ? s.keys2 : s.keys, *v1 = alt ? s.vals2 : s.vals;
-        uint32_t *k2 = alt ? s.keys : s.keys2, *v2 = alt ? s.vals : s.vals2;
-        e = launch_map_keys(v1, u.nbr_ids, u.row_of, k1, pairs, st);
-        bool alt2 = false;
-        if (e == cudaSuccess)
-            e = radix_sort_pairs(k1, v1, k2, v2, pairs, u.row_bits, s.tmp, s.tmp_bytes, st, &alt2);
-        if (e != cudaSuccess) return e;
-        k_place_fwd<<<sms * 2, 256, 0, st>>>(alt2 ? v2 : v1, pairs, u.nbr_ids, u.nbr_cos, u.scale,
-                                             u.first, u.M, u.row_of, u.in_ptr_old, u.in_ptr_new,
-                                             s.fwd_off, u.in_src_new, u.in_aff_new, u.rstat,
-                                             u.in_w_new);
+    MoveEdges mv{nnz_old, u.in_src_old, u.in_aff_old, u.in_w_old, u.in_src_new, u.in_aff_new,
+                 u.in_w_new, u.M, u.touched, u.ext_of, u.rstat};
+    e = launch_move_edges(mv, u.in_ptr_old, fwd, pairs, alt_r ? rk2 : rk, recip_rows, s.move, st,
+                          &L);
+    if (e != cudaSuccess) return e;
+    k_place_fwd<<<sms * 2, 256, 0, st>>>(fwd, order, pairs, u.nbr_cos, u.scale, u.first, u.M,
+                                         u.row_of, u.in_ptr_old, u.in_ptr_new, u.in_src_new,
+                                         u.in_aff_new, u.rstat, u.in_w_new);
+    if (u.reciprocal) {
+        k_place_recip<<<sms * 2, 256, 0, st>>>(u.nbr_ids, u.nbr_cos, u.scale, u.first, u.n_new,
+                                               u.M, u.row_of, u.in_ptr_new, u.in_src_new,
+                                               u.in_aff_new, u.rstat, u.in_w_new);
         ++L;
-        if (u.reciprocal) {
-            k_place_recip<<<sms * 2, 256, 0, st>>>(u.nbr_ids, u.nbr_cos, u.scale, u.first, u.n_new,
-                                                   u.M, u.row_of, u.in_ptr_new, u.in_src_new,
-                                                   u.in_aff_new, u.rstat, u.in_w_new);
-            ++L;
-        }
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
     }
     if (launches) *launches += L;
     return cudaGetLastError();

@@ -501,18 +501,6 @@ __global__ void k_mm_release(MmTables t, int64_t n_pages, const int32_t *__restr
         }
 }
 
-// first index of the sorted keys[0, count) holding a key >= v
-__device__ __forceinline__ int64_t lower_bound_u32(const uint32_t *__restrict__ keys, int64_t count,
-                                                   uint32_t v) {
-    int64_t lo = 0, hi = count;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (keys[mid] < v) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
 // Every namespace (partition) starts on a fresh page: at the first
 // position of each run of equal namespace keys, the pages that run fills
 // (ceil(run / P)); zero elsewhere.  An exclusive scan of these gives each
@@ -524,7 +512,7 @@ __global__ void k_mm_part_pages(const uint32_t *__restrict__ ns_sorted, int64_t 
         const uint32_t k = ns_sorted[i];
         int64_t v = 0;
         if (i == 0 || ns_sorted[i - 1] != k) {
-            const int64_t end = k == 0xffffffffu ? count : lower_bound_u32(ns_sorted, count, k + 1);
+            const int64_t end = lower_bound_u32(ns_sorted, count, (uint64_t)k + 1);
             v = (end - i + per_page - 1) / per_page;
         }
         part_pages[i] = v;

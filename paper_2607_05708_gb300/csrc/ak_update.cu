@@ -75,7 +75,8 @@ static akashic_status_t relate_top_m_batched(const UpdateArgs &a, cudaStream_t s
 // store, then ONE tensor-core pass over all rows x all new chunks whose
 // epilogue keeps only the keys above the bounds, then an exact selection
 // of the M best among them.  The dots are never written to memory.
-akashic_status_t relate_top_m(const UpdateArgs &a, cudaStream_t st, int *launches) {
+akashic_status_t relate_top_m(const UpdateArgs &a, cudaStream_t st, int *launches,
+                              int *dev_status) {
     // every row of the store is scored; rows holding chunks >= first are
     // masked in the selection (rows are in page order, not ID order)
     const int64_t n = a.n_rows;
@@ -141,7 +142,11 @@ akashic_status_t relate_top_m(const UpdateArgs &a, cudaStream_t st, int *launche
         if (rc == AKASHIC_OK && e == cudaSuccess)
             e = launch_dots_filter(a.emb, n, a.dim, qp, n_ct, a.n_new, a.ext_of, a.first, bound,
                                    cnt, buf, cap, a.status, st, launches, a.dead_row);
-        // buffers that overflowed fall back to the exact batched path
+        // the merge is queued before the host knows whether a buffer
+        // overflowed (then the exact batched path starts over)
+        if (rc == AKASHIC_OK && e == cudaSuccess)
+            e = launch_buf_merge_signed(cnt, buf, cap, a.n_new, a.M, a.nbr_ids, a.nbr_cos,
+                                        a.status, st, launches);
         unsigned int max_cnt = 0;
         if (rc == AKASHIC_OK && e == cudaSuccess) {
             unsigned int *h = (unsigned int *)malloc((size_t)a.n_new * 4);
@@ -149,99 +154,83 @@ akashic_status_t relate_top_m(const UpdateArgs &a, cudaStream_t st, int *launche
                 rc = AKASHIC_ENOMEM;
             } else {
                 e = cudaMemcpyAsync(h, cnt, (size_t)a.n_new * 4, cudaMemcpyDeviceToHost, st);
+                if (e == cudaSuccess)
+                    e = cudaMemcpyAsync(dev_status, a.status, 4, cudaMemcpyDeviceToHost, st);
                 if (e == cudaSuccess) e = cudaStreamSynchronize(st);
                 for (int64_t c = 0; e == cudaSuccess && c < a.n_new; ++c)
                     max_cnt = h[c] > max_cnt ? h[c] : max_cnt;
                 free(h);
             }
         }
-        overflow = (int64_t)max_cnt > cap;
-        if (e == cudaSuccess && rc == AKASHIC_OK && !overflow)
-            e = launch_buf_merge_signed(cnt, buf, cap, a.n_new, a.M, a.nbr_ids, a.nbr_cos,
-                                        a.status, st, launches);
-        if (e == cudaSuccess && rc == AKASHIC_OK) e = cudaStreamSynchronize(st);
+        overflow = (int64_t)max_cnt > cap && *dev_status == 0;
         if (e != cudaSuccess && rc == AKASHIC_OK) rc = AKASHIC_ECUDA;
     }
-    if (rc == AKASHIC_OK && overflow) rc = relate_top_m_batched(a, st, launches);
+    if (rc == AKASHIC_OK && overflow) {
+        rc = relate_top_m_batched(a, st, launches);
+        if (rc == AKASHIC_OK && cudaMemcpy(dev_status, a.status, 4, cudaMemcpyDeviceToHost) !=
+                                    cudaSuccess)
+            rc = AKASHIC_ECUDA;
+    }
     return rc;
 }
 
 // ------------------------------------------------------------------ CSR insert
-// new degree of every row: old degree, + M for new rows, + reciprocal count
-__global__ void k_new_degree(const int64_t *__restrict__ rp, int64_t n_rows, int64_t first,
-                             int64_t n_new, int M, const int64_t *__restrict__ recip,
-                             int64_t *__restrict__ deg) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_rows;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t d = rp[i + 1] - rp[i];
-        if (i >= first && i < first + n_new) d += M;
-        if (recip) d += recip[i];
-        deg[i] = d;
+// The update's preconditions, by a thread a new chunk: EINVAL if the range's
+// rows have out-edges, EDEVICE if an edge points at one of its chunks (its
+// reciprocal edge would be a repeat).
+__global__ void k_check_new_rows(const int64_t *__restrict__ rp, const int64_t *__restrict__ in_ptr,
+                                 const int32_t *__restrict__ row_of, int64_t first, int64_t n_new,
+                                 int *status) {
+    if (rp[first] != rp[first + n_new]) {
+        set_status(status, AKASHIC_EINVAL);
+        return;
+    }
+    for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < n_new;
+         a += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t r = row_of[first + a];
+        if (in_ptr[r + 1] != in_ptr[r]) set_status(status, AKASHIC_EDEVICE);
     }
 }
 
-__global__ void k_count_recip(const int32_t *__restrict__ nbr, int64_t pairs,
-                              unsigned long long *__restrict__ recip) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < pairs;
-         p += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&recip[nbr[p]], 1ull);
+cudaError_t launch_check_new_rows(const int64_t *rp, const int64_t *in_ptr, const int32_t *row_of,
+                                  int64_t first, int64_t n_new, int *status, cudaStream_t st) {
+    const int64_t want = ceil_div<int64_t>(n_new, 256), cap = device_sm_count();
+    k_check_new_rows<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(rp, in_ptr, row_of, first,
+                                                                         n_new, status);
+    return cudaGetLastError();
 }
 
-// Old edges keep their order at the front of each row.  Edge-parallel:
-// chunks of CHUNK_E old edges are dealt round-robin to the warps; a warp
-// finds the rows of a chunk at once (chunk_rows), then issues all of a
-// lane's loads for the chunk before any store; edge e of row r goes to
-// nrp[r] + (e - rp[r]).
-__global__ __launch_bounds__(256) void k_copy_old_rows(
-    const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
-    const float *__restrict__ aff, int64_t n_rows, const int64_t *__restrict__ nrp,
-    int32_t *__restrict__ ncol, float *__restrict__ naff, int64_t new_lo, int64_t new_hi,
-    int *status) {
-    __shared__ int rid_s[8][CHUNK_E];
-    constexpr int PER = CHUNK_E / 32;
-    const int lane = threadIdx.x & 31;
-    int *rid = rid_s[threadIdx.x >> 5];
-    const int64_t nnz = rp[n_rows];
-    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t n_chunks = (nnz + CHUNK_E - 1) / CHUNK_E;
-    // chunks dealt round-robin to the warps; the lanes find the first rows
-    // of a warp's next 32 chunks at once, one binary search each
-    int64_t first = 0;
-    int i = 0;
-    for (int64_t c = w0; c < n_chunks; c += nw, ++i) {
-        if ((i & 31) == 0) {
-            const int64_t cl = c + (int64_t)lane * nw;
-            first = cl < n_chunks ? edge_row(rp, n_rows, cl * CHUNK_E) : 0;
-        }
-        const int64_t base = c * CHUNK_E;
-        const int64_t r_lo = __shfl_sync(0xffffffffu, first, i & 31);
-        {
-            int rows[PER];
-            chunk_rows(rp, n_rows, nnz, base, r_lo, rid, rows);
-            int32_t cv[PER];
-            float av[PER];
-            int64_t pos[PER];
-#pragma unroll
-            for (int j = 0; j < PER; ++j) {
-                const int64_t e = base + 32 * j + lane;
-                const int64_t row = r_lo + rows[j];
-                const bool ok = e < nnz;
-                cv[j] = ok ? col[e] : 0;
-                av[j] = ok ? aff[e] : 0.f;
-                pos[j] = ok ? e + (nrp[row] - rp[row]) : -1;
-            }
-#pragma unroll
-            for (int j = 0; j < PER; ++j) {
-                if (pos[j] < 0) continue;
-                // an existing edge into a new chunk would make a reciprocal
-                // edge a repeat
-                if (cv[j] >= new_lo && cv[j] < new_hi) set_status(status, AKASHIC_EDEVICE);
-                ncol[pos[j]] = cv[j];
-                naff[pos[j]] = av[j];
-            }
-            __syncwarp();
-        }
+// keys[p] = map ? map[ids[p]] : ids[p], vals[p] = p.
+__global__ void k_pair_keys(const int32_t *__restrict__ ids, const int32_t *__restrict__ map,
+                            int64_t pairs, uint32_t *__restrict__ keys,
+                            uint32_t *__restrict__ vals) {
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < pairs;
+         p += (int64_t)gridDim.x * blockDim.x) {
+        keys[p] = (uint32_t)(map ? map[ids[p]] : ids[p]);
+        vals[p] = (uint32_t)p;
+    }
+}
+
+cudaError_t launch_pair_keys(const int32_t *ids, const int32_t *map, int64_t pairs, uint32_t *keys,
+                             uint32_t *vals, cudaStream_t st) {
+    if (pairs <= 0) return cudaSuccess;
+    const int64_t want = ceil_div<int64_t>(pairs, 256), cap = (int64_t)device_sm_count() * 4;
+    k_pair_keys<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(ids, map, pairs, keys, vals);
+    return cudaGetLastError();
+}
+
+// New row starts: the old ones moved by the new rows before the row (M edges
+// each) and by the reciprocal edges of the rows before it, counted in the
+// sorted target IDs (a search of cached words a row instead of counting,
+// adding up and scanning arrays of all rows).
+__global__ void k_new_row_ptr(const int64_t *__restrict__ rp, int64_t n_rows, int64_t first,
+                              int64_t n_new, int M, const uint32_t *__restrict__ tgt,
+                              int64_t recips, int64_t *__restrict__ nrp) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= n_rows;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        int64_t before = i - first;
+        before = before < 0 ? 0 : (before > n_new ? n_new : before);
+        nrp[i] = rp[i] + before * M + lower_bound_u32(tgt, recips, (uint64_t)i);
     }
 }
 
@@ -269,88 +258,123 @@ __global__ void k_fill_new_rows(const int32_t *__restrict__ nbr, const float *__
 
 // Reciprocal edges j -> new chunk, appended after row j's old edges in
 // ascending new-chunk order.  `order` lists the (new, slot) pair indices
-// stably sorted by target j, so pairs of one j come in ascending new ID.
+// stably sorted by target j (tgt), so pairs of one j come in ascending new ID.
 __global__ void k_fill_recip(const uint32_t *__restrict__ order, const uint32_t *__restrict__ tgt,
-                             int64_t pairs, const int32_t *__restrict__ nbr,
-                             const float *__restrict__ cosv, int64_t first, int M, float scale,
-                             const int64_t *__restrict__ rp, const int64_t *__restrict__ recip_off,
+                             int64_t pairs, const float *__restrict__ cosv, int64_t first, int M,
+                             float scale, const int64_t *__restrict__ rp,
                              const int64_t *__restrict__ nrp, int32_t *__restrict__ ncol,
                              float *__restrict__ naff) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < pairs;
          p += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t pair = order[p];
         const int64_t j = tgt[p];
-        const int64_t rank = p - recip_off[j];
+        const int64_t rank = p - lower_bound_u32(tgt, p, (uint64_t)j);
         const int64_t pos = nrp[j] + (rp[j + 1] - rp[j]) + rank;
         ncol[pos] = (int32_t)(first + pair / M);
         naff[pos] = scale * cosv[pair];
-        (void)nbr;
+    }
+}
+
+__global__ void k_first_row(int64_t first, uint32_t *__restrict__ out) { *out = (uint32_t)first; }
+
+// The softmax of the rows that gained edges (the new rows, then each target's
+// row, at its first pair), eight lanes a row in k_row_softmax's order, and
+// their rows' bits in touched.
+__global__ __launch_bounds__(256) void k_gained_softmax(const uint32_t *__restrict__ tgt,
+                                                        int64_t recips, int64_t first,
+                                                        int64_t n_new,
+                                                        const int64_t *__restrict__ nrp,
+                                                        const float *__restrict__ naff,
+                                                        const int32_t *__restrict__ row_of,
+                                                        float *__restrict__ nw_,
+                                                        float2 *__restrict__ rstat,
+                                                        uint32_t *__restrict__ touched) {
+    constexpr int L = 8;
+    const int lane = threadIdx.x & 31, sub = lane % L;
+    const int64_t items = n_new + recips;
+    const int64_t step = ((int64_t)gridDim.x * blockDim.x) / L;
+    const int64_t warp0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (32 / L);
+    for (int64_t i0 = warp0; i0 < items; i0 += step) {   // (warp-uniform)
+        const int64_t i = i0 + lane / L;
+        int64_t r = -1;
+        if (i < n_new) {
+            r = first + i;
+        } else if (i < items) {
+            const int64_t p = i - n_new;
+            if (p == 0 || tgt[p - 1] != tgt[p]) r = tgt[p];
+        }
+        const int64_t a = r >= 0 ? nrp[r] : 0, b = r >= 0 ? nrp[r + 1] : 0;
+        float m = -INFINITY;
+        for (int64_t e = a + sub; e < b; e += L) m = fmaxf(m, naff[e]);
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        float s = 0.f;
+        for (int64_t e = a + sub; e < b; e += L) s += expf(naff[e] - m);
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (b > a) {
+            const float2 stat = make_float2(m, 1.f / s);
+            if (sub == 0) {
+                rstat[r] = stat;
+                const uint32_t row = (uint32_t)row_of[r];
+                atomicOr(&touched[row >> 5], 1u << (row & 31));
+            }
+            for (int64_t e = a + sub; e < b; e += L) nw_[e] = row_softmax_weight(naff[e], stat);
+        }
     }
 }
 
 akashic_status_t csr_insert(const UpdateArgs &a, const int64_t *rp, const int32_t *col,
-                            const float *aff, int64_t nnz, int64_t *new_rp, int32_t *new_col,
-                            float *new_aff, cudaStream_t st, int *launches) {
-    const int64_t n_rows = a.n_rows, pairs = a.n_new * a.M;
+                            const float *aff, const float *w, int64_t nnz, int64_t *new_rp,
+                            int32_t *new_col, float *new_aff, float *new_w, float2 *rstat,
+                            uint32_t *touched, cudaStream_t st, int *launches) {
+    const int64_t n_rows = a.n_rows, pairs = a.n_new * a.M, recips = a.reciprocal ? pairs : 0;
     const int sms = device_sm_count();
-    const size_t tmp_bytes = (radix_tmp_bytes(pairs) > scan_tmp_bytes(n_rows + 1)
-                                  ? radix_tmp_bytes(pairs)
-                                  : scan_tmp_bytes(n_rows + 1)) + 4096;
-    int64_t *deg = (int64_t *)a.get(SCR_DEG, (size_t)(n_rows + 1) * 8);
-    int64_t *recip = (int64_t *)a.get(SCR_RECIP, (size_t)(n_rows + 1) * 8);
-    int64_t *recip_off = (int64_t *)a.get(SCR_RECIP_OFF, (size_t)(n_rows + 1) * 8);
+    const size_t tmp_bytes = radix_tmp_bytes(pairs) + 4096;
     uint32_t *keys = (uint32_t *)a.get(SCR_KEYS, (size_t)pairs * 4 + 16);
     uint32_t *vals = (uint32_t *)a.get(SCR_VALS, (size_t)pairs * 4 + 16);
     uint32_t *keys2 = (uint32_t *)a.get(SCR_KEYS2, (size_t)pairs * 4 + 16);
     uint32_t *vals2 = (uint32_t *)a.get(SCR_VALS2, (size_t)pairs * 4 + 16);
     void *tmp = a.get(SCR_TMP, tmp_bytes);
-    akashic_status_t rc = (deg && recip && recip_off && keys && vals && keys2 && vals2 && tmp)
-                              ? AKASHIC_OK : AKASHIC_ENOMEM;
-    cudaError_t e = cudaSuccess;
-    int L = 0;
-    if (rc == AKASHIC_OK) {
-        cudaMemsetAsync(recip, 0, (size_t)(n_rows + 1) * 8, st);
-        if (a.reciprocal)
-            k_count_recip<<<sms * 4, 256, 0, st>>>(a.nbr_ids, pairs, (unsigned long long *)recip);
-        k_new_degree<<<sms * 4, 256, 0, st>>>(rp, n_rows, a.first, a.n_new, a.M,
-                                              a.reciprocal ? recip : nullptr, deg);
-        L += 3;
+    uint32_t *words = (uint32_t *)a.get(SCR_MOVE, (size_t)(1 + move_words(nnz, pairs, a.n_new)) * 4);
+    if (!keys || !vals || !keys2 || !vals2 || !tmp || !words) return AKASHIC_ENOMEM;
+    cudaError_t e = cudaMemsetAsync(touched, 0, (size_t)ceil_div<int64_t>(n_rows, 32) * 4, st);
+    int L = 5;
+    bool alt = false;
+    if (e == cudaSuccess && recips > 0) {
+        int bits = 0;
+        while (bits < 32 && ((int64_t)1 << bits) <= a.first - 1) ++bits;
+        e = launch_pair_keys(a.nbr_ids, nullptr, pairs, keys, vals, st);
+        if (e == cudaSuccess)
+            e = radix_sort_pairs(keys, vals, keys2, vals2, pairs, bits, tmp, tmp_bytes, st, &alt, &L);
+        L += 2;
+    }
+    const uint32_t *tgt = alt ? keys2 : keys, *order = alt ? vals2 : vals;
+    if (e == cudaSuccess) {
+        k_new_row_ptr<<<sms * 8, 256, 0, st>>>(rp, n_rows, a.first, a.n_new, a.M, tgt, recips,
+                                               new_rp);
+        // old edges keep their order at the front of each row, and their weights
+        // (the rows that gain edges get theirs anew below); the new rows' edges
+        // go in as one block before row first's place
+        k_first_row<<<1, 1, 0, st>>>(a.first, words);
+        MoveEdges mv{nnz, col, aff, w, new_col, new_aff, new_w, a.n_new * a.M, nullptr, nullptr,
+                     nullptr};
+        e = launch_move_edges(mv, rp, tgt, recips, words, 1, words + 1, st, &L);
+    }
+    if (e == cudaSuccess) {
+        k_fill_new_rows<<<sms * 2, 256, 0, st>>>(a.nbr_ids, a.nbr_cos, a.first, a.n_new, a.M,
+                                                 a.scale, new_rp, new_col, new_aff);
+        if (recips > 0)
+            k_fill_recip<<<sms * 2, 256, 0, st>>>(order, tgt, pairs, a.nbr_cos, a.first, a.M,
+                                                  a.scale, rp, new_rp, new_col, new_aff);
+        const int64_t want = ceil_div<int64_t>((a.n_new + recips) * 8, 256);
+        const int64_t cap = (int64_t)sms * 16;
+        k_gained_softmax<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(
+            tgt, recips, a.first, a.n_new, new_rp, new_aff, a.row_of, new_w, rstat, touched);
         e = cudaGetLastError();
-        if (e == cudaSuccess) e = scan_exclusive(deg, new_rp, n_rows, tmp, tmp_bytes, st);
-        if (e == cudaSuccess) {
-            const int64_t warps = ceil_div<int64_t>(nnz, CHUNK_E);
-            const int64_t g = ceil_div<int64_t>(warps > 0 ? warps : 1, 8);
-            k_copy_old_rows<<<(unsigned)(g < (int64_t)sms * 6 ? g : (int64_t)sms * 6), 256, 0,
-                              st>>>(rp, col, aff, n_rows, new_rp, new_col, new_aff, a.first,
-                                    a.first + a.n_new, a.status);
-            k_fill_new_rows<<<sms * 2, 256, 0, st>>>(a.nbr_ids, a.nbr_cos, a.first, a.n_new, a.M,
-                                                     a.scale, new_rp, new_col, new_aff);
-            L += 2;
-            e = cudaGetLastError();
-        }
-        if (e == cudaSuccess && a.reciprocal && pairs > 0) {
-            e = scan_exclusive(recip, recip_off, n_rows, tmp, tmp_bytes, st);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(keys, a.nbr_ids, (size_t)pairs * 4,
-                                                      cudaMemcpyDeviceToDevice, st);
-            if (e == cudaSuccess) e = launch_iota(vals, pairs, st);
-            bool alt = false;
-            int bits = 0;
-            while (bits < 32 && ((int64_t)1 << bits) <= a.first - 1) ++bits;
-            if (e == cudaSuccess)
-                e = radix_sort_pairs(keys, vals, keys2, vals2, pairs, bits, tmp, tmp_bytes, st, &alt);
-            if (e == cudaSuccess) {
-                k_fill_recip<<<sms * 2, 256, 0, st>>>(alt ? vals2 : vals, alt ? keys2 : keys, pairs,
-                                                      a.nbr_ids, a.nbr_cos, a.first, a.M, a.scale, rp,
-                                                      recip_off, new_rp, new_col, new_aff);
-                L += 1;
-                e = cudaGetLastError();
-            }
-        }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) rc = AKASHIC_ECUDA;
     }
     if (launches) *launches += L;
-    return rc;
+    return e == cudaSuccess ? AKASHIC_OK : AKASHIC_ECUDA;
 }
 
 }  // namespace ak

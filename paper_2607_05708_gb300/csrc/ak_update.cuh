@@ -9,9 +9,9 @@ namespace ak {
 enum UpdateScratchSlot {
     SCR_QP = 0, SCR_EXTS, SCR_WS, SCR_BOUND, SCR_CNT, SCR_BUF,              // relate (fused)
     SCR_DOTS, SCR_CAND,                                                      // relate (batched)
-    SCR_DEG, SCR_RECIP, SCR_RECIP_OFF, SCR_KEYS, SCR_VALS, SCR_KEYS2, SCR_VALS2, SCR_TMP,
+    SCR_KEYS, SCR_VALS, SCR_KEYS2, SCR_VALS2, SCR_TMP,
     SCR_NBR_IDS, SCR_NBR_COS,                                                // update results
-    SCR_IN_INC, SCR_IN_DEG, SCR_IN_OFF, SCR_IN_RSTAT,                        // transpose patch
+    SCR_TOUCHED, SCR_IN_ROWS, SCR_MOVE,                                      // graph insert
     SCR_DEAD_S,                                                              // relate sample
     SCR_DEL,                                                                 // deletion
     SCR_MM_G, SCR_MM_GN, SCR_MM_CAND, SCR_MM_MOVING, SCR_MM_POS, SCR_MM_PARENT,  // memory
@@ -47,14 +47,24 @@ struct UpdateArgs {
     void *get(int slot, size_t bytes) const { return scratch(scratch_ctx, slot, bytes); }
 };
 
-// a6: top-M prior neighbours of every new chunk by <e_new, e_prior>.
-akashic_status_t relate_top_m(const UpdateArgs &a, cudaStream_t st, int *launches);
+// The update's preconditions into the status word: EINVAL if the range's rows
+// have out-edges, EDEVICE if an edge points at one of its chunks.
+cudaError_t launch_check_new_rows(const int64_t *rp, const int64_t *in_ptr, const int32_t *row_of,
+                                  int64_t first, int64_t n_new, int *status, cudaStream_t st);
+
+// a6: top-M prior neighbours of every new chunk by <e_new, e_prior>.  Waits
+// once for the stream; *dev_status (host) = the status word then.
+akashic_status_t relate_top_m(const UpdateArgs &a, cudaStream_t st, int *launches,
+                              int *dev_status);
 
 // a7: new out-edge CSR = old edges + M out-edges per new chunk (+ reciprocal
-// edges appended to the chosen rows), columns ascending in every row.
-// new_rp has n_rows+1 entries; new_col/new_aff have room for the result.
+// edges appended to the chosen rows), columns ascending in every row, with the
+// weights (and rstat) of the rows that gained edges anew; touched gets those
+// rows' bits.  new_rp has n_rows+1 entries; new_col / new_aff / new_w have room
+// for the result.  Does not wait.
 akashic_status_t csr_insert(const UpdateArgs &a, const int64_t *rp, const int32_t *col,
-                            const float *aff, int64_t nnz, int64_t *new_rp, int32_t *new_col,
-                            float *new_aff, cudaStream_t st, int *launches);
+                            const float *aff, const float *w, int64_t nnz, int64_t *new_rp,
+                            int32_t *new_col, float *new_aff, float *new_w, float2 *rstat,
+                            uint32_t *touched, cudaStream_t st, int *launches);
 
 }  // namespace ak
