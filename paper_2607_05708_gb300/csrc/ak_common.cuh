@@ -18,11 +18,15 @@ __device__ __forceinline__ void set_status(int *status, int code) {
 }
 
 // ------------------------------------------------------------------ dependent launches
-// The retrieval's kernels are launched with programmatic stream
-// serialisation (launch_pdl): each may be scheduled while the kernel before
-// it in the stream drains, and waits here, before it touches global memory,
-// until that kernel has completed and its writes are visible (a kernel
-// launched without the attribute returns from the wait at once).
+// The kernels of a retrieval and of the graph's and the pages' upkeep are
+// launched with programmatic stream serialisation (launch_pdl): each may be
+// scheduled while the kernel before it in the stream drains, and waits here,
+// before it touches global memory, until that kernel has completed and its
+// writes are visible (a kernel launched without the attribute returns from the
+// wait at once).  Every thread waits before anything else, so that a kernel's
+// end says that all before it have ended.  An upkeep call is a chain of 10 to 45
+// short kernels: 40 chunks added to 262,144 712 -> 640 us, 200 deleted from
+// 524,288 575 -> 547.
 __device__ __forceinline__ void griddep_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }

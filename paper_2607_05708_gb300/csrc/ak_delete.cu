@@ -17,6 +17,7 @@ __global__ void k_mark_dead(const int64_t *__restrict__ ids, int64_t n, int64_t 
                             const int32_t *__restrict__ row_of, int32_t *__restrict__ dead_row,
                             int *status, const int32_t *__restrict__ page_row,
                             int32_t *__restrict__ page_live) {
+    griddep_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t id = ids[i];
@@ -33,6 +34,7 @@ __global__ void k_mark_dead(const int64_t *__restrict__ ids, int64_t n, int64_t 
 __global__ void k_dead_bits(const int32_t *__restrict__ dead_row,
                             const int32_t *__restrict__ ext_of, int64_t n,
                             uint32_t *__restrict__ by_row, uint32_t *__restrict__ by_id) {
+    griddep_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     // warp-uniform trip count: whole words
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < ((n + 31) & ~(int64_t)31);
@@ -50,7 +52,8 @@ __global__ void k_dead_bits(const int32_t *__restrict__ dead_row,
 cudaError_t launch_dead_bits(const int32_t *dead_row, const int32_t *ext_of, int64_t n,
                              uint32_t *by_row, uint32_t *by_id, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    k_dead_bits<<<device_sm_count() * 4, 256, 0, st>>>(dead_row, ext_of, n, by_row, by_id);
+    launch_pdl(k_dead_bits, dim3((unsigned)(device_sm_count() * 4)), dim3(256), 0, st, dead_row,
+               ext_of, n, by_row, by_id);
     return cudaGetLastError();
 }
 
@@ -60,6 +63,7 @@ cudaError_t launch_dead_bits(const int32_t *dead_row, const int32_t *ext_of, int
 __global__ void k_drop_rows(const int64_t *__restrict__ ids, int64_t n, int64_t n_total,
                             const int32_t *__restrict__ row_of, const int64_t *__restrict__ ptr,
                             uint32_t *__restrict__ drop_bits) {
+    griddep_wait();
     for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
         const int64_t id = ids[i];
         if (id < 0 || id >= n_total) continue;
@@ -87,6 +91,7 @@ constexpr int DROP_TILE = 8 * 32 * DROP_WORDS;
 int64_t drop_tiles(int64_t nnz) { return ceil_div<int64_t>(nnz, DROP_TILE); }
 
 __global__ __launch_bounds__(256) void k_drop_mark(const DropDead d) {
+    griddep_wait();
     __shared__ int warp_n[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t e0 = (int64_t)blockIdx.x * DROP_TILE + warp * 32 * DROP_WORDS;
@@ -120,6 +125,7 @@ __global__ __launch_bounds__(256) void k_drop_mark(const DropDead d) {
 }
 
 __global__ __launch_bounds__(256, 4) void k_drop_edges(const DropDead d) {
+    griddep_wait();
     __shared__ int warp_n[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -182,6 +188,7 @@ __global__ __launch_bounds__(256) void k_drop_row_ptr(const DropDead d,
                                                       float2 *__restrict__ rstat,
                                                       const int32_t *__restrict__ row_of,
                                                       uint32_t *__restrict__ touched) {
+    griddep_wait();
     constexpr int L = 8;
     const int lane = threadIdx.x & 31, sub = lane % L;
     const int64_t step = ((int64_t)gridDim.x * blockDim.x) / L;
@@ -247,8 +254,8 @@ cudaError_t launch_mark_dead(const int64_t *ids, int64_t n, int64_t n_total, con
                              int32_t *dead_row, int *status, cudaStream_t st,
                              const int32_t *page_row, int32_t *page_live) {
     if (n <= 0) return cudaSuccess;
-    k_mark_dead<<<device_sm_count(), 256, 0, st>>>(ids, n, n_total, row_of, dead_row, status,
-                                                   page_row, page_live);
+    launch_pdl(k_mark_dead, dim3((unsigned)(device_sm_count())), dim3(256), 0, st, ids, n, n_total,
+               row_of, dead_row, status, page_row, page_live);
     return cudaGetLastError();
 }
 
@@ -257,12 +264,12 @@ cudaError_t launch_drop_dead_edges(const DropDead &d, cudaStream_t st) {
     if (d.nnz <= 0) return cudaErrorInvalidValue;
     if (d.n_ids > 0) {
         const int64_t g = d.n_ids < (int64_t)sms * 16 ? d.n_ids : (int64_t)sms * 16;
-        k_drop_rows<<<(unsigned)g, 128, 0, st>>>(d.ids, d.n_ids, d.n_total, d.own_row_of, d.ptr,
-                                                 d.drop_bits);
+        launch_pdl(k_drop_rows, dim3((unsigned)g), dim3(128), 0, st, d.ids, d.n_ids, d.n_total,
+                   d.own_row_of, d.ptr, d.drop_bits);
     }
     const unsigned tiles = (unsigned)drop_tiles(d.nnz);
-    k_drop_mark<<<tiles, 256, 0, st>>>(d);
-    k_drop_edges<<<tiles, 256, 0, st>>>(d);
+    launch_pdl(k_drop_mark, dim3(tiles), dim3(256), 0, st, d);
+    launch_pdl(k_drop_edges, dim3(tiles), dim3(256), 0, st, d);
     return cudaGetLastError();
 }
 
@@ -270,8 +277,8 @@ cudaError_t launch_drop_row_ptr(const DropDead &d, int64_t *ptr_out, float *w, f
                                 const int32_t *row_of, uint32_t *touched, cudaStream_t st) {
     const int64_t want = ceil_div<int64_t>((d.n_rows + 1) * 8, 256);
     const int64_t cap = (int64_t)device_sm_count() * 16;
-    k_drop_row_ptr<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(d, ptr_out, w, rstat,
-                                                                       row_of, touched);
+    launch_pdl(k_drop_row_ptr, dim3((unsigned)(want < cap ? want : cap)), dim3(256), 0, st, d,
+               ptr_out, w, rstat, row_of, touched);
     return cudaGetLastError();
 }
 

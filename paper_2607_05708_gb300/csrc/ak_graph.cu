@@ -103,6 +103,7 @@ __device__ __forceinline__ int64_t block_sum_scan(int64_t v, int64_t *wsum) {
 __global__ __launch_bounds__(SCAN_THREADS) void k_scan_reduce(const int64_t *__restrict__ in,
                                                               int64_t n,
                                                               int64_t *__restrict__ tile_sum) {
+    griddep_wait();
     __shared__ int64_t wsum[SCAN_THREADS / 32];
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
     int64_t s = 0;
@@ -118,6 +119,7 @@ __global__ __launch_bounds__(SCAN_THREADS) void k_scan_reduce(const int64_t *__r
 __global__ __launch_bounds__(SCAN_THREADS) void k_scan_down(const int64_t *__restrict__ in,
                                                             int64_t *__restrict__ out, int64_t n,
                                                             const int64_t *__restrict__ tile_sum) {
+    griddep_wait();
     __shared__ int64_t wsum[SCAN_THREADS / 32];
     int64_t pre = 0;
     for (int64_t t = threadIdx.x; t < (int64_t)blockIdx.x; t += SCAN_THREADS) pre += tile_sum[t];
@@ -180,8 +182,9 @@ cudaError_t scan_exclusive(const int64_t *in, int64_t *out, int64_t n, void *tmp
     const int64_t tiles = ceil_div<int64_t>(n, SCAN_TILE);
     if (n > 0 && tiles <= SCAN_FLAT_TILES) {
         int64_t *sums = (int64_t *)tmp;
-        if (tiles > 1) k_scan_reduce<<<(unsigned)tiles, SCAN_THREADS, 0, st>>>(in, n, sums);
-        k_scan_down<<<(unsigned)tiles, SCAN_THREADS, 0, st>>>(in, out, n, sums);
+        if (tiles > 1) launch_pdl(k_scan_reduce, dim3((unsigned)tiles), dim3(SCAN_THREADS), 0, st,
+                                  in, n, sums);
+        launch_pdl(k_scan_down, dim3((unsigned)tiles), dim3(SCAN_THREADS), 0, st, in, out, n, sums);
         if (launches) *launches += tiles > 1 ? 2 : 1;
         return cudaGetLastError();
     }
@@ -304,6 +307,7 @@ __global__ __launch_bounds__(RS_THREADS) void k_rs_hist32(const uint32_t *__rest
                                                           int n_tiles, int *__restrict__ hist,
                                                           int *__restrict__ zero1,
                                                           int *__restrict__ zero2) {
+    griddep_wait();
     __shared__ int h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
@@ -324,6 +328,7 @@ __global__ __launch_bounds__(RS_THREADS) void k_rs_scatter_small(
     uint32_t mask, int n_tiles, const int *__restrict__ hcur, int *__restrict__ hnext,
     int shift_next, uint32_t mask_next, int *__restrict__ hzero, uint32_t *__restrict__ okeys,
     uint32_t *__restrict__ ovals) {
+    griddep_wait();
     __shared__ int cnt[RS_WARPS][256];
     __shared__ int pre[RS_WARPS][256];
     __shared__ int off_s[256];
@@ -392,6 +397,7 @@ __global__ __launch_bounds__(128) void k_sort_one(const uint32_t *__restrict__ k
                                                   const uint32_t *__restrict__ vals, int n,
                                                   uint32_t mask, uint32_t *__restrict__ okeys,
                                                   uint32_t *__restrict__ ovals) {
+    griddep_wait();
     __shared__ uint4 x4[RS_ONE / 4];
     uint32_t *x = reinterpret_cast<uint32_t *>(x4);
     for (int i = threadIdx.x; i < ((n + 3) & ~3); i += 128) x[i] = i < n ? keys[i] & mask : ~0u;
@@ -428,8 +434,8 @@ cudaError_t radix_sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt,
     if (n <= 1 || bits <= 0) return cudaSuccess;
     if (tmp_bytes < radix_tmp_bytes(n)) return cudaErrorInvalidValue;
     if (n <= RS_ONE) {
-        k_sort_one<<<(unsigned)ceil_div<int64_t>(n, 128), 128, 0, st>>>(
-            keys, vals, (int)n, bits >= 32 ? 0xffffffffu : (1u << bits) - 1u, keys_alt, vals_alt);
+        launch_pdl(k_sort_one, dim3((unsigned)ceil_div<int64_t>(n, 128)), dim3(128), 0, st, keys,
+                   vals, (int)n, bits >= 32 ? 0xffffffffu : (1u << bits) - 1u, keys_alt, vals_alt);
         if (launches) *launches += 1;
         *result_in_alt = true;
         return cudaGetLastError();
@@ -446,16 +452,17 @@ cudaError_t radix_sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt,
         const int64_t ms = 256 * s_tiles;
         int *h[3] = {(int *)tmp, (int *)tmp + ms, (int *)tmp + 2 * ms};
         const int nt = (int)s_tiles;
-        k_rs_hist32<<<nt, RS_THREADS, 0, st>>>(ki, n, 0, bits < 8 ? (1u << bits) - 1u : 0xffu, nt,
-                                               h[0], h[1], h[2]);
+        launch_pdl(k_rs_hist32, dim3(nt), dim3(RS_THREADS), 0, st, ki, n, 0,
+                   bits < 8 ? (1u << bits) - 1u : 0xffu, nt, h[0], h[1], h[2]);
         if (launches) *launches += 1;
         for (int p = 0, sh = 0; sh < bits; ++p, sh += 8) {
             const int nb = bits - sh < 8 ? bits - sh : 8;
             const int shn = sh + 8;
             const int nbn = bits - shn < 8 ? bits - shn : 8;
-            k_rs_scatter_small<<<nt, RS_THREADS, 0, st>>>(
-                ki, vi, n, sh, (1u << nb) - 1u, nt, h[p % 3], shn < bits ? h[(p + 1) % 3] : nullptr,
-                shn, shn < bits ? (1u << nbn) - 1u : 0u, p >= 1 ? h[(p + 2) % 3] : nullptr, ko, vo);
+            launch_pdl(k_rs_scatter_small, dim3(nt), dim3(RS_THREADS), 0, st, ki, vi, n, sh,
+                       (1u << nb) - 1u, nt, h[p % 3], shn < bits ? h[(p + 1) % 3] : nullptr, shn,
+                       shn < bits ? (1u << nbn) - 1u : 0u, p >= 1 ? h[(p + 2) % 3] : nullptr, ko,
+                       vo);
             if (launches) *launches += 1;
             cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return e;
@@ -667,6 +674,7 @@ __global__ void k_batch_layout(const uint32_t *__restrict__ order, int64_t first
                                uint16_t *__restrict__ emb, const int32_t *__restrict__ page_in,
                                int64_t first_page, int per_page, int32_t *__restrict__ page_row,
                                int32_t *__restrict__ ext_of, int32_t *__restrict__ row_of) {
+    griddep_wait();
     const int lane = threadIdx.x & 31;
     int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -689,9 +697,8 @@ cudaError_t launch_batch_layout(const uint32_t *order, int64_t first, int64_t n,
                                 int64_t first_page, int per_page, int32_t *page_row,
                                 int32_t *ext_of, int32_t *row_of, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    k_batch_layout<<<device_sm_count() * 8, 256, 0, st>>>(order, first, n, dim, emb_in, emb,
-                                                          page_in, first_page, per_page, page_row,
-                                                          ext_of, row_of);
+    launch_pdl(k_batch_layout, dim3((unsigned)(device_sm_count() * 8)), dim3(256), 0, st, order,
+               first, n, dim, emb_in, emb, page_in, first_page, per_page, page_row, ext_of, row_of);
     return cudaGetLastError();
 }
 
@@ -764,6 +771,7 @@ __global__ __launch_bounds__(256) void k_heavy_rows(const int64_t *__restrict__ 
                                                     int64_t split_t, int32_t *__restrict__ rows,
                                                     int64_t *__restrict__ n_rows,
                                                     int32_t *__restrict__ counts) {
+    griddep_wait();
     const int t = threadIdx.x;
     const int64_t tile = blockIdx.x;
     if (WRITE && counts[tile] == 0 && tile != gridDim.x - 1) return;
@@ -797,6 +805,7 @@ __global__ __launch_bounds__(256) void k_hub_segs(SplitParams sp,
                                                   const int32_t *__restrict__ rows,
                                                   const int64_t *__restrict__ n_rows,
                                                   int64_t max_hubs, int64_t *__restrict__ nseg) {
+    griddep_wait();
     const int lane = threadIdx.x & 31;
     const int64_t n = *n_rows, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -820,6 +829,7 @@ __global__ void k_hub_fill(SplitParams sp, const int64_t *__restrict__ in_ptr,
                            uint32_t *__restrict__ seg_win, uint32_t *__restrict__ seg_id,
                            int32_t *__restrict__ slot_split, uint32_t *__restrict__ row_key,
                            uint32_t *__restrict__ row_id) {
+    griddep_wait();
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n_rows; i += nw) {
@@ -846,6 +856,7 @@ __global__ void k_seg_permute(const uint32_t *__restrict__ order, const int64_t 
                               const int64_t *__restrict__ e1, int64_t n_segs,
                               int64_t *__restrict__ e0s, int64_t *__restrict__ e1s,
                               int32_t *__restrict__ slot) {
+    griddep_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_segs;
          i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t o = order[i];
@@ -870,11 +881,13 @@ cudaError_t launch_hub_count(const SplitParams &sp, const int64_t *in_ptr, const
     }
     int32_t *tc = (int32_t *)scratch;
     int64_t *nseg = scratch + ceil_div<int64_t>(tiles, 2);
-    k_heavy_rows<false><<<(unsigned)tiles, 256, 0, st>>>(in_ptr, n, sp.split_t, rows, counts, tc);
-    k_heavy_rows<true><<<(unsigned)tiles, 256, 0, st>>>(in_ptr, n, sp.split_t, rows, counts, tc);
+    launch_pdl(k_heavy_rows<false>, dim3((unsigned)tiles), dim3(256), 0, st, in_ptr, n, sp.split_t,
+               rows, counts, tc);
+    launch_pdl(k_heavy_rows<true>, dim3((unsigned)tiles), dim3(256), 0, st, in_ptr, n, sp.split_t,
+               rows, counts, tc);
     const int64_t want = ceil_div<int64_t>(max_hubs, 8), cap = (int64_t)device_sm_count() * 8;
-    k_hub_segs<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(sp, in_ptr, in_src, rows, counts,
-                                                                    max_hubs, nseg);
+    launch_pdl(k_hub_segs, dim3((unsigned)(want < cap ? want : cap)), dim3(256), 0, st, sp, in_ptr,
+               in_src, rows, counts, max_hubs, nseg);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return scan_exclusive(nseg, slot0, max_hubs, nseg + max_hubs, scan_tmp_bytes(max_hubs), st);
@@ -888,9 +901,9 @@ cudaError_t launch_hub_fill(const SplitParams &sp, const int64_t *in_ptr, const 
                             cudaStream_t st) {
     if (n_rows <= 0) return cudaSuccess;
     const int64_t want = ceil_div<int64_t>(n_rows, 4), cap = (int64_t)device_sm_count() * 16;
-    k_hub_fill<<<(unsigned)(want < cap ? want : cap), 128, 0, st>>>(
-        sp, in_ptr, in_src, rows, slot0, n_rows, n_segs, split_row, split_slot0, seg_e0, seg_e1,
-        seg_win, seg_id, slot_split, row_key, row_id);
+    launch_pdl(k_hub_fill, dim3((unsigned)(want < cap ? want : cap)), dim3(128), 0, st, sp, in_ptr,
+               in_src, rows, slot0, n_rows, n_segs, split_row, split_slot0, seg_e0, seg_e1,
+               seg_win, seg_id, slot_split, row_key, row_id);
     return cudaGetLastError();
 }
 
@@ -898,7 +911,8 @@ cudaError_t launch_seg_permute(const uint32_t *order, const int64_t *e0, const i
                                int64_t n_segs, int64_t *e0s, int64_t *e1s, int32_t *slot,
                                cudaStream_t st) {
     if (n_segs <= 0) return cudaSuccess;
-    k_seg_permute<<<device_sm_count() * 2, 256, 0, st>>>(order, e0, e1, n_segs, e0s, e1s, slot);
+    launch_pdl(k_seg_permute, dim3((unsigned)(device_sm_count() * 2)), dim3(256), 0, st, order, e0,
+               e1, n_segs, e0s, e1s, slot);
     return cudaGetLastError();
 }
 

@@ -26,6 +26,7 @@ __global__ void k_new_in_ptr(const int64_t *__restrict__ in_ptr_old, int64_t n,
                              const uint32_t *__restrict__ fwd, int64_t pairs,
                              const uint32_t *__restrict__ new_rows, int64_t n_new, int M,
                              int64_t *__restrict__ in_ptr_new) {
+    griddep_wait();
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r <= n;
          r += (int64_t)gridDim.x * blockDim.x)
         in_ptr_new[r] = in_ptr_old[r] + lower_bound_u32(fwd, pairs, (uint64_t)r) +
@@ -34,6 +35,7 @@ __global__ void k_new_in_ptr(const int64_t *__restrict__ in_ptr_old, int64_t n,
 
 __global__ void k_row_keys(const int32_t *__restrict__ row_of, int64_t first, int64_t n_new,
                            uint32_t *__restrict__ keys, uint32_t *__restrict__ vals) {
+    griddep_wait();
     for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < n_new;
          a += (int64_t)gridDim.x * blockDim.x) {
         keys[a] = (uint32_t)row_of[first + a];
@@ -57,6 +59,7 @@ constexpr int MOVE_PER = 8, MOVE_TILE = 256 * MOVE_PER;
 // cut[p] = ptr[sorted[p] + end], p < count
 __global__ void k_move_cuts(const int64_t *__restrict__ ptr, const uint32_t *__restrict__ sorted,
                             int64_t count, int end, uint32_t *__restrict__ cut) {
+    griddep_wait();
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < count;
          p += (int64_t)gridDim.x * blockDim.x)
         cut[p] = (uint32_t)ptr[sorted[p] + end];
@@ -66,6 +69,7 @@ __global__ void k_move_cuts(const int64_t *__restrict__ ptr, const uint32_t *__r
 __global__ void k_move_tiles(const uint32_t *__restrict__ cut, int64_t n_cut,
                              const uint32_t *__restrict__ cut2, int64_t n_cut2, int64_t tiles,
                              int32_t *__restrict__ tile_cut, int32_t *__restrict__ tile_cut2) {
+    griddep_wait();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t > tiles) return;
     tile_cut[t] = (int32_t)lower_bound_u32(cut, n_cut, (uint64_t)t * MOVE_TILE);
@@ -77,6 +81,7 @@ __global__ __launch_bounds__(256, 4) void k_move_edges(const MoveEdges m,
                                                        const uint32_t *__restrict__ cut2,
                                                        const int32_t *__restrict__ tile_cut,
                                                        const int32_t *__restrict__ tile_cut2) {
+    griddep_wait();
     const int64_t tile = blockIdx.x, e0 = tile * MOVE_TILE + threadIdx.x;
     int32_t t[MOVE_PER];
     float v[MOVE_PER], w[MOVE_PER];
@@ -144,11 +149,13 @@ cudaError_t launch_move_edges(const MoveEdges &m, const int64_t *ptr, const uint
         const int64_t want = ceil_div<int64_t>(n, 256);
         return (unsigned)(want < cap ? want : cap);
     };
-    if (pairs > 0) k_move_cuts<<<grid(pairs), 256, 0, st>>>(ptr, sorted, pairs, 1, cut);
-    if (n_rows2 > 0) k_move_cuts<<<grid(n_rows2), 256, 0, st>>>(ptr, rows2, n_rows2, 0, cut2);
-    k_move_tiles<<<(unsigned)ceil_div<int64_t>(tiles + 1, 256), 256, 0, st>>>(cut, pairs, cut2,
-                                                                             n_rows2, tiles, tc, tc2);
-    k_move_edges<<<(unsigned)tiles, 256, 0, st>>>(m, cut, cut2, tc, tc2);
+    if (pairs > 0) launch_pdl(k_move_cuts, dim3((unsigned)(grid(pairs))), dim3(256), 0, st, ptr,
+                              sorted, pairs, 1, cut);
+    if (n_rows2 > 0) launch_pdl(k_move_cuts, dim3((unsigned)(grid(n_rows2))), dim3(256), 0, st,
+                                ptr, rows2, n_rows2, 0, cut2);
+    launch_pdl(k_move_tiles, dim3((unsigned)ceil_div<int64_t>(tiles + 1, 256)), dim3(256), 0, st,
+               cut, pairs, cut2, n_rows2, tiles, tc, tc2);
+    launch_pdl(k_move_edges, dim3((unsigned)tiles), dim3(256), 0, st, m, cut, cut2, tc, tc2);
     if (launches) *launches += 2 + (pairs > 0) + (n_rows2 > 0);
     return cudaGetLastError();
 }
@@ -162,6 +169,7 @@ __global__ void k_place_fwd(const uint32_t *__restrict__ fwd, const uint32_t *__
                             const int64_t *__restrict__ in_ptr_new, int32_t *__restrict__ src_new,
                             float *__restrict__ aff_new, const float2 *__restrict__ rstat,
                             float *__restrict__ w_new) {
+    griddep_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pairs;
          i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t p = order[i], rt = fwd[i];
@@ -185,6 +193,7 @@ __global__ void k_place_recip(const int32_t *__restrict__ nbr_ids, const float *
                               const int64_t *__restrict__ in_ptr_new, int32_t *__restrict__ src_new,
                               float *__restrict__ aff_new, const float2 *__restrict__ rstat,
                               float *__restrict__ w_new) {
+    griddep_wait();
     const int lane = threadIdx.x & 31;
     int64_t a = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -219,29 +228,29 @@ cudaError_t launch_in_edges_update(const InEdgeUpdate &u, const InEdgeScratch &s
     uint32_t *rk = s.rows, *rv = rk + u.n_new, *rk2 = rv + u.n_new, *rv2 = rk2 + u.n_new;
     if (e == cudaSuccess && recip_rows > 0) {
         const int64_t want = ceil_div<int64_t>(u.n_new, 256);
-        k_row_keys<<<(unsigned)(want < sms ? want : sms), 256, 0, st>>>(u.row_of, u.first, u.n_new,
-                                                                        rk, rv);
+        launch_pdl(k_row_keys, dim3((unsigned)(want < sms ? want : sms)), dim3(256), 0, st,
+                   u.row_of, u.first, u.n_new, rk, rv);
         e = radix_sort_pairs(rk, rv, rk2, rv2, u.n_new, u.row_bits, s.tmp, s.tmp_bytes, st, &alt_r,
                              &L);
         ++L;
     }
     if (e != cudaSuccess) return e;
     const uint32_t *fwd = alt ? s.keys2 : s.keys, *order = alt ? s.vals2 : s.vals;
-    k_new_in_ptr<<<sms * 8, 256, 0, st>>>(u.in_ptr_old, u.n, fwd, pairs, alt_r ? rk2 : rk,
-                                          recip_rows, u.M, u.in_ptr_new);
+    launch_pdl(k_new_in_ptr, dim3((unsigned)(sms * 8)), dim3(256), 0, st, u.in_ptr_old, u.n, fwd,
+               pairs, alt_r ? rk2 : rk, recip_rows, u.M, u.in_ptr_new);
     const int64_t nnz_old = u.nnz_new - pairs * (u.reciprocal ? 2 : 1);
     MoveEdges mv{nnz_old, u.in_src_old, u.in_aff_old, u.in_w_old, u.in_src_new, u.in_aff_new,
                  u.in_w_new, u.M, u.touched, u.ext_of, u.rstat};
     e = launch_move_edges(mv, u.in_ptr_old, fwd, pairs, alt_r ? rk2 : rk, recip_rows, s.move, st,
                           &L);
     if (e != cudaSuccess) return e;
-    k_place_fwd<<<sms * 2, 256, 0, st>>>(fwd, order, pairs, u.nbr_cos, u.scale, u.first, u.M,
-                                         u.row_of, u.in_ptr_old, u.in_ptr_new, u.in_src_new,
-                                         u.in_aff_new, u.rstat, u.in_w_new);
+    launch_pdl(k_place_fwd, dim3((unsigned)(sms * 2)), dim3(256), 0, st, fwd, order, pairs,
+               u.nbr_cos, u.scale, u.first, u.M, u.row_of, u.in_ptr_old, u.in_ptr_new,
+               u.in_src_new, u.in_aff_new, u.rstat, u.in_w_new);
     if (u.reciprocal) {
-        k_place_recip<<<sms * 2, 256, 0, st>>>(u.nbr_ids, u.nbr_cos, u.scale, u.first, u.n_new,
-                                               u.M, u.row_of, u.in_ptr_new, u.in_src_new,
-                                               u.in_aff_new, u.rstat, u.in_w_new);
+        launch_pdl(k_place_recip, dim3((unsigned)(sms * 2)), dim3(256), 0, st, u.nbr_ids,
+                   u.nbr_cos, u.scale, u.first, u.n_new, u.M, u.row_of, u.in_ptr_new, u.in_src_new,
+                   u.in_aff_new, u.rstat, u.in_w_new);
         ++L;
     }
     if (launches) *launches += L;

@@ -102,6 +102,7 @@ __device__ int mm_request_set(const int64_t *__restrict__ S, int r, int s_len, i
 __global__ void k_mm_count(const int64_t *__restrict__ S, int n_req, int s_len, int64_t n,
                            const int32_t *__restrict__ row_of,
                            const int32_t *__restrict__ dead_row, MmTables t, int *status) {
+    griddep_wait();
     __shared__ int32_t sets[8][MM_MAX_S];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int r = blockIdx.x * 8 + w; r < n_req; r += gridDim.x * 8) {
@@ -122,6 +123,7 @@ __global__ void k_mm_colocate(const int64_t *__restrict__ S, int n_req, int s_le
                               const int32_t *__restrict__ row_of,
                               const int32_t *__restrict__ dead_row, MmTables t, float tau,
                               int32_t *__restrict__ g_out, int32_t *__restrict__ g_n) {
+    griddep_wait();
     __shared__ int32_t sets[8][MM_MAX_S];
     __shared__ int flags[8][MM_MAX_S];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -169,6 +171,7 @@ __global__ __launch_bounds__(1024) void k_mm_relocate(const int32_t *__restrict_
                                                       int32_t *page_row, MmTables t,
                                                       int64_t next_page, int per_page,
                                                       const int *status, int64_t *result) {
+    griddep_wait();
     __shared__ int need[32];
     __shared__ int64_t next_s, writes_s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -242,6 +245,7 @@ __global__ __launch_bounds__(1024) void k_mm_relocate(const int32_t *__restrict_
 
 // ------------------------------------------------------------------ compaction
 __global__ void k_mm_candidates(MmTables t, int64_t n_pages, float theta, int32_t *__restrict__ cand) {
+    griddep_wait();
     // warp-uniform trip count, so the whole warp takes part in every ballot
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n_pages;
@@ -269,6 +273,7 @@ __global__ __launch_bounds__(256) void k_mm_moving(int64_t n, const int32_t *__r
                                                    const int32_t *__restrict__ cand,
                                                    uint32_t *__restrict__ moving,
                                                    int32_t *__restrict__ counts) {
+    griddep_wait();
     const int t = threadIdx.x;
     int64_t row[4];
 #pragma unroll
@@ -308,6 +313,7 @@ __global__ __launch_bounds__(256) void k_mm_list(int64_t n, const int32_t *__res
                                                  uint32_t *__restrict__ ns_key,
                                                  unsigned long long *__restrict__ count,
                                                  const int32_t *__restrict__ counts) {
+    griddep_wait();
     const int t = threadIdx.x;
     const int64_t tile = blockIdx.x;
     const int own = counts[tile];
@@ -349,6 +355,7 @@ __global__ void k_mm_union(MmTables t, const uint32_t *__restrict__ moving,
                            const unsigned long long *__restrict__ count,
                            const int32_t *__restrict__ row_of, const int32_t *__restrict__ ns_row,
                            float tau, int32_t *__restrict__ parent, int *status) {
+    griddep_wait();
     for (int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; h < t.co_cap;
          h += (int64_t)gridDim.x * blockDim.x) {
         const unsigned long long key = t.co_key[h];
@@ -374,6 +381,7 @@ __global__ void k_mm_union(MmTables t, const uint32_t *__restrict__ moving,
 // chunks arrive in ID order
 __global__ void k_mm_roots(const uint32_t *__restrict__ ids, int64_t count,
                            const int32_t *__restrict__ parent, uint32_t *__restrict__ root_key) {
+    griddep_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x)
         root_key[i] = (uint32_t)mm_find((volatile int32_t *)parent, (int32_t)ids[i]);
@@ -401,6 +409,7 @@ __global__ __launch_bounds__(1024) void k_mm_repack_small(const uint32_t *__rest
                                                           int32_t *__restrict__ page_row,
                                                           MmTables t, int64_t first_page,
                                                           int per_page, int64_t *new_pages) {
+    griddep_wait();
     __shared__ unsigned long long key[MM_SMALL];   // (namespace, root)
     __shared__ uint16_t at[MM_SMALL];              // place in ids
     __shared__ int32_t run_page[MM_SMALL];         // at a run's head: its first page
@@ -493,6 +502,7 @@ cudaError_t launch_mm_ns_keys(const uint32_t *ids, int64_t count, const int32_t 
 }
 
 __global__ void k_mm_release(MmTables t, int64_t n_pages, const int32_t *__restrict__ cand) {
+    griddep_wait();
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n_pages;
          p += (int64_t)gridDim.x * blockDim.x)
         if (cand[p]) {
@@ -547,6 +557,7 @@ __global__ void k_mm_repack(const uint32_t *__restrict__ order_ids,
 // new rows [first, first+n): their pages gain a live slot each
 __global__ void k_mm_count_pages(const int32_t *__restrict__ page_row, int64_t first, int64_t n,
                                  MmTables t) {
+    griddep_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t p = page_row[first + i];
@@ -609,8 +620,9 @@ cudaError_t launch_mm_count(const int64_t *S, int n_req, int s_len, int64_t n,
                             int *status, cudaStream_t st) {
     if (n_req <= 0) return cudaSuccess;
     const int grid = (int)ceil_div<int64_t>(n_req, 8);
-    k_mm_count<<<grid < device_sm_count() * 8 ? grid : device_sm_count() * 8, 256, 0, st>>>(
-        S, n_req, s_len, n, row_of, dead_row, t, status);
+    launch_pdl(k_mm_count,
+               dim3((unsigned)(grid < device_sm_count() * 8 ? grid : device_sm_count() * 8)),
+               dim3(256), 0, st, S, n_req, s_len, n, row_of, dead_row, t, status);
     return cudaGetLastError();
 }
 
@@ -621,12 +633,13 @@ cudaError_t launch_mm_relocate(const int64_t *S, int n_req, int s_len, int64_t n
                                cudaStream_t st) {
     if (n_req <= 0) return cudaSuccess;
     const int grid = (int)ceil_div<int64_t>(n_req, 8);
-    k_mm_colocate<<<grid < device_sm_count() * 8 ? grid : device_sm_count() * 8, 256, 0, st>>>(
-        S, n_req, s_len, n, row_of, dead_row, t, tau, g_buf, g_n);
+    launch_pdl(k_mm_colocate,
+               dim3((unsigned)(grid < device_sm_count() * 8 ? grid : device_sm_count() * 8)),
+               dim3(256), 0, st, S, n_req, s_len, n, row_of, dead_row, t, tau, g_buf, g_n);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_mm_relocate<<<1, 1024, 0, st>>>(g_buf, g_n, n_req, page_row, t, next_page, per_page, status,
-                                      result);
+    launch_pdl(k_mm_relocate, dim3(1), dim3(1024), 0, st, g_buf, g_n, n_req, page_row, t,
+               next_page, per_page, status, result);
     return cudaGetLastError();
 }
 
@@ -635,7 +648,8 @@ cudaError_t launch_mm_candidates(const MmTables &t, int64_t n_pages, float theta
     cudaError_t e = cudaMemsetAsync(t.released, 0, 8, st);
     if (e != cudaSuccess || n_pages <= 0) return e;
     const int64_t want = ceil_div<int64_t>(n_pages, 256), cap = (int64_t)device_sm_count() * 2;
-    k_mm_candidates<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(t, n_pages, theta, cand);
+    launch_pdl(k_mm_candidates, dim3((unsigned)(want < cap ? want : cap)), dim3(256), 0, st, t,
+               n_pages, theta, cand);
     return cudaGetLastError();
 }
 
@@ -648,24 +662,26 @@ cudaError_t launch_mm_collect(const MmTables &t, int64_t n, const int32_t *row_o
                               cudaStream_t st) {
     if (n <= 0) return cudaErrorInvalidValue;
     const unsigned tiles = (unsigned)mm_tiles(n);
-    k_mm_moving<<<tiles, 256, 0, st>>>(n, row_of, dead_row, page_row, cand, moving, counts);
-    k_mm_list<<<tiles, 256, 0, st>>>(n, row_of, ns_row, moving, parent, ids, ns_key,
-                                     t.released + 1, counts);
+    launch_pdl(k_mm_moving, dim3(tiles), dim3(256), 0, st, n, row_of, dead_row, page_row, cand,
+               moving, counts);
+    launch_pdl(k_mm_list, dim3(tiles), dim3(256), 0, st, n, row_of, ns_row, moving, parent, ids,
+               ns_key, t.released + 1, counts);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mm_union(const MmTables &t, const uint32_t *moving, const int32_t *row_of,
                             const int32_t *ns_row, float tau, int32_t *parent, int *status,
                             cudaStream_t st) {
-    k_mm_union<<<device_sm_count() * 8, 256, 0, st>>>(t, moving, t.released + 1, row_of, ns_row,
-                                                      tau, parent, status);
+    launch_pdl(k_mm_union, dim3((unsigned)(device_sm_count() * 8)), dim3(256), 0, st, t, moving,
+               t.released + 1, row_of, ns_row, tau, parent, status);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mm_roots(const uint32_t *ids, int64_t count, const int32_t *parent,
                             uint32_t *root_key, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
-    k_mm_roots<<<device_sm_count() * 2, 256, 0, st>>>(ids, count, parent, root_key);
+    launch_pdl(k_mm_roots, dim3((unsigned)(device_sm_count() * 2)), dim3(256), 0, st, ids, count,
+               parent, root_key);
     return cudaGetLastError();
 }
 
@@ -676,9 +692,10 @@ cudaError_t launch_mm_repack_small(const MmTables &t, int64_t n_pages, const int
                                    int32_t *page_row, int64_t first_page, int per_page,
                                    int64_t *new_pages, cudaStream_t st) {
     if (count < 1 || count > MM_SMALL) return cudaErrorInvalidValue;
-    if (n_pages > 0) k_mm_release<<<device_sm_count() * 2, 256, 0, st>>>(t, n_pages, cand);
-    k_mm_repack_small<<<1, 1024, 0, st>>>(ids, ns_key, (int)count, parent, row_of, page_row, t,
-                                          first_page, per_page, new_pages);
+    if (n_pages > 0) launch_pdl(k_mm_release, dim3((unsigned)(device_sm_count() * 2)), dim3(256),
+                                0, st, t, n_pages, cand);
+    launch_pdl(k_mm_repack_small, dim3(1), dim3(1024), 0, st, ids, ns_key, (int)count, parent,
+               row_of, page_row, t, first_page, per_page, new_pages);
     return cudaGetLastError();
 }
 
@@ -688,7 +705,8 @@ cudaError_t launch_mm_release_repack(const MmTables &t, int64_t n_pages, const i
                                      const int32_t *row_of, int32_t *page_row, int64_t first_page,
                                      int per_page, cudaStream_t st) {
     const int sms = device_sm_count();
-    if (n_pages > 0) k_mm_release<<<sms * 2, 256, 0, st>>>(t, n_pages, cand);
+    if (n_pages > 0) launch_pdl(k_mm_release, dim3((unsigned)(sms * 2)), dim3(256), 0, st, t,
+                                n_pages, cand);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || count <= 0) return e;
     k_mm_repack<<<sms * 2, 256, 0, st>>>(order_ids, ns_sorted, part_base, count, row_of, page_row,
@@ -699,7 +717,8 @@ cudaError_t launch_mm_release_repack(const MmTables &t, int64_t n_pages, const i
 cudaError_t launch_mm_count_pages(const int32_t *page_row, int64_t first, int64_t n,
                                   const MmTables &t, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    k_mm_count_pages<<<device_sm_count() * 2, 256, 0, st>>>(page_row, first, n, t);
+    launch_pdl(k_mm_count_pages, dim3((unsigned)(device_sm_count() * 2)), dim3(256), 0, st,
+               page_row, first, n, t);
     return cudaGetLastError();
 }
 

@@ -73,6 +73,7 @@ cudaError_t launch_prep_queries(const uint16_t *q, int b, int bp, int dim, float
 // One warp per row; the running maximum only grows (appends never shrink it).
 __global__ void k_row_norm_max(const uint16_t *__restrict__ emb, int64_t n, int dim,
                                float *max_norm) {
+    griddep_wait();
     const int lane = threadIdx.x & 31;
     int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -95,7 +96,7 @@ cudaError_t launch_row_norm_max(const uint16_t *emb, int64_t n, int dim, float *
     if (n <= 0) return cudaSuccess;
     int64_t warps = n < (int64_t)152 * 64 ? n : (int64_t)152 * 64;
     int grid = (int)ceil_div<int64_t>(warps * 32, 256);
-    k_row_norm_max<<<grid, 256, 0, st>>>(emb, n, dim, max_norm);
+    launch_pdl(k_row_norm_max, dim3(grid), dim3(256), 0, st, emb, n, dim, max_norm);
     return cudaGetLastError();
 }
 

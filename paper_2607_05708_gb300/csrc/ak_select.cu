@@ -360,6 +360,7 @@ template <int W>
 __global__ __launch_bounds__(W * 32) void k_sample_kth_split(
     const uint32_t *__restrict__ keys_t, int64_t n_sample, int b, int k,
     unsigned long long *__restrict__ bound, unsigned int *__restrict__ cnt) {
+    griddep_wait();
     static_assert(W * KS_KMAX <= KS_BUF, "the warps' survivors fit a buffer");
     __shared__ uint32_t buf[W][KS_BUF];
     __shared__ int lens[W];
@@ -430,9 +431,11 @@ cudaError_t launch_sample_kth_keys(const uint32_t *keys_t, int64_t n_sample, int
                                    int *launches) {
     if (k < 1 || k > KS_KMAX || bp < 1 || b > bp) return cudaErrorInvalidValue;
     if (b <= 2 * device_sm_count())
-        k_sample_kth_split<8><<<bp, 256, 0, st>>>(keys_t, n_sample, b, k, bound, cnt);
+        launch_pdl(k_sample_kth_split<8>, dim3(bp), dim3(256), 0, st, keys_t, n_sample, b, k,
+                   bound, cnt);
     else
-        k_sample_kth_split<4><<<bp, 128, 0, st>>>(keys_t, n_sample, b, k, bound, cnt);
+        launch_pdl(k_sample_kth_split<4>, dim3(bp), dim3(128), 0, st, keys_t, n_sample, b, k,
+                   bound, cnt);
     if (launches) *launches += 1;
     return cudaGetLastError();
 }
@@ -799,6 +802,7 @@ __global__ __launch_bounds__(SEL_THREADS) void k_topm_merge(
 __global__ __launch_bounds__(SEL_THREADS) void k_buf_merge_signed(
     const unsigned int *__restrict__ cnt, const unsigned long long *__restrict__ buf, int64_t cap,
     int k, int32_t *__restrict__ nbr_ids, float *__restrict__ nbr_cos, int *status) {
+    griddep_wait();
     __shared__ int hist[256 * (SEL_THREADS / 32)];
     __shared__ unsigned long long stage[SEL_STAGE];
     __shared__ unsigned long long win[64];
@@ -832,8 +836,8 @@ cudaError_t launch_buf_merge_signed(const unsigned int *cnt, const unsigned long
                                     int64_t cap, int64_t n_cols, int k, int32_t *nbr_ids,
                                     float *nbr_cos, int *status, cudaStream_t st, int *launches) {
     if (n_cols <= 0) return cudaSuccess;
-    k_buf_merge_signed<<<(unsigned)n_cols, SEL_THREADS, 0, st>>>(cnt, buf, cap, k, nbr_ids,
-                                                                 nbr_cos, status);
+    launch_pdl(k_buf_merge_signed, dim3((unsigned)n_cols), dim3(SEL_THREADS), 0, st, cnt, buf, cap,
+               k, nbr_ids, nbr_cos, status);
     if (launches) *launches += 1;
     return cudaGetLastError();
 }

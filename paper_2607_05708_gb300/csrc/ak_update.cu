@@ -11,6 +11,7 @@ namespace ak {
 // zero-padded bp-row block.
 __global__ void k_gather_rows(const uint16_t *__restrict__ emb, const int32_t *__restrict__ row_of,
                               int64_t c0, int b, int bp, int dim, uint16_t *__restrict__ dst) {
+    griddep_wait();
     const int64_t total = (int64_t)bp * dim;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -21,6 +22,7 @@ __global__ void k_gather_rows(const uint16_t *__restrict__ emb, const int32_t *_
 
 __global__ void k_ext_sample(const int32_t *__restrict__ ext_of, int64_t n_sample, int64_t stride,
                              int32_t *__restrict__ out) {
+    griddep_wait();
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n_sample;
          v += (int64_t)gridDim.x * blockDim.x)
         out[v] = ext_of[v * stride];
@@ -29,7 +31,8 @@ __global__ void k_ext_sample(const int32_t *__restrict__ ext_of, int64_t n_sampl
 cudaError_t launch_ext_sample(const int32_t *ext_of, int64_t n_sample, int64_t stride,
                               int32_t *out, cudaStream_t st) {
     if (n_sample <= 0) return cudaSuccess;
-    k_ext_sample<<<device_sm_count(), 256, 0, st>>>(ext_of, n_sample, stride, out);
+    launch_pdl(k_ext_sample, dim3((unsigned)(device_sm_count())), dim3(256), 0, st, ext_of,
+               n_sample, stride, out);
     return cudaGetLastError();
 }
 
@@ -54,8 +57,8 @@ static akashic_status_t relate_top_m_batched(const UpdateArgs &a, cudaStream_t s
         const int b = (int)(a.n_new - off < 256 ? a.n_new - off : 256);
         int bp = 32;
         while (bp < b) bp <<= 1;
-        k_gather_rows<<<device_sm_count(), 256, 0, st>>>(a.emb, a.row_of, a.first + off, b, bp,
-                                                          a.dim, qp);
+        launch_pdl(k_gather_rows, dim3((unsigned)(device_sm_count())), dim3(256), 0, st, a.emb,
+                   a.row_of, a.first + off, b, bp, a.dim, qp);
         e = cudaGetLastError();
         if (e == cudaSuccess)
             e = launch_dots(a.emb, n_old, 1, a.dim, qp, bp, 1, dots, a.status, st, launches);
@@ -111,9 +114,9 @@ akashic_status_t relate_top_m(const UpdateArgs &a, cudaStream_t st, int *launche
     cudaError_t e = cudaSuccess;
     bool overflow = false;
     if (rc == AKASHIC_OK) {
-        k_gather_rows<<<sms * 2, 256, 0, st>>>(a.emb, a.row_of, a.first, (int)a.n_new, (int)n_pad,
-                                               a.dim, qp);
-        k_ext_sample<<<sms, 256, 0, st>>>(a.ext_of, n_sample, stride, ext_s);
+        launch_pdl(k_gather_rows, dim3((unsigned)(sms * 2)), dim3(256), 0, st, a.emb, a.row_of,
+                   a.first, (int)a.n_new, (int)n_pad, a.dim, qp);
+        launch_pdl(k_ext_sample, dim3(sms), dim3(256), 0, st, a.ext_of, n_sample, stride, ext_s);
         e = cudaGetLastError();
         // deleted chunks are never neighbours: their sample rows carry no key
         const int32_t *dead_s = nullptr;
@@ -122,7 +125,8 @@ akashic_status_t relate_top_m(const UpdateArgs &a, cudaStream_t st, int *launche
             if (!ds) {
                 rc = AKASHIC_ENOMEM;
             } else {
-                k_ext_sample<<<sms, 256, 0, st>>>(a.dead_row, n_sample, stride, ds);
+                launch_pdl(k_ext_sample, dim3(sms), dim3(256), 0, st, a.dead_row, n_sample, stride,
+                           ds);
                 e = cudaGetLastError();
                 dead_s = ds;
             }
@@ -181,6 +185,7 @@ akashic_status_t relate_top_m(const UpdateArgs &a, cudaStream_t st, int *launche
 __global__ void k_check_new_rows(const int64_t *__restrict__ rp, const int64_t *__restrict__ in_ptr,
                                  const int32_t *__restrict__ row_of, int64_t first, int64_t n_new,
                                  int *status) {
+    griddep_wait();
     if (rp[first] != rp[first + n_new]) {
         set_status(status, AKASHIC_EINVAL);
         return;
@@ -195,8 +200,8 @@ __global__ void k_check_new_rows(const int64_t *__restrict__ rp, const int64_t *
 cudaError_t launch_check_new_rows(const int64_t *rp, const int64_t *in_ptr, const int32_t *row_of,
                                   int64_t first, int64_t n_new, int *status, cudaStream_t st) {
     const int64_t want = ceil_div<int64_t>(n_new, 256), cap = device_sm_count();
-    k_check_new_rows<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(rp, in_ptr, row_of, first,
-                                                                         n_new, status);
+    launch_pdl(k_check_new_rows, dim3((unsigned)(want < cap ? want : cap)), dim3(256), 0, st, rp,
+               in_ptr, row_of, first, n_new, status);
     return cudaGetLastError();
 }
 
@@ -204,6 +209,7 @@ cudaError_t launch_check_new_rows(const int64_t *rp, const int64_t *in_ptr, cons
 __global__ void k_pair_keys(const int32_t *__restrict__ ids, const int32_t *__restrict__ map,
                             int64_t pairs, uint32_t *__restrict__ keys,
                             uint32_t *__restrict__ vals) {
+    griddep_wait();
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < pairs;
          p += (int64_t)gridDim.x * blockDim.x) {
         keys[p] = (uint32_t)(map ? map[ids[p]] : ids[p]);
@@ -215,7 +221,8 @@ cudaError_t launch_pair_keys(const int32_t *ids, const int32_t *map, int64_t pai
                              uint32_t *vals, cudaStream_t st) {
     if (pairs <= 0) return cudaSuccess;
     const int64_t want = ceil_div<int64_t>(pairs, 256), cap = (int64_t)device_sm_count() * 4;
-    k_pair_keys<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(ids, map, pairs, keys, vals);
+    launch_pdl(k_pair_keys, dim3((unsigned)(want < cap ? want : cap)), dim3(256), 0, st, ids, map,
+               pairs, keys, vals);
     return cudaGetLastError();
 }
 
@@ -226,6 +233,7 @@ cudaError_t launch_pair_keys(const int32_t *ids, const int32_t *map, int64_t pai
 __global__ void k_new_row_ptr(const int64_t *__restrict__ rp, int64_t n_rows, int64_t first,
                               int64_t n_new, int M, const uint32_t *__restrict__ tgt,
                               int64_t recips, int64_t *__restrict__ nrp) {
+    griddep_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= n_rows;
          i += (int64_t)gridDim.x * blockDim.x) {
         int64_t before = i - first;
@@ -240,6 +248,7 @@ __global__ void k_fill_new_rows(const int32_t *__restrict__ nbr, const float *__
                                 int64_t first, int64_t n_new, int M, float scale,
                                 const int64_t *__restrict__ nrp, int32_t *__restrict__ ncol,
                                 float *__restrict__ naff) {
+    griddep_wait();
     const int lane = threadIdx.x & 31;
     int64_t a = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -264,6 +273,7 @@ __global__ void k_fill_recip(const uint32_t *__restrict__ order, const uint32_t 
                              float scale, const int64_t *__restrict__ rp,
                              const int64_t *__restrict__ nrp, int32_t *__restrict__ ncol,
                              float *__restrict__ naff) {
+    griddep_wait();
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < pairs;
          p += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t pair = order[p];
@@ -275,7 +285,8 @@ __global__ void k_fill_recip(const uint32_t *__restrict__ order, const uint32_t 
     }
 }
 
-__global__ void k_first_row(int64_t first, uint32_t *__restrict__ out) { *out = (uint32_t)first; }
+__global__ void k_first_row(int64_t first, uint32_t *__restrict__ out) {
+    griddep_wait(); *out = (uint32_t)first; }
 
 // The softmax of the rows that gained edges (the new rows, then each target's
 // row, at its first pair), eight lanes a row in k_row_softmax's order, and
@@ -289,6 +300,7 @@ __global__ __launch_bounds__(256) void k_gained_softmax(const uint32_t *__restri
                                                         float *__restrict__ nw_,
                                                         float2 *__restrict__ rstat,
                                                         uint32_t *__restrict__ touched) {
+    griddep_wait();
     constexpr int L = 8;
     const int lane = threadIdx.x & 31, sub = lane % L;
     const int64_t items = n_new + recips;
@@ -351,26 +363,26 @@ akashic_status_t csr_insert(const UpdateArgs &a, const int64_t *rp, const int32_
     }
     const uint32_t *tgt = alt ? keys2 : keys, *order = alt ? vals2 : vals;
     if (e == cudaSuccess) {
-        k_new_row_ptr<<<sms * 8, 256, 0, st>>>(rp, n_rows, a.first, a.n_new, a.M, tgt, recips,
-                                               new_rp);
+        launch_pdl(k_new_row_ptr, dim3((unsigned)(sms * 8)), dim3(256), 0, st, rp, n_rows, a.first,
+                   a.n_new, a.M, tgt, recips, new_rp);
         // old edges keep their order at the front of each row, and their weights
         // (the rows that gain edges get theirs anew below); the new rows' edges
         // go in as one block before row first's place
-        k_first_row<<<1, 1, 0, st>>>(a.first, words);
+        launch_pdl(k_first_row, dim3(1), dim3(1), 0, st, a.first, words);
         MoveEdges mv{nnz, col, aff, w, new_col, new_aff, new_w, a.n_new * a.M, nullptr, nullptr,
                      nullptr};
         e = launch_move_edges(mv, rp, tgt, recips, words, 1, words + 1, st, &L);
     }
     if (e == cudaSuccess) {
-        k_fill_new_rows<<<sms * 2, 256, 0, st>>>(a.nbr_ids, a.nbr_cos, a.first, a.n_new, a.M,
-                                                 a.scale, new_rp, new_col, new_aff);
+        launch_pdl(k_fill_new_rows, dim3((unsigned)(sms * 2)), dim3(256), 0, st, a.nbr_ids,
+                   a.nbr_cos, a.first, a.n_new, a.M, a.scale, new_rp, new_col, new_aff);
         if (recips > 0)
-            k_fill_recip<<<sms * 2, 256, 0, st>>>(order, tgt, pairs, a.nbr_cos, a.first, a.M,
-                                                  a.scale, rp, new_rp, new_col, new_aff);
+            launch_pdl(k_fill_recip, dim3((unsigned)(sms * 2)), dim3(256), 0, st, order, tgt,
+                       pairs, a.nbr_cos, a.first, a.M, a.scale, rp, new_rp, new_col, new_aff);
         const int64_t want = ceil_div<int64_t>((a.n_new + recips) * 8, 256);
         const int64_t cap = (int64_t)sms * 16;
-        k_gained_softmax<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(
-            tgt, recips, a.first, a.n_new, new_rp, new_aff, a.row_of, new_w, rstat, touched);
+        launch_pdl(k_gained_softmax, dim3((unsigned)(want < cap ? want : cap)), dim3(256), 0, st,
+                   tgt, recips, a.first, a.n_new, new_rp, new_aff, a.row_of, new_w, rstat, touched);
         e = cudaGetLastError();
     }
     if (launches) *launches += L;
