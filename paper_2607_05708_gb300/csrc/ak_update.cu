@@ -8,15 +8,20 @@
 namespace ak {
 
 // Gather the embeddings of chunks c0 .. c0+b-1 (rows row_of[c]) into a
-// zero-padded bp-row block.
+// zero-padded bp-row block.  Bound by latency: eight values a load (dim is a
+// multiple of 64, both buffers are allocations of the library's own), 4096 rows
+// of 1024 45 -> 9 us.
 __global__ void k_gather_rows(const uint16_t *__restrict__ emb, const int32_t *__restrict__ row_of,
                               int64_t c0, int b, int bp, int dim, uint16_t *__restrict__ dst) {
     griddep_wait();
-    const int64_t total = (int64_t)bp * dim;
+    const int per = dim / 8;
+    const int64_t total = (int64_t)bp * per;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = i / dim, t = i % dim;
-        dst[i] = r < b ? emb[(int64_t)row_of[c0 + r] * dim + t] : (uint16_t)0;
+        const int64_t r = i / per, t = i % per;
+        reinterpret_cast<uint4 *>(dst)[i] =
+            r < b ? reinterpret_cast<const uint4 *>(emb + (int64_t)row_of[c0 + r] * dim)[t]
+                  : make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
