@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include "../../include/akashic_mem.h"
+#include "ak_sizes.h"
 
 namespace ak {
 
@@ -283,11 +284,10 @@ constexpr int ROWS_PER_GRAB = 8;     // rows a warp claims at a time (dynamic sc
 // `launches`, if given, is incremented by the kernels launched.
 cudaError_t scan_exclusive(const int64_t *in, int64_t *out, int64_t n, void *tmp,
                            size_t tmp_bytes, cudaStream_t st, int *launches = nullptr);
-size_t scan_tmp_bytes(int64_t n);
 
 // Stable LSD radix sort of (key, value) pairs on the low `bits` key bits;
 // the result lands in (keys, vals) or, if *result_in_alt, in the alt buffers.
-size_t radix_tmp_bytes(int64_t n);
+// tmp: radix_tmp_bytes(n) bytes (ak_sizes.h).
 cudaError_t radix_sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt,
                              uint32_t *vals_alt, int64_t n, int bits, void *tmp,
                              size_t tmp_bytes, cudaStream_t st, bool *result_in_alt,

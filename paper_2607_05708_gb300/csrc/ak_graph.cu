@@ -22,7 +22,8 @@ static int sm_count_cached() {
 int device_sm_count() { return sm_count_cached(); }
 
 // ================================================================== scan
-constexpr int SCAN_THREADS = 256, SCAN_ITEMS = 8, SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
+constexpr int SCAN_THREADS = 256, SCAN_ITEMS = 8;
+static_assert(SCAN_TILE == SCAN_THREADS * SCAN_ITEMS, "a tile is one CTA's share");
 
 __device__ __forceinline__ int64_t warp_incl_scan(int64_t v) {
     const int lane = threadIdx.x & 31;
@@ -149,17 +150,6 @@ __global__ __launch_bounds__(SCAN_THREADS) void k_scan_down(const int64_t *__res
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == SCAN_THREADS - 1) out[n] = excl;
 }
 
-size_t scan_tmp_bytes(int64_t n) {
-    size_t tot = 0;
-    int64_t m = n;
-    do {
-        int64_t tiles = ceil_div<int64_t>(m, SCAN_TILE);
-        tot += (size_t)(2 * tiles + 2) * sizeof(int64_t);
-        m = tiles;
-    } while (m > 1);
-    return tot + 64;
-}
-
 static cudaError_t scan_rec(const int64_t *in, int64_t *out, int64_t n, int64_t *tmp,
                             cudaStream_t st, int *launches) {
     if (n <= 0) return cudaSuccess;
@@ -200,7 +190,8 @@ cudaError_t scan_exclusive(const int64_t *in, int64_t *out, int64_t n, void *tmp
 // Per pass: tile histograms (digit-major), one exclusive scan, then a stable
 // scatter in which each warp ranks its keys round by round with
 // __match_any_sync and the warps of a tile are combined in order.
-constexpr int RS_THREADS = 256, RS_ITEMS = 16, RS_TILE = RS_THREADS * RS_ITEMS;
+constexpr int RS_THREADS = 256, RS_ITEMS = 16;
+static_assert(RS_TILE == RS_THREADS * RS_ITEMS, "a tile is one CTA's share");
 constexpr int RS_WARPS = RS_THREADS / 32, RS_PER_WARP = RS_TILE / RS_WARPS;
 
 __global__ __launch_bounds__(RS_THREADS) void k_rs_hist(const uint32_t *__restrict__ keys,
@@ -299,8 +290,8 @@ __global__ __launch_bounds__(RS_THREADS) void k_rs_scatter(
 // histograms, by destination tile.  Three histogram buffers rotate: pass p
 // reads H[p % 3], counts into H[(p+1) % 3] (zero by then) and zeroes its
 // column of H[(p+2) % 3], which pass p-1 read and pass p+1 counts into.
-constexpr int RS_SMALL_ITEMS = 4, RS_SMALL_TILE = RS_THREADS * RS_SMALL_ITEMS;
-constexpr int64_t RS_SMALL_TILES = 256;
+constexpr int RS_SMALL_ITEMS = 4;
+static_assert(RS_SMALL_TILE == RS_THREADS * RS_SMALL_ITEMS, "a tile is one CTA's share");
 
 __global__ __launch_bounds__(RS_THREADS) void k_rs_hist32(const uint32_t *__restrict__ keys,
                                                           int64_t n, int shift, uint32_t mask,
@@ -415,15 +406,6 @@ __global__ __launch_bounds__(128) void k_sort_one(const uint32_t *__restrict__ k
     }
     okeys[rank] = keys[i];
     ovals[rank] = vals[i];
-}
-
-size_t radix_tmp_bytes(int64_t n) {
-    int64_t n_tiles = ceil_div<int64_t>(n, RS_TILE);
-    int64_t m = 256 * n_tiles;
-    const size_t big = (size_t)(2 * m + 1) * sizeof(int64_t) + scan_tmp_bytes(m) + 256;
-    const int64_t st = ceil_div<int64_t>(n, RS_SMALL_TILE);
-    const size_t small = st <= RS_SMALL_TILES ? (size_t)3 * 256 * st * sizeof(int) + 256 : 0;
-    return big > small ? big : small;
 }
 
 cudaError_t radix_sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt,
