@@ -79,6 +79,11 @@ struct DevBuf {
     template <typename T> T *as() const { return (T *)p; }
 };
 
+static void swap_bufs(DevBuf &x, DevBuf &y) {
+    std::swap(x.p, y.p);
+    std::swap(x.cap, y.cap);
+}
+
 // Words of StreamScratch::words: u's extremes [2], the kept lists' lengths
 // (int64 [2]), the hops' work queues ([2] a hop), the candidates' flags.
 constexpr int CW_EXT = 0, CW_KEPT = 2, CW_QUEUE = 6, CW_REACH = CW_QUEUE + 2 * AKASHIC_MAX_HOPS,
@@ -336,10 +341,8 @@ static akashic_status_t mm_ensure_pairs(akashic_mem *m, int64_t more, cudaStream
     DevBuf nk, nv;
     AK_TRY(nk.ensure((size_t)cap * 8));
     AK_TRY(nv.ensure((size_t)cap * 4));
-    std::swap(m->co_key.p, nk.p);
-    std::swap(m->co_key.cap, nk.cap);
-    std::swap(m->co_val.p, nv.p);
-    std::swap(m->co_val.cap, nv.cap);
+    swap_bufs(m->co_key, nk);
+    swap_bufs(m->co_val, nv);
     const int64_t old_cap = m->co_cap;
     m->co_cap = cap;
     CUDA_TRY(launch_mm_rehash(nk.as<unsigned long long>(), nv.as<uint32_t>(), old_cap,
@@ -775,6 +778,30 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
     uint32_t *touched =
         (uint32_t *)store_scratch(m, SCR_TOUCHED, (size_t)ceil_div<int64_t>(m->n, 32) * 4);
     if (!touched) return fail(AKASHIC_ENOMEM, "update: out of device memory");
+    // the transpose is patched (or built anew, where there is none), into spares
+    // that are taken now too: both lists change together or not at all (csr_insert
+    // is done with the slots that it shares, of the same sizes)
+    const int64_t nnz_old = m->nnz, pairs = n * (int64_t)M;
+    const bool patch = m->inc_transpose && nnz_old > 0;
+    DevBuf &ptr2 = m->in_ptr2, &src2 = m->in_src2, &aff2 = m->in_aff2, &w2 = m->in_w2;
+    const size_t tb = radix_tmp_bytes(pairs) + 4096;   // pairs >= n: the new rows' sort too
+    InEdgeScratch sc{};
+    if (patch) {
+        AK_TRY(ensure_spare(ptr2, (size_t)(m->cap + 1) * 8));
+        AK_TRY(ensure_spare(src2, (size_t)nnz_new * 4));
+        AK_TRY(ensure_spare(aff2, (size_t)nnz_new * 4));
+        AK_TRY(ensure_spare(w2, (size_t)nnz_new * 4));
+        auto get = [&](int slot, size_t bytes) {
+            return (uint32_t *)store_scratch(m, slot, bytes);
+        };
+        sc = InEdgeScratch{get(SCR_KEYS, (size_t)pairs * 4 + 16), get(SCR_VALS, (size_t)pairs * 4 + 16),
+                           get(SCR_KEYS2, (size_t)pairs * 4 + 16), get(SCR_VALS2, (size_t)pairs * 4 + 16),
+                           get(SCR_IN_ROWS, (size_t)n * 16),
+                           get(SCR_MOVE, (size_t)(1 + move_words(nnz_old, pairs, n)) * 4),
+                           get(SCR_TMP, tb), tb};
+        if (!sc.keys || !sc.vals || !sc.keys2 || !sc.vals2 || !sc.rows || !sc.move || !sc.tmp)
+            return fail(AKASHIC_ENOMEM, "update: out of device memory");
+    }
     {
         // rows [first, first+n) must have no out-edges and no in-edges: checked on
         // the device, read back with the top-M's outcome, before anything changes
@@ -799,39 +826,11 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
             if (r != AKASHIC_OK) return fail(r, "update: CSR insert failed");
         }
         PhaseScope pt(m, AKASHIC_PHASE_TRANSPOSE, st);
-        std::swap(m->row_ptr.p, nrp.p);
-        std::swap(m->row_ptr.cap, nrp.cap);
-        std::swap(m->col.p, ncol.p);
-        std::swap(m->col.cap, ncol.cap);
-        std::swap(m->aff.p, naff.p);
-        std::swap(m->aff.cap, naff.cap);
-        std::swap(m->w.p, m->w2.p);
-        std::swap(m->w.cap, m->w2.cap);
-        const int64_t nnz_old = m->nnz;
-        m->nnz = nnz_new;
-        if (!m->inc_transpose || nnz_old == 0) {
-            AK_TRY(rebuild_in_edges(m, st));
-        } else {
-            // patch the transpose: old lists moved, new edges placed, weights
-            // recomputed from the logits (ak_inedges.cu)
-            DevBuf &ptr2 = m->in_ptr2, &src2 = m->in_src2, &aff2 = m->in_aff2, &w2 = m->in_w2;
-            const int64_t rows = m->n, pairs = n * (int64_t)M;
-            AK_TRY(ensure_spare(ptr2, (size_t)(m->cap + 1) * 8));
-            AK_TRY(ensure_spare(src2, (size_t)nnz_new * 4));
-            AK_TRY(ensure_spare(aff2, (size_t)nnz_new * 4));
-            AK_TRY(ensure_spare(w2, (size_t)nnz_new * 4));
-            const size_t tb = radix_tmp_bytes(pairs) + 4096;
-            void *p_rows = store_scratch(m, SCR_IN_ROWS, (size_t)n * 16);
-            void *p_k = store_scratch(m, SCR_KEYS, (size_t)pairs * 4 + 16);
-            void *p_v = store_scratch(m, SCR_VALS, (size_t)pairs * 4 + 16);
-            void *p_k2 = store_scratch(m, SCR_KEYS2, (size_t)pairs * 4 + 16);
-            void *p_v2 = store_scratch(m, SCR_VALS2, (size_t)pairs * 4 + 16);
-            void *p_tmp = store_scratch(m, SCR_TMP, tb);
-            void *p_move = store_scratch(m, SCR_MOVE, (size_t)(1 + move_words(nnz_old, pairs, n)) * 4);
-            if (!p_rows || !p_move || !p_k || !p_v || !p_k2 || !p_v2 || !p_tmp)
-                return fail(AKASHIC_ENOMEM, "update: out of device memory");
+        if (patch) {
+            // old lists moved, new edges placed, weights recomputed from the
+            // logits (ak_inedges.cu)
             InEdgeUpdate u;
-            u.n = rows;
+            u.n = m->n;
             u.nnz_new = nnz_new;
             u.in_ptr_old = m->in_ptr.as<int64_t>();
             u.in_src_old = m->in_src.as<int32_t>();
@@ -849,25 +848,28 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
             u.n_new = n;
             u.M = M;
             u.reciprocal = reciprocal != 0;
-            u.row_bits = bits_for(rows - 1);
+            u.row_bits = bits_for(m->n - 1);
             u.row_of = m->row_of.as<int32_t>();
             u.ext_of = m->ext_of.as<int32_t>();
             u.rstat = m->rstat.as<float2>();
-            InEdgeScratch sc{(uint32_t *)p_k, (uint32_t *)p_v, (uint32_t *)p_k2, (uint32_t *)p_v2,
-                             (uint32_t *)p_rows, (uint32_t *)p_move, p_tmp, tb};
             CUDA_TRY(launch_in_edges_update(u, sc, st, &pt.launches));
-            std::swap(m->in_ptr.p, ptr2.p);
-            std::swap(m->in_ptr.cap, ptr2.cap);
-            std::swap(m->in_src.p, src2.p);
-            std::swap(m->in_src.cap, src2.cap);
-            std::swap(m->in_aff.p, aff2.p);
-            std::swap(m->in_aff.cap, aff2.cap);
-            std::swap(m->in_w.p, w2.p);
-            std::swap(m->in_w.cap, w2.cap);
+            swap_bufs(m->in_ptr, ptr2);
+            swap_bufs(m->in_src, src2);
+            swap_bufs(m->in_aff, aff2);
+            swap_bufs(m->in_w, w2);
+        }
+        swap_bufs(m->row_ptr, nrp);
+        swap_bufs(m->col, ncol);
+        swap_bufs(m->aff, naff);
+        swap_bufs(m->w, m->w2);
+        m->nnz = nnz_new;
+        if (patch) {
             pt.end();
             ph.launches += pt.launches;
             PhaseScope phub(m, AKASHIC_PHASE_HUB_PLAN, st);
             AK_TRY(build_split_plan(m, st));
+        } else {
+            AK_TRY(rebuild_in_edges(m, st));
         }
     }
     CUDA_TRY(cudaStreamSynchronize(st));
@@ -1011,18 +1013,14 @@ akashic_status_t akashic_mem_delete(akashic_mem_t *m, const int64_t *ids, int64_
                                  st));
     CUDA_TRY(cudaStreamSynchronize(st));
     m->nnz = nnz_new;
-    auto swap = [](DevBuf &x, DevBuf &y) {
-        std::swap(x.p, y.p);
-        std::swap(x.cap, y.cap);
-    };
-    swap(m->row_ptr, m->rp2);
-    swap(m->col, m->col2);
-    swap(m->aff, m->aff2);
-    swap(m->w, m->w2);
-    swap(m->in_ptr, m->in_ptr2);
-    swap(m->in_src, m->in_src2);
-    swap(m->in_aff, m->in_aff2);
-    swap(m->in_w, m->in_w2);
+    swap_bufs(m->row_ptr, m->rp2);
+    swap_bufs(m->col, m->col2);
+    swap_bufs(m->aff, m->aff2);
+    swap_bufs(m->w, m->w2);
+    swap_bufs(m->in_ptr, m->in_ptr2);
+    swap_bufs(m->in_src, m->in_src2);
+    swap_bufs(m->in_aff, m->in_aff2);
+    swap_bufs(m->in_w, m->in_w2);
     AK_TRY(build_split_plan(m, st));
     return check_status(m, st, "delete");
 }
