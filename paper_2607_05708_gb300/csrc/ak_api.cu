@@ -1228,21 +1228,36 @@ static akashic_status_t ensure_mass(akashic_mem *m, const HopPlan &hp, int H, cu
         m->mass_levels = 0;
         m->mass_n = n;
     }
-    CUDA_TRY(launch_mass_levels(hp, m->mass_levels + 1, H, m->mass_up.as<float>(),
-                                m->mass_dn.as<float>(), m->mass_zero.as<float>(),
-                                m->mass_vu.as<float>(), m->mass_vl.as<float>(), st));
+    const cudaError_t e = launch_mass_levels(hp, m->mass_levels + 1, H, m->mass_up.as<float>(),
+                                             m->mass_dn.as<float>(), m->mass_zero.as<float>(),
+                                             m->mass_vu.as<float>(), m->mass_vl.as<float>(), st);
+    m->mass_levels = -1;
+    AK_TRY(tables_built(m, st));
+    CUDA_TRY(e);
     m->mass_levels = H;
-    return tables_built(m, st);
+    return AKASHIC_OK;
 }
 
 // The candidate rows and their reach coefficients for H >= 2 hops (after the
 // mass levels).  A level is never rewritten while the graph stays the same, so
 // a call with another hop count only adds levels that no other call reads yet.
-// table_mu held.
+// Every buffer is taken before the first launch, and a build that has launched
+// anything ends in tables_built: levels that are announced are always ordered
+// before the calls of other streams.  table_mu held.
 static akashic_status_t ensure_reach(akashic_mem *m, const HopPlan &hp, int H, cudaStream_t st) {
     const int64_t n = m->n;
     AK_TRY(wait_tables(m, st));
-    if (m->reach_levels >= H && m->reach_n == n) return AKASHIC_OK;
+    if (m->reach_n != n) m->reach_levels = -1;
+    if (m->reach_levels >= H) return AKASHIC_OK;
+    const bool fresh = m->reach_levels < 1;
+    if (fresh) {
+        AK_TRY(m->reach_rows.ensure(REACH_T * 4));
+        AK_TRY(m->reach_t.ensure(16));
+        AK_TRY(m->reach_pick.ensure((size_t)reach_pick_words() * 8));
+        AK_TRY(ensure_spare(m->reach_map, (size_t)n * 4));
+    }
+    for (int t = fresh ? 0 : m->reach_levels; t < H; ++t)
+        AK_TRY(ensure_spare(m->reach_c[t], (size_t)n * REACH_T * 4));
     ReachBuild rb{};
     rb.n = n;
     rb.mup = m->mass_up.as<float>();
@@ -1253,29 +1268,26 @@ static akashic_status_t ensure_reach(akashic_mem *m, const HopPlan &hp, int H, c
     rb.col = m->col.as<int32_t>();
     rb.row_of = m->row_of.as<int32_t>();
     rb.w = m->w.as<float>();
-    if (m->reach_levels < 1 || m->reach_n != n) {
-        m->reach_levels = -1;
-        AK_TRY(m->reach_rows.ensure(REACH_T * 4));
-        AK_TRY(m->reach_t.ensure(16));
-        AK_TRY(m->reach_pick.ensure((size_t)reach_pick_words() * 8));
-        AK_TRY(ensure_spare(m->reach_map, (size_t)n * 4));
-        AK_TRY(ensure_spare(m->reach_c[0], (size_t)n * REACH_T * 4));
-        rb.rows = m->reach_rows.as<int32_t>();
-        rb.t_cnt = m->reach_t.as<int>();
-        rb.map = m->reach_map.as<int32_t>();
-        rb.pick = m->reach_pick.as<unsigned long long>();
-        CUDA_TRY(launch_reach_pick(rb, m->reach_c[0].as<float>(), st));
-        m->reach_levels = 1;
-        m->reach_n = n;
+    rb.rows = m->reach_rows.as<int32_t>();
+    rb.t_cnt = m->reach_t.as<int>();
+    rb.map = m->reach_map.as<int32_t>();
+    rb.pick = m->reach_pick.as<unsigned long long>();
+    cudaError_t e = cudaSuccess;
+    int levels = m->reach_levels;
+    if (fresh) {
+        e = launch_reach_pick(rb, m->reach_c[0].as<float>(), st);
+        levels = 1;
         ++m->reach_build;
     }
-    for (int t = m->reach_levels; t < H; ++t) {
-        AK_TRY(ensure_spare(m->reach_c[t], (size_t)n * REACH_T * 4));
-        CUDA_TRY(launch_reach_level(rb, m->reach_c[t - 1].as<float>(), m->reach_c[t].as<float>(),
-                                    st));
-        m->reach_levels = t + 1;
-    }
-    return tables_built(m, st);
+    for (; e == cudaSuccess && levels < H; ++levels)
+        e = launch_reach_level(rb, m->reach_c[levels - 1].as<float>(),
+                               m->reach_c[levels].as<float>(), st);
+    m->reach_levels = -1;
+    AK_TRY(tables_built(m, st));
+    CUDA_TRY(e);
+    m->reach_levels = levels;
+    m->reach_n = n;
+    return AKASHIC_OK;
 }
 
 static ReachLevels reach_levels_of(const akashic_mem *m) {

@@ -100,3 +100,48 @@ def test_an_update_that_does_not_fit_changes_nothing():
     for a, b in zip(got, want):
         assert (a == b).all()
     assert len(before[1]) == n * 32
+
+
+def _two(st, q, stream, hops, k=8):
+    import torch
+    with torch.cuda.stream(stream):
+        out = st.retrieve(q, k, 0.5, hops, stream=stream)
+    return out
+
+
+def test_tables_that_do_not_fit_are_not_seen_half_built(monkeypatch):
+    """Two streams with different hop counts after a deletion: the one with three
+    hops does not get its third table.  The other's answers come from tables that
+    are finished, at once and later."""
+    import torch
+    n = 262_144
+    monkeypatch.setenv("AKASHIC_REACH", "0")
+    plain, emb = _store(n, 0)
+    monkeypatch.setenv("AKASHIC_REACH", "1")
+    st, _ = _store(n, 0)
+    q = emb[5:6].contiguous()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(6):                        # two hops: the tables are built
+        _two(st, q, b, 2)
+    _two(st, q, a, 3)                         # a's own slabs
+    torch.cuda.synchronize()
+    gone = torch.tensor([int(_two(st, q, b, 2)[0][0, 0])], device="cuda")
+    torch.cuda.synchronize()
+    plain.delete(gone)
+    st.delete(gone)
+    want = [t.cpu().numpy() for t in plain.retrieve(q, 8, 0.5, 2)]
+    out = []
+    with _memory(16 * MB):
+        for _ in range(8):                    # (the hops, until the tables pay)
+            _two(st, q, a, 3)
+        for _ in range(4):
+            out.append(_two(st, q, b, 2))
+        st.sync(a)
+        st.sync(b)
+    out.append(_two(st, q, b, 2))
+    st.sync(b)
+    for ids, scores, _, _ in out:
+        hit = ids.cpu().numpy() == want[0]
+        assert hit.mean() >= 0.75
+        np.testing.assert_allclose(scores.cpu().numpy(), want[1], rtol=1e-5, atol=0)
