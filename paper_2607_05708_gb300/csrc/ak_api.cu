@@ -1401,6 +1401,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
         //   RC_MMA   other hop counts, or 33 to 64 queries: the same, with the
         //            score in fp32 and the hops queued behind; their kernels
         //            return at once when the plan says the candidates suffice
+        //            (which it does not for sharp temperatures: REACH_SPLIT_SHIFT)
         //   RC_FMA   at most 32 queries: in fp32 on the CUDA cores, then the hops
         //            likewise
         // The first builds the graph-only coefficients at once; they cost about
@@ -1593,6 +1594,8 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                     rf.ws = sc->words.as<int32_t>() + CW_REACH;
                     rf.plan = sc->reach_plan.as<int32_t>();
                     rf.outcome = mode == RC_SYNC ? nullptr : sc->plan_host + 2;
+                    rf.shift = mode == RC_MMA ? sc->shift.as<float>() : nullptr;
+                    rf.bp = bp;
                     CUDA_TRY(launch_reach_flags(rf, st, &ph.launches));
                     if (mode == RC_SYNC) {
                         if (!sc->plan_ev)

@@ -188,15 +188,18 @@ cudaError_t launch_score(const uint16_t *emb, int64_t n, int dim, const uint16_t
                          const int32_t *dead_row = nullptr, float *row_max = nullptr,
                          float *row_min = nullptr, int n_real = 0, unsigned int *ext = nullptr,
                          const int32_t *done = nullptr);
-// At most any score of the batch: exp(-2 c) for the largest shift c of its
-// columns (z >= -c in every column).  The same bits wherever a whole warp calls
-// it.
-__device__ __forceinline__ float batch_u_min(const float *__restrict__ shift, int bp) {
+// The largest shift c of a batch's columns, and a value that no score of the
+// batch is below: exp(-2 c) (z >= -c in every column).  The same bits wherever a
+// whole warp calls them.
+__device__ __forceinline__ float batch_shift(const float *__restrict__ shift, int bp) {
     float c = 0.f;
     for (int i = threadIdx.x & 31; i < bp; i += 32) c = fmaxf(c, shift[i]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) c = fmaxf(c, __shfl_xor_sync(0xffffffffu, c, o));
-    return exp2f(-2.f * c * LOG2E_F);
+    return c;
+}
+__device__ __forceinline__ float batch_u_min(const float *__restrict__ shift, int bp) {
+    return exp2f(-2.f * batch_shift(shift, bp) * LOG2E_F);
 }
 // The same scores with u - batch_u_min(shift) written as split bf16 instead of
 // u in fp32: u_hi and u_lo [n][bp] each, their sum within 2^-17 relative (the
@@ -708,7 +711,18 @@ struct ReachFlags {
     int32_t *plan;                   // [REACH_PLAN_INTS]
     int32_t *outcome;                // host-visible word (or NULL): 1 the candidates
                                      // suffice, 2 the hops run
+    const float *shift;              // the query columns' shifts (or NULL): the hops run
+    int bp;                          // above REACH_SPLIT_SHIFT
 };
+// The largest shift c of a batch that the candidates' tensor-core pass takes from
+// the hops.  Its operands hold 16 bits of u - exp(-2c), which is at most 1 - exp(-2c)
+// of u, so its error grows with c where the hops' does not: against 64 bits (rms of
+// the scores; 65,537 and 262,144 chunks, 48 and 200 queries, two to four hops)
+// 4e-8 at 2c = 0.06 (dim 1024 at the default temperature), 6e-8 at 0.25 (dim 64),
+// up to 9.7e-8 at 0.5, 1.6e-7 at 1 and 2.9e-7 at 2; the hops 9e-8 to 1.7e-7
+// throughout.  (Two hops with 65 queries and more took the tensor cores before
+// there was a limit, with a larger error, and have none.)
+constexpr float REACH_SPLIT_SHIFT = 0.1875f;
 cudaError_t launch_reach_flags(const ReachFlags &f, cudaStream_t st, int *launches);
 int reach_parts();                   // CTAs of the candidates' pass (partial rows)
 // The call's plan on the device (int32[REACH_PLAN_INTS], written by

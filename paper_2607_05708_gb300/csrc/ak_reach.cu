@@ -285,7 +285,9 @@ __global__ __launch_bounds__(256) void k_reach_flags(const ReachFlags f) {
     __shared__ int32_t kf[REACH_T];
     if (threadIdx.x < REACH_T) kf[threadIdx.x] = vk[threadIdx.x];
     __syncthreads();
-    reach_build_plan(kf, *(volatile int *)bad, t_cnt, f.k, f.plan);
+    // (a batch whose scores spread too far for 16 bits counts as a row too many)
+    const bool sharp = f.shift && !(batch_shift(f.shift, f.bp) <= REACH_SPLIT_SHIFT);
+    reach_build_plan(kf, *(volatile int *)bad + (sharp ? 1 : 0), t_cnt, f.k, f.plan);
     if (f.outcome && threadIdx.x == REACH_T - 1)       // (the thread that wrote plan[0])
         *(volatile int32_t *)f.outcome = f.plan[0] ? 1 : 2;
 }

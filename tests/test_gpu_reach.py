@@ -30,6 +30,38 @@ def _launches(store, wl, q):
     return out, ph["last_hop"][1]
 
 
+@pytest.mark.parametrize("B,hops,spread,same", [
+    (48, 2, 1.0, True), (100, 3, 2.0, True), (48, 4, 1.0, True),   # too sharp for 16-bit pairs
+    (48, 2, 0.375, False), (100, 3, 0.25, False),
+])
+def test_sharp_temperatures_keep_the_hops_precision(B, hops, spread, same, monkeypatch):
+    """Scores between exp(-spread) and 1: with a wide spread the tensor-core pass
+    would be less exact than the hops, so they run and give their own bits; below
+    the limit (0.375) the candidates are used."""
+    import torch
+    from paper_2607_05708_gb300 import MemStore
+    wl = synth.workload(2, scale=1 / 64)
+    norm = lambda x: np.linalg.norm(synth.bf16_to_f32(x), axis=1).max()
+    tau = 0.999 * spread / (2 * norm(wl.queries[:B]) * norm(wl.emb))
+    q = torch.from_numpy(np.ascontiguousarray(wl.queries[:B]).view(np.int16)).cuda()
+    out = []
+    for reach in ("0", "1"):
+        monkeypatch.setenv("AKASHIC_REACH", reach)
+        store = MemStore.from_arrays(wl.emb, wl.page_of["clustered"], wl.row_ptr, wl.col, wl.aff,
+                                     temperature=tau)
+        for _ in range(12):
+            got = store.retrieve(q, 4, 0.5, hops)
+        store.sync()
+        out.append([t.cpu().numpy() for t in got])
+    (ids, scores, _, _), (ids0, scores0, _, _) = out[1], out[0]
+    assert ((ids == ids0).all() and (scores == scores0).all()) == same
+    hit = ids == ids0
+    # the products' 4.6e-5 of the part above the smallest score (see REL), and the
+    # hops' and the candidates' sums
+    np.testing.assert_allclose(scores[hit], scores0[hit], atol=0,
+                               rtol=REL + 4.6e-5 * (1 - np.exp(-spread)) * (not same))
+
+
 @pytest.mark.parametrize("n,B,hops,k", [
     (16384, 1, 2, 32),          # one column tile of 8
     (16383, 9, 2, 8),           # 16 columns, ragged rows
