@@ -144,12 +144,20 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
  * Does not synchronise, with one exception: with hops = 2, alpha > 0, no
  * scope and 65 to 256 queries in a batch of 128 or 256, the host waits once
  * per batch for the device's decision between the two-hop path from reach
- * coefficients and the hops (an event recorded after a 12-byte copy, not the
+ * coefficients and the hops (an event recorded after an 8-byte copy, not the
  * whole stream; the candidates' pass is already queued behind it, so the
  * GPU does not idle).  The other calls with two to four hops decide on the
  * device.
  * Graph-only tables built by a call on one stream are waited for (an event,
- * not a host wait) by calls on every other stream. */
+ * not a host wait) by calls on every other stream.
+ * The two paths round differently, so scores may differ in their last bits, and
+ * chunks of nearly equal score in their order, between calls that take one and
+ * the other.  Which one a call takes follows from the store and the calls made
+ * before it, not from when those finish: calls with two to four hops (but two
+ * hops with 65 queries and more) run the hops until these have cost as much as
+ * the tables since the graph last changed; a call that the candidates do not
+ * suffice for is followed by 15 of the same alpha, hops, k and width on its
+ * stream that run the hops. */
 akashic_status_t akashic_mem_retrieve(akashic_mem_t *m, const uint16_t *q, int32_t B, int32_t k,
                                       float alpha, int32_t hops, int64_t *ids, float *scores,
                                       int32_t *page_ids, int32_t *n_pages, void *stream);

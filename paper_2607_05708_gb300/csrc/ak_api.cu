@@ -85,9 +85,10 @@ static void swap_bufs(DevBuf &x, DevBuf &y) {
 }
 
 // Words of StreamScratch::words: u's extremes [2], the kept lists' lengths
-// (int64 [2]), the hops' work queues ([2] a hop), the candidates' flags.
+// (int64 [2]), the hops' work queues ([2] a hop), the candidates' flags, whether
+// this call skips the candidates.
 constexpr int CW_EXT = 0, CW_KEPT = 2, CW_QUEUE = 6, CW_REACH = CW_QUEUE + 2 * AKASHIC_MAX_HOPS,
-              CW_COUNT = CW_REACH + REACH_WS;
+              CW_SKIP = CW_REACH + REACH_WS, CW_COUNT = CW_SKIP + 1;
 
 struct StreamScratch {
     DevBuf qp, shift, u, sa, sb, zpart, partial, cand;
@@ -109,14 +110,41 @@ struct StreamScratch {
     // their copy (the host waits for that point only)
     int32_t *plan_host = nullptr;
     cudaEvent_t plan_ev = nullptr;
-    // the fp32 pass: the combined coefficients and their key; the last
-    // attempt's outcome (plan_host[2], written by the device) and its key
+    // the fp32 pass: the combined coefficients and their key
     DevBuf coef_f, cf_sum;
     int64_t no_room_n = -1;      // rows at which the tables did not fit
-    uint64_t cf_build = ~0ull, try_build = ~0ull;
-    float cf_alpha = -1.f, try_alpha = -1.f;
-    int cf_H = 0, try_H = 0, try_k = 0, try_skip = 0;
-    int64_t cf_n = -1, try_n = -1;
+    uint64_t cf_build = ~0ull;
+    float cf_alpha = -1.f;
+    int cf_H = 0;
+    int64_t cf_n = -1;
+    // the calls that could use the candidates, by key (try_skips): a key's number
+    // and theirs; its mark on the device and the copy the host sees
+    struct TryKey {
+        uint64_t build = ~0ull, used = 0;
+        int64_t n = -1;
+        float alpha = -1.f;
+        int H = 0, k = 0, mode = 0;
+        uint32_t number = 0, calls = 0;
+    };
+    static constexpr int TRY_KEYS = 8;
+    TryKey keys[TRY_KEYS];
+    uint32_t key_numbers = 0;
+    uint64_t key_uses = 0;
+    DevBuf tried;                // [TRY_KEYS]
+    unsigned long long *told = nullptr;
+    TryKey &try_key(uint64_t build, int64_t n, float alpha, int H, int k, int mode) {
+        TryKey *at = keys;
+        for (TryKey &t : keys) {
+            if (t.build == build && t.n == n && t.alpha == alpha && t.H == H && t.k == k &&
+                t.mode == mode && t.calls < (1u << 30)) {
+                t.used = ++key_uses;
+                return t;
+            }
+            if (t.used < at->used) at = &t;
+        }
+        *at = TryKey{build, ++key_uses, n, alpha, H, k, mode, ++key_numbers, 0};
+        return *at;
+    }
     ~StreamScratch() {
         if (plan_host) cudaFreeHost(plan_host);
         if (plan_ev) cudaEventDestroy(plan_ev);
@@ -1296,11 +1324,15 @@ static ReachLevels reach_levels_of(const akashic_mem *m) {
     return c;
 }
 
-// The pinned words a stream's plans are read back through.
-static akashic_status_t plan_words(StreamScratch *sc) {
+// The pinned words a stream's plans are read back through, and its marks.
+static akashic_status_t plan_words(StreamScratch *sc, cudaStream_t st) {
     if (sc->plan_host) return AKASHIC_OK;
-    CUDA_TRY(cudaMallocHost((void **)&sc->plan_host, 16));
-    memset(sc->plan_host, 0, 16);
+    constexpr size_t marks = StreamScratch::TRY_KEYS * sizeof(unsigned long long);
+    AK_TRY(sc->tried.ensure(marks));
+    CUDA_TRY(cudaMemsetAsync(sc->tried.p, 0, marks, st));
+    CUDA_TRY(cudaMallocHost((void **)&sc->plan_host, 16 + marks));
+    memset(sc->plan_host, 0, 16 + marks);
+    sc->told = (unsigned long long *)(sc->plan_host + 4);
     return AKASHIC_OK;
 }
 
@@ -1413,6 +1445,8 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
         // 262,147 chunks, 24 queries 384 -> 142; 262,144 chunks, 200 queries, three
         // hops 1589 -> 237 (564 in fp32).
         enum { RUN_HOPS, RC_SYNC, RC_MMA, RC_FMA } mode = RUN_HOPS;
+        unsigned long long now = 0;   // this call's number, and where its key's mark
+        int mark = 0;                 // stands (RC_MMA, RC_FMA)
         if (bounds) {
             std::lock_guard<std::mutex> lk(m->table_mu);
             AK_TRY(ensure_mass(m, hp, eff_hops, st));
@@ -1449,29 +1483,15 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                         sc->no_room_n = n;   // not again on this stream at this size
                     }
                 }
-                // where the candidates did not suffice (the device has said so
-                // by now, or has not yet), the next 15 calls like it run the
-                // hops alone
+                // where the candidates did not suffice, the next calls like it
+                // run the hops alone (try_skips)
                 if (go) {
-                    AK_TRY(plan_words(sc));
-                    volatile int32_t *outcome = sc->plan_host + 2;
-                    if (sc->try_build != m->reach_build || sc->try_alpha != alpha ||
-                        sc->try_H != eff_hops || sc->try_k != k || sc->try_n != n) {
-                        sc->try_build = m->reach_build;
-                        sc->try_alpha = alpha;
-                        sc->try_H = eff_hops;
-                        sc->try_k = k;
-                        sc->try_n = n;
-                        sc->try_skip = 0;
-                        *outcome = 0;
-                    } else if (sc->try_skip > 0) {
-                        --sc->try_skip;
-                        go = false;
-                    } else if (*outcome == 2) {
-                        sc->try_skip = 14;
-                        *outcome = 0;
-                        go = false;
-                    }
+                    AK_TRY(plan_words(sc, st));
+                    StreamScratch::TryKey &t = sc->try_key(m->reach_build, n, alpha, eff_hops, k,
+                                                           bp == 32 ? RC_FMA : RC_MMA);
+                    mark = (int)(&t - sc->keys);
+                    now = ((unsigned long long)t.number << 32) | t.calls++;
+                    go = !try_skips(((volatile unsigned long long *)sc->told)[mark], now);
                 }
                 if (go) mode = bp == 32 ? RC_FMA : RC_MMA;
             }
@@ -1480,6 +1500,9 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
         // which the score GEMM writes in the bytes of the fp32 slab (hi [n][bp],
         // then lo [n][bp])
         const bool split_u = mode == RC_SYNC || mode == RC_MMA;
+        // (the hops queued behind; the call's word says whether to skip the rest)
+        const bool queued = mode == RC_MMA || mode == RC_FMA;
+        const int32_t *skip = queued ? sc->words.as<int32_t>() + CW_SKIP : nullptr;
         uint16_t *u_hi = split_u ? sc->u.as<uint16_t>() : nullptr;
         uint16_t *u_lo = split_u ? u_hi + (size_t)n * bp : nullptr;
         auto score_fp32 = [&](int *launches, const int32_t *done) -> cudaError_t {
@@ -1499,7 +1522,9 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                                          sc->qp.as<uint16_t>(), sc->shift.as<float>(),
                                          m->status.as<int>(), st,
                                          sc->words.as<unsigned int>(),
-                                         eff_hops >= 1 ? CW_COUNT : 0));
+                                         eff_hops >= 1 ? CW_COUNT : 0, CW_SKIP,
+                                         queued ? sc->tried.as<unsigned long long>() + mark : nullptr,
+                                         now));
             ph.launches += 1;
             if (split_u)
                 CUDA_TRY(launch_score_split(m->emb.as<uint16_t>(), n, m->dim,
@@ -1507,7 +1532,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                                             m->tau, u_hi, u_lo, sc->zpart.as<float>(),
                                             m->status.as<int>(), st, &ph.launches, &zrows, ns.dead,
                                             sc->rmax_u.as<float>(), sc->rmin_u.as<float>(), b,
-                                            ext));
+                                            ext, skip));
             else if (!dense_fused)
                 CUDA_TRY(score_fp32(&ph.launches, nullptr));
         }
@@ -1576,7 +1601,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
             if (mode != RUN_HOPS) {
                 {
                     PhaseScope ph(m, AKASHIC_PHASE_BOUND, st);
-                    AK_TRY(plan_words(sc));
+                    AK_TRY(plan_words(sc, st));
                     AK_TRY(sc->reach_plan.ensure(REACH_PLAN_INTS * 4));
                     ReachFlags rf{};
                     rf.u0 = rb.u0;
@@ -1593,7 +1618,12 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                     rf.t_cnt = m->reach_t.as<int>();
                     rf.ws = sc->words.as<int32_t>() + CW_REACH;
                     rf.plan = sc->reach_plan.as<int32_t>();
-                    rf.outcome = mode == RC_SYNC ? nullptr : sc->plan_host + 2;
+                    rf.skip = skip;
+                    if (queued) {
+                        rf.tried = sc->tried.as<unsigned long long>() + mark;
+                        rf.told = sc->told + mark;
+                        rf.again = now + TRY_AGAIN;
+                    }
                     rf.shift = mode == RC_MMA ? sc->shift.as<float>() : nullptr;
                     rf.bp = bp;
                     CUDA_TRY(launch_reach_flags(rf, st, &ph.launches));

@@ -209,7 +209,8 @@ cudaError_t launch_score_split(const uint16_t *emb, int64_t n, int dim, const ui
                                const float *shift, float tau, uint16_t *u_hi, uint16_t *u_lo,
                                float *zpart, int *status, cudaStream_t st, int *launches,
                                int *zrows, const int32_t *dead_row, float *row_max,
-                               float *row_min, int n_real, unsigned int *ext);
+                               float *row_min, int n_real, unsigned int *ext,
+                               const int32_t *done);
 
 // The score on every stride-th row only: out[v, c] = u[v*stride, c] for
 // v < n_sample (same kernel and arithmetic as launch_score, so the values
@@ -258,11 +259,26 @@ cudaError_t launch_dots_keys_t(const uint16_t *emb, int64_t n, int64_t row_strid
 
 // Query preparation: pad q (b rows) to bp rows of zeros and compute
 // shift[c] = tau * |q_c| * max_norm (0 for padding); flags ERANGE.
-// zero (or NULL): n_zero words set to 0 (the call's counters).
+// zero (or NULL): n_zero words set to 0 (the call's counters), but zero[skip_at]
+// (where tried is given) to 1 if the mark *tried says to skip call `now`.
 cudaError_t launch_prep_queries(const uint16_t *q, int b, int bp, int dim, float tau,
                                 const float *max_norm, uint16_t *qp, float *shift, int *status,
                                 cudaStream_t st, unsigned int *zero = nullptr,
-                                int n_zero = 0);
+                                int n_zero = 0, int skip_at = 0,
+                                const unsigned long long *tried = nullptr,
+                                unsigned long long now = 0);
+// When calls on a stream try the candidates.  The calls with one key (graph,
+// alpha, hops, k) since it last changed are numbered; a mark is (key's number <<
+// 32 | call's number).  Where the candidates do not suffice for a call, the
+// device leaves the mark of the next call to try them, TRY_AGAIN calls later, and
+// those before it run the hops alone.  So what a call does follows from the calls
+// before it and never from when they end.  The host reads the mark too, as it
+// stands, to spare the launches that a skipping call's kernels would return from.
+constexpr unsigned int TRY_AGAIN = 16;
+__host__ __device__ __forceinline__ bool try_skips(unsigned long long tried,
+                                                   unsigned long long now) {
+    return (tried >> 32) == (now >> 32) && tried > now;
+}
 
 // Running maximum of row norms of emb[0..n) into *max_norm (monotone).
 cudaError_t launch_row_norm_max(const uint16_t *emb, int64_t n, int dim, float *max_norm,
@@ -709,8 +725,9 @@ struct ReachFlags {
     const int *t_cnt;                // candidates (device)
     int32_t *ws;
     int32_t *plan;                   // [REACH_PLAN_INTS]
-    int32_t *outcome;                // host-visible word (or NULL): 1 the candidates
-                                     // suffice, 2 the hops run
+    const int32_t *skip;             // or NULL: with skip[0] = 1 the hops run, unseen
+    unsigned long long *tried, *told;    // or NULL: where the candidates do not
+    unsigned long long again;            // suffice get the mark `again` (told: host)
     const float *shift;              // the query columns' shifts (or NULL): the hops run
     int bp;                          // above REACH_SPLIT_SHIFT
 };

@@ -221,6 +221,10 @@ __global__ __launch_bounds__(256) void k_reach_flags(const ReachFlags f) {
     __shared__ float floor_s;
     __shared__ unsigned int lb_s[REACH_T];
     griddep_wait();
+    if (f.skip && f.skip[0] == 1) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) f.plan[0] = 0;
+        return;
+    }
     int32_t *keep = f.ws, *bad = f.ws + REACH_T, *done = f.ws + REACH_T + 1;
     const int t_cnt = *f.t_cnt;
     {
@@ -288,8 +292,10 @@ __global__ __launch_bounds__(256) void k_reach_flags(const ReachFlags f) {
     // (a batch whose scores spread too far for 16 bits counts as a row too many)
     const bool sharp = f.shift && !(batch_shift(f.shift, f.bp) <= REACH_SPLIT_SHIFT);
     reach_build_plan(kf, *(volatile int *)bad + (sharp ? 1 : 0), t_cnt, f.k, f.plan);
-    if (f.outcome && threadIdx.x == REACH_T - 1)       // (the thread that wrote plan[0])
-        *(volatile int32_t *)f.outcome = f.plan[0] ? 1 : 2;
+    if (f.tried && threadIdx.x == REACH_T - 1 && f.plan[0] == 0) {   // (it wrote plan[0])
+        *f.tried = f.again;
+        *(volatile unsigned long long *)f.told = f.again;
+    }
 }
 
 cudaError_t launch_reach_flags(const ReachFlags &f, cudaStream_t st, int *launches) {

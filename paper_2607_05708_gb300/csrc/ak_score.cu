@@ -17,11 +17,14 @@ template <bool VEC>
 __global__ void k_prep_queries(const uint16_t *__restrict__ q, int b, int dim, float tau,
                                const float *__restrict__ max_norm, uint16_t *__restrict__ qp,
                                float *__restrict__ shift, int *status,
-                               unsigned int *__restrict__ zero, int n_zero) {
+                               unsigned int *__restrict__ zero, int n_zero, int skip_at,
+                               const unsigned long long *__restrict__ tried,
+                               unsigned long long now) {
     griddep_wait();
     const int c = blockIdx.x;
     if (c == 0)
-        for (int i = threadIdx.x; i < n_zero; i += blockDim.x) zero[i] = 0u;
+        for (int i = threadIdx.x; i < n_zero; i += blockDim.x)
+            zero[i] = tried && i == skip_at && try_skips(*tried, now) ? 1u : 0u;
     __shared__ float red[32];
     float ss = 0.f;
     if constexpr (VEC) {
@@ -60,12 +63,13 @@ __global__ void k_prep_queries(const uint16_t *__restrict__ q, int b, int dim, f
 
 cudaError_t launch_prep_queries(const uint16_t *q, int b, int bp, int dim, float tau,
                                 const float *max_norm, uint16_t *qp, float *shift, int *status,
-                                cudaStream_t st, unsigned int *zero, int n_zero) {
+                                cudaStream_t st, unsigned int *zero, int n_zero, int skip_at,
+                                const unsigned long long *tried, unsigned long long now) {
     if (n_zero < 0 || (n_zero > 0 && !zero)) return cudaErrorInvalidValue;
     const bool vec = ((uintptr_t)q & 15) == 0 && dim % 8 == 0;
     cudaError_t e = launch_pdl(vec ? k_prep_queries<true> : k_prep_queries<false>, dim3(bp),
                                dim3(128), 0, st, q, b, dim, tau, max_norm, qp, shift, status,
-                               zero, n_zero);
+                               zero, n_zero, skip_at, tried, now);
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
@@ -930,8 +934,10 @@ cudaError_t launch_score_split(const uint16_t *emb, int64_t n, int dim, const ui
                                const float *shift, float tau, uint16_t *u_hi, uint16_t *u_lo,
                                float *zpart, int *status, cudaStream_t st, int *launches,
                                int *zrows, const int32_t *dead_row, float *row_max,
-                               float *row_min, int n_real, unsigned int *ext) {
+                               float *row_min, int n_real, unsigned int *ext,
+                               const int32_t *done) {
     GemmEpi ep{};
+    ep.done = done;
     ep.dead_row = dead_row;
     ep.row_max = row_max;
     ep.row_min = row_min;

@@ -100,20 +100,59 @@ def test_equals_the_hops(n, B, hops, k, monkeypatch):
 
 
 def test_candidates_that_do_not_suffice():
-    """300 rows of equal in-weight above the split limit: more rows reach the
-    floor than there are candidates, so every call goes through the hops."""
+    """304 rows of the same in-weight above the split limit, and no links among them:
+    more rows reach the floor than there are candidates, so every call goes through
+    the hops."""
     base = synth.workload(2, scale=1 / 64)
     n = base.n
     rng = np.random.default_rng(3)
-    hubs = np.sort(rng.choice(n, 300, replace=False))
-    col = np.sort(np.stack([rng.permutation(hubs)[:8] for _ in range(n)]), axis=1)
-    ok = col != np.arange(n)[:, None]
-    rp = np.concatenate([[0], np.cumsum(ok.sum(1))]).astype(np.int64)
-    wl = dataclasses.replace(base, row_ptr=rp, col=col[ok].astype(np.int32),
-                             aff=np.zeros(int(ok.sum()), np.float32), k=16, hops=2)
+    hubs = rng.choice(n, 304, replace=False)
+    col = np.sort(hubs[(np.arange(8 * n) % 304).reshape(n, 8)], axis=1)   # 431 each, +-1
+    ok = ~np.isin(np.arange(n), hubs)
+    rp = np.concatenate([[0], np.cumsum(8 * ok)]).astype(np.int64)
+    wl = dataclasses.replace(base, row_ptr=rp, col=col[ok].astype(np.int32).ravel(),
+                             aff=np.zeros(8 * int(ok.sum()), np.float32), k=16, hops=2)
     q = wl.queries[:20]
     store = gpu_store(wl, "clustered")
     ref = oracle_retrieve(wl, "clustered", queries=q)
-    for _ in range(24):
-        _, got = gpu_retrieve(wl, "clustered", store=store, queries=q)
+    seen = []
+    for _ in range(40):
+        got, launches = _launches(store, wl, q)
         assert_retrieval_parity(wl, "clustered", got, ref)
+        seen.append(launches)
+    # the hops until they have cost as much as the tables (192 columns x hops, 64 a
+    # call); the candidates tried (first combined, two launches more), the hops run
+    # behind them; 15 calls of hops alone
+    assert seen == ([2] * 3 + [7] + [2] * 15 + ([5] + [2] * 15) * 2)[:40], seen
+
+
+def test_the_path_does_not_depend_on_timing():
+    """Batches whose candidates suffice and batches (too sharp) whose do not, under
+    one key: enqueued at once they take the paths that they take one by one."""
+    import torch
+    from paper_2607_05708_gb300 import MemStore
+    wl = synth.workload(2, scale=1 / 64)
+    norm = lambda x: np.linalg.norm(synth.bf16_to_f32(x), axis=1).max()
+    soft = wl.queries[:48]
+    sharp = synth.to_bf16(2 * synth.bf16_to_f32(soft))
+    tau = 0.25 / (2 * norm(soft) * norm(wl.emb))             # 0.25 and 0.5 about 0.375
+    qs = [torch.from_numpy(np.ascontiguousarray(x).view(np.int16)).cuda() for x in (soft, sharp)]
+    turns = np.random.default_rng(5).random(60) < 0.15       # True: the sharp one
+    out = []
+    for wait in (True, False):
+        store = MemStore.from_arrays(wl.emb, wl.page_of["clustered"], wl.row_ptr, wl.col, wl.aff,
+                                     temperature=tau)
+        bufs = [(torch.empty((48, 4), dtype=torch.int64, device="cuda"),
+                 torch.empty((48, 4), device="cuda")) for _ in turns]
+        torch.cuda.synchronize()
+        for t, (ids, scores) in zip(turns, bufs):
+            store.retrieve(qs[int(t)], 4, 0.5, 2, ids=ids, scores=scores)
+            if wait:
+                store.sync()
+        store.sync()
+        out.append([(i.cpu().numpy(), s.cpu().numpy()) for i, s in bufs])
+    for (i0, s0), (i1, s1) in zip(*out):
+        assert (i0 == i1).all() and (s0 == s1).all()
+    # both paths were taken by the soft batch
+    bits = {s.tobytes() for (_, s), t in zip(out[0], turns) if not t}
+    assert len(bits) == 2
