@@ -157,7 +157,12 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
  * hops with 65 queries and more) run the hops until these have cost as much as
  * the tables since the graph last changed; a call that the candidates do not
  * suffice for is followed by 15 of the same alpha, hops, k and width on its
- * stream that run the hops. */
+ * stream that run the hops.
+ * The tables take 512 bytes a chunk and hop for the store, and 512 a chunk for
+ * each stream and form of it that uses them.  They are taken only while as much
+ * device memory stays free (two hops with 65 queries and more: while there is
+ * room), else the hops run; and they are freed when another allocation of the
+ * store or of its retrievals does not fit and no call is using them. */
 akashic_status_t akashic_mem_retrieve(akashic_mem_t *m, const uint16_t *q, int32_t B, int32_t k,
                                       float alpha, int32_t hops, int64_t *ids, float *scores,
                                       int32_t *page_ids, int32_t *n_pages, void *stream);

@@ -7,6 +7,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <atomic>
 #include <mutex>
 #include <string>
 #include <unordered_map>
@@ -47,11 +48,24 @@ static akashic_status_t fail(akashic_status_t st, const char *fmt, ...) {
     } while (0)
 
 // ------------------------------------------------------------------ device buffers
+// The store whose reach tables an allocation of this thread may have freed when
+// the device has no room for it (Reclaim; release_tables frees them, if it can).
+static thread_local akashic_mem *g_reclaim = nullptr;
+static bool release_tables(akashic_mem *m);
+struct Reclaim {
+    akashic_mem *prev = g_reclaim;
+    explicit Reclaim(akashic_mem *m) { g_reclaim = m; }
+    ~Reclaim() { g_reclaim = prev; }
+};
+
 struct DevBuf {
     void *p = nullptr;
     size_t cap = 0;
-    ~DevBuf() {
+    ~DevBuf() { release(); }
+    void release() {
         if (p) cudaFree(p);
+        p = nullptr;
+        cap = 0;
     }
     // Grow to at least `bytes`; contents are not preserved unless keep.
     akashic_status_t ensure(size_t bytes, bool keep = false, cudaStream_t st = 0) {
@@ -59,6 +73,10 @@ struct DevBuf {
         size_t want = bytes < 256 ? 256 : bytes;
         void *q = nullptr;
         cudaError_t e = cudaMalloc(&q, want);
+        if (e == cudaErrorMemoryAllocation && g_reclaim) {
+            cudaGetLastError();
+            if (release_tables(g_reclaim)) e = cudaMalloc(&q, want);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(AKASHIC_ENOMEM, "device allocation of %zu bytes failed", want);
@@ -112,7 +130,7 @@ struct StreamScratch {
     cudaEvent_t plan_ev = nullptr;
     // the fp32 pass: the combined coefficients and their key
     DevBuf coef_f, cf_sum;
-    int64_t no_room_n = -1;      // rows at which the tables did not fit
+    int64_t no_room_n = -1, no_room_sync_n = -1;   // rows at which the tables did not fit
     uint64_t cf_build = ~0ull;
     float cf_alpha = -1.f;
     int cf_H = 0;
@@ -217,6 +235,8 @@ struct akashic_mem {
     int64_t hop_work_n = -1;  // graph (or the number of rows) last changed
     uint64_t reach_build = 0; // incremented by every rebuild
     bool reach_on = true;     // AKASHIC_REACH=0: always run the hops
+    std::atomic<int> table_users{0};   // calls between taking the tables (table_mu) and
+                                       // having queued all that reads them
     // the mass levels and reach tables are built by whichever retrieve needs
     // them first, on its own stream: table_mu serialises the builders and
     // every retrieve that reads them waits on table_ev, recorded after the
@@ -390,6 +410,45 @@ struct Tmp {
 // Grow a spare buffer with 1/4 headroom (contents not kept).
 static akashic_status_t ensure_spare(DevBuf &b, size_t bytes) {
     return bytes > b.cap ? b.ensure(bytes + bytes / 4) : AKASHIC_OK;
+}
+
+// The reach tables of the store and of its streams, freed unless a call is using
+// them (cudaFree waits for the kernels that do); none is built again for this many
+// rows.  True if there was something to free.  table_mu held.
+static bool release_tables_locked(akashic_mem *m) {
+    if (m->table_users.load() != 0) return false;
+    size_t freed = 0;
+    auto drop = [&](DevBuf &b) {
+        freed += b.cap;
+        b.release();
+    };
+    for (DevBuf &b : m->reach_c) drop(b);
+    drop(m->reach_map);
+    m->reach_levels = -1;
+    std::lock_guard<std::mutex> lk(m->mu);
+    for (auto &kv : m->scratch) {
+        StreamScratch *sc = kv.second;
+        for (DevBuf *b : {&sc->coef_hi, &sc->coef_lo, &sc->coef_sum, &sc->coef_f, &sc->cf_sum,
+                          &sc->reach_part})
+            drop(*b);
+        sc->coef_build = sc->cf_build = ~0ull;
+        sc->no_room_n = m->n;
+    }
+    return freed > 0;
+}
+static bool release_tables(akashic_mem *m) {
+    std::lock_guard<std::mutex> lk(m->table_mu);
+    return release_tables_locked(m);
+}
+
+// Rows that a table is sized for when it grows: a quarter more, to the capacity.
+static int64_t table_rows(const akashic_mem *m) {
+    const int64_t room = m->n + m->n / 4;
+    return room < m->cap ? room : m->cap;
+}
+
+static akashic_status_t ensure_table(DevBuf &b, size_t now, size_t grown) {
+    return now > b.cap ? b.ensure(grown) : AKASHIC_OK;
 }
 
 static akashic_status_t build_split_plan(akashic_mem *m, cudaStream_t st);
@@ -662,6 +721,7 @@ akashic_status_t akashic_mem_append_chunks(akashic_mem_t *m, const uint16_t *emb
     if (first_id_out) *first_id_out = m->n;
     if (n == 0) return AKASHIC_OK;
     DeviceGuard g(m->device);
+    Reclaim reclaim(m);
     cudaStream_t st = (cudaStream_t)stream;
     const int64_t first = m->n;
     PhaseScope ph(m, AKASHIC_PHASE_GRAPH, st);
@@ -776,6 +836,7 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
         return fail(AKASHIC_EINVAL, "update: M must be in [1, min(64, first)]");
     if (n == 0) return AKASHIC_OK;
     DeviceGuard g(m->device);
+    Reclaim reclaim(m);
     cudaStream_t st = (cudaStream_t)stream;
     UpdateArgs ua;
     ua.emb = m->emb.as<uint16_t>();
@@ -958,6 +1019,7 @@ akashic_status_t akashic_mem_delete(akashic_mem_t *m, const int64_t *ids, int64_
     if (n == 0) return AKASHIC_OK;
     if (!ids) return fail(AKASHIC_EINVAL, "delete: NULL ids");
     DeviceGuard g(m->device);
+    Reclaim reclaim(m);
     cudaStream_t st = (cudaStream_t)stream;
     // check every ID first, so that a bad list changes nothing
     CUDA_TRY(launch_mark_dead(ids, n, m->n, m->row_of.as<int32_t>(), nullptr,
@@ -1063,6 +1125,7 @@ akashic_status_t akashic_mem_relocate(akashic_mem_t *m, const int64_t *S, int32_
     if (n_req == 0) return AKASHIC_OK;
     if (!S) return fail(AKASHIC_EINVAL, "relocate: NULL S");
     DeviceGuard g(m->device);
+    Reclaim reclaim(m);
     cudaStream_t st = (cudaStream_t)stream;
     PhaseScope ph(m, AKASHIC_PHASE_RELOCATE, st);
     const int64_t pairs = (int64_t)n_req * s_len * (s_len - 1) / 2;
@@ -1101,6 +1164,7 @@ akashic_status_t akashic_mem_compact_pages(akashic_mem_t *m, float theta, float 
     if (!(tau_assoc >= 0.f && tau_assoc <= 1.f))
         return fail(AKASHIC_EINVAL, "compact: tau_assoc must lie in [0, 1]");
     DeviceGuard g(m->device);
+    Reclaim reclaim(m);
     cudaStream_t st = (cudaStream_t)stream;
     const int64_t n = m->n, pages = m->next_page;
     if (released) *released = 0;
@@ -1282,10 +1346,11 @@ static akashic_status_t ensure_reach(akashic_mem *m, const HopPlan &hp, int H, c
         AK_TRY(m->reach_rows.ensure(REACH_T * 4));
         AK_TRY(m->reach_t.ensure(16));
         AK_TRY(m->reach_pick.ensure((size_t)reach_pick_words() * 8));
-        AK_TRY(ensure_spare(m->reach_map, (size_t)n * 4));
+        AK_TRY(ensure_table(m->reach_map, (size_t)n * 4, (size_t)table_rows(m) * 4));
     }
     for (int t = fresh ? 0 : m->reach_levels; t < H; ++t)
-        AK_TRY(ensure_spare(m->reach_c[t], (size_t)n * REACH_T * 4));
+        AK_TRY(ensure_table(m->reach_c[t], (size_t)n * REACH_T * 4,
+                            (size_t)table_rows(m) * REACH_T * 4));
     ReachBuild rb{};
     rb.n = n;
     rb.mup = m->mass_up.as<float>();
@@ -1318,6 +1383,51 @@ static akashic_status_t ensure_reach(akashic_mem *m, const HopPlan &hp, int H, c
     return AKASHIC_OK;
 }
 
+// All that a call of width bp and H hops keeps for its candidates: its stream's
+// coefficients and partials, the store's tables.  polite: only while the device
+// keeps as much free as this takes, else ENOMEM and nothing taken.  table_mu held.
+static akashic_status_t take_tables(akashic_mem *m, StreamScratch *sc, const HopPlan &hp, int H,
+                                    int bp, bool polite, cudaStream_t st) {
+    const int64_t n = m->n, room = table_rows(m);
+    const size_t parts =
+        (size_t)(bp == 32 ? reach_fma_parts(n) : reach_parts()) * REACH_T * bp * 4;
+    const auto coef = [&](int64_t rows) {
+        return bp == 32 ? (size_t)rows * REACH_T * 4 : (size_t)reach_pad_rows(rows) * REACH_T * 2;
+    };
+    const auto sum = [](int64_t rows) { return (size_t)reach_sum_words(rows) * 8; };
+    struct {
+        DevBuf *b;
+        size_t now, grown;
+    } own[] = {{&sc->reach_part, parts, parts},
+               {bp == 32 ? &sc->coef_f : &sc->coef_hi, coef(n), coef(room)},
+               {bp == 32 ? &sc->cf_sum : &sc->coef_sum, sum(n), sum(room)},
+               {&sc->coef_lo, bp == 32 ? 0 : coef(n), coef(room)}};
+    if (polite) {
+        size_t need = 0, left = 0, all = 0;
+        for (const auto &o : own) need += o.now > o.b->cap ? o.grown : 0;
+        for (int t = 0; t < H; ++t)
+            if ((size_t)n * REACH_T * 4 > m->reach_c[t].cap) need += (size_t)room * REACH_T * 4;
+        if (need > 0) {
+            CUDA_TRY(cudaMemGetInfo(&left, &all));
+            if (left < 2 * need) return AKASHIC_ENOMEM;
+        }
+    }
+    for (const auto &o : own) AK_TRY(ensure_table(*o.b, o.now, o.grown));
+    return ensure_reach(m, hp, H, st);
+}
+
+// A call that uses the tables, until it has queued all that reads them.
+struct TableUse {
+    akashic_mem *m = nullptr;
+    void take(akashic_mem *of) {
+        m = of;
+        m->table_users.fetch_add(1);
+    }
+    ~TableUse() {
+        if (m) m->table_users.fetch_sub(1);
+    }
+};
+
 static ReachLevels reach_levels_of(const akashic_mem *m) {
     ReachLevels c{};
     for (int t = 0; t < REACH_MAX_H; ++t) c.level[t] = m->reach_c[t].as<float>();
@@ -1348,6 +1458,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
     if (hops < 0 || hops > AKASHIC_MAX_HOPS) return fail(AKASHIC_EINVAL, "retrieve: hops must be in [0, 16]");
     if (!(alpha >= 0.f) || !isfinite(alpha)) return fail(AKASHIC_EINVAL, "retrieve: alpha must be finite and >= 0");
     DeviceGuard g(m->device);
+    Reclaim reclaim(m);
     cudaStream_t st = (cudaStream_t)stream;
     StreamScratch *sc = scratch_for(m, stream);
     if (!sc) return fail(AKASHIC_ENOMEM, "retrieve: host allocation failed");
@@ -1447,13 +1558,24 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
         enum { RUN_HOPS, RC_SYNC, RC_MMA, RC_FMA } mode = RUN_HOPS;
         unsigned long long now = 0;   // this call's number, and where its key's mark
         int mark = 0;                 // stands (RC_MMA, RC_FMA)
+        TableUse use;
         if (bounds) {
             std::lock_guard<std::mutex> lk(m->table_mu);
-            AK_TRY(ensure_mass(m, hp, eff_hops, st));
+            Reclaim locked(nullptr);
+            akashic_status_t r = ensure_mass(m, hp, eff_hops, st);
+            if (r == AKASHIC_ENOMEM && release_tables_locked(m)) r = ensure_mass(m, hp, eff_hops, st);
+            AK_TRY(r);
             const bool can = !q_ns && m->reach_on && eff_hops >= 2 && eff_hops <= REACH_MAX_H;
+            // (no room for the tables: the hops run, as they would without, and the
+            // stream does not ask again at this size)
             if (can && eff_hops == 2 && bp >= 128 && m->n_split > 0) {
-                AK_TRY(ensure_reach(m, hp, eff_hops, st));
-                mode = RC_SYNC;
+                r = sc->no_room_sync_n == n ? AKASHIC_ENOMEM
+                                            : take_tables(m, sc, hp, eff_hops, bp, false, st);
+                if (r == AKASHIC_ENOMEM && sc->no_room_sync_n != n && release_tables_locked(m))
+                    r = take_tables(m, sc, hp, eff_hops, bp, false, st);
+                if (r == AKASHIC_OK) mode = RC_SYNC;
+                else if (r == AKASHIC_ENOMEM) sc->no_room_sync_n = n;
+                else return r;
             } else if (can && !direct && m->n_split >= k && sc->no_room_n != n) {
                 bool go = m->reach_levels >= eff_hops && m->reach_n == n;
                 if (!go) {
@@ -1463,25 +1585,10 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                     if (!go) m->hop_work += (double)eff_hops * bp;
                 }
                 if (go) {
-                    // no room for the tables: the hops run, as they would without
-                    const size_t cb = (size_t)REACH_T * reach_pad_rows(n) * 2;
-                    const int parts = bp == 32 ? reach_fma_parts(n) : reach_parts();
-                    akashic_status_t r = ensure_reach(m, hp, eff_hops, st);
-                    if (r == AKASHIC_OK)
-                        r = ensure_spare(sc->reach_part, (size_t)parts * REACH_T * bp * 4);
-                    if (r == AKASHIC_OK)
-                        r = bp == 32 ? ensure_spare(sc->coef_f, (size_t)n * REACH_T * 4)
-                                     : ensure_spare(sc->coef_hi, cb);
-                    if (r == AKASHIC_OK && bp != 32) r = ensure_spare(sc->coef_lo, cb);
-                    if (r == AKASHIC_OK)
-                        r = ensure_spare(bp == 32 ? sc->cf_sum : sc->coef_sum,
-                                         (size_t)reach_sum_words(n) * 8);
-                    if (r != AKASHIC_OK && r != AKASHIC_ENOMEM) return r;
-                    if (r == AKASHIC_ENOMEM) {
-                        g_last_error.clear();
-                        go = false;
-                        sc->no_room_n = n;   // not again on this stream at this size
-                    }
+                    r = take_tables(m, sc, hp, eff_hops, bp, true, st);
+                    if (r == AKASHIC_ENOMEM) sc->no_room_n = n;
+                    else if (r != AKASHIC_OK) return r;
+                    go = r == AKASHIC_OK;
                 }
                 // where the candidates did not suffice, the next calls like it
                 // run the hops alone (try_skips)
@@ -1495,6 +1602,8 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                 }
                 if (go) mode = bp == 32 ? RC_FMA : RC_MMA;
             }
+            g_last_error.clear();
+            if (mode != RUN_HOPS) use.take(m);
         }
         // on the tensor cores the candidates' pass loads u - m as split bf16,
         // which the score GEMM writes in the bytes of the fp32 slab (hi [n][bp],
@@ -1663,14 +1772,8 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                                               sc->reach_part.as<float>(), cnt, ws + sp.off_buf,
                                               sp.cap, st, &ph.launches));
                 } else {
-                    AK_TRY(ensure_spare(sc->reach_part,
-                                        (size_t)reach_parts() * REACH_T * bp * 4));
                     if (sc->coef_build != m->reach_build || sc->coef_alpha != alpha ||
                         sc->coef_H != eff_hops || sc->coef_n != n) {
-                        const size_t cb = (size_t)REACH_T * reach_pad_rows(n) * 2;
-                        AK_TRY(ensure_spare(sc->coef_hi, cb));
-                        AK_TRY(ensure_spare(sc->coef_lo, cb));
-                        AK_TRY(ensure_spare(sc->coef_sum, (size_t)reach_sum_words(n) * 8));
                         CUDA_TRY(launch_reach_pack(reach_levels_of(m), n, eff_hops, alpha,
                                                    sc->coef_hi.as<uint16_t>(),
                                                    sc->coef_lo.as<uint16_t>(),

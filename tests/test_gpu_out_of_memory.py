@@ -145,3 +145,64 @@ def test_tables_that_do_not_fit_are_not_seen_half_built(monkeypatch):
         hit = ids.cpu().numpy() == want[0]
         assert hit.mean() >= 0.75
         np.testing.assert_allclose(scores.cpu().numpy(), want[1], rtol=1e-5, atol=0)
+
+
+def _candidates(st, q, stream=None):
+    """Whether a call of two hops queues the candidates' pass."""
+    st.set_profiling(True)
+    st.phase_times()
+    st.retrieve(q, 8, 0.5, 2, stream=stream)
+    st.sync(stream)
+    ph = st.phase_times()
+    st.set_profiling(False)
+    return ph["last_hop"][1] > 2
+
+
+def test_tables_give_way(monkeypatch):
+    """An update and a wide retrieval that fit only in the place of the tables."""
+    import torch
+    n, new = 262_144, 256
+    monkeypatch.setenv("AKASHIC_REACH", "0")
+    plain, emb = _store(n, new)
+    monkeypatch.setenv("AKASHIC_REACH", "1")
+    st, _ = _store(n, new)
+    few, many = emb[5:6].contiguous(), emb[:256].contiguous()
+    wide = [t.cpu().numpy() for t in plain.retrieve(many, 5, 0.5, 0)]
+    first = [t.cpu().numpy() for t in plain.retrieve(few, 8, 0.5, 2)]
+    assert [_candidates(st, few) for _ in range(5)][-1]
+    with _memory(16 * MB):                       # the tables are 0.4 GB, the slab 0.27
+        got = [t.cpu().numpy() for t in st.retrieve(many, 5, 0.5, 0)]
+        st.sync()
+        assert not any(_candidates(st, few) for _ in range(8))
+        out = [t.cpu().numpy() for t in st.retrieve(few, 8, 0.5, 2)]
+    for a, b in zip(got, wide):
+        assert (a == b).all()
+    for a, b in zip(out, first):
+        assert (a == b).all()                    # the hops: the same bits
+    st, _ = _store(n, new)
+    assert [_candidates(st, few) for _ in range(5)][-1]
+    plain.append_chunks(emb[n:])
+    plain.update_relations(n, new, 32, True)
+    want = _csr(plain)
+    with _memory(48 * MB):                       # (an update takes 0.35 GB)
+        st.append_chunks(emb[n:])
+        st.update_relations(n, new, 32, True)
+    for a, b in zip(_csr(st), want):
+        assert (a == b).all()
+
+
+def test_tables_leave_as_much_free():
+    """The tables of one query and two hops (three tables of 512 bytes a chunk) are
+    not taken where less than twice that is free."""
+    import torch
+    n = 262_144
+    st, emb = _store(n, 0)
+    q = emb[5:6].contiguous()
+    st.retrieve(q, 8, 0.5, 2)                    # the slabs
+    st.sync()
+    with _memory(3 * 512 * n * 3 // 2):
+        free = torch.cuda.mem_get_info()[0]
+        assert not any(_candidates(st, q) for _ in range(8))
+        assert torch.cuda.mem_get_info()[0] > free - 8 * MB      # (the outputs)
+    st, _ = _store(n, 0)
+    assert [_candidates(st, q) for _ in range(8)][-1]
