@@ -103,10 +103,11 @@ static void swap_bufs(DevBuf &x, DevBuf &y) {
 }
 
 // Words of StreamScratch::words: u's extremes [2], the kept lists' lengths
-// (int64 [2]), the hops' work queues ([2] a hop), the candidates' flags, whether
-// this call skips the candidates.
-constexpr int CW_EXT = 0, CW_KEPT = 2, CW_QUEUE = 6, CW_REACH = CW_QUEUE + 2 * AKASHIC_MAX_HOPS,
-              CW_SKIP = CW_REACH + REACH_WS, CW_COUNT = CW_SKIP + 1;
+// (int64 [2]), whether this call skips the candidates (away from the flags' counters,
+// which every CTA of k_reach_flags adds to: 1.2 us a call beside them), the hops'
+// work queues ([2] a hop), the candidates' flags.
+constexpr int CW_EXT = 0, CW_KEPT = 2, CW_SKIP = 6, CW_QUEUE = 8,
+              CW_REACH = CW_QUEUE + 2 * AKASHIC_MAX_HOPS, CW_COUNT = CW_REACH + REACH_WS;
 
 struct StreamScratch {
     DevBuf qp, shift, u, sa, sb, zpart, partial, cand;

@@ -221,12 +221,12 @@ __global__ __launch_bounds__(256) void k_reach_flags(const ReachFlags f) {
     __shared__ float floor_s;
     __shared__ unsigned int lb_s[REACH_T];
     griddep_wait();
-    if (f.skip && f.skip[0] == 1) {
+    int32_t *keep = f.ws, *bad = f.ws + REACH_T, *done = f.ws + REACH_T + 1;
+    const int t_cnt = *f.t_cnt, skip = f.skip ? f.skip[0] : 0;   // (one wait for both)
+    if (skip == 1) {
         if (blockIdx.x == 0 && threadIdx.x == 0) f.plan[0] = 0;
         return;
     }
-    int32_t *keep = f.ws, *bad = f.ws + REACH_T, *done = f.ws + REACH_T + 1;
-    const int t_cnt = *f.t_cnt;
     {
         const int t = threadIdx.x;
         unsigned int lb = 0u;                            // (bounds are >= 0)

@@ -22,9 +22,10 @@ __global__ void k_prep_queries(const uint16_t *__restrict__ q, int b, int dim, f
                                unsigned long long now) {
     griddep_wait();
     const int c = blockIdx.x;
+    // (the mark is needed at the end only)
+    const unsigned long long mark = c == 0 && tried && threadIdx.x == 0 ? *tried : 0ull;
     if (c == 0)
-        for (int i = threadIdx.x; i < n_zero; i += blockDim.x)
-            zero[i] = tried && i == skip_at && try_skips(*tried, now) ? 1u : 0u;
+        for (int i = threadIdx.x; i < n_zero; i += blockDim.x) zero[i] = 0u;
     __shared__ float red[32];
     float ss = 0.f;
     if constexpr (VEC) {
@@ -58,6 +59,7 @@ __global__ void k_prep_queries(const uint16_t *__restrict__ q, int b, int dim, f
         float s = (c < b) ? tau * sqrtf(tot) * (*max_norm) : 0.f;
         shift[c] = s;
         if (!(2.f * s <= 80.f)) set_status(status, AKASHIC_ERANGE);
+        if (try_skips(mark, now)) zero[skip_at] = 1u;
     }
 }
 
