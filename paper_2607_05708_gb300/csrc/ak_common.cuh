@@ -336,9 +336,10 @@ __device__ __forceinline__ int64_t lower_bound_u32(const uint32_t *__restrict__ 
     }
     return lo;
 }
-// keys[p] = map ? map[ids[p]] : ids[p], vals[p] = p, p < pairs.
-cudaError_t launch_pair_keys(const int32_t *ids, const int32_t *map, int64_t pairs, uint32_t *keys,
-                             uint32_t *vals, cudaStream_t st);
+// Pairs p (M a new chunk) as sort items: key map ? map[ids[p]] : ids[p], value p;
+// in their own order or (order) in that of the new chunks order[0], order[1], ...
+cudaError_t launch_pair_keys(const int32_t *ids, const int32_t *map, const uint32_t *order, int M,
+                             int64_t pairs, uint32_t *keys, uint32_t *vals, cudaStream_t st);
 // The store keeps chunks in HBM in page order: row r holds chunk ext_of[r],
 // chunk c lives in row row_of[c].  The out-edge CSR stays in chunk IDs; the
 // in-edge transpose used by propagation is in rows.

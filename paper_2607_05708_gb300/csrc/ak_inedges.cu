@@ -160,8 +160,10 @@ cudaError_t launch_move_edges(const MoveEdges &m, const int64_t *ptr, const uint
     return cudaGetLastError();
 }
 
-// Forward edges c -> t, pairs sorted by the row of t (fwd): after the row's old
-// list, by source row (rank by counting among the row's new sources).
+// Forward edges c -> t, pairs sorted by the row of t (fwd), those of one row by the
+// row of c: after the row's old list, in that order.  (A place counted among the
+// row's pairs instead took every one of them a scan of all: the square of the new
+// chunks that chose one target.)
 __global__ void k_place_fwd(const uint32_t *__restrict__ fwd, const uint32_t *__restrict__ order,
                             int64_t pairs, const float *__restrict__ nbr_cos, float scale,
                             int64_t first, int M, const int32_t *__restrict__ row_of,
@@ -173,13 +175,10 @@ __global__ void k_place_fwd(const uint32_t *__restrict__ fwd, const uint32_t *__
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pairs;
          i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t p = order[i], rt = fwd[i];
-        const int32_t rs = row_of[first + p / M];
-        int64_t rank = 0;
-        for (int64_t q = lower_bound_u32(fwd, i, rt); q < pairs && fwd[q] == rt; ++q)
-            rank += row_of[first + order[q] / M] < rs ? 1 : 0;
+        const int64_t rank = i - lower_bound_u32(fwd, i, rt);
         const int64_t pos = in_ptr_new[rt] + (in_ptr_old[rt + 1] - in_ptr_old[rt]) + rank;
         const float a = scale * nbr_cos[p];
-        src_new[pos] = rs;
+        src_new[pos] = row_of[first + p / M];
         aff_new[pos] = a;
         w_new[pos] = row_softmax_weight(a, rstat[first + p / M]);   // source: chunk first + p / M
     }
@@ -217,32 +216,31 @@ cudaError_t launch_in_edges_update(const InEdgeUpdate &u, const InEdgeScratch &s
     const int sms = device_sm_count();
     const int64_t pairs = u.n_new * u.M;
     if (pairs <= 0) return cudaErrorInvalidValue;
-    int L = 3;
-    // forward pairs by target row; the new rows, which get M edges each
+    int L = 4;
+    // the new rows (each gets M reciprocal edges), then the forward pairs by target
+    // row: taken in the order of the new rows, as the sort is stable
     bool alt = false, alt_r = false;
-    cudaError_t e = launch_pair_keys(u.nbr_ids, u.row_of, pairs, s.keys, s.vals, st);
+    uint32_t *rk = s.rows, *rv = rk + u.n_new, *rk2 = rv + u.n_new, *rv2 = rk2 + u.n_new;
+    const int64_t want = ceil_div<int64_t>(u.n_new, 256);
+    launch_pdl(k_row_keys, dim3((unsigned)(want < sms ? want : sms)), dim3(256), 0, st, u.row_of,
+               u.first, u.n_new, rk, rv);
+    cudaError_t e = radix_sort_pairs(rk, rv, rk2, rv2, u.n_new, u.row_bits, s.tmp, s.tmp_bytes, st,
+                                     &alt_r, &L);
+    const uint32_t *rows = alt_r ? rk2 : rk, *by_row = alt_r ? rv2 : rv;
+    if (e == cudaSuccess)
+        e = launch_pair_keys(u.nbr_ids, u.row_of, by_row, u.M, pairs, s.keys, s.vals, st);
     if (e == cudaSuccess)
         e = radix_sort_pairs(s.keys, s.vals, s.keys2, s.vals2, pairs, u.row_bits, s.tmp,
                              s.tmp_bytes, st, &alt, &L);
     const int64_t recip_rows = u.reciprocal ? u.n_new : 0;
-    uint32_t *rk = s.rows, *rv = rk + u.n_new, *rk2 = rv + u.n_new, *rv2 = rk2 + u.n_new;
-    if (e == cudaSuccess && recip_rows > 0) {
-        const int64_t want = ceil_div<int64_t>(u.n_new, 256);
-        launch_pdl(k_row_keys, dim3((unsigned)(want < sms ? want : sms)), dim3(256), 0, st,
-                   u.row_of, u.first, u.n_new, rk, rv);
-        e = radix_sort_pairs(rk, rv, rk2, rv2, u.n_new, u.row_bits, s.tmp, s.tmp_bytes, st, &alt_r,
-                             &L);
-        ++L;
-    }
     if (e != cudaSuccess) return e;
     const uint32_t *fwd = alt ? s.keys2 : s.keys, *order = alt ? s.vals2 : s.vals;
     launch_pdl(k_new_in_ptr, dim3((unsigned)(sms * 8)), dim3(256), 0, st, u.in_ptr_old, u.n, fwd,
-               pairs, alt_r ? rk2 : rk, recip_rows, u.M, u.in_ptr_new);
+               pairs, rows, recip_rows, u.M, u.in_ptr_new);
     const int64_t nnz_old = u.nnz_new - pairs * (u.reciprocal ? 2 : 1);
     MoveEdges mv{nnz_old, u.in_src_old, u.in_aff_old, u.in_w_old, u.in_src_new, u.in_aff_new,
                  u.in_w_new, u.M, u.touched, u.ext_of, u.rstat};
-    e = launch_move_edges(mv, u.in_ptr_old, fwd, pairs, alt_r ? rk2 : rk, recip_rows, s.move, st,
-                          &L);
+    e = launch_move_edges(mv, u.in_ptr_old, fwd, pairs, rows, recip_rows, s.move, st, &L);
     if (e != cudaSuccess) return e;
     launch_pdl(k_place_fwd, dim3((unsigned)(sms * 2)), dim3(256), 0, st, fwd, order, pairs,
                u.nbr_cos, u.scale, u.first, u.M, u.row_of, u.in_ptr_old, u.in_ptr_new,

@@ -210,24 +210,24 @@ cudaError_t launch_check_new_rows(const int64_t *rp, const int64_t *in_ptr, cons
     return cudaGetLastError();
 }
 
-// keys[p] = map ? map[ids[p]] : ids[p], vals[p] = p.
 __global__ void k_pair_keys(const int32_t *__restrict__ ids, const int32_t *__restrict__ map,
-                            int64_t pairs, uint32_t *__restrict__ keys,
-                            uint32_t *__restrict__ vals) {
+                            const uint32_t *__restrict__ order, int M, int64_t pairs,
+                            uint32_t *__restrict__ keys, uint32_t *__restrict__ vals) {
     griddep_wait();
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < pairs;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        keys[p] = (uint32_t)(map ? map[ids[p]] : ids[p]);
-        vals[p] = (uint32_t)p;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pairs;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t p = order ? (int64_t)order[i / M] * M + i % M : i;
+        keys[i] = (uint32_t)(map ? map[ids[p]] : ids[p]);
+        vals[i] = (uint32_t)p;
     }
 }
 
-cudaError_t launch_pair_keys(const int32_t *ids, const int32_t *map, int64_t pairs, uint32_t *keys,
-                             uint32_t *vals, cudaStream_t st) {
+cudaError_t launch_pair_keys(const int32_t *ids, const int32_t *map, const uint32_t *order, int M,
+                             int64_t pairs, uint32_t *keys, uint32_t *vals, cudaStream_t st) {
     if (pairs <= 0) return cudaSuccess;
     const int64_t want = ceil_div<int64_t>(pairs, 256), cap = (int64_t)device_sm_count() * 4;
     launch_pdl(k_pair_keys, dim3((unsigned)(want < cap ? want : cap)), dim3(256), 0, st, ids, map,
-               pairs, keys, vals);
+               order, M, pairs, keys, vals);
     return cudaGetLastError();
 }
 
@@ -361,7 +361,7 @@ akashic_status_t csr_insert(const UpdateArgs &a, const int64_t *rp, const int32_
     if (e == cudaSuccess && recips > 0) {
         int bits = 0;
         while (bits < 32 && ((int64_t)1 << bits) <= a.first - 1) ++bits;
-        e = launch_pair_keys(a.nbr_ids, nullptr, pairs, keys, vals, st);
+        e = launch_pair_keys(a.nbr_ids, nullptr, nullptr, a.M, pairs, keys, vals, st);
         if (e == cudaSuccess)
             e = radix_sort_pairs(keys, vals, keys2, vals2, pairs, bits, tmp, tmp_bytes, st, &alt, &L);
         L += 2;
