@@ -1036,7 +1036,7 @@ akashic_status_t akashic_mem_delete(akashic_mem_t *m, const int64_t *ids, int64_
     // the compaction's scratch; what has to start at zero comes first
     const size_t rb = (size_t)ceil_div<int64_t>(rows, 32) * 4;
     const size_t eb = (size_t)ceil_div<int64_t>(nnz, 32) * 4;
-    const size_t cb = (size_t)drop_tiles(nnz) * 4;
+    const size_t cb = (size_t)drop_words(nnz) * 4;
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t zero = 2 * up(rb) + 2 * up(eb);
     uint8_t *scr = (uint8_t *)store_scratch(m, SCR_DEL, zero + up(rb) + 2 * up(eb) + up(cb));
@@ -1175,7 +1175,7 @@ akashic_status_t akashic_mem_compact_pages(akashic_mem_t *m, float theta, float 
     int32_t *cand = (int32_t *)store_scratch(m, SCR_MM_CAND, (size_t)(pages + 1) * 4);
     uint32_t *moving = (uint32_t *)store_scratch(m, SCR_MM_MOVING, (size_t)ceil_div<int64_t>(n, 32) * 4);
     int32_t *parent = (int32_t *)store_scratch(m, SCR_MM_PARENT, (size_t)n * 4);
-    int32_t *counts = (int32_t *)store_scratch(m, SCR_MM_COUNTS, (size_t)mm_tiles(n) * 4);
+    int32_t *counts = (int32_t *)store_scratch(m, SCR_MM_COUNTS, (size_t)mm_words(n) * 4);
     uint32_t *ids = (uint32_t *)store_scratch(m, SCR_MM_IDS, (size_t)n * 4 + 16);
     uint32_t *nsk = (uint32_t *)store_scratch(m, SCR_MM_NSK, (size_t)n * 4 + 16);
     if (!cand || !moving || !parent || !counts || !ids || !nsk)

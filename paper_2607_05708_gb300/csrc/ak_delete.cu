@@ -88,7 +88,8 @@ __global__ void k_drop_rows(const int64_t *__restrict__ ids, int64_t n, int64_t 
 // list's 470 MB take 88 us.)
 constexpr int DROP_WORDS = 16;                          // a warp
 constexpr int DROP_TILE = 8 * 32 * DROP_WORDS;
-int64_t drop_tiles(int64_t nnz) { return ceil_div<int64_t>(nnz, DROP_TILE); }
+static int64_t drop_tiles(int64_t nnz) { return ceil_div<int64_t>(nnz, DROP_TILE); }
+int64_t drop_words(int64_t nnz) { return tile_words(drop_tiles(nnz)); }
 
 __global__ __launch_bounds__(256) void k_drop_mark(const DropDead d) {
     griddep_wait();
@@ -269,6 +270,8 @@ cudaError_t launch_drop_dead_edges(const DropDead &d, cudaStream_t st) {
     }
     const unsigned tiles = (unsigned)drop_tiles(d.nnz);
     launch_pdl(k_drop_mark, dim3(tiles), dim3(256), 0, st, d);
+    cudaError_t e = launch_tile_groups(d.counts, tiles, st);
+    if (e != cudaSuccess) return e;
     launch_pdl(k_drop_edges, dim3(tiles), dim3(256), 0, st, d);
     return cudaGetLastError();
 }

@@ -21,6 +21,34 @@ static int sm_count_cached() {
 }
 int device_sm_count() { return sm_count_cached(); }
 
+// ================================================================== ordered tiles
+// groups[g] = the sum of the counts of tiles 1024 g .. (see tile_base).
+__global__ __launch_bounds__(256) void k_tile_groups(int32_t *__restrict__ counts, int64_t tiles) {
+    griddep_wait();
+    __shared__ int part[8];
+    const int64_t t0 = (int64_t)blockIdx.x * TILE_GROUP;
+    int s = 0;
+#pragma unroll
+    for (int q = 0; q < TILE_GROUP / 256; ++q) {
+        const int64_t t = t0 + q * 256 + threadIdx.x;
+        s += t < tiles ? counts[t] : 0;
+    }
+    s = (int)__reduce_add_sync(0xffffffffu, (unsigned)s);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) s += part[w];
+        counts[tiles + blockIdx.x] = s;
+    }
+}
+
+cudaError_t launch_tile_groups(int32_t *counts, int64_t tiles, cudaStream_t st, int *launches) {
+    if (tiles <= TILE_FLAT) return cudaSuccess;
+    if (launches) *launches += 1;
+    return launch_pdl(k_tile_groups, dim3((unsigned)ceil_div<int64_t>(tiles, TILE_GROUP)),
+                      dim3(256), 0, st, counts, tiles);
+}
+
 // ================================================================== scan
 constexpr int SCAN_THREADS = 256, SCAN_ITEMS = 8;
 static_assert(SCAN_TILE == SCAN_THREADS * SCAN_ITEMS, "a tile is one CTA's share");
@@ -849,7 +877,7 @@ __global__ void k_seg_permute(const uint32_t *__restrict__ order, const int64_t 
 }
 
 int64_t hub_plan_words(int64_t n, int64_t max_hubs) {
-    return ceil_div<int64_t>(ceil_div<int64_t>(n, HEAVY_TILE), 2) + max_hubs +
+    return ceil_div<int64_t>(tile_words(ceil_div<int64_t>(n, HEAVY_TILE)), 2) + max_hubs +
            (int64_t)(scan_tmp_bytes(max_hubs) / 8) + 1;
 }
 
@@ -862,15 +890,17 @@ cudaError_t launch_hub_count(const SplitParams &sp, const int64_t *in_ptr, const
         return e == cudaSuccess ? cudaMemsetAsync(slot0 + (max_hubs > 0 ? max_hubs : 0), 0, 8, st) : e;
     }
     int32_t *tc = (int32_t *)scratch;
-    int64_t *nseg = scratch + ceil_div<int64_t>(tiles, 2);
+    int64_t *nseg = scratch + ceil_div<int64_t>(tile_words(tiles), 2);
     launch_pdl(k_heavy_rows<false>, dim3((unsigned)tiles), dim3(256), 0, st, in_ptr, n, sp.split_t,
                rows, counts, tc);
+    cudaError_t e = launch_tile_groups(tc, tiles, st);
+    if (e != cudaSuccess) return e;
     launch_pdl(k_heavy_rows<true>, dim3((unsigned)tiles), dim3(256), 0, st, in_ptr, n, sp.split_t,
                rows, counts, tc);
     const int64_t want = ceil_div<int64_t>(max_hubs, 8), cap = (int64_t)device_sm_count() * 8;
     launch_pdl(k_hub_segs, dim3((unsigned)(want < cap ? want : cap)), dim3(256), 0, st, sp, in_ptr,
                in_src, rows, counts, max_hubs, nseg);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return scan_exclusive(nseg, slot0, max_hubs, nseg + max_hubs, scan_tmp_bytes(max_hubs), st);
 }
@@ -1322,7 +1352,9 @@ __global__ __launch_bounds__(256) void k_keep_list(int64_t row_tiles, int64_t se
 static int64_t keep_tiles(const HopPlan &p) {
     return ceil_div<int64_t>(p.n, KEEP_TILE) + ceil_div<int64_t>(p.n_segs, KEEP_TILE);
 }
-int64_t keep_words(const HopPlan &p) { return keep_tiles(p) * (1 + KEEP_TILE / 32); }
+int64_t keep_words(const HopPlan &p) {
+    return tile_words(keep_tiles(p)) + keep_tiles(p) * (KEEP_TILE / 32);
+}
 
 cudaError_t launch_keep(const HopPlan &p, const RowBounds &rb, const float *floor_p,
                         const NsFloors *nf, int32_t *split_skip, int32_t *kept_rows,
@@ -1331,11 +1363,12 @@ cudaError_t launch_keep(const HopPlan &p, const RowBounds &rb, const float *floo
     static_assert(KEEP_TILE == 1024, "tile_places");
     const int64_t tiles = keep_tiles(p), row_tiles = ceil_div<int64_t>(p.n, KEEP_TILE);
     const NsFloors f = nf ? *nf : NsFloors{};
-    uint32_t *bits = (uint32_t *)(words + tiles);
+    uint32_t *bits = (uint32_t *)(words + tile_words(tiles));
     cudaError_t e = launch_pdl(
         k_keep_mark, dim3((unsigned)(tiles + ceil_div<int64_t>(p.n_split_rows, KEEP_TILE))),
         dim3(256), 0, st, rb, floor_p, f, p.in_ptr, p.split.split_t, p.n_split_rows, p.split_row,
         p.n_segs, p.seg_slot, p.slot_split, split_skip, words, bits, p.done);
+    if (e == cudaSuccess) e = launch_tile_groups(words, tiles, st, launches);
     if (e == cudaSuccess)
         e = launch_pdl(k_keep_list, dim3((unsigned)tiles), dim3(256), 0, st, row_tiles,
                        tiles - row_tiles, (const int32_t *)words, (const uint32_t *)bits, kept_rows,

@@ -653,7 +653,8 @@ cudaError_t launch_mm_candidates(const MmTables &t, int64_t n_pages, float theta
     return cudaGetLastError();
 }
 
-int64_t mm_tiles(int64_t n) { return ceil_div<int64_t>(n, MM_TILE); }
+static int64_t mm_tiles(int64_t n) { return ceil_div<int64_t>(n, MM_TILE); }
+int64_t mm_words(int64_t n) { return tile_words(mm_tiles(n)); }
 
 cudaError_t launch_mm_collect(const MmTables &t, int64_t n, const int32_t *row_of,
                               const int32_t *dead_row, const int32_t *page_row,
@@ -664,6 +665,8 @@ cudaError_t launch_mm_collect(const MmTables &t, int64_t n, const int32_t *row_o
     const unsigned tiles = (unsigned)mm_tiles(n);
     launch_pdl(k_mm_moving, dim3(tiles), dim3(256), 0, st, n, row_of, dead_row, page_row, cand,
                moving, counts);
+    cudaError_t e = launch_tile_groups(counts, tiles, st);
+    if (e != cudaSuccess) return e;
     launch_pdl(k_mm_list, dim3(tiles), dim3(256), 0, st, n, row_of, ns_row, moving, parent, ids,
                ns_key, t.released + 1, counts);
     return cudaGetLastError();
