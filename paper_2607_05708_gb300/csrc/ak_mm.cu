@@ -63,6 +63,11 @@ __device__ __forceinline__ bool mm_assoc(uint32_t co, int32_t sa, int32_t sb, fl
     return co > 0u && (double)co >= (double)tau * uni;
 }
 
+// Pages of per_page slots that `chunks` chunks fill (per_page up to 2^31 - 1).
+__device__ __forceinline__ int mm_pages(int chunks, int per_page) {
+    return (int)(((int64_t)chunks + per_page - 1) / per_page);
+}
+
 // The distinct valid chunks of request r (order of first appearance): IDs
 // in [0, n), not deleted, first occurrence only.  Warp-cooperative; returns
 // the count (same in every lane); set[] in shared memory.
@@ -227,7 +232,7 @@ __global__ __launch_bounds__(1024) void k_mm_relocate(const int32_t *__restrict_
                     atomicAdd(&t.page_live[q], 1);
                 }
                 if (lane == 0) {
-                    next_s = next + (ng + per_page - 1) / per_page;
+                    next_s = next + mm_pages(ng, per_page);
                     writes_s += ng;
                 }
             }
@@ -459,7 +464,7 @@ __global__ __launch_bounds__(1024) void k_mm_repack_small(const uint32_t *__rest
             }
             len[h] = lo - i;
         }
-        pages += (len[h] + per_page - 1) / per_page;
+        pages += mm_pages(len[h], per_page);
     }
     // base pages: exclusive scan of the runs' pages over the threads
     int incl = pages;
@@ -476,7 +481,7 @@ __global__ __launch_bounds__(1024) void k_mm_repack_small(const uint32_t *__rest
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         if (head[h]) run_page[2 * tid + h] = base;
-        base += (len[h] + per_page - 1) / per_page;
+        base += mm_pages(len[h], per_page);
     }
     __syncthreads();
     // place i: its run's head is the first place with its namespace

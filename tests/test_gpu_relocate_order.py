@@ -75,3 +75,24 @@ def test_compaction_sizes(pages, keep, namespaces):
     for tau in (0.3, 0.0):
         assert st.compact_pages(0.75, tau) == len(mm.compact(0.75, tau))
         _check(st, mm)
+
+
+@pytest.mark.parametrize("P", [2 ** 31 - 1, 2 ** 31 - 3, 2 ** 30])
+def test_pages_of_any_size(P):
+    """Relocation and compaction with the largest chunks_per_page: a group is one
+    page, a namespace's share of a compaction one."""
+    import torch
+    n = 400
+    page_of = np.arange(n) // 40
+    ns = np.arange(n) % 4 - 2
+    st, mm = _store(n, 64, page_of, P, ns), MemoryManager(page_of, P, ns_of=ns)
+    S = np.arange(96).reshape(12, 8) * 4
+    st.relocate(torch.from_numpy(S).cuda(), 0.5)
+    mm.relocate(S, 0.5)
+    _check(st, mm)
+    gone = np.array([i for i in range(n) if i % 40 > 9], np.int64)
+    st.delete(torch.from_numpy(gone).cuda())
+    mm.delete(gone)
+    for _ in range(2):
+        assert st.compact_pages(0.75, 0.5) == len(mm.compact(0.75, 0.5))
+        _check(st, mm)
