@@ -361,6 +361,7 @@ __global__ void k_mm_union(MmTables t, const uint32_t *__restrict__ moving,
                            const int32_t *__restrict__ row_of, const int32_t *__restrict__ ns_row,
                            float tau, int32_t *__restrict__ parent, int *status) {
     griddep_wait();
+    if (*count < 2) return;   // no pair of them: the table need not be looked through
     for (int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; h < t.co_cap;
          h += (int64_t)gridDim.x * blockDim.x) {
         const unsigned long long key = t.co_key[h];
