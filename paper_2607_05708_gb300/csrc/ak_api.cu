@@ -111,7 +111,7 @@ constexpr int CW_EXT = 0, CW_KEPT = 2, CW_SKIP = 6, CW_QUEUE = 8,
 
 struct StreamScratch {
     DevBuf qp, shift, u, sa, sb, zpart, partial, cand;
-    DevBuf words;                // a call's counters (CallWords), zeroed by its first kernel
+    DevBuf words;                // a call's counters (CW_*), zeroed by its first kernel
     DevBuf samp, ext_s, zsamp;   // retrieval without hops: the score's row sample
     DevBuf qns, ns_s, dead_s;    // scope: per query column, per sample row
     DevBuf rmax_u, rmin_u;       // u's row maxima / minima over the real queries
@@ -901,7 +901,10 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
         int code = 0;
         akashic_status_t r = relate_top_m(ua, st, &ph.launches, &code);
         if (r != AKASHIC_OK) return fail(r, "update: relation GEMM / top-M failed");
-        if (code != 0) return check_status(m, st, "update");
+        if (code != 0)
+            return check_status(m, st, code == AKASHIC_EINVAL
+                                           ? "update: rows [first, first+n) already have out-edges"
+                                           : "update");
     }
     {
         PhaseScope ph(m, AKASHIC_PHASE_GRAPH, st);
