@@ -195,7 +195,7 @@ int64_t score_tiles(int64_t n);
 // row_max / row_min (optional, together): [n] the largest and smallest u of
 // each row over the first n_real columns (the real queries), for the
 // propagation's row bounds; with them, ext (optional, [2], zeroed before)
-// gets their extremes in launch_final_bounds' encoding.
+// gets their extremes (RowBounds::ext).
 // One thread waits on a barrier that nothing signals, giving up after
 // `polls` polls like every bounded wait (ETIMEOUT into *status).
 cudaError_t launch_wait_timeout_check(int *status, uint32_t polls, cudaStream_t st);
@@ -736,7 +736,7 @@ constexpr int REACH_WS = REACH_T + 2;
 struct ReachFlags {
     const float *u0, *l0;            // u's row maxima / minima [n]
     const float *mup, *mdn;          // mass levels [H + 1][n]
-    const unsigned int *ext;         // Umax / Lmin (launch_final_bounds' encoding)
+    const unsigned int *ext;         // Umax / Lmin (RowBounds::ext)
     int64_t n;
     int H;
     float alpha;
@@ -847,13 +847,12 @@ cudaError_t launch_select_signed(const SelectPlan &sp, const float *s, int b,
                                  unsigned long long *ws, const int32_t *ext_of, int64_t id_limit,
                                  int64_t c_base, int32_t *nbr_ids, float *nbr_cos, int *status,
                                  cudaStream_t st, int *launches, NsScope ns = NsScope{});
-// Bound pass alone over signed values: bound[c] for the b real columns
-// (the k-th largest sampled key; padding columns get an all-ones bound).
-// Bound only, unsigned keys (retrieval): ws + sp.off_bound gets the bound,
-// the column counts are cleared.  For a filter fused into the score, from
-// the sampled score slab `s`, or (s == NULL) into the last hop, from the keys
-// that launch_hop_sample left at ws + sp.off_tr.  `slack` lowers each bound by that many units of the
-// score's last place (margin for a sample computed by another launch).
+// Bound pass alone (retrieval): ws + sp.off_bound gets the k-th largest sampled
+// key of the b real columns (padding columns an all-ones bound), the column counts
+// are cleared.  For a filter fused into the score, from the sampled score slab
+// `s`, or (s == NULL) into the last hop, from the keys that launch_hop_sample left
+// at ws + sp.off_tr.  `slack` lowers each bound by that many units of the score's
+// last place (margin for a sample computed by another launch).
 cudaError_t launch_sample_bound(const SelectPlan &sp, const float *s, int b,
                                 const int32_t *ext_of, unsigned long long *ws, cudaStream_t st,
                                 int *launches, uint32_t slack = 0, NsScope ns = NsScope{},
@@ -897,10 +896,6 @@ cudaError_t launch_topk_direct(const float *s, int64_t n, int bp, int b, int k,
                                const int32_t *row_of, const int32_t *page_row, int64_t *ids,
                                float *scores, int32_t *page_ids, int32_t *n_pages, int *status,
                                NsScope ns, int sort_by_time, cudaStream_t st, int *launches);
-cudaError_t launch_sample_bound_signed(const SelectPlan &sp, const float *s, int b,
-                                       const int32_t *ext_of, int64_t id_limit,
-                                       unsigned long long *ws, unsigned long long *bound,
-                                       cudaStream_t st, int *launches, NsScope ns = NsScope{});
 // bound[c] = the k-th largest of the n_sample keys keys_t[c][*] (k <= 64) as a
 // key with the chunk-ID half zero, 0 if fewer than k keys are nonzero; ~0
 // for the padding columns b <= c < bp; cnt[c] = 0.  One CTA a column.

@@ -1,4 +1,4 @@
-// Two-hop scores of the top-k candidates without the hops.
+// Scores of the top-k candidates for two to four hops, without the hops.
 //
 // Unrolling the hop recursion s^(h) = u + alpha R^T s^(h-1) (the relation
 // propagation of §4.1, R_ki = w(k -> i)) gives, for a row j,
@@ -9,8 +9,10 @@
 // upper bound reaches the top-k floor can be selected; when all of them lie
 // in a small set of heavy candidate rows whose coefficients are kept, their
 // final scores for every query come from one pass over the score slab u,
-// and the hops are not run.  The selection is the same as the hops' (the
-// values differ only by fp32 summation order).
+// and the hops are not run.  The selection is the same as the hops' up to
+// scores that are equal within the two paths' roundings: sums in another order, and
+// on the tensor cores coefficients and u as pairs of bf16 (16 bits; see
+// REACH_SPLIT_SHIFT).
 #include <cuda_bf16.h>
 
 #include "ak_common.cuh"

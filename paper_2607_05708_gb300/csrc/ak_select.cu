@@ -1123,30 +1123,12 @@ static cudaError_t bound_and_filter(const SelectPlan &sp, const float *s, int b,
     return cudaGetLastError();
 }
 
-template <bool SIGNED>
-static cudaError_t sample_bound(const SelectPlan &sp, const float *s, int b,
-                                const int32_t *ext_of, int64_t id_limit,
-                                unsigned long long *ws, unsigned long long *bound,
-                                cudaStream_t st, int *launches, uint32_t slack = 0,
-                                NsScope ns = NsScope{}, const int32_t *done = nullptr) {
-    cudaError_t e = launch_kth<SIGNED>(sp, s, b, ext_of, id_limit, ws, bound,
-                                       (unsigned int *)(ws + sp.off_cnt), st, slack, ns, done);
-    if (launches) *launches += s ? 2 : 1;
-    return e;
-}
-
-cudaError_t launch_sample_bound_signed(const SelectPlan &sp, const float *s, int b,
-                                       const int32_t *ext_of, int64_t id_limit,
-                                       unsigned long long *ws, unsigned long long *bound,
-                                       cudaStream_t st, int *launches, NsScope ns) {
-    return sample_bound<true>(sp, s, b, ext_of, id_limit, ws, bound, st, launches, 0, ns);
-}
-
 cudaError_t launch_sample_bound(const SelectPlan &sp, const float *s, int b,
                                 const int32_t *ext_of, unsigned long long *ws, cudaStream_t st,
                                 int *launches, uint32_t slack, NsScope ns, const int32_t *done) {
-    return sample_bound<false>(sp, s, b, ext_of, (int64_t)1 << 40, ws, ws + sp.off_bound, st,
-                               launches, slack, ns, done);
+    if (launches) *launches += s ? 2 : 1;
+    return launch_kth<false>(sp, s, b, ext_of, (int64_t)1 << 40, ws, ws + sp.off_bound,
+                             (unsigned int *)(ws + sp.off_cnt), st, slack, ns, done);
 }
 
 cudaError_t launch_select(const SelectPlan &sp, const float *s, int b, unsigned long long *ws,
