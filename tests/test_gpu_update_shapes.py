@@ -136,3 +136,30 @@ def test_many_new_chunks_of_few_targets(n, new, M, recip):
     wl = dataclasses.replace(synth.workload(2, scale=1 / 64), emb=emb, hops=1, k=k,
                              row_ptr=rp, col=col, aff=aff, page_of={"p": page})
     assert_retrieval_parity(wl, "p", got, ref)
+
+
+def test_refused_updates_say_why_and_change_nothing():
+    """Rows that have out-edges, and a chunk that an edge points at already."""
+    import torch
+    from paper_2607_05708_gb300 import AkashicError, MemStore
+    rng = np.random.default_rng(2)
+    emb = torch.from_numpy(synth.to_bf16(rng.normal(0, 0.1, (300, 64)).astype(np.float32))
+                           .view(np.int16)).cuda()
+    st = MemStore(64, 300, chunks_per_page=16)
+    st.append_chunks(emb[:200])
+    st.update_relations(100, 100, 4, True)
+    rp = torch.zeros(51, dtype=torch.int64, device="cuda")
+    rp[10:] = 1                                          # chunk 209 links to 220
+    st.append_chunks(emb[200:250], None, rp, torch.tensor([220], dtype=torch.int32, device="cuda"),
+                     torch.ones(1, device="cuda"))
+    before = [t.cpu().numpy() for t in st.export_csr()]
+    for first, n, code, why in ((150, 20, "EINVAL", "already have out-edges"),
+                                (200, 50, "EINVAL", "already have out-edges"),
+                                (210, 40, "EDEVICE", "update")):
+        with pytest.raises(AkashicError, match=why) as e:
+            st.update_relations(first, n, 4, True)
+        assert e.value.code == code
+        for a, b in zip(st.export_csr(), before):
+            assert (a.cpu().numpy() == b).all()
+    st.sync()                                            # nothing is left in the status word
+    st.update_relations(221, 29, 4, True)
