@@ -1556,9 +1556,10 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
         // than the hops of such a batch.  For the others they are built once the
         // hops have cost that much since the graph changed, so that a graph that
         // changes every few calls costs at most twice the hops alone.  One GB300,
-        // hops -> candidates: 1,048,576 chunks, 1 query, two hops 1533 -> 440 us;
-        // 262,147 chunks, 24 queries 384 -> 142; 262,144 chunks, 200 queries, three
-        // hops 1589 -> 237 (564 in fp32).
+        // hops -> candidates on a graph that stays: 1,048,576 chunks, 1 query, two
+        // hops 1533 -> 440 us (the call that builds the tables 3439, the fourth after
+        // a change); 262,147 chunks, 24 queries 384 -> 142 (913, the fourth); 262,144
+        // chunks, 200 queries, three hops 1589 -> 237 (1593, the second; 564 in fp32).
         enum { RUN_HOPS, RC_SYNC, RC_MMA, RC_FMA } mode = RUN_HOPS;
         unsigned long long now = 0;   // this call's number, and where its key's mark
         int mark = 0;                 // stands (RC_MMA, RC_FMA)
