@@ -155,7 +155,8 @@ akashic_status_t akashic_mem_update_relations(akashic_mem_t *m, int64_t first, i
  * the other.  Which one a call takes follows from the store and the calls made
  * before it, not from when those finish: calls with two to four hops (but two
  * hops with 65 queries and more) run the hops until these have cost as much as
- * the tables since the graph last changed; a call that the candidates do not
+ * the tables since the graph last changed (up to 16 times as much where earlier
+ * tables were dropped before they paid); a call that the candidates do not
  * suffice for is followed by 15 of the same alpha, hops, k and width on its
  * stream that run the hops.
  * The tables take 512 bytes a chunk and hop for the store, and 512 a chunk for

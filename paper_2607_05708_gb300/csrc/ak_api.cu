@@ -234,6 +234,10 @@ struct akashic_mem {
     int64_t reach_n = -1;     // rows they were computed for
     double hop_work = 0;      // query columns x hops run through the hops since the
     int64_t hop_work_n = -1;  // graph (or the number of rows) last changed
+    // what the tables of this graph had to save to pay (0: none built for small
+    // batches), what they have saved (in the same unit), and how many times that
+    // cost the hops have to reach before tables are built (table_turn)
+    double table_cost = 0, table_saved = 0, table_wait = 1;
     uint64_t reach_build = 0; // incremented by every rebuild
     bool reach_on = true;     // AKASHIC_REACH=0: always run the hops
     std::atomic<int> table_users{0};   // calls between taking the tables (table_mu) and
@@ -442,6 +446,17 @@ static bool release_tables(akashic_mem *m) {
     return release_tables_locked(m);
 }
 
+// The graph, or the number of rows, has changed: the work done on it starts over.
+// Where its tables had not saved what they cost, the next ones are built after twice
+// as much work (16 times at most), else after the least again.
+static void table_turn(akashic_mem *m) {
+    if (m->table_cost > 0) {
+        const bool paid = m->table_saved >= m->table_cost;
+        m->table_wait = paid ? 1 : (m->table_wait < 16 ? 2 * m->table_wait : 16);
+    }
+    m->table_cost = m->table_saved = m->hop_work = 0;
+}
+
 // Rows that a table is sized for when it grows: a quarter more, to the capacity.
 static int64_t table_rows(const akashic_mem *m) {
     const int64_t room = m->n + m->n / 4;
@@ -510,7 +525,7 @@ static akashic_status_t build_split_plan(akashic_mem *m, cudaStream_t st) {
     const int64_t n = m->n;
     m->mass_levels = -1;   // the graph changed
     m->reach_levels = -1;
-    m->hop_work = 0;
+    table_turn(m);
     // temporaries from the store's scratch (slots SCR_SPLIT0..11)
     akashic_status_t sc_rc = AKASHIC_OK;
     auto get = [&](int i, size_t bytes) -> Tmp {
@@ -1554,8 +1569,9 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
         // The first builds the graph-only coefficients at once; they cost about
         // what the hops cost over 128 columns a level past the first, far less
         // than the hops of such a batch.  For the others they are built once the
-        // hops have cost that much since the graph changed, so that a graph that
-        // changes every few calls costs at most twice the hops alone.  One GB300,
+        // hops have cost that much since the graph changed, and later where the
+        // tables of the graphs before did not pay (table_turn), so that a graph
+        // that changes every few calls soon costs no more than the hops.  One GB300,
         // hops -> candidates on a graph that stays: 1,048,576 chunks, 1 query, two
         // hops 1533 -> 440 us (the call that builds the tables 3439, the fourth after
         // a change); 262,147 chunks, 24 queries 384 -> 142 (913, the fourth); 262,144
@@ -1582,18 +1598,19 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                 else if (r == AKASHIC_ENOMEM) sc->no_room_sync_n = n;
                 else return r;
             } else if (can && !direct && m->n_split >= k && sc->no_room_n != n) {
+                const double work = (double)eff_hops * bp, cost = REACH_T * (eff_hops - 1) + 64;
+                if (m->hop_work_n != n) table_turn(m);
+                m->hop_work_n = n;
                 bool go = m->reach_levels >= eff_hops && m->reach_n == n;
-                if (!go) {
-                    if (m->hop_work_n != n) m->hop_work = 0;
-                    m->hop_work_n = n;
-                    go = m->hop_work >= REACH_T * (eff_hops - 1) + 64;
-                    if (!go) m->hop_work += (double)eff_hops * bp;
-                }
+                const bool build = !go && m->hop_work >= cost * m->table_wait;
+                if (!go && !build) m->hop_work += work;
+                go = go || build;
                 if (go) {
                     r = take_tables(m, sc, hp, eff_hops, bp, true, st);
                     if (r == AKASHIC_ENOMEM) sc->no_room_n = n;
                     else if (r != AKASHIC_OK) return r;
                     go = r == AKASHIC_OK;
+                    if (go && build) m->table_cost += cost;
                 }
                 // where the candidates did not suffice, the next calls like it
                 // run the hops alone (try_skips)
@@ -1606,6 +1623,7 @@ static akashic_status_t retrieve_impl(akashic_mem *m, const uint16_t *q, int32_t
                     go = !try_skips(((volatile unsigned long long *)sc->told)[mark], now);
                 }
                 if (go) mode = bp == 32 ? RC_FMA : RC_MMA;
+                if (go) m->table_saved += work;
             }
             g_last_error.clear();
             if (mode != RUN_HOPS) use.take(m);

@@ -126,6 +126,29 @@ def test_candidates_that_do_not_suffice():
     assert seen == ([2] * 3 + [7] + [2] * 15 + ([5] + [2] * 15) * 2)[:40], seen
 
 
+def test_tables_wait_where_they_did_not_pay():
+    """A store that is written every few reads builds tables once, then does without;
+    once it is read long enough again, they come after the least work again."""
+    import torch
+    wl = synth.workload(2, scale=1 / 64)
+    q = wl.queries[:20]
+    store = gpu_store(wl, "clustered")
+    victims = iter(range(100, 200))
+
+    def reads(n):
+        seen = [_launches(store, wl, q)[1] for _ in range(n)]
+        store.delete(torch.tensor([next(victims)], device="cuda"))
+        return [x > 2 for x in seen]
+
+    hops, cand = [False], [True]
+    assert reads(4) == hops * 3 + cand          # built, used once
+    assert reads(4) == hops * 4                 # twice the work now
+    assert reads(8) == hops * 6 + cand * 2      # again dropped too early
+    assert reads(12) == hops * 12               # four times
+    assert reads(16) == hops * 12 + cand * 4    # they pay (3 calls' work saved)
+    assert reads(4) == hops * 3 + cand
+
+
 def test_the_path_does_not_depend_on_timing():
     """Batches whose candidates suffice and batches (too sharp) whose do not, under
     one key: enqueued at once they take the paths that they take one by one."""
