@@ -3,11 +3,10 @@ another way, and leave the store as it was.  The memory is taken by ordinary
 allocations beside the store, in blocks that are given back one by one, so that
 every allocation of a call gets to fail."""
 import contextlib
+import ctypes
 
 import numpy as np
 import pytest
-
-import synth
 
 pytestmark = pytest.mark.gpu
 
@@ -15,41 +14,49 @@ MB = 1 << 20
 
 
 class _Held:
-    """All free device memory but `left` bytes, and blocks to give back."""
+    """All free device memory but `left` bytes, and blocks to give back; from the
+    driver, so that a block given back is free at once."""
 
     def __init__(self, left, blocks, size):
         import torch
         torch.cuda.synchronize()
         torch.cuda.empty_cache()
-        new = lambda b: torch.empty(b, dtype=torch.uint8, device="cuda")
-        self.blocks = [new(size) for _ in range(blocks)]
-        self.rest, part = [], 1 << 38
+        self.cuda = ctypes.CDLL("libcuda.so.1")
+        self.blocks, self.rest, part = [], [], 1 << 38
+        while len(self.blocks) < blocks:
+            self.blocks.append(self._new(size))
+            assert self.blocks[-1], "no room to begin with"
         while part >= 8 * MB:                 # the rest in pieces of a power of two
-            free = torch.cuda.mem_get_info()[0]
-            if free - left < part:
-                part >>= 1
-                continue
-            try:
-                self.rest.append(new(part))
-            except torch.OutOfMemoryError:    # no piece of that size in one
+            fits = torch.cuda.mem_get_info()[0] - left >= part
+            p = self._new(part) if fits else None
+            if p:
+                self.rest.append(p)
+            else:                             # (or no piece of that size in one)
                 part >>= 1
 
+    def _new(self, size):
+        p = ctypes.c_uint64()
+        rc = self.cuda.cuMemAlloc_v2(ctypes.byref(p), ctypes.c_size_t(size))
+        assert rc in (0, 2), rc               # CUDA_SUCCESS, CUDA_ERROR_OUT_OF_MEMORY
+        return p if rc == 0 else None
+
     def give_back(self):
-        import torch
-        self.blocks.pop()
-        torch.cuda.empty_cache()
+        assert self.cuda.cuMemFree_v2(self.blocks.pop()) == 0
+
+    def give_all(self):
+        self.blocks, rest = [], self.blocks + self.rest
+        self.rest = []
+        for p in rest:
+            assert self.cuda.cuMemFree_v2(p) == 0
 
 
 @contextlib.contextmanager
 def _memory(left, blocks=0, size=16 * MB):
-    import torch
     held = _Held(left, blocks, size)
     try:
         yield held
     finally:
-        held.blocks.clear()
-        held.rest.clear()
-        torch.cuda.empty_cache()
+        held.give_all()
 
 
 def _store(n, room, dim=64, links=32, seed=3, **kw):
